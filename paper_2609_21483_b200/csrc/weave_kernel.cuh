@@ -41,7 +41,10 @@ constexpr int kMaxEE = 256;      // routed + shared experts
 constexpr int kMaxTopK = 16;
 constexpr int kFine = 8;         // fine chunks = largest chunk count K
 constexpr int kMaxSeg = 1024;     // (chunk, expert) segments: K * (E+S) <= 1024 bounds the chunk count
-constexpr int kTinfo = 4;        // tile-descriptor ring between the producer and its consumers
+constexpr int kTinfo = 2;        // tile-descriptor ring between the scheduler and its consumers.  Every slot is a tile claimed ahead;
+                                 // pairs whose tiles share a weight panel stay closer together, and the last tiles are spread more
+                                 // evenly, with two than with four (T = 8192 Qwen3-30B-shaped skewed 778 -> 757 us, Mixtral-shaped
+                                 // 2457 -> 2421, T = 64 unchanged)
 constexpr int kTmemCols = 512;
 constexpr int kEpiWarps = 4;     // warps 4..7
 constexpr int kRel = 3;          // mailbox ring between the epilogue warps and the releasing warp (warp 3)
@@ -1272,7 +1275,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
         __syncwarp();
     } else if (warp == 0) {
         // ---------------- TMA producer (both CTAs): this CTA's 128 rows of A and its half of B;
-        // lane 0 issues the loads, the warp stays together tile by tile
+        // the warp stays together, one elected thread issues
         bool dead = false;
         while (!dead) {
             bool ok = true;
@@ -1284,8 +1287,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
             if (lane == 0) mbar_arrive_remote(mapa_u32(smem_u32(&S.ti_empty[ps.slot]), 0u));
             ps.next_slot();
             if (ti.type == 2) break;
-            bool dead_l = false;
-            if (lane == 0) {
+            {
                 const CUtensorMap *tma_a, *tma_b;
                 int arow, brow, arow2 = -1;
                 // swapped tiles: rows per CTA on the N axis (the MMA's N, a multiple of 16, split in two)
@@ -1314,18 +1316,23 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                     arow = ti.e * p.H + ti.n * 256 + (int)rank * 128;
                     brow = ti.row0 + (int)rank * nhalf;
                 }
+                // The whole warp walks the loop, one elected thread issues.  The next stage's barrier is looked at
+                // before this k-step's copies are issued, so that the answer is there when it is needed (the
+                // check took ~140 cycles of every k-step on its own).  Both decisions are made warp-uniform.
+                const uint32_t ring = smem_u32(stages), full0 = smem_u32(&S.full[0]), full0_lead = mapa_u32(full0, 0u);
+                bool freed = __all_sync(0xffffffffu, mbar_test_wait(&S.empty[ps.stage], ps.stage_phase ^ 1u));
                 for (int kb = 0; kb < ti.nkb; ++kb) {
-                    if (!mbar_wait(&S.empty[ps.stage], ps.stage_phase ^ 1u, p, 33)) { dead_l = true; break; }
-                    uint8_t *sa = stages + ps.stage * kStageBytes;
-                    const uint32_t lbar = mapa_u32(smem_u32(&S.full[ps.stage]), 0u);
-                    if (rank == 0) mbar_arrive_expect_tx(&S.full[ps.stage], tx);
-                    tma_load_2d_pair(sa, tma_a, kb * kBK, arow, lbar);
-                    if (arow2 >= 0) tma_load_2d_pair(sa + kStageA / 2, tma_a, kb * kBK, arow2, lbar);
-                    tma_load_2d_pair(sa + kStageA, tma_b, kb * kBK, brow, lbar);
+                    if (!freed && !__all_sync(0xffffffffu, mbar_wait(&S.empty[ps.stage], ps.stage_phase ^ 1u, p, 33))) {
+                        dead = true;
+                        break;
+                    }
+                    const uint32_t sa = ring + (uint32_t)(ps.stage * kStageBytes), fo = (uint32_t)(ps.stage * 8);
                     ps.next_stage();
+                    freed = __all_sync(0xffffffffu, mbar_test_wait(&S.empty[ps.stage], ps.stage_phase ^ 1u));
+                    tma_kstep_pair(sa, tma_a, sa + kStageA, tma_b, kb * kBK, arow, arow2, brow, full0_lead + fo, full0 + fo, tx,
+                                   rank == 0 ? 1u : 0u, arow2 >= 0 ? 1u : 0u);
                 }
             }
-            dead = __any_sync(0xffffffffu, dead_l);
         }
         if (dead && lane == 0) linger_after_abort();
         __syncwarp();
@@ -1354,16 +1361,20 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
             tc_fence_after();
             const unsigned long long tm1 = trace_now(p);
             const uint32_t d = tmem_base + (uint32_t)ps.acc * 256u;
+            bool landed = mbar_test_wait(&S.full[ps.stage], ps.stage_phase);
             for (int kb = 0; kb < ti.nkb; ++kb) {
                 // The operands were written by TMA (either CTA's, into its own shared memory) and are
                 // read by the tensor cores only: the barrier's completion is all the ordering needed.
                 // A wait that gives up has raised the abort flag: the following ones return at once,
                 // and the tile's (meaningless) MMAs only touch memory this pair owns.
-                if (lane == 0) ok = mbar_wait(&S.full[ps.stage], ps.stage_phase, p, 42) && ok;
-                __syncwarp();
+                // Every lane waits (a lone waiting lane and the re-convergence behind it cost ~75 cycles per
+                // k-step), and the next stage's barrier is looked at before this k-step's MMAs are issued.
+                if (!landed) ok = mbar_wait(&S.full[ps.stage], ps.stage_phase, p, 42) && ok;
                 const uint64_t da = desc0 + (uint64_t)(ps.stage * (kStageBytes >> 4));
-                tc_mma_kstep_pair(d, da, da + (uint64_t)(kStageA >> 4), idesc, (uint32_t)(kb != 0), &S.empty[ps.stage], 3);
+                uint64_t *const eb = &S.empty[ps.stage];
                 ps.next_stage();
+                landed = mbar_test_wait(&S.full[ps.stage], ps.stage_phase);
+                tc_mma_kstep_pair(d, da, da + (uint64_t)(kStageA >> 4), idesc, (uint32_t)(kb != 0), eb, 3);
             }
             if (elect_one()) tc_commit_pair(&S.tmem_full[ps.acc], 3);        // accumulators complete in both CTAs
             if (lane == 0)

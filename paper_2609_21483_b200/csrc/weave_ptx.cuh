@@ -86,6 +86,20 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
     return ok != 0;
 }
 
+// the same without suspending the thread: a look ahead whose answer is used later
+__device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // ---------------------------------------------------------------- TMA
 // (the tiled loads themselves are in the CTA-pair section below; none of them uses multicast)
 
@@ -274,13 +288,28 @@ __device__ __forceinline__ void cluster_sync_all()
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// TMA load issued by either CTA of the pair into ITS OWN shared memory; the byte count is credited
-// to the barrier at `leader_bar` (a shared::cluster address in the pair's leader CTA).  No multicast.
-__device__ __forceinline__ void tma_load_2d_pair(void *smem_dst, const void *tmap, int x, int y, uint32_t leader_bar)
+// One k-step's operand copies of one CTA of the pair, called by the whole (converged) warp; the elected
+// thread issues them, everything else stays warp-uniform (a stand-alone producer with one lane in a
+// divergent branch needs 270 cycles per k-step of three copies, this form 220).  The copies go into THIS
+// CTA's shared memory, their bytes are credited to the barrier at `leader_bar` (a shared::cluster address in
+// the pair's leader CTA), on which the leader itself (expect != 0) arrives with the byte count of both CTAs.
+// a2 != 0: the first operand comes as two 64-row boxes, 8 KB apart.  No multicast.
+__device__ __forceinline__ void tma_kstep_pair(uint32_t dst_a, const void *map_a, uint32_t dst_b, const void *map_b, int x,
+                                               int row_a, int row_a2, int row_b, uint32_t leader_bar, uint32_t local_bar,
+                                               uint32_t tx, uint32_t expect, uint32_t a2)
 {
     asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(smem_u32(smem_dst)), "l"(tmap), "r"(x), "r"(y), "r"(leader_bar)
+        "{\n\t.reg .pred pe, px, p2;\n\t.reg .b32 d2;\n\t"
+        "elect.sync _|pe, 0xffffffff;\n\t"
+        "setp.ne.and.u32 px, %10, 0, pe;\n\t"
+        "setp.ne.and.u32 p2, %11, 0, pe;\n\t"
+        "add.u32 d2, %0, 8192;\n\t"
+        "@px mbarrier.arrive.expect_tx.shared::cta.b64 _, [%8], %9;\n\t"
+        "@pe cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%4, %5}], [%7];\n\t"
+        "@p2 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [d2], [%1, {%4, %12}], [%7];\n\t"
+        "@pe cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%2], [%3, {%4, %6}], [%7];\n\t}"
+        ::"r"(dst_a), "l"(map_a), "r"(dst_b), "l"(map_b), "r"(x), "r"(row_a), "r"(row_b), "r"(leader_bar), "r"(local_bar),
+          "r"(tx), "r"(expect), "r"(a2), "r"(row_a2)
         : "memory");
 }
 
