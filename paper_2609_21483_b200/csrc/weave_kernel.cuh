@@ -61,12 +61,11 @@ enum { kModeAuto = 0, kModeFixed = 1, kModeSerial = 2 };
 struct Ctl {
     unsigned bar_count;   // grid-barrier arrivals
     unsigned q_disp;      // next dispatch tile
-    unsigned q_gemm;      // next GEMM tile (chunk-pipeline DAG order)
+    unsigned q_gemm[2];   // next GEMM tile (chunk-pipeline DAG order) of either list
     unsigned q_comb;      // next combine tile
     unsigned fix_done;    // routing blocks whose rows are final
     unsigned exit_count;
     unsigned abort;       // set by the first wait that gives up; every wait polls it
-    unsigned pad0;
     unsigned y_done[kFine];  // per chunk: epilogue-warp arrivals of finished gemm1 tiles
     unsigned q_pull;      // expert-parallel share: next block of remote tokens to stage
     unsigned pull_done;   // ... blocks staged
@@ -132,6 +131,8 @@ struct KParams {
     const float *tf;      // [n_sm+1] FLOP/us
     uint4 *trace;         // optional [n_sm][trace_cap] event records (nullptr = off)
     int trace_cap;
+    unsigned die_mask[32]; // bit smid: which half of the chip (die) the SM sits on
+    int two_dies;          // 0: not known, one list of GEMM tiles
     int4 *wait_log;       // [n_sm][8 warps]: written only by a wait that gives up or is cut short by the abort word
 };
 
@@ -183,6 +184,7 @@ struct SmemTail {
     int chunk_pt0[kFine + 1];
     int chunk_nswap[kFine];      // per chunk: segments with an odd number of m-blocks
     int chunk_tile0[kFine + 1];
+    int split_pt, split_seg;     // K = 1: pair tiles [0, split_pt) = segments [0, split_seg) are list 0, the rest list 1
     int offsets[kMaxEE + 1];
     int seg_mb0[kMaxSeg + 1];
     int seg_pt0[kMaxSeg + 1];    // prefix of pair tiles: ceil(m-blocks / 2) per segment
@@ -698,18 +700,28 @@ __device__ __forceinline__ void decode_mblock(const SmemTail &S, int EE, int mb,
 // DRAM traffic on the Mixtral-shaped layer), and alternating gemm1 with gemm0 units (+1 % at
 // I = 512, -9 % on the Qwen3-235B-shaped stack: two weight working sets in L2).
 // Host-callable so that the order can be checked without a GPU.
-__host__ __device__ __forceinline__ void decode_pair_tile(const SmemTail &S, const KParams &p, int g, TileInfo &lead,
+// With one chunk the queue is cut into two lists at an expert's boundary (split_seg), one for each half of the
+// chip, see the set-up; `list` says which one g counts in.
+__host__ __device__ __forceinline__ void decode_pair_tile(const SmemTail &S, const KParams &p, int list, int g, TileInfo &lead,
                                                           TileInfo &peer)
 {
-    int j = 0;
-    while (j + 1 < S.K && g >= S.chunk_tile0[j + 1]) ++j;
-    int local = g - S.chunk_tile0[j];
-    const int cpt0 = S.chunk_pt0[j];
-    const int nptj = S.chunk_pt0[j + 1] - cpt0;
+    int j = 0, local = g, cpt0, nptj, lo, hi;
+    if (S.K == 1) {
+        cpt0 = list ? S.split_pt : 0;
+        nptj = (list ? S.chunk_pt0[1] : S.split_pt) - cpt0;
+        lo = list ? S.split_seg : 0;
+        hi = list ? p.EE : S.split_seg;
+    } else {
+        while (j + 1 < S.K && g >= S.chunk_tile0[j + 1]) ++j;
+        local = g - S.chunk_tile0[j];
+        cpt0 = S.chunk_pt0[j];
+        nptj = S.chunk_pt0[j + 1] - cpt0;
+        lo = j * p.EE;
+        hi = lo + p.EE;
+    }
     int type = 0, nt = p.nt0;
     if (local >= nptj * p.nt0) { type = 1; local -= nptj * p.nt0; nt = p.nt1; }
-    // largest s of the chunk with (seg_pt0[s] - cpt0) * nt <= local (empty segments share a start)
-    int lo = j * p.EE, hi = (j + 1) * p.EE;
+    // largest s of the list with (seg_pt0[s] - cpt0) * nt <= local (empty segments share a start)
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
         if ((S.seg_pt0[mid] - cpt0) * nt <= local) lo = mid; else hi = mid;
@@ -1207,7 +1219,7 @@ __device__ __forceinline__ void staged_store_32(const uint32_t (&o)[16], uint32_
 // budget = how many pair tiles this CTA pair may claim (the steal count for a movement pair).
 // Called by both CTAs of a pair with the same arguments.
 __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_t *stages, uint32_t tmem_base,
-                                           const TmaMaps *tm, int budget, PipeState &ps)
+                                           const TmaMaps *tm, int budget, int die, PipeState &ps)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_ctarank();      // 0 = leader (issues the MMAs), 1 = peer
@@ -1220,13 +1232,28 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
         // kTinfo tiles ahead of the MMAs, so claim and flag latencies stay off the critical path.
         if (lane == 0) {
             int taken = 0;
-            int g_next = (budget > 0 || S.elastic) ? (int)atomicAdd(&p.ctl->q_gemm, 1u) : 0x7fffffff;
+            // this die's list first; when it has run out, the other one's.  A tile waits only for tiles before it in
+            // its own list and for the dispatch, so of all claimed tiles the one claimed first can always proceed.
+            const int per_pt = p.nt0 + p.nt1;
+            const int n_list0 = S.K == 1 ? S.split_pt * per_pt : S.n_gemm;
+            int list = n_list0 == S.n_gemm ? 0 : die;
+            bool second = false;
+            auto claim = [&]() -> int {
+                for (;;) {
+                    const int c = (int)atomicAdd(&p.ctl->q_gemm[list], 1u);
+                    if (c < (list ? S.n_gemm - n_list0 : n_list0)) return c;
+                    if (second) return 0x7fffffff;
+                    second = true;
+                    list ^= 1;
+                }
+            };
+            int g_next = (budget > 0 || S.elastic) ? claim() : 0x7fffffff;
             for (;;) {
                 const int g = g_next;
                 const unsigned long long tp0 = trace_now(p);
                 TileInfo tl, tp;
                 if (g >= S.n_gemm) { tl.type = tp.type = 2; tl.mb = tp.mb = -1; tl.nrows = tp.nrows = 0; }
-                else decode_pair_tile(S, p, g, tl, tp);
+                else decode_pair_tile(S, p, list, g, tl, tp);
                 if (!mbar_wait(&S.ti_empty[ps.slot], ps.slot_phase ^ 1u, p, 30)) break;
                 S.ti[ps.slot] = tl;
                 {
@@ -1248,7 +1275,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                             more = ld_acquire_u32(&p.ctl->y_done[ch]) < y_done_target(S, p, ch);
                         }
                     }
-                    g_next = more ? (int)atomicAdd(&p.ctl->q_gemm, 1u) : 0x7fffffff;
+                    g_next = more ? claim() : 0x7fffffff;
                     bool ok;
                     const bool two = tp.mb != tl.mb;         // a regular pair tile has two m-blocks
                     if (tl.type == 0 || tl.type == 3) {
@@ -1699,6 +1726,9 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
     float cm_bw = 0.f, cm_tf = 0.f, cm_bw_n = 0.f, cm_tf_n = 0.f;
     if (cm_ok) { cm_bw = p.bw[cm_c]; cm_tf = p.tf[n_sm - cm_c]; }
     if (p.mode == kModeAuto) { cm_bw_n = p.bw[n_sm]; cm_tf_n = p.tf[n_sm]; }
+    unsigned smid;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+    const int die = p.two_dies && smid < 1024u ? (int)((p.die_mask[smid >> 5] >> (smid & 31u)) & 1u) : 0;
     const int P = p.T * (p.k + p.S);
     // Eq. 1-3 (single-GPU reading: every pair moves through HBM)
     const float B = (float)(2 * p.H);
@@ -1894,7 +1924,20 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
                 S.seg_row0[j * EE + tid] = run_row;
                 S.seg_rows[j * EE + tid] = rows;
             }
+            // One chunk: the two lists meet at the expert boundary nearest to half of the pair tiles.  Each half of the
+            // chip has an L2 of its own that caches what its SMs read, wherever it lives; with whole experts on one
+            // half, a weight panel and the expert's rows cross to the other half once instead of being fetched by
+            // both (under the power cap every byte moved costs time: Mixtral-shaped T = 4096 2421 -> 2362 us,
+            // Qwen3-30B-shaped T = 8192 skewed 778 -> 760; no difference where nothing is shared, T = 64).
+            if (K == 1 && tid < EE && p.two_dies) {
+                const int mypt = (mbs + 1) >> 1, before = ptot - 2 * pex, after = 2 * (pex + mypt) - ptot;
+                if (before >= 0 && after > 0) {
+                    S.split_pt = before <= after ? pex : pex + mypt;
+                    S.split_seg = before <= after ? tid : tid + 1;
+                }
+            }
             if (tid == 0) {
+                if (K > 1 || !p.two_dies || ptot == 0) { S.split_pt = ptot; S.split_seg = EE; }
                 S.chunk_mb0[j] = mb_base;
                 S.chunk_pt0[j] = pt_base;
                 S.chunk_tile0[j] = pt_base * (p.nt0 + p.nt1);
@@ -2004,7 +2047,7 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         if (dmax > 0) dispatch_phase(p, S, stages, dmax, n_disp, p.nblk <= kLocalBlocks);
         if (serial) alive = grid_barrier(p, S, bar0 + (unsigned)n_sm, 2);
         const int budget = (mover && plan_kind != kPlanPhased) ? plan_steal : 0x7fffffff;
-        if (alive && (budget > 0 || S.elastic)) gemm_phase(p, S, stages, tmem_base, &tm, budget, ps);
+        if (alive && (budget > 0 || S.elastic)) gemm_phase(p, S, stages, tmem_base, &tm, budget, die, ps);
         if (serial) alive = alive && grid_barrier(p, S, bar0 + 2u * (unsigned)n_sm, 3);
         if (alive) combine_phase(p, S, stages);
     }
@@ -2029,6 +2072,30 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         for (int i = tid; i < p.nmb_max; i += kThreads) { p.xe_ready[i] = 0u; p.h_ready[i] = 0u; }
         unsigned *z = reinterpret_cast<unsigned *>(p.ctl);
         if (tid < kCtlZeroWords) z[tid] = 0u;
+    }
+}
+
+// ------------------------------------------------------------------------------------ which half an SM sits on
+
+// One warp per SM: the shortest of kDieTries round trips of an atomic on each of kDieLines lines.  An atomic is done
+// in the L2 that the line belongs to: 320-410 cycles from the SMs of that half of the chip, 690-810 from the
+// others (148 SMs, idle chip), whereas loads take the same time from both once either side has cached them.
+constexpr int kDieLines = 8, kDieTries = 6, kMaxSm = 1024;
+__global__ void __launch_bounds__(32, 1) weave_die_probe_kernel(unsigned *lines, int stride_words, unsigned *out)
+{
+    unsigned smid;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+    if (threadIdx.x != 0 || smid >= (unsigned)kMaxSm) return;
+    for (int a = 0; a < kDieLines; ++a) {
+        unsigned best = 0xFFFFFFFFu;
+        for (int r = 0; r < kDieTries; ++r) {
+            const long long t0 = clock64();
+            const unsigned v = atomicAdd(lines + a * stride_words, 0u);      // (the lines hold zeros)
+            if (v != 0u) out[smid * kDieLines + a] = v;      // never taken: holds the second reading back until the value is here
+            const long long t1 = clock64();
+            if (r > 0) best = min(best, (unsigned)(t1 - t0));
+        }
+        out[smid * kDieLines + a] = best;
     }
 }
 

@@ -4,6 +4,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -115,6 +116,8 @@ struct weave_moe {
     void *trace;
     int trace_cap;
     int ep_rank, ep_size;
+    unsigned die_mask[32];      // see find_dies()
+    int two_dies;
     // pipelined host path: copy streams and per-slot events, created on first use
     bool pipe_ready;
     unsigned long long pipe_calls;
@@ -178,6 +181,48 @@ void default_tables(int n_sm, std::vector<float> &bw, std::vector<float> &tf)
     }
     bw[0] = bw[1];
     tf[0] = tf[1];
+}
+
+// Which half of the chip each SM sits on, from the latencies of weave_die_probe_kernel: on every line the SMs fall
+// into a near and a far group with a wide gap between them, and all lines have to agree on the grouping.  Returns
+// 1 and the mask (bit smid), or 0 (no such grouping: one list of GEMM tiles serves the whole chip).  `scratch`: at
+// least 64 KB of zeroed device memory, left with the latencies in its first half.
+int find_dies(int n_sm, uint8_t *scratch, unsigned (&mask)[32])
+{
+    memset(mask, 0, sizeof(mask));
+    const int smem = 120 * 1024;      // one block per SM
+    if (cudaFuncSetAttribute(weave_die_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 0;
+    unsigned *out = reinterpret_cast<unsigned *>(scratch);
+    weave_die_probe_kernel<<<n_sm, 32, smem>>>(reinterpret_cast<unsigned *>(scratch + kMaxSm * kDieLines * 4), 1024, out);
+    std::vector<unsigned> lat((size_t)kMaxSm * kDieLines);
+    if (cudaGetLastError() != cudaSuccess ||
+        cudaMemcpy(lat.data(), out, lat.size() * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
+        return 0;
+    std::vector<int> sms;
+    for (int i = 0; i < kMaxSm; ++i)
+        if (lat[(size_t)i * kDieLines]) sms.push_back(i);
+    const int n = (int)sms.size();
+    if (n < 8) return 0;
+    std::vector<int> votes(n, 0);
+    int lines = 0;
+    for (int a = 0; a < kDieLines; ++a) {
+        std::vector<unsigned> v;
+        for (int i : sms) v.push_back(lat[(size_t)i * kDieLines + a]);
+        std::sort(v.begin(), v.end());
+        int cut = n / 4;      // the widest gap with at least a quarter of the SMs on either side
+        for (int i = n / 4; i < n - n / 4; ++i)
+            if (v[i] - v[i - 1] > v[cut] - v[cut - 1]) cut = i;
+        if (5 * (v[cut] - v[cut - 1]) < v[0]) continue;
+        ++lines;
+        const bool first = lat[(size_t)sms[0] * kDieLines + a] >= v[cut];
+        for (int i = 0; i < n; ++i) votes[i] += ((lat[(size_t)sms[i] * kDieLines + a] >= v[cut]) != first) ? 1 : -1;
+    }
+    if (lines < kDieLines / 2) return 0;
+    for (int i = 0; i < n; ++i) {
+        if (votes[i] != lines && votes[i] != -lines) return 0;
+        if (votes[i] > 0) mask[sms[i] >> 5] |= 1u << (sms[i] & 31);
+    }
+    return 1;
 }
 
 int upload_tables(weave_moe *h, const float *bw, const float *tf)
@@ -284,6 +329,10 @@ int weave_moe_create(const weave_moe_config *cfg, weave_moe_t *out)
 
     e = cudaMemset(h->ws, 0, L.zero_end);
     if (e != cudaSuccess) { int rc = cuda_fail(h, e); delete h; return rc; }
+    static_assert(sizeof(int4) * kWaitLogSlots >= 64 * 1024, "the probe borrows the wait log");
+    h->two_dies = find_dies(prop.multiProcessorCount, h->ws + L.wait_log, h->die_mask);
+    e = cudaMemset(h->ws + L.wait_log, 0, sizeof(int4) * kWaitLogSlots);
+    if (e != cudaSuccess) { int rc = cuda_fail(h, e); delete h; return rc; }
     std::vector<float> bw, tf;
     default_tables(h->n_sm, bw, tf);
     int rc = upload_tables(h, bw.data(), tf.data());
@@ -348,6 +397,8 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     p.trace = reinterpret_cast<uint4 *>(h->trace);
     p.trace_cap = h->trace_cap;
     p.wait_log = reinterpret_cast<int4 *>(ws + L.wait_log);
+    memcpy(p.die_mask, h->die_mask, sizeof(p.die_mask));
+    p.two_dies = h->two_dies;
 
     void *args[] = {&p, &h->tm};
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -692,10 +743,11 @@ int weave_moe_debug_gemm_queue(const int32_t *rows, int num_segments, int num_ch
     S.seg_mb0[num_chunks * num_segments] = mb; S.seg_pt0[num_chunks * num_segments] = pt;
     S.chunk_mb0[num_chunks] = mb; S.chunk_pt0[num_chunks] = pt; S.chunk_tile0[num_chunks] = pt * (nt0 + nt1);
     S.K = num_chunks;
+    S.split_pt = pt; S.split_seg = num_segments;      // (one list: the order inside either of two is this one's)
     const int n = pt * (nt0 + nt1);
     for (int g = 0; g < n && g < max_tiles && out; ++g) {
         TileInfo tl, tp;
-        decode_pair_tile(S, p, g, tl, tp);
+        decode_pair_tile(S, p, 0, g, tl, tp);
         int32_t *o = out + (size_t)g * 6;
         o[0] = tl.type; o[1] = tl.mb; o[2] = tl.type >= 3 ? -1 : tp.mb; o[3] = tl.n; o[4] = tl.chunk; o[5] = tl.nrows;
     }
@@ -727,6 +779,8 @@ struct StaticDevice {
     const float *tables;  // device address of g_static_tables on this device
     size_t usable;
     int n_sm;
+    unsigned die_mask[32];
+    int two_dies;
     EncodeTiledFn encode;
 };
 constexpr int kMaxDevices = 64;
@@ -765,6 +819,8 @@ int static_setup(int dev, StaticDevice **out)
         if (cudaFuncSetAttribute(weave_moe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) !=
             cudaSuccess)
             return WEAVE_ERR_CUDA;
+        if (cudaMemset(d.base, 0, 64 * 1024) != cudaSuccess) return WEAVE_ERR_CUDA;
+        d.two_dies = find_dies(prop.multiProcessorCount, d.base, d.die_mask);
         void *fnp = nullptr;
         cudaDriverEntryPointQueryResult qres;
         if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fnp, cudaEnableDefault, &qres) != cudaSuccess || !fnp ||
@@ -824,6 +880,8 @@ int weave_moe_forward_static(int hidden, int ffn, int num_experts, int top_k, in
     h.elastic = -1;
     h.bw_dev = sd->tables;
     h.tf_dev = sd->tables + 1024;
+    memcpy(h.die_mask, sd->die_mask, sizeof(h.die_mask));
+    h.two_dies = sd->two_dies;
     const int EE = num_experts + num_shared;
     int r = 0;
     r = encode_maps(sd->encode, &h.tm, h.ws + L.xe, h.ws + L.hbuf, gate_up, down, (uint64_t)L.p_max, (uint64_t)EE,

@@ -530,3 +530,24 @@ def test_small_batches_on_both_sides_of_the_every_cta_routing_limit(T, sched):
     s = {"auto": None, "serial": (pk.SCHED_SERIAL, 0, 1, 0), "fixed_k2": (pk.SCHED_FIXED, 24, 2, 3)}[sched]
     moe, _, _ = run_case(cfg, sched=s)
     moe.close()
+
+
+@pytest.mark.parametrize("rows", ["one_expert", "first_heavy", "last_heavy", "two_equal", "one_row_each"])
+@pytest.mark.parametrize("ffn", [128, 384])
+def test_load_distributions_around_the_cut_between_the_two_tile_lists(rows, ffn):
+    """The GEMM queue of one chunk is cut at an expert's boundary near half of its tiles.  Loads that put
+    the cut at either end (one list empty), behind a heavy expert, between equals and among one-row experts;
+    k = 1 and crafted logits, whole output against the oracle, the same bits with chunks (one list)."""
+    E = 16
+    T = {"one_expert": 300, "first_heavy": 700, "last_heavy": 700, "two_equal": 512, "one_row_each": E}[rows]
+    cfg = _small(f"cut_{rows}_{ffn}", T, 256, ffn, E, 1, cfg_id=950)
+    want = {"one_expert": np.full(T, 5), "first_heavy": np.where(np.arange(T) < 600, 0, np.arange(T) % E),
+            "last_heavy": np.where(np.arange(T) < 600, E - 1, np.arange(T) % E), "two_equal": np.arange(T) % 2 + 7,
+            "one_row_each": np.arange(T)}[rows]
+    inp = wl.make_inputs(cfg)
+    inp.logits[np.arange(T), want] = 50.0
+    dev = to_dev(inp)
+    moe, out, _ = run_case(cfg, inp=inp, dev_tensors=dev)
+    _, chunked, _ = run_case(cfg, sched=(pk.SCHED_FIXED, 20, 2, 1), inp=inp, dev_tensors=dev, moe=moe)
+    assert torch.equal(out.view(torch.int16), chunked.view(torch.int16))
+    moe.close()
