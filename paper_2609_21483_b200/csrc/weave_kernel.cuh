@@ -786,7 +786,7 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
     const unsigned long long *lmask = local_route ? reinterpret_cast<const unsigned long long *>(stages + kStages * kStageBytes) : nullptr;
     MoveScratch &M = move_scratch(stages);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    fence_proxy_async();      // the buffers held routing scratch written with ordinary stores
+    fence_proxy_async_shared();      // the buffers held routing scratch written with ordinary stores
     __syncthreads();
     const uint32_t rowb = (uint32_t)p.H * 2u;
     const int R = max(1, kMvBuf / (int)rowb);     // rows per buffer
@@ -994,7 +994,7 @@ __device__ __forceinline__ void combine_phase(const KParams &p, SmemTail &S, uin
 {
     MoveScratch &M = move_scratch(stages);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    fence_proxy_async();
+    fence_proxy_async_shared();
     __syncthreads();
     const int kk = p.k + p.S;
     const int W = min(p.H, ((kMvBuf / (2 * kk)) / 64) * 64);     // columns per piece (128-byte multiple)
@@ -1223,7 +1223,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_ctarank();      // 0 = leader (issues the MMAs), 1 = peer
-    fence_proxy_async();     // the stage buffers were last touched by ordinary stores (routing scratch)
+    fence_proxy_async_shared();     // the stage buffers were last touched by ordinary stores (routing scratch)
     __syncthreads();
 
     if (warp == 2 && rank == 0) {
@@ -1263,19 +1263,6 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                     for (int w = 0; w < (int)(sizeof(TileInfo) / 4); ++w) st_cluster_u32(dst + 4 * w, src[w]);
                 }
                 if (tl.type != 2) {
-                    ++taken;
-                    bool more = taken < budget;
-                    if (!more && S.elastic) {
-                        // the steal quota is used up: keep taking GEMM tiles for as long as the next
-                        // combine chunk has not been produced yet (nothing else to do meanwhile)
-                        const unsigned qc = ld_relaxed_u32(&p.ctl->q_comb);
-                        if (qc >= (unsigned)S.n_comb) more = true;
-                        else {
-                            const int ch = ((((int)qc * S.comb_tok / kRouteBlock) * kFine) / p.nblk) / (kFine / S.K);
-                            more = ld_acquire_u32(&p.ctl->y_done[ch]) < y_done_target(S, p, ch);
-                        }
-                    }
-                    g_next = more ? claim() : 0x7fffffff;
                     bool ok;
                     const bool two = tp.mb != tl.mb;         // a regular pair tile has two m-blocks
                     if (tl.type == 0 || tl.type == 3) {
@@ -1297,6 +1284,20 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 mbar_arrive_cluster(mapa_u32(smem_u32(&S.ti_full[ps.slot]), 1u));
                 ps.next_slot();
                 if (tl.type == 2) break;
+                // the next claim's round trip (or two, where one list has run out) comes after the hand-over
+                ++taken;
+                bool more = taken < budget;
+                if (!more && S.elastic) {
+                    // the steal quota is used up: keep taking GEMM tiles for as long as the next
+                    // combine chunk has not been produced yet (nothing else to do meanwhile)
+                    const unsigned qc = ld_relaxed_u32(&p.ctl->q_comb);
+                    if (qc >= (unsigned)S.n_comb) more = true;
+                    else {
+                        const int ch = ((((int)qc * S.comb_tok / kRouteBlock) * kFine) / p.nblk) / (kFine / S.K);
+                        more = ld_acquire_u32(&p.ctl->y_done[ch]) < y_done_target(S, p, ch);
+                    }
+                }
+                g_next = more ? claim() : 0x7fffffff;
             }
         }
         __syncwarp();

@@ -49,9 +49,11 @@ __device__ __forceinline__ unsigned atom_acqrel_add_u32(unsigned *p, unsigned v)
 
 // generic-proxy writes (st.global by any SM, made visible through a flag) -> async-proxy reads
 // (TMA) and back
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
-// the same restricted to global memory (about a third of the full fence's ~1900 cycles): for hand-overs of rows in
-// global memory between ordinary stores or bulk stores on one SM and tensor-map loads on another
+// (restricted to one state space: the unrestricted fence takes ~1900 cycles)
+// shared memory: for stage buffers that were last touched by ordinary stores and are filled by bulk or tensor copies next
+__device__ __forceinline__ void fence_proxy_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// global memory (about a third of the full fence): for hand-overs of rows in global memory between ordinary stores or
+// bulk stores on one SM and tensor-map loads on another
 __device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
 // ---------------------------------------------------------------- mbarrier

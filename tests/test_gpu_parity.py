@@ -551,3 +551,22 @@ def test_load_distributions_around_the_cut_between_the_two_tile_lists(rows, ffn)
     _, chunked, _ = run_case(cfg, sched=(pk.SCHED_FIXED, 20, 2, 1), inp=inp, dev_tensors=dev, moe=moe)
     assert torch.equal(out.view(torch.int16), chunked.view(torch.int16))
     moe.close()
+
+
+@pytest.mark.parametrize("T", [1, 8, 9, 16, 17, 32, 33, 48, 49, 64])
+@pytest.mark.parametrize("E,k,S", [(4, 1, 0), (5, 5, 1), (130, 8, 2), (256, 16, 0)])
+def test_batches_whose_gate_up_tiles_read_x_itself(T, E, k, S):
+    """One routing block under the phased plan: the gate/up tiles multiply all tokens and keep the expert's
+    rows, routing uses 32, 16, 8 or 4 threads per token.  T around each of those limits and around the row
+    boxes of 8, 16 and 32; experts below and above a warp's width, odd counts; whole output against the oracle,
+    and the dispatched rows are still written."""
+    cfg = _small(f"direct_T{T}_E{E}", T, 256, 256, E, k, S, cfg_id=960 + E)
+    inp = wl.make_inputs(cfg)
+    dev = to_dev(inp)
+    moe, out, _ = run_case(cfg, inp=inp, dev_tensors=dev)
+    assert moe.plan()["kind"] == pk.PLAN_PHASED
+    xe, tok = moe.intermediates(T)["xe"].view(torch.int16), moe.routing(T)["token_of"].long()
+    assert torch.equal(xe, dev[0].view(torch.int16)[tok])
+    _, serial, _ = run_case(cfg, sched=(pk.SCHED_SERIAL, 0, 1, 0), inp=inp, dev_tensors=dev, moe=moe)
+    assert torch.equal(out.view(torch.int16), serial.view(torch.int16))
+    moe.close()
