@@ -94,7 +94,8 @@ enum { kPlanSplit = 0, kPlanDispatchAll = 1, kPlanPhased = 2, kPlanRejoin = 3 };
 
 struct KParams {
     int T, H, I, E, S, k, EE;
-    int nblk;             // routing blocks = ceil(T / 64)
+    int nblk;             // 64-token blocks = ceil(T / 64): the unit of the chunks, of small batches and of the expert-parallel share
+    int lg_rb, nrb;       // routing blocks of 1 << lg_rb tokens: 64, or 32 or 16 (8) where that gives no more blocks than CTAs
     int mode, fixed_c, fixed_K, fixed_steal;
     int nt0, nt1;         // n-tiles per m-block: I / 128, ceil(H / 256)
     int nmb_max;          // allocated length of the per-m-block flag arrays
@@ -115,7 +116,7 @@ struct KParams {
     __nv_bfloat16 *out;
     Ctl *ctl;
     unsigned *fcnt;       // [8][256] rows per (fine chunk, expert); zero at entry
-    int *hist;            // [nblk][256]
+    int *hist;            // [nrb][256]; shares its place with y, whose rows are written long after the last look at it
     int *topk_idx;        // [T][k]
     float *gates;         // [T][k]
     int *row_of;          // [T][k]
@@ -341,11 +342,8 @@ __device__ __forceinline__ unsigned long long block_excl_scan_packed(unsigned lo
 // the two halves of a grid barrier, for a caller that has work to do between arriving and waiting
 __device__ __forceinline__ void grid_barrier_arrive(const KParams &p)
 {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        red_release_add_u32(&p.ctl->bar_count, 1u);
-    }
+    __syncthreads();      // (the release is cumulative: it covers what the other threads wrote before the block barrier)
+    if (threadIdx.x == 0) red_release_add_u32(&p.ctl->bar_count, 1u);
 }
 __device__ __forceinline__ bool grid_barrier_wait(const KParams &p, SmemTail &S, unsigned target, int where)
 {
@@ -357,7 +355,6 @@ __device__ __forceinline__ bool grid_barrier(const KParams &p, SmemTail &S, unsi
 {
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
         red_release_add_u32(&p.ctl->bar_count, 1u);
         S.bcast[2] = flag_wait_ge(&p.ctl->bar_count, target, p, where) ? 1 : 0;
     }
@@ -419,17 +416,17 @@ __device__ __forceinline__ int route_row_stride(int E) { return ((E + 27) / 32) 
 __device__ __forceinline__ void stage_logits_issue(const KParams &p, int b, float *lg_s)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int ntok = min(kRouteBlock, p.T - b * kRouteBlock);
+    const int t0 = b << p.lg_rb, ntok = min(1 << p.lg_rb, p.T - t0);
     const int stride = route_row_stride(p.E);
     if ((p.E & 3) == 0) {      // rows are 16-byte multiples: both sides of every copy are 16-byte aligned
         const int per_row = p.E >> 2;
         for (int i = threadIdx.x; i < ntok * per_row; i += kThreads) {
             const int r = i / per_row, c = (i - r * per_row) << 2;
-            cp_async_16(smem_u32(lg_s + r * stride + c), p.logits + (size_t)(b * kRouteBlock + r) * p.E + c);
+            cp_async_16(smem_u32(lg_s + r * stride + c), p.logits + (size_t)(t0 + r) * p.E + c);
         }
     } else {
         for (int r = warp; r < ntok; r += kThreads / 32) {
-            const float *src = p.logits + (size_t)(b * kRouteBlock + r) * p.E;
+            const float *src = p.logits + (size_t)(t0 + r) * p.E;
             for (int c = lane; c < p.E; c += 32) cp_async_4(smem_u32(lg_s + r * stride + c), src + c);
         }
     }
@@ -452,18 +449,22 @@ __device__ __forceinline__ void stage_logits_issue(const KParams &p, int b, floa
 // that is not inlined sees generic pointers, and generic atomics that land in shared memory take a slow
 // path); inlined it is 1-3 us per layer faster on the small batches.
 struct RouteArgs {
-    int T, E, k, ep_size, ep_rank, ep_tshard;
+    int lg_rb, T, E, k, ep_size, ep_rank, ep_tshard;
     int *status;
     int *topk_idx;
     float *gates;
 };
-__device__ __forceinline__ void route_block_quads(int T, int E, int k, int ep_size, int ep_rank, int ep_tshard, int *status,
+// kQuad: 64-token blocks, four threads per token.  Otherwise 32, 16 or 8 tokens with 8, 16 or 32 threads each: a thread
+// then goes through E / 8 to E / 32 experts instead of E / 4 (routing of a block, staging included: E = 256, k = 8, T = 1023 12.5 -> 7.4 us, E = 128, T = 1 7.8 -> 5.8).
+template <bool kQuad>
+__device__ __forceinline__ void route_block(int lg_rb, int T, int E, int k, int ep_size, int ep_rank, int ep_tshard, int *status,
                                                int *topk_idx, float *gates, int b, uint32_t lg_s, uint32_t r_mask,
                                                uint32_t r_idx, uint32_t r_cnt, uint32_t r_p, bool write_out)
 {
-    static_assert(kThreads == 4 * kRouteBlock, "four threads per token of a routing block");
-    const int tl = threadIdx.x >> 2, q = threadIdx.x & 3;
-    const int t = b * kRouteBlock + tl;
+    static_assert(kThreads == 4 * kRouteBlock, "four threads per token of a 64-token routing block");
+    const int lg = kQuad ? 2 : 8 - lg_rb, G = 1 << lg;      // G threads per token
+    const int tl = threadIdx.x >> lg, q = threadIdx.x & (G - 1);
+    const int t = (b << (kQuad ? 6 : lg_rb)) + tl;
     const bool valid = t < T;
     const int e_lo = ep_size > 1 ? ep_rank * (E / ep_size) : 0;
     const int e_hi = ep_size > 1 ? e_lo + E / ep_size : E;
@@ -475,7 +476,7 @@ __device__ __forceinline__ void route_block_quads(int T, int E, int k, int ep_si
     int be = 0x7fffffff;      // expert of this thread's best key
     bool bad = false;
 #pragma unroll 2
-    for (int e = q; e < E; e += 4) {
+    for (int e = q; e < E; e += G) {
         float x = ld_shared_f32(row + 4u * (uint32_t)e);
         const bool nf = !(fabsf(x) <= 3.402823466e38f);      // NaN or +-inf: flag it, keep indices in range
         bad = bad || (valid && nf);
@@ -492,8 +493,8 @@ __device__ __forceinline__ void route_block_quads(int T, int E, int k, int ep_si
     for (int j = 0; j < k; ++j) {
         unsigned hk = bk;
         int hi = bk ? be : 0x7fffffff;
-#pragma unroll
-        for (int o = 1; o <= 2; o <<= 1) {
+#pragma unroll kQuad ? 2 : 1
+        for (int o = 1; o < G; o <<= 1) {
             const unsigned ok = __shfl_xor_sync(0xffffffffu, hk, o);
             const int oi = __shfl_xor_sync(0xffffffffu, hi, o);
             if (ok > hk || (ok == hk && oi < hi)) { hk = ok; hi = oi; }
@@ -507,7 +508,7 @@ __device__ __forceinline__ void route_block_quads(int T, int E, int k, int ep_si
         // all k selected experts
         const bool local = hi >= e_lo && hi < e_hi;
         nloc += local ? 1 : 0;
-        if (valid && (j & 3) == q) {
+        if (valid && (j & (G - 1)) == q) {
             st_shared_u32(r_p + 4u * (uint32_t)(tl * kMaxTopK + j), __float_as_uint(pj));
             if (write_out) {
                 topk_idx[(size_t)t * k + j] = hi;
@@ -516,11 +517,11 @@ __device__ __forceinline__ void route_block_quads(int T, int E, int k, int ep_si
             if (local) red_shared_or_u32(r_mask + 8u * (uint32_t)hi + 4u * (uint32_t)(tl >> 5), 1u << (tl & 31));
         }
         // the owner takes its winner out and looks for its next best
-        if ((hi & 3) == q && hk != 0u) {
+        if ((hi & (G - 1)) == q && hk != 0u) {
             st_shared_u32(row + 4u * (uint32_t)hi, 0u);
             bk = 0u; be = 0x7fffffff;
 #pragma unroll 4
-            for (int e = q; e < E; e += 4) {
+            for (int e = q; e < E; e += G) {
                 const unsigned c = ld_shared_u32(row + 4u * (uint32_t)e);
                 if (c > bk) { bk = c; be = e; }
             }
@@ -529,7 +530,7 @@ __device__ __forceinline__ void route_block_quads(int T, int E, int k, int ep_si
     __syncwarp();
     if (valid) {
         if (write_out)
-            for (int j = q; j < k; j += 4)
+            for (int j = q; j < k; j += G)
                 gates[(size_t)t * k + j] = __fdiv_rn(__uint_as_float(ld_shared_u32(r_p + 4u * (uint32_t)(tl * kMaxTopK + j))), sum);
         if (ep_size > 1 && q == 0 && nloc) {
             if (t / ep_tshard == ep_rank) red_shared_add_u32(r_cnt, (uint32_t)nloc);
@@ -795,7 +796,7 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
         int b = 0;
         uint32_t ph = 0;
         bool ok = true;
-        if (lane == 0 && lmask == nullptr) ok = flag_wait_ge(&p.ctl->fix_done, (unsigned)p.nblk, p, 10);
+        if (lane == 0 && lmask == nullptr) ok = flag_wait_ge(&p.ctl->fix_done, (unsigned)p.nrb, p, 10);
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (p.ep_size > 1) {
             // expert-parallel share: first every remote token that has an expert here is copied ONCE
@@ -1017,7 +1018,7 @@ __device__ __forceinline__ void combine_phase(const KParams &p, SmemTail &S, uin
             // the tile's rows and gates are final once the permutation is; they are fetched before the wait for
             // the chunk's last GEMM tile, so that only the row copies themselves follow that wait
             if (!perm_final) {
-                if (lane == 0) ok = flag_wait_ge(&p.ctl->fix_done, (unsigned)p.nblk, p, 20);
+                if (lane == 0) ok = flag_wait_ge(&p.ctl->fix_done, (unsigned)p.nrb, p, 20);
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok) break;
                 perm_final = true;
@@ -1667,7 +1668,7 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
     float *lg_s = reinterpret_cast<float *>(stages + 2048 + kLocalBlocks * kRouteBlock * kMaxTopK * 4);   // [64][route_row_stride(E)]
     {
         const int b_first = p.nblk <= kLocalBlocks ? 0 : (int)blockIdx.x;
-        if (b_first < p.nblk) stage_logits_issue(p, b_first, lg_s);
+        if (b_first < p.nrb) stage_logits_issue(p, b_first, lg_s);
     }
 
     if (tid == 0) {
@@ -1740,7 +1741,7 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
     ma.alpha = p.alpha; ma.eff[0] = p.eff[0]; ma.eff[1] = p.eff[1]; ma.eff[2] = p.eff[2]; ma.eff[3] = p.eff[3];
     ma.kinds = p.kinds; ma.c_min = p.c_min; ma.c_step = p.c_step;
     RouteArgs ra;
-    ra.T = p.T; ra.E = p.E; ra.k = p.k; ra.ep_size = p.ep_size; ra.ep_rank = p.ep_rank; ra.ep_tshard = p.ep_tshard;
+    ra.lg_rb = p.lg_rb; ra.T = p.T; ra.E = p.E; ra.k = p.k; ra.ep_size = p.ep_size; ra.ep_rank = p.ep_rank; ra.ep_tshard = p.ep_tshard;
     ra.status = &p.ctl->status; ra.topk_idx = p.topk_idx; ra.gates = p.gates;
     PlanPick pick;
     pick.c = n_sm; pick.ki = 0; pick.kind = kPlanSplit; pick.t = 0.f;
@@ -1749,7 +1750,7 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
     // ================= phase R: routing
     for (int it = 0;; ++it) {
         const int b = local_route ? it : (int)blockIdx.x + it * n_sm;
-        if (b >= p.nblk) break;
+        if (b >= p.nrb) break;
         const int slot = local_route ? b : 0;
         unsigned long long *r_mask = lmask + slot * (kMaxEE + 1);
         const bool writer = !local_route || b == (int)blockIdx.x;
@@ -1766,20 +1767,21 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         {
             const uint32_t a0 = smem_u32(lg_s), a1 = smem_u32(r_mask), a2 = smem_u32(idx_b), a3 = smem_u32(r_cnt + 2 * slot),
                            a4 = smem_u32(r_p);
-            route_block_quads(ra.T, ra.E, ra.k, ra.ep_size, ra.ep_rank, ra.ep_tshard, ra.status, ra.topk_idx, ra.gates, b, a0, a1, a2, a3, a4, writer);
+            if (ra.lg_rb == 6)
+                route_block<true>(6, ra.T, ra.E, ra.k, ra.ep_size, ra.ep_rank, ra.ep_tshard, ra.status, ra.topk_idx, ra.gates, b, a0, a1, a2, a3, a4, writer);
+            else
+                route_block<false>(ra.lg_rb, ra.T, ra.E, ra.k, ra.ep_size, ra.ep_rank, ra.ep_tshard, ra.status, ra.topk_idx, ra.gates, b, a0, a1, a2, a3, a4, writer);
         }
         __syncthreads();
-        if (p.nblk > n_sm) {
+        if (p.nrb > n_sm) {
             // this CTA routes several blocks and its scratch is reused: the in-block rank of each (token,
             // slot) - tokens before it in the block that chose the same expert - goes out to global memory
-            for (int pi = tid; pi < kRouteBlock * p.k; pi += kThreads) {
-                const int tl = pi / p.k, j = pi - tl * p.k;
-                const int t = b * kRouteBlock + tl;
-                if (t < p.T) {
+            const int tl = tid >> 2, t = b * kRouteBlock + tl;      // (64-token blocks then)
+            if (t < p.T)
+                for (int j = tid & 3; j < p.k; j += 4) {
                     const int e = idx_b[tl * kMaxTopK + j];     // -1: the expert lives on another rank
                     p.row_of[(size_t)t * p.k + j] = e >= 0 ? __popcll(r_mask[e] & ((1ull << tl) - 1ull)) : -1;
                 }
-            }
         }
         if (ep && writer && tid == 0) p.uniq_mask[b] = r_mask[kMaxEE];
         if (!local_route) {
@@ -1789,8 +1791,8 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
                 if (r_cnt[1]) atomicAdd(&p.ctl->x_in, (unsigned)r_cnt[1]);
                 if (um) atomicAdd(&p.ctl->x_in_uniq, (unsigned)__popcll(um));
             }
-            const int ntok = min(kRouteBlock, p.T - b * kRouteBlock);
-            const int f = (b * kFine) / p.nblk;
+            const int ntok = min(1 << p.lg_rb, p.T - (b << p.lg_rb));
+            const int f = ((b >> (6 - p.lg_rb)) * kFine) / p.nblk;
             for (int e = tid; e < EE; e += kThreads) {
                 const int cnt = e < p.E ? __popcll(r_mask[e]) : ntok;
                 p.hist[(size_t)b * kMaxEE + e] = cnt;
@@ -1978,8 +1980,8 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
     // ================= permutation fix-up: in-block rank + rows of earlier blocks + expert offset
     if (alive) {
         int fixed = 0;
-        const bool from_smem = p.nblk <= n_sm;      // this CTA's block is still in its shared memory
-        for (int b = blockIdx.x; b < p.nblk; b += n_sm) {
+        const bool from_smem = p.nrb <= n_sm;      // this CTA's block is still in its shared memory
+        for (int b = blockIdx.x; b < p.nrb; b += n_sm) {
             const int slot = local_route ? b : 0;
             const unsigned long long *r_mask = lmask + slot * (kMaxEE + 1);
             const int *idx_b = r_idx + slot * kRouteBlock * kMaxTopK;
@@ -1988,43 +1990,37 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
                 if (local_route) {
                     for (int bb = 0; bb < b; ++bb) base += __popcll(lmask[bb * (kMaxEE + 1) + tid]);
                 } else {
-                    const int f = (b * kFine) / p.nblk;
-                    const int bstart = (f * p.nblk + kFine - 1) / kFine;
+                    const int f = ((b >> (6 - p.lg_rb)) * kFine) / p.nblk;
+                    const int bstart = ((f * p.nblk + kFine - 1) / kFine) << (6 - p.lg_rb);
 #pragma unroll
                     for (int ff = 0; ff < kFine; ++ff) if (ff < f) base += cf[ff];
+#pragma unroll 4
                     for (int bb = bstart; bb < b; ++bb) base += __ldcg(p.hist + (size_t)bb * kMaxEE + tid);
                 }
                 r_base[tid] = base;
             }
             __syncthreads();
-            for (int pi = tid; pi < kRouteBlock * p.k; pi += kThreads) {
-                const int tl = pi / p.k, j = pi - tl * p.k;
-                const int t = b * kRouteBlock + tl;
-                if (t < p.T) {
-                    const int e = from_smem ? idx_b[tl * kMaxTopK + j] : __ldcg(p.topk_idx + (size_t)t * p.k + j);
-                    const int rk = from_smem ? (e >= 0 ? __popcll(r_mask[e] & ((1ull << tl) - 1ull)) : -1)
-                                             : __ldcg(p.row_of + (size_t)t * p.k + j);
+            // the threads that routed a token place its rows (no divisions: this stands between routing and dispatch)
+            const int lg = 8 - p.lg_rb, tl = tid >> lg, t = (b << p.lg_rb) + tl;
+            if (t < p.T) {
+                for (int j = tid & ((1 << lg) - 1); j < p.k; j += 1 << lg) {
+                    const size_t at = (size_t)t * p.k + j;
+                    const int e = from_smem ? idx_b[tl * kMaxTopK + j] : __ldcg(p.topk_idx + at);
+                    const int rk = from_smem ? (e >= 0 ? __popcll(r_mask[e] & ((1ull << tl) - 1ull)) : -1) : __ldcg(p.row_of + at);
                     if (rk >= 0) {
                         const int r = rk + r_base[e];
-                        p.row_of[(size_t)t * p.k + j] = r;
+                        p.row_of[at] = r;
                         p.token_of[r] = t;
                     } else if (from_smem) {
-                        p.row_of[(size_t)t * p.k + j] = -1;
+                        p.row_of[at] = -1;
                     }
                 }
-            }
-            for (int pi = tid; pi < kRouteBlock * p.S; pi += kThreads) {
-                const int tl = pi / p.S, s = pi - tl * p.S;
-                const int t = b * kRouteBlock + tl;
-                if (t < p.T) p.token_of[S.offsets[p.E + s] + t] = t;
+                for (int s = tid & ((1 << lg) - 1); s < p.S; s += 1 << lg) p.token_of[S.offsets[p.E + s] + t] = t;
             }
             __syncthreads();
             ++fixed;
         }
-        if (tid == 0 && fixed) {
-            __threadfence();
-            red_release_add_u32(&p.ctl->fix_done, (unsigned)fixed);
-        }
+        if (tid == 0 && fixed) red_release_add_u32(&p.ctl->fix_done, (unsigned)fixed);
     }
 
     if (tid == 0) trace_ev(p, S, kEvFixup, 0u, tk3, trace_now(p), 0u);
@@ -2063,7 +2059,6 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         if (p.trace)     // last record of the CTA's slice: how many events were written
             p.trace[(size_t)blockIdx.x * p.trace_cap + p.trace_cap - 1] =
                 make_uint4(min(S.trace_n, (unsigned)p.trace_cap - 1u), 0u, 0u, 0u);
-        __threadfence();
         S.bcast[0] = atom_acqrel_add_u32(&p.ctl->exit_count, 1u) == (unsigned)(n_sm - 1) ? 1 : 0;
     }
     __syncthreads();

@@ -358,6 +358,13 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     p.T = T; p.H = c.hidden; p.I = c.ffn; p.E = c.num_experts; p.S = c.num_shared; p.k = c.top_k;
     p.EE = c.num_experts + c.num_shared;
     p.nblk = (T + kRouteBlock - 1) / kRouteBlock;
+    // Routing blocks of 16 or 32 tokens, with 16 or 8 threads per token, while each still has a CTA to itself (an
+    // expert-parallel share stages its remote tokens by 64).  A batch of at most 64 tokens is one block, routed by every
+    // CTA for itself, with as many threads per token as there are.
+    p.lg_rb = 6;
+    if (p.nblk <= kLocalBlocks) p.lg_rb = T <= 8 ? 3 : T <= 16 ? 4 : T <= 32 ? 5 : 6;
+    else if (h->ep_size == 1) p.lg_rb = T <= 16 * h->n_cta ? 4 : T <= 32 * h->n_cta ? 5 : 6;
+    p.nrb = (T + (1 << p.lg_rb) - 1) >> p.lg_rb;
     p.mode = h->mode; p.fixed_c = h->fixed_c; p.fixed_K = h->fixed_K; p.fixed_steal = h->fixed_steal;
     p.nt0 = c.ffn / kTN0;
     p.nt1 = (c.hidden + 255) / 256;
@@ -375,7 +382,7 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     uint8_t *ws = h->ws;
     p.ctl = reinterpret_cast<Ctl *>(ws + L.ctl);
     p.fcnt = reinterpret_cast<unsigned *>(ws + L.fcnt);
-    p.hist = reinterpret_cast<int *>(ws + L.hist);
+    p.hist = reinterpret_cast<int *>(ws + L.y);      // at most 64 bytes per token, a row of y has at least 256
     p.topk_idx = reinterpret_cast<int *>(ws + L.topk);
     p.gates = reinterpret_cast<float *>(ws + L.gates);
     p.row_of = reinterpret_cast<int *>(ws + L.row_of);

@@ -570,3 +570,18 @@ def test_batches_whose_gate_up_tiles_read_x_itself(T, E, k, S):
     _, serial, _ = run_case(cfg, sched=(pk.SCHED_SERIAL, 0, 1, 0), inp=inp, dev_tensors=dev, moe=moe)
     assert torch.equal(out.view(torch.int16), serial.view(torch.int16))
     moe.close()
+
+
+@pytest.mark.parametrize("T", [1, 8, 9, 16, 17, 32, 33, 65, 80, 2367, 2368, 2369, 4737])
+@pytest.mark.parametrize("E,k,S", [(4, 1, 0), (5, 5, 1), (130, 8, 2), (256, 16, 0)])
+def test_routing_blocks_of_every_size(T, E, k, S):
+    """Routing blocks of 8, 16, 32 and 64 tokens (32 to 4 threads per token): T around the limits between them and
+    around whole blocks, experts fewer than a token's threads, odd counts, k up to the limit.  Routing, counts,
+    offsets and permutation bit for bit, outputs on a sample; the same with two chunks."""
+    cfg = _small(f"rb_T{T}_E{E}", T, 128, 128, E, k, S, cfg_id=970 + E)
+    inp = wl.make_inputs(cfg)
+    dev = to_dev(inp)
+    moe, out, _ = run_case(cfg, inp=inp, dev_tensors=dev, n_sample=None if T < 100 else 16, budget=64)
+    _, chunked, _ = run_case(cfg, sched=(pk.SCHED_FIXED, 20, 2, 1), inp=inp, dev_tensors=dev, moe=moe, n_sample=4, budget=16)
+    assert torch.equal(out.view(torch.int16), chunked.view(torch.int16))
+    moe.close()
