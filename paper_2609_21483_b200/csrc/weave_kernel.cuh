@@ -32,10 +32,11 @@ constexpr int kStages = 6;
 constexpr int kStageA = kBM * kBK * 2;                  // 16 KB: this CTA's 128 rows of A
 constexpr int kStageB = 128 * kBK * 2;                  // 16 KB: this CTA's half (128 rows) of the 256-row B tile
 constexpr int kStageBytes = kStageA + kStageB;          // 32 KB
-constexpr int kEpiStageBytes = 4 * 2 * 32 * 64;         // epilogue staging: per warp two buffers of 32 rows x 64 bytes
+constexpr int kEpiStageBytes = 4 * 4096;                // epilogue staging, per warp: 32 rows x 64 bytes, and two 1 KB exchange buffers
 constexpr int kRouteBlock = 64;  // tokens per routing block (one 64-bit mask per expert)
 constexpr int kLocalBlocks = 1;  // a batch of at most this many routing blocks is routed by every CTA for itself
                                  // (measured at two blocks: routing both in every CTA costs more than the grid barrier saves)
+constexpr int kDirectTokens = 32; // largest batch whose gate/up tiles read x itself
 constexpr int kCombTile = 16;    // tokens per combine tile (fewer when the batch would give fewer tiles than SMs)
 constexpr int kMaxEE = 256;      // routed + shared experts
 constexpr int kMaxTopK = 16;
@@ -106,6 +107,7 @@ struct KParams {
     unsigned long long *uniq_mask;   // [nblk] remote tokens of the block that have a local expert
     int elastic_steal;    // movement pairs keep stealing past their quota while no combine chunk is ready
     int kinds;            // bit mask of the plan kinds the cost model may choose (bit kPlanSplit, ...)
+    int direct;           // the gate/up tiles may read x itself (T <= kDirectTokens, see the kernel body); tm.x is set
     int withhold_mb;      // test hook: this m-block's "dispatched" flag is never published (-1 = off)
     int c_min, c_max, c_step;
     float alpha;
@@ -166,7 +168,7 @@ struct SmemTail {
     uint64_t ti_full[kTinfo], ti_empty[kTinfo];
     uint64_t dv_full[kStages], dv_empty[kStages];   // dispatch: loader -> storer ring over the stage buffers
     uint64_t cb_full[kStages], cb_empty[kStages];   // combine: loader -> reducing warps
-    uint64_t xg_full, xg_empty;                     // swapped gemm0 epilogue: up warps -> gate warps
+    uint64_t xg[2];                                 // swapped gemm0 epilogue: a gate and an up warp trade values
     uint64_t rel_full[kRel], rel_empty[kRel];       // epilogue warps -> releasing warp: a tile's stores are issued
     unsigned *rel_flag[kRel];                       // the ready counter that tile arrives on, and by how much
     unsigned rel_cnt[kRel];
@@ -203,6 +205,7 @@ struct MoveScratch {
 };
 static_assert(sizeof(MoveScratch) <= kEpiStageBytes / 2, "movement scratch must fit half of the staging area");
 static_assert(kLocalBlocks * (kMaxEE + 1) * 8 <= kEpiStageBytes / 2, "the routing masks must fit the other half");
+static_assert(kLocalBlocks * kMaxEE * 8 <= 2048, "the masks that the direct gate/up tiles read end below the first exchange buffer");
 static_assert(kFine == 8, "chunk of a fine chunk = f >> (3 - log2 K)");
 __device__ __forceinline__ MoveScratch &move_scratch(uint8_t *stages)
 {
@@ -470,6 +473,7 @@ __device__ __forceinline__ void route_block(int lg_rb, int T, int E, int k, int 
     const int e_hi = ep_size > 1 ? e_lo + E / ep_size : E;
     const uint32_t row = lg_s + 4u * (uint32_t)(tl * route_row_stride(E));      // this token's logits, then keys
 
+    if (!__any_sync(0xffffffffu, valid)) return;      // (a warp without a token)
     // keys: 0 = nothing there; every finite logit maps to a key >= 1 that orders like the float
     // (a token past the end keeps all-zero keys: its quad then selects nothing and writes nothing)
     unsigned bk = 0u;
@@ -493,11 +497,17 @@ __device__ __forceinline__ void route_block(int lg_rb, int T, int E, int k, int 
     for (int j = 0; j < k; ++j) {
         unsigned hk = bk;
         int hi = bk ? be : 0x7fffffff;
+        if (!kQuad && lg == 5) {      // a whole warp per token: two reductions in hardware
+            const unsigned top = __reduce_max_sync(0xffffffffu, hk);
+            hi = (int)__reduce_min_sync(0xffffffffu, hk == top ? (unsigned)hi : 0x7fffffffu);
+            hk = top;
+        } else {
 #pragma unroll kQuad ? 2 : 1
-        for (int o = 1; o < G; o <<= 1) {
-            const unsigned ok = __shfl_xor_sync(0xffffffffu, hk, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, hi, o);
-            if (ok > hk || (ok == hk && oi < hi)) { hk = ok; hi = oi; }
+            for (int o = 1; o < G; o <<= 1) {
+                const unsigned ok = __shfl_xor_sync(0xffffffffu, hk, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, hi, o);
+                if (ok > hk || (ok == hk && oi < hi)) { hk = ok; hi = oi; }
+            }
         }
         // every thread of the quad knows slot j now; thread j mod 4 writes it down
         const float v = float_from_order_key(hk);
@@ -1128,7 +1138,8 @@ __device__ __forceinline__ void combine_phase(const KParams &p, SmemTail &S, uin
 // Tensor maps of the GEMM operands: bf16 matrices, boxes of 64 columns (one 128-byte swizzle row) by
 // 128 rows (64 rows for the gate and up halves of a swapped tile's weight operand; 8, 16, 32 or 64
 // rows for a swapped tile's row operand, whichever covers its half of the m-block's rows).
-struct TmaMaps { CUtensorMap xe, wgu, h, wd, wgu64, xe_n[4], h_n[4]; };
+// x: the input itself, boxes of half the batch's tokens rounded up to 8 or 16 (only where KParams::direct is set).
+struct TmaMaps { CUtensorMap xe, wgu, h, wd, wgu64, xe_n[4], h_n[4], x; };
 
 struct PipeState {     // per-role ring positions; they persist across the tiles of a phase
     int stage = 0;  uint32_t stage_phase = 0;
@@ -1218,9 +1229,10 @@ __device__ __forceinline__ void staged_store_32(const uint32_t (&o)[16], uint32_
 }
 
 // budget = how many pair tiles this CTA pair may claim (the steal count for a movement pair).
-// Called by both CTAs of a pair with the same arguments.
+// Called by both CTAs of a pair with the same arguments.  direct: the gate/up tiles take the batch's tokens themselves
+// as their row operand (all tiles are swapped ones then).
 __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_t *stages, uint32_t tmem_base,
-                                           const TmaMaps *tm, int budget, int die, PipeState &ps)
+                                           const TmaMaps *tm, int budget, int die, bool direct, PipeState &ps)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_ctarank();      // 0 = leader (issues the MMAs), 1 = peer
@@ -1266,7 +1278,9 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 if (tl.type != 2) {
                     bool ok;
                     const bool two = tp.mb != tl.mb;         // a regular pair tile has two m-blocks
-                    if (tl.type == 0 || tl.type == 3) {
+                    if (direct && tl.type == 3) {
+                        ok = true;               // x was there before the launch
+                    } else if (tl.type == 0 || tl.type == 3) {
                         ok = flag_wait_ge(&p.xe_ready[tl.mb], 1u, p, 31);
                         if (ok && two) ok = flag_wait_ge(&p.xe_ready[tp.mb], 1u, p, 31);
                     } else {
@@ -1278,14 +1292,14 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                     // the tile's input rows may have been written with ordinary stores on other SMs and
                     // are read by TMA next: the cross-proxy fence sits here, after the acquire and before
                     // the hand-over to the producers, off their critical path
-                    fence_proxy_async_global();
+                    if (!(direct && tl.type == 3)) fence_proxy_async_global();
                     trace_ev(p, S, kEvGemmLoad, (unsigned)g, tp0, trace_now(p), 0u);
                 }
                 mbar_arrive(&S.ti_full[ps.slot]);
                 mbar_arrive_cluster(mapa_u32(smem_u32(&S.ti_full[ps.slot]), 1u));
                 ps.next_slot();
                 if (tl.type == 2) break;
-                // the next claim's round trip (or two, where one list has run out) comes after the hand-over
+                // the next claim's round trip comes after the hand-over
                 ++taken;
                 bool more = taken < budget;
                 if (!more && S.elastic) {
@@ -1320,7 +1334,8 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 const CUtensorMap *tma_a, *tma_b;
                 int arow, brow, arow2 = -1;
                 // swapped tiles: rows per CTA on the N axis (the MMA's N, a multiple of 16, split in two)
-                const int nhalf = (((ti.nrows + 15) >> 4) << 4) >> 1;
+                const bool from_x = direct && ti.type == 3;
+                const int nhalf = ((((from_x ? p.T : ti.nrows) + 15) >> 4) << 4) >> 1;
                 // ... fetched with the smallest box that covers them (the copy engine takes in a fixed
                 // number of rows per cycle, so rows nobody reads cost as much as the others)
                 const int bi = nhalf <= 8 ? 0 : nhalf <= 16 ? 1 : nhalf <= 32 ? 2 : 3;
@@ -1339,6 +1354,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                     arow = ti.e * 2 * p.I + ti.n * kTN0 + (int)rank * 64;
                     arow2 = arow + p.I;
                     brow = ti.row0 + (int)rank * nhalf;
+                    if (from_x) { tma_b = &tm->x; brow = (int)rank * nhalf; }
                 } else {                     // M axis: this CTA's 128 of the n-tile's 256 out-columns
                     tma_a = &tm->wd; tma_b = &tm->h_n[bi];
                     tx = 2u * (kStageA + (1024u << bi));
@@ -1382,7 +1398,8 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
             ps.next_slot();
             if (ti.type == 2) break;
             // regular tiles: 256 rows x 256 columns; swapped tiles: 256 weight rows x (rows rounded up to 16)
-            const uint32_t idesc = umma_idesc_bf16(2 * kBM, ti.type >= 3 ? (uint32_t)(((ti.nrows + 15) >> 4) << 4) : 256u);
+            const int n_op = direct && ti.type == 3 ? p.T : ti.nrows;
+            const uint32_t idesc = umma_idesc_bf16(2 * kBM, ti.type >= 3 ? (uint32_t)(((n_op + 15) >> 4) << 4) : 256u);
             // timeline record of this tile: extra = time spent waiting for a free accumulator (ns)
             const unsigned long long tm0 = trace_now(p);
             if (lane == 0) ok = mbar_wait_cluster(&S.tmem_empty[ps.acc], ps.acc_phase ^ 1u, p, 41);
@@ -1455,78 +1472,98 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
             const int rows_valid = ti.nrows - q * 32;          // rows of this warp's quadrant that exist
             const uint32_t epi_stage = smem_u32(stages + kStages * kStageBytes) + (uint32_t)q * 4096u;   // this warp's staging (2 x 2 KB)
             bool acc_released = false;
+            auto release_acc = [&]() {       // the tile's last TMEM load has landed: the accumulator goes back to the issuer
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_remote(mapa_u32(smem_u32(&S.tmem_empty[ps.acc]), 0u));
+                acc_released = true;
+            };
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)ps.acc * 256u;
             if (ti.type == 3) {
-                // swapped gemm0: lanes 0..63 hold the gate projection of this CTA's 64 h-columns, lanes
-                // 64..127 the up projection; TMEM columns are the m-block's rows.  The up warps hand
-                // their values to the gate warps through the staging buffer, 16 rows at a time.
-                // each up warp (q = 2, 3) writes into its OWN 2 KB staging region, [32][16] fp32, and gate
-                // warp q - 2 reads it; a warp's region is never written by anybody else, so a warp that
-                // is still busy with the previous tile cannot be overrun
-                const uint32_t xs = smem_u32(stages + kStages * kStageBytes) + (uint32_t)(2 + (q & 1)) * 4096u;
+                // swapped gemm0: lanes 0..63 hold the gate projection of this CTA's 64 h-columns, lanes 64..127 the up
+                // projection; TMEM columns are the m-block's rows.  Gate warp q and up warp q + 2 trade halves of every
+                // 16 rows through shared memory, 1 KB each way: the gate warp finishes rows 0..7, the up warp rows
+                // 8..15.  Each warp writes only its own two buffers (the upper half of its staging area), in turn; it
+                // fills one again two batches later, after a barrier at which the partner arrived with the older
+                // batch's values already used in stores.
+                // (With the gate warps alone doing the arithmetic and the stores 64 rows took 5.5 us.)
+                //
+                // direct: TMEM columns are the batch's tokens, and the expert's rows are those with a bit in its mask.
+                const int up = q >> 1;
+                const uint32_t xbase = smem_u32(stages + kStages * kStageBytes) + 2048u + (uint32_t)lane * 16u;
+                const uint32_t xmine = xbase + (uint32_t)q * 4096u, xtheirs = xbase + (uint32_t)(q ^ 2) * 4096u;
+                uint64_t *const xbar = &S.xg[q & 1];
                 const int col = ti.n * kTN0 + (int)rank * 64 + (q & 1) * 32 + lane;      // this thread's h-column
-                const int nch = (ti.nrows + 15) >> 4;
-                for (int c = 0; c < nch && !dead; ++c) {
-                    uint32_t v[16];
-                    tmem_ld_32x16(taddr + c * 16, v);
-                    tmem_ld_wait16(v);
-                    if (q >= 2) {
-                        if (!mbar_wait(&S.xg_empty, xg_phase ^ 1u, p, 52)) dead = true;
+                const int ncol = direct ? p.T : ti.nrows;
+                unsigned long long sel = ~0ull;                  // direct: the tokens of this expert
+                if (direct) {
+                    sel = (2ull << (p.T - 1)) - 1ull;
+                    if (ti.e < p.E) sel = *reinterpret_cast<const unsigned long long *>(stages + kStages * kStageBytes + 8 * ti.e);
+                }
+                for (int c0 = 0; c0 < ncol && !dead; c0 += 32) {
+                    uint32_t v[32];
+                    tmem_ld_32x32(taddr + c0, v);
+                    tmem_ld_wait32(v);
+                    if (c0 + 32 >= ncol) release_acc();
+#pragma unroll
+                    for (int b = 0; b < 2; ++b) {
+                        const int c = c0 + 16 * b;
+                        if (c >= ncol || (direct && ((sel >> c) & 0xFFFFull) == 0ull)) continue;      // (the same for both warps)
+                        const uint32_t xo = xg_phase ? 1024u : 0u;
+                        if (up) {
+                            st_shared_v4(xmine + xo, make_uint4(v[16 * b], v[16 * b + 1], v[16 * b + 2], v[16 * b + 3]));
+                            st_shared_v4(xmine + xo + 512u, make_uint4(v[16 * b + 4], v[16 * b + 5], v[16 * b + 6], v[16 * b + 7]));
+                        } else {
+                            st_shared_v4(xmine + xo, make_uint4(v[16 * b + 8], v[16 * b + 9], v[16 * b + 10], v[16 * b + 11]));
+                            st_shared_v4(xmine + xo + 512u, make_uint4(v[16 * b + 12], v[16 * b + 13], v[16 * b + 14], v[16 * b + 15]));
+                        }
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(xbar);
+                        if (!mbar_wait(xbar, xg_phase, p, 53)) dead = true;
                         dead = __any_sync(0xffffffffu, dead);
                         if (dead) break;
+                        xg_phase ^= 1u;
+                        const uint4 t0 = ld_shared_v4(xtheirs + xo), t1 = ld_shared_v4(xtheirs + xo + 512u);
+                        const uint32_t o[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+                        // this warp's eight rows of the batch, as bits (warp-uniform: a row that is not there costs a branch)
+                        const int r0 = c + 8 * up;
+                        unsigned rows8 = (unsigned)(sel >> r0) & 0xFFu;
+                        if (!direct) rows8 = ncol - r0 >= 8 ? 0xFFu : (1u << max(0, ncol - r0)) - 1u;
+                        const int first = direct ? __popcll(sel & ((1ull << r0) - 1ull)) : r0;
+                        __nv_bfloat16 *dst = p.hbuf + (size_t)(ti.row0 + first) * p.I + col;
+                        __nv_bfloat16 hv[8];
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            st_shared_v4(xs + (uint32_t)(lane * 64 + i * 16),
-                                         make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&S.xg_full);
-                    } else {
-                        if (!mbar_wait(&S.xg_full, xg_phase, p, 53)) dead = true;
-                        dead = __any_sync(0xffffffffu, dead);
-                        if (dead) break;
-                        uint32_t u[16];
+                        for (int i = 0; i < 8; ++i)
+                            hv[i] = __float2bfloat16_rn(silu_mul(__uint_as_float(up ? o[i] : v[16 * b + i]), __uint_as_float(up ? v[16 * b + 8 + i] : o[i])));
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const uint4 t4 = ld_shared_v4(xs + (uint32_t)(lane * 64 + i * 16));
-                            u[4 * i] = t4.x; u[4 * i + 1] = t4.y; u[4 * i + 2] = t4.z; u[4 * i + 3] = t4.w;
-                        }
-                        // the four vector loads have landed before the region is handed back to the up warp
-                        // (see tile_info_landed: the values are not used until after the arrival)
-                        *reinterpret_cast<volatile int *>(&S.scan_w[warp]) = (int)(u[0] ^ u[4] ^ u[8] ^ u[12]);
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&S.xg_empty);
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const int tok = c * 16 + j;
-                            if (tok < ti.nrows)
-                                p.hbuf[(size_t)(ti.row0 + tok) * p.I + col] =
-                                    __float2bfloat16_rn(silu_mul(__uint_as_float(v[j]), __uint_as_float(u[j])));
-                        }
+                        for (int i = 0; i < 8; ++i)
+                            if ((rows8 >> i) & 1u) {
+                                *dst = hv[i];
+                                dst += p.I;
+                            }
+                        // (values that no row used have to land all the same before the partner fills the buffer again)
+                        *reinterpret_cast<volatile int *>(&S.scan_w[warp]) = (int)(o[0] ^ o[4]);
                     }
-                    xg_phase ^= 1u;
                 }
                 if (dead) break;
-                // an up warp may reuse its staging region in the next tile only after the gate warps
-                // have read the last chunk
-                if (q >= 2) {
-                    if (!mbar_wait(&S.xg_empty, xg_phase ^ 1u, p, 54)) dead = true;
-                    dead = __any_sync(0xffffffffu, dead);
-                    if (dead) break;
-                }
             } else if (ti.type == 4) {
                 // swapped gemm1: lane = one of this CTA's 128 out-columns, TMEM columns = the m-block's rows
-                const int col = ti.n * 256 + (int)rank * 128 + q * 32 + lane;
-                const int nch = (ti.nrows + 15) >> 4;
                 if (ti.n * 256 + (int)rank * 128 < p.H) {
-                    for (int c = 0; c < nch; ++c) {
-                        uint32_t v[16];
-                        tmem_ld_32x16(taddr + c * 16, v);
-                        tmem_ld_wait16(v);
+                    __nv_bfloat16 *dst = p.y + (size_t)ti.row0 * p.H + ti.n * 256 + (int)rank * 128 + q * 32 + lane;
+                    for (int c0 = 0; c0 < ti.nrows; c0 += 32) {
+                        uint32_t v[32];
+                        tmem_ld_32x32(taddr + c0, v);
+                        tmem_ld_wait32(v);
+                        if (c0 + 32 >= ti.nrows) release_acc();
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const int tok = c * 16 + j;
-                            if (tok < ti.nrows)
-                                p.y[(size_t)(ti.row0 + tok) * p.H + col] = __float2bfloat16_rn(__uint_as_float(v[j]));
+                        for (int g = 0; g < 4; ++g) {
+                            if (c0 + 8 * g >= ti.nrows) break;
+                            __nv_bfloat16 *dg = dst + (size_t)(c0 + 8 * g) * p.H;
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                if (c0 + 8 * g + j < ti.nrows) *dg = __float2bfloat16_rn(__uint_as_float(v[8 * g + j]));
+                                dg += p.H;
+                            }
                         }
                     }
                 }
@@ -1549,10 +1586,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                             tmem_ld_32x32(taddr + (c + 1) * 32, gr[(c + 1) & 1]);
                             tmem_ld_32x32(taddr + 128 + (c + 1) * 32, ur[(c + 1) & 1]);
                         } else {
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive_remote(mapa_u32(smem_u32(&S.tmem_empty[ps.acc]), 0u));
-                            acc_released = true;
+                            release_acc();
                         }
 #pragma unroll
                         for (int i = 0; i < 16; ++i)
@@ -1578,12 +1612,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                                 tmem_ld_wait64(ar[0]);
                                 reg_fence64(ar[1]);
                             }
-                            if (c + 2 >= nb && !acc_released) {      // every load of the tile has landed
-                                tc_fence_before();
-                                __syncwarp();
-                                if (lane == 0) mbar_arrive_remote(mapa_u32(smem_u32(&S.tmem_empty[ps.acc]), 0u));
-                                acc_released = true;
-                            }
+                            if (c + 2 >= nb && !acc_released) release_acc();      // every load of the tile has landed
 #pragma unroll
                             for (int hh = 0; hh < 2; ++hh) {
 #pragma unroll
@@ -1608,8 +1637,8 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 if (q == 0) trace_ev(p, S, kEvGemmEpi, (unsigned)(ti.mb & 0xFFFFFF), te0, trace_now(p),
                                      (unsigned)(ti.type << 16 | (int)min(65535ull, te1 - te0)));
             }
-            // a swapped gemm0 tile is stored by the two gate warps of each CTA (4 arrivals per m-block
-            // and n-tile over the pair, like a regular tile); a swapped gemm1 tile by all 8 warps
+            // 4 arrivals per m-block and gemm0 n-tile: from the m-block's own CTA of a regular tile, 2 from each CTA of
+            // a swapped one; a swapped gemm1 tile makes 4 from each CTA (see y_done_target)
             const bool g0 = ti.type == 0 || ti.type == 3;
             if (!post(g0 ? &p.h_ready[ti.mb] : &p.ctl->y_done[ti.chunk], ti.type == 3 ? 2u : (unsigned)kEpiWarps)) dead = true;
             ps.next_acc();
@@ -1618,6 +1647,29 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
         // ---------------- releasing warp (both CTAs): makes the tiles' arrivals on the ready counters
         int rs = 0;
         uint32_t rph = 0;
+        if (direct) {
+            // nothing reads the dispatched rows here, but the caller may ask for them: token t's row of x goes to its
+            // rows of Xe, the token's experts spread over `parts` CTAs
+            const unsigned long long *mask = reinterpret_cast<const unsigned long long *>(stages + kStages * kStageBytes);
+            const int parts = max(1, (int)gridDim.x / p.T), vecs = p.H >> 3;
+            for (int w = blockIdx.x; w < p.T * parts; w += gridDim.x) {
+                const int t = w % p.T;
+                int n = 0;
+                for (int e0 = 0; e0 < p.EE; e0 += 32) {
+                    const int e = e0 + lane;
+                    unsigned mine = __ballot_sync(0xffffffffu, e < p.EE && (e >= p.E || ((mask[e] >> t) & 1ull)));
+                    for (; mine; mine &= mine - 1u, ++n) {
+                        if (n % parts != w / p.T) continue;
+                        const int es = e0 + __ffs((int)mine) - 1;
+                        const int r = S.offsets[es] + (es < p.E ? __popcll(mask[es] & ((1ull << t) - 1ull)) : t);
+                        const uint4 *src = reinterpret_cast<const uint4 *>(p.x + (size_t)t * p.H);
+                        uint4 *dst = reinterpret_cast<uint4 *>(p.xe + (size_t)r * p.H);
+#pragma unroll 4
+                        for (int i = lane; i < vecs; i += 32) dst[i] = __ldg(src + i);
+                    }
+                }
+            }
+        }
         while (true) {
             if (!mbar_wait(&S.rel_full[rs], rph, p, 57)) break;
             unsigned *flag = S.rel_flag[rs];
@@ -1685,12 +1737,13 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         // tile descriptor consumed: leader's producer + MMA + 4 epilogue warps, peer's producer + 4 warps
 #pragma unroll 1
         for (int i = 0; i < kTinfo; ++i) { mbar_init(&S.ti_full[i], 1); mbar_init(&S.ti_empty[i], 3 + 2 * kEpiWarps); }
-        mbar_init(&S.xg_full, 2); mbar_init(&S.xg_empty, 2);
+        mbar_init(&S.xg[0], 2); mbar_init(&S.xg[1], 2);
 #pragma unroll 1
         for (int i = 0; i < kRel; ++i) { mbar_init(&S.rel_full[i], kEpiWarps); mbar_init(&S.rel_empty[i], 1); }
         fence_mbar_init();
         tma_prefetch_desc(&tm.xe); tma_prefetch_desc(&tm.wgu); tma_prefetch_desc(&tm.h); tma_prefetch_desc(&tm.wd);
         tma_prefetch_desc(&tm.wgu64);
+        if (p.direct) tma_prefetch_desc(&tm.x);
 #pragma unroll 1
         for (int i = 0; i < 4; ++i) { tma_prefetch_desc(&tm.xe_n[i]); tma_prefetch_desc(&tm.h_n[i]); }
     }
@@ -2041,10 +2094,18 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         const bool two_roles = plan_kind == kPlanSplit || plan_kind == kPlanRejoin;
         const int dmax = (mover || !two_roles) ? 0x7fffffff : (S.elastic ? 1 : 0);
         const int n_disp = (!two_roles || S.elastic) ? n_sm : plan_c;       // who dispatches at all
-        if (dmax > 0) dispatch_phase(p, S, stages, dmax, n_disp, p.nblk <= kLocalBlocks);
+        // A batch of at most 32 tokens under the phased plan: N = T columns cost a swapped tile's MMA no more than the
+        // expert's few rows do (an instruction takes 48 cycles up to N = 64, and the weights set the pace), so the
+        // gate/up tiles multiply ALL tokens, straight from x, and their epilogue keeps the expert's rows.  Nothing waits
+        // for a dispatch then (4-5 us); the GEMM phase's releasing warps write Xe, for whoever asks for it, before
+        // they have tiles to release.  T = 1 Qwen3-30B-shaped 46.8 -> 40.3 us, T = 7 DSv2-Lite-shaped 119.1 -> 112.7,
+        // T = 27 149.4 -> 146.7.  At T = 64 a launch by itself gains as much (199.9 -> 197.8) but under load the
+        // additional columns and rows cost power (202.8 -> 205.9 after half a second): hence the limit.
+        const bool direct = p.direct && plan_kind == kPlanPhased;
+        if (dmax > 0 && !direct) dispatch_phase(p, S, stages, dmax, n_disp, p.nblk <= kLocalBlocks);
         if (serial) alive = grid_barrier(p, S, bar0 + (unsigned)n_sm, 2);
         const int budget = (mover && plan_kind != kPlanPhased) ? plan_steal : 0x7fffffff;
-        if (alive && (budget > 0 || S.elastic)) gemm_phase(p, S, stages, tmem_base, &tm, budget, die, ps);
+        if (alive && (budget > 0 || S.elastic)) gemm_phase(p, S, stages, tmem_base, &tm, budget, die, direct, ps);
         if (serial) alive = alive && grid_barrier(p, S, bar0 + 2u * (unsigned)n_sm, 3);
         if (alive) combine_phase(p, S, stages);
     }

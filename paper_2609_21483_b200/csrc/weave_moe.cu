@@ -124,6 +124,7 @@ struct weave_moe {
     cudaStream_t pipe_h2d, pipe_d2h;
     cudaEvent_t pipe_in_ready[2], pipe_k_done[2], pipe_out_done[2];
     TmaMaps tm;
+    EncodeTiledFn encode;
 };
 
 namespace {
@@ -326,6 +327,7 @@ int weave_moe_create(const weave_moe_config *cfg, weave_moe_t *out)
     r = encode_maps(enc, &h->tm, h->ws + L.xe, h->ws + L.hbuf, cfg->gate_up, cfg->down, (uint64_t)L.p_max, (uint64_t)EE,
                     (uint64_t)cfg->hidden, (uint64_t)cfg->ffn);
     if (r) { h->last_cuda_error = r; delete h; return WEAVE_ERR_CUDA; }
+    h->encode = enc;
 
     e = cudaMemset(h->ws, 0, L.zero_end);
     if (e != cudaSuccess) { int rc = cuda_fail(h, e); delete h; return rc; }
@@ -406,6 +408,16 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     p.wait_log = reinterpret_cast<int4 *>(ws + L.wait_log);
     memcpy(p.die_mask, h->die_mask, sizeof(p.die_mask));
     p.two_dies = h->two_dies;
+
+    // A small batch under AUTO: its gate/up tiles may read x itself (kernel body).  Not in an expert-parallel share, whose
+    // remote tokens are to be read from their staged copies, and not under the withheld-flag hook, which is about a wait
+    // that does not exist then.
+    p.direct = T <= kDirectTokens && h->mode == WEAVE_SCHED_AUTO && h->ep_size == 1 && h->withhold_mb < 0 ? 1 : 0;
+    if (p.direct) {
+        const int half = (T + 15) / 16 * 8;      // rows per CTA of the pair
+        const int r = encode_map(h->encode, &h->tm.x, x, (uint64_t)T, (uint64_t)c.hidden, false, half <= 8 ? 8 : 16);
+        if (r) { h->last_cuda_error = r; return WEAVE_ERR_CUDA; }
+    }
 
     void *args[] = {&p, &h->tm};
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -889,6 +901,7 @@ int weave_moe_forward_static(int hidden, int ffn, int num_experts, int top_k, in
     h.tf_dev = sd->tables + 1024;
     memcpy(h.die_mask, sd->die_mask, sizeof(h.die_mask));
     h.two_dies = sd->two_dies;
+    h.encode = sd->encode;
     const int EE = num_experts + num_shared;
     int r = 0;
     r = encode_maps(sd->encode, &h.tm, h.ws + L.xe, h.ws + L.hbuf, gate_up, down, (uint64_t)L.p_max, (uint64_t)EE,
