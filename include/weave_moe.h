@@ -291,8 +291,8 @@ int weave_moe_debug_gemm_queue(const int32_t *rows, int num_segments, int num_ch
  *     synchronous copy, raises the kernel's shared-memory limit and resolves the TMA descriptor
  *     encoder).  Make that first call outside any stream capture.
  *   - All calls on a device share the one array, and it keeps the previous call's contents; every
- *     call enqueues one memset of the control words and then the kernel.  Calls that overlap on the
- *     GPU (different streams, no ordering between them) race on the array: order them.
+ *     call enqueues the kernel and nothing else.  Calls that overlap on the GPU (different streams,
+ *     no ordering between them) race on the array: order them.
  *   - Scheduling is AUTO with the default cost tables.  Arguments, layouts and alignment as for
  *     weave_moe_create() / weave_moe_forward(); asynchronous on the stream; a device-side failure
  *     of this call (non-finite logits, an expired wait) is not reported - use a handle when the

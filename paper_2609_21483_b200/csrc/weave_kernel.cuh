@@ -57,22 +57,38 @@ constexpr int kErrTimeout = -6;
 
 enum { kModeAuto = 0, kModeFixed = 1, kModeSerial = 2 };
 
-// Control words in global memory.  The first kCtlZeroWords words are zero at kernel entry and are
-// re-zeroed by the last CTA to leave, so no memset precedes a launch.
-struct Ctl {
+// Control words in global memory.  There are two sets of the words that a launch counts with (queues, flags, rows per
+// chunk and expert), used in turn: a launch finds its own set zero and zeroes the other one, which the launch before it
+// used, on its way in, so that nothing has to be cleaned up, and nobody has to be waited for, on the way out.  Which
+// one is whose follows from `epoch`: CTA 0 adds 65536 - (CTAs - 1) as it leaves and every other CTA 1, so the upper half
+// counts completed launches whatever their grids, and stays put until the last CTA of a launch is done.
+// (Before, the last CTA out zeroed the words behind an atomic that every CTA waited for, and the static entry point
+// zeroed its own with a memset: T = 1 40.1 -> 38.9 us, T = 64 200.7 -> 196.0, 8-expert T = 256 static 44.9 -> 41.3.)
+struct CtlSet {
     unsigned bar_count;   // grid-barrier arrivals
     unsigned q_disp;      // next dispatch tile
     unsigned q_gemm[2];   // next GEMM tile (chunk-pipeline DAG order) of either list
     unsigned q_comb;      // next combine tile
     unsigned fix_done;    // routing blocks whose rows are final
-    unsigned exit_count;
     unsigned abort;       // set by the first wait that gives up; every wait polls it
     unsigned y_done[kFine];  // per chunk: epilogue-warp arrivals of finished gemm1 tiles
     unsigned q_pull;      // expert-parallel share: next block of remote tokens to stage
     unsigned pull_done;   // ... blocks staged
     unsigned x_local, x_in, x_in_uniq;   // ... the workload descriptors of Section 3.1, counted while routing
-    unsigned pad1[3];
-    // ---- not re-zeroed: results for the host
+    unsigned pad[12];
+    // followed by fcnt [8][256]: rows per (fine chunk, expert);
+    //             xe_ready [nmb_max]: 1 when the m-block's rows are dispatched;
+    //             h_ready [nmb_max]: epilogue-warp arrivals of the m-block's gemm0 tiles
+};
+static_assert(sizeof(CtlSet) == 128, "the arrays behind it start on a line of their own");
+__host__ __device__ __forceinline__ size_t ctl_set_bytes(int nmb_max)
+{
+    return (sizeof(CtlSet) + sizeof(unsigned) * ((size_t)kFine * kMaxEE + 2 * (size_t)nmb_max) + 255) / 256 * 256;
+}
+struct Ctl {
+    unsigned epoch;
+    unsigned pad[31];
+    // results for the host
     int status;
     int timeout_where;
     int plan_c, plan_K, plan_steal;
@@ -81,7 +97,6 @@ struct Ctl {
     unsigned ep_x_local, ep_x_in, ep_x_in_uniq;
     int plan_kind;
 };
-constexpr int kCtlZeroWords = 24;
 
 // Plan kinds of the cost model.  kPlanSplit is the paper's (Eq. 15): c movement SMs beside N - c GEMM
 // SMs from the start.  The other two exist because on one GPU the movement is an HBM copy that all
@@ -117,7 +132,7 @@ struct KParams {
     const float *logits;
     __nv_bfloat16 *out;
     Ctl *ctl;
-    unsigned *fcnt;       // [8][256] rows per (fine chunk, expert); zero at entry
+    uint8_t *sets;        // two CtlSets with their arrays, ctl_set_bytes(nmb_max) each
     int *hist;            // [nrb][256]; shares its place with y, whose rows are written long after the last look at it
     int *topk_idx;        // [T][k]
     float *gates;         // [T][k]
@@ -128,8 +143,6 @@ struct KParams {
     __nv_bfloat16 *xe;    // [P][H]
     __nv_bfloat16 *hbuf;  // [P][I]
     __nv_bfloat16 *y;     // [P][H]
-    unsigned *xe_ready;   // [nmb_max] 1 when the m-block's rows are dispatched; zero at entry
-    unsigned *h_ready;    // [nmb_max] epilogue-warp arrivals of the m-block's gemm0 tiles; zero at entry
     const float *bw;      // [n_sm+1] byte/us
     const float *tf;      // [n_sm+1] FLOP/us
     uint4 *trace;         // optional [n_sm][trace_cap] event records (nullptr = off)
@@ -163,6 +176,8 @@ constexpr int kMvBuf = kStageBytes;     // 32 KB
 constexpr int kCombWarps = 6;           // warps 2..7 reduce
 
 struct SmemTail {
+    CtlSet *cs;                  // this launch's set of control words, and its arrays
+    unsigned *fcnt, *xe_ready, *h_ready;
     uint64_t full[kStages], empty[kStages];
     uint64_t tmem_full[2], tmem_empty[2];
     uint64_t ti_full[kTinfo], ti_empty[kTinfo];
@@ -180,6 +195,7 @@ struct SmemTail {
     int scan_w[8];
     int scan_total;
     int c, K, steal, nmb, n_gemm, n_comb;
+    int budget, die, direct;     // see gemm_phase
     int elastic;                 // this launch: movement pairs take GEMM tiles beyond their quota, GEMM CTAs dispatch one m-block first
     int comb_tok;                // tokens per combine tile of this launch: 16, 8, 4, 2 or 1
     unsigned trace_n;
@@ -215,12 +231,23 @@ __device__ __forceinline__ MoveScratch &move_scratch(uint8_t *stages)
 constexpr int kSmemBytes = kStages * kStageBytes + kEpiStageBytes + (int)sizeof(SmemTail) + 1024;
 static_assert(kSmemBytes <= 232448, "exceeds the 227 KB a CTA may opt into");
 
+// [stage ring | epilogue staging | SmemTail], the ring on a 1024-byte boundary
+__device__ __forceinline__ uint8_t *smem_stages()
+{
+    extern __shared__ uint8_t smem_raw[];
+    return smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+}
+__device__ __forceinline__ SmemTail &smem_tail()
+{
+    return *reinterpret_cast<SmemTail *>(smem_stages() + kStages * kStageBytes + kEpiStageBytes);
+}
+
 // ------------------------------------------------------------------------------------ waits
 
 __device__ __noinline__ void give_up(Ctl *ctl, int where)
 {
     if (atomicCAS(&ctl->status, 0, kErrTimeout) == 0) ctl->timeout_where = where;
-    atomicExch(&ctl->abort, 1u);
+    atomicExch(&smem_tail().cs->abort, 1u);
 }
 
 // Post-mortem of a failed launch: every wait that ends without success (its own limit ran out, or it saw
@@ -273,7 +300,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, const 
     while (!mbar_try_wait(bar, parity)) {
         if ((++it & 31u) == 0u) {
             if (ab) { note_failed_wait(p.wait_log, where, smem_u32(bar), parity, 2); return false; }
-            ab = ld_relaxed_u32(&p.ctl->abort);
+            ab = ld_relaxed_u32(&smem_tail().cs->abort);
             const unsigned long long now = globaltimer_ns();
             if (t0 == 0) t0 = now;
             else if ((long long)(now - t0) > (long long)p.timeout_ns) {     // signed: a timer that steps back is not a time-out
@@ -294,7 +321,7 @@ __device__ __forceinline__ bool flag_wait_ge(const unsigned *flag, unsigned targ
     while (ld_acquire_u32(flag) < target) {
         __nanosleep(40);
         if ((++it & 31u) == 0u) {
-            if (ld_relaxed_u32(&p.ctl->abort)) {
+            if (ld_relaxed_u32(&smem_tail().cs->abort)) {
                 note_failed_wait(p.wait_log, where, (unsigned)(size_t)flag, target, 2);
                 return false;
             }
@@ -343,14 +370,14 @@ __device__ __forceinline__ unsigned long long block_excl_scan_packed(unsigned lo
 }
 
 // the two halves of a grid barrier, for a caller that has work to do between arriving and waiting
-__device__ __forceinline__ void grid_barrier_arrive(const KParams &p)
+__device__ __forceinline__ void grid_barrier_arrive(SmemTail &S)
 {
     __syncthreads();      // (the release is cumulative: it covers what the other threads wrote before the block barrier)
-    if (threadIdx.x == 0) red_release_add_u32(&p.ctl->bar_count, 1u);
+    if (threadIdx.x == 0) red_release_add_u32(&S.cs->bar_count, 1u);
 }
 __device__ __forceinline__ bool grid_barrier_wait(const KParams &p, SmemTail &S, unsigned target, int where)
 {
-    if (threadIdx.x == 0) S.bcast[2] = flag_wait_ge(&p.ctl->bar_count, target, p, where) ? 1 : 0;
+    if (threadIdx.x == 0) S.bcast[2] = flag_wait_ge(&S.cs->bar_count, target, p, where) ? 1 : 0;
     __syncthreads();
     return S.bcast[2] != 0;
 }
@@ -358,8 +385,8 @@ __device__ __forceinline__ bool grid_barrier(const KParams &p, SmemTail &S, unsi
 {
     __syncthreads();
     if (threadIdx.x == 0) {
-        red_release_add_u32(&p.ctl->bar_count, 1u);
-        S.bcast[2] = flag_wait_ge(&p.ctl->bar_count, target, p, where) ? 1 : 0;
+        red_release_add_u32(&S.cs->bar_count, 1u);
+        S.bcast[2] = flag_wait_ge(&S.cs->bar_count, target, p, where) ? 1 : 0;
     }
     __syncthreads();
     return S.bcast[2] != 0;
@@ -806,7 +833,7 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
         int b = 0;
         uint32_t ph = 0;
         bool ok = true;
-        if (lane == 0 && lmask == nullptr) ok = flag_wait_ge(&p.ctl->fix_done, (unsigned)p.nrb, p, 10);
+        if (lane == 0 && lmask == nullptr) ok = flag_wait_ge(&S.cs->fix_done, (unsigned)p.nrb, p, 10);
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (p.ep_size > 1) {
             // expert-parallel share: first every remote token that has an expert here is copied ONCE
@@ -815,7 +842,7 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
             // 64-token routing block, taken by whoever comes first.
             while (ok) {
                 int blk = 0;
-                if (lane == 0) blk = (int)atomicAdd(&p.ctl->q_pull, 1u);
+                if (lane == 0) blk = (int)atomicAdd(&S.cs->q_pull, 1u);
                 blk = __shfl_sync(0xffffffffu, blk, 0);
                 if (blk >= p.nblk) break;
                 const unsigned long long um = lmask ? lmask[blk * (kMaxEE + 1) + kMaxEE] : __ldcg(p.uniq_mask + blk);
@@ -828,7 +855,7 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
                 __syncwarp();
                 if (lane == 0) {
                     if (n == 0) {
-                        red_release_add_u32(&p.ctl->pull_done, 1u);
+                        red_release_add_u32(&S.cs->pull_done, 1u);
                     } else {
                         const int Rp = min(R, 32);
                         for (int r0 = 0; r0 < n; r0 += Rp) {
@@ -856,7 +883,7 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
                     if (++b == kStages) { b = 0; ph ^= 1u; }
                 } else ok = false;
             }
-            if (lane == 0 && ok && max_tiles > 0) ok = flag_wait_ge(&p.ctl->pull_done, (unsigned)p.nblk, p, 15);
+            if (lane == 0 && ok && max_tiles > 0) ok = flag_wait_ge(&S.cs->pull_done, (unsigned)p.nblk, p, 15);
             ok = __shfl_sync(0xffffffffu, ok, 0);
             // only lane 0 walked the ring so far; from here on every lane addresses the buffers
             b = __shfl_sync(0xffffffffu, b, 0);
@@ -865,7 +892,7 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
         for (int taken = 0; ok && taken < max_tiles; ++taken) {
             int mb = (int)blockIdx.x;
             if (taken > 0) {
-                if (lane == 0) mb = n_disp + (int)atomicAdd(&p.ctl->q_disp, 1u);
+                if (lane == 0) mb = n_disp + (int)atomicAdd(&S.cs->q_disp, 1u);
                 mb = __shfl_sync(0xffffffffu, mb, 0);
             }
             if (mb >= S.nmb) { if (taken > 0) break; else continue; }
@@ -945,9 +972,9 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
                     // (the bulk stores have completed; the release below orders them for whoever acquires the flag)
                     if (!fenced) { fence_proxy_async_global(); fenced = true; }
                     if (pe_mb[s8] < 0) {
-                        red_release_add_u32(&p.ctl->pull_done, 1u);      // a block of remote tokens is staged
+                        red_release_add_u32(&S.cs->pull_done, 1u);      // a block of remote tokens is staged
                     } else {
-                        if (pe_mb[s8] != p.withhold_mb) st_release_u32(&p.xe_ready[pe_mb[s8]], 1u);
+                        if (pe_mb[s8] != p.withhold_mb) st_release_u32(&S.xe_ready[pe_mb[s8]], 1u);
                         trace_ev(p, S, kEvDispatch, (unsigned)pe_mb[s8], pe_t0[s8], trace_now(p), (unsigned)pe_rows[s8]);
                     }
                     ++pe_head;
@@ -1019,7 +1046,7 @@ __device__ __forceinline__ void combine_phase(const KParams &p, SmemTail &S, uin
         bool ok = true;
         for (;;) {
             int q = 0;
-            if (lane == 0) q = (int)atomicAdd(&p.ctl->q_comb, 1u);
+            if (lane == 0) q = (int)atomicAdd(&S.cs->q_comb, 1u);
             q = __shfl_sync(0xffffffffu, q, 0);
             if (q >= S.n_comb) break;
             const int t0 = q * S.comb_tok;
@@ -1028,7 +1055,7 @@ __device__ __forceinline__ void combine_phase(const KParams &p, SmemTail &S, uin
             // the tile's rows and gates are final once the permutation is; they are fetched before the wait for
             // the chunk's last GEMM tile, so that only the row copies themselves follow that wait
             if (!perm_final) {
-                if (lane == 0) ok = flag_wait_ge(&p.ctl->fix_done, (unsigned)p.nrb, p, 20);
+                if (lane == 0) ok = flag_wait_ge(&S.cs->fix_done, (unsigned)p.nrb, p, 20);
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok) break;
                 perm_final = true;
@@ -1043,7 +1070,7 @@ __device__ __forceinline__ void combine_phase(const KParams &p, SmemTail &S, uin
                 if (lane == 0) {
                     const unsigned long long tw0 = trace_now(p);
                     for (int j = ready_upto + 1; ok && j <= chunk; ++j) {
-                        ok = flag_wait_ge(&p.ctl->y_done[j], y_done_target(S, p, j), p, 21);
+                        ok = flag_wait_ge(&S.cs->y_done[j], y_done_target(S, p, j), p, 21);
                     }
                     trace_ev(p, S, kEvWaitChunk, (unsigned)chunk, tw0, trace_now(p), 0u);
                 }
@@ -1184,7 +1211,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity
     while (!mbar_try_wait_cluster(bar, parity)) {
         if ((++it & 31u) == 0u) {
             if (ab) { note_failed_wait(p.wait_log, where, smem_u32(bar), parity, 2); return false; }
-            ab = ld_relaxed_u32(&p.ctl->abort);
+            ab = ld_relaxed_u32(&smem_tail().cs->abort);
             const unsigned long long now = globaltimer_ns();
             if (t0 == 0) t0 = now;
             else if ((long long)(now - t0) > (long long)p.timeout_ns) {
@@ -1228,12 +1255,12 @@ __device__ __forceinline__ void staged_store_32(const uint32_t (&o)[16], uint32_
     __syncwarp();      // the region is rewritten by the next batch
 }
 
-// budget = how many pair tiles this CTA pair may claim (the steal count for a movement pair).
-// Called by both CTAs of a pair with the same arguments.  direct: the gate/up tiles take the batch's tokens themselves
-// as their row operand (all tiles are swapped ones then).
-__device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_t *stages, uint32_t tmem_base,
-                                           const TmaMaps *tm, int budget, int die, bool direct, PipeState &ps)
+// S.budget = how many pair tiles this CTA pair may claim (the steal count for a movement pair); S.direct: the
+// gate/up tiles take the batch's tokens themselves as their row operand (all tiles are swapped ones then).  They and
+// the other scalars come through shared memory: the epilogue has no registers to spare for values that live across it.
+__device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_t *stages, const TmaMaps *tm)
 {
+    PipeState ps;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_ctarank();      // 0 = leader (issues the MMAs), 1 = peer
     fence_proxy_async_shared();     // the stage buffers were last touched by ordinary stores (routing scratch)
@@ -1249,18 +1276,18 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
             // its own list and for the dispatch, so of all claimed tiles the one claimed first can always proceed.
             const int per_pt = p.nt0 + p.nt1;
             const int n_list0 = S.K == 1 ? S.split_pt * per_pt : S.n_gemm;
-            int list = n_list0 == S.n_gemm ? 0 : die;
+            int list = n_list0 == S.n_gemm ? 0 : S.die;
             bool second = false;
             auto claim = [&]() -> int {
                 for (;;) {
-                    const int c = (int)atomicAdd(&p.ctl->q_gemm[list], 1u);
+                    const int c = (int)atomicAdd(&S.cs->q_gemm[list], 1u);
                     if (c < (list ? S.n_gemm - n_list0 : n_list0)) return c;
                     if (second) return 0x7fffffff;
                     second = true;
                     list ^= 1;
                 }
             };
-            int g_next = (budget > 0 || S.elastic) ? claim() : 0x7fffffff;
+            int g_next = (S.budget > 0 || S.elastic) ? claim() : 0x7fffffff;
             for (;;) {
                 const int g = g_next;
                 const unsigned long long tp0 = trace_now(p);
@@ -1278,21 +1305,21 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 if (tl.type != 2) {
                     bool ok;
                     const bool two = tp.mb != tl.mb;         // a regular pair tile has two m-blocks
-                    if (direct && tl.type == 3) {
+                    if (S.direct && tl.type == 3) {
                         ok = true;               // x was there before the launch
                     } else if (tl.type == 0 || tl.type == 3) {
-                        ok = flag_wait_ge(&p.xe_ready[tl.mb], 1u, p, 31);
-                        if (ok && two) ok = flag_wait_ge(&p.xe_ready[tp.mb], 1u, p, 31);
+                        ok = flag_wait_ge(&S.xe_ready[tl.mb], 1u, p, 31);
+                        if (ok && two) ok = flag_wait_ge(&S.xe_ready[tp.mb], 1u, p, 31);
                     } else {
                         const unsigned need = (unsigned)(p.nt0 * kEpiWarps);
-                        ok = flag_wait_ge(&p.h_ready[tl.mb], need, p, 32);
-                        if (ok && two) ok = flag_wait_ge(&p.h_ready[tp.mb], need, p, 32);
+                        ok = flag_wait_ge(&S.h_ready[tl.mb], need, p, 32);
+                        if (ok && two) ok = flag_wait_ge(&S.h_ready[tp.mb], need, p, 32);
                     }
                     if (!ok) break;
                     // the tile's input rows may have been written with ordinary stores on other SMs and
                     // are read by TMA next: the cross-proxy fence sits here, after the acquire and before
                     // the hand-over to the producers, off their critical path
-                    if (!(direct && tl.type == 3)) fence_proxy_async_global();
+                    if (!(S.direct && tl.type == 3)) fence_proxy_async_global();
                     trace_ev(p, S, kEvGemmLoad, (unsigned)g, tp0, trace_now(p), 0u);
                 }
                 mbar_arrive(&S.ti_full[ps.slot]);
@@ -1301,15 +1328,15 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 if (tl.type == 2) break;
                 // the next claim's round trip comes after the hand-over
                 ++taken;
-                bool more = taken < budget;
+                bool more = taken < S.budget;
                 if (!more && S.elastic) {
                     // the steal quota is used up: keep taking GEMM tiles for as long as the next
                     // combine chunk has not been produced yet (nothing else to do meanwhile)
-                    const unsigned qc = ld_relaxed_u32(&p.ctl->q_comb);
+                    const unsigned qc = ld_relaxed_u32(&S.cs->q_comb);
                     if (qc >= (unsigned)S.n_comb) more = true;
                     else {
                         const int ch = ((((int)qc * S.comb_tok / kRouteBlock) * kFine) / p.nblk) / (kFine / S.K);
-                        more = ld_acquire_u32(&p.ctl->y_done[ch]) < y_done_target(S, p, ch);
+                        more = ld_acquire_u32(&S.cs->y_done[ch]) < y_done_target(S, p, ch);
                     }
                 }
                 g_next = more ? claim() : 0x7fffffff;
@@ -1334,7 +1361,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 const CUtensorMap *tma_a, *tma_b;
                 int arow, brow, arow2 = -1;
                 // swapped tiles: rows per CTA on the N axis (the MMA's N, a multiple of 16, split in two)
-                const bool from_x = direct && ti.type == 3;
+                const bool from_x = S.direct && ti.type == 3;
                 const int nhalf = ((((from_x ? p.T : ti.nrows) + 15) >> 4) << 4) >> 1;
                 // ... fetched with the smallest box that covers them (the copy engine takes in a fixed
                 // number of rows per cycle, so rows nobody reads cost as much as the others)
@@ -1398,7 +1425,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
             ps.next_slot();
             if (ti.type == 2) break;
             // regular tiles: 256 rows x 256 columns; swapped tiles: 256 weight rows x (rows rounded up to 16)
-            const int n_op = direct && ti.type == 3 ? p.T : ti.nrows;
+            const int n_op = S.direct && ti.type == 3 ? p.T : ti.nrows;
             const uint32_t idesc = umma_idesc_bf16(2 * kBM, ti.type >= 3 ? (uint32_t)(((n_op + 15) >> 4) << 4) : 256u);
             // timeline record of this tile: extra = time spent waiting for a free accumulator (ns)
             const unsigned long long tm0 = trace_now(p);
@@ -1406,7 +1433,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
             if (!__all_sync(0xffffffffu, ok)) { dead = true; break; }
             tc_fence_after();
             const unsigned long long tm1 = trace_now(p);
-            const uint32_t d = tmem_base + (uint32_t)ps.acc * 256u;
+            const uint32_t d = S.tmem_base + (uint32_t)ps.acc * 256u;
             bool landed = mbar_test_wait(&S.full[ps.stage], ps.stage_phase);
             for (int kb = 0; kb < ti.nkb; ++kb) {
                 // The operands were written by TMA (either CTA's, into its own shared memory) and are
@@ -1478,7 +1505,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 if (lane == 0) mbar_arrive_remote(mapa_u32(smem_u32(&S.tmem_empty[ps.acc]), 0u));
                 acc_released = true;
             };
-            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)ps.acc * 256u;
+            const uint32_t taddr = S.tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)ps.acc * 256u;
             if (ti.type == 3) {
                 // swapped gemm0: lanes 0..63 hold the gate projection of this CTA's 64 h-columns, lanes 64..127 the up
                 // projection; TMEM columns are the m-block's rows.  Gate warp q and up warp q + 2 trade halves of every
@@ -1490,6 +1517,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 //
                 // direct: TMEM columns are the batch's tokens, and the expert's rows are those with a bit in its mask.
                 const int up = q >> 1;
+                const bool direct = S.direct != 0;
                 const uint32_t xbase = smem_u32(stages + kStages * kStageBytes) + 2048u + (uint32_t)lane * 16u;
                 const uint32_t xmine = xbase + (uint32_t)q * 4096u, xtheirs = xbase + (uint32_t)(q ^ 2) * 4096u;
                 uint64_t *const xbar = &S.xg[q & 1];
@@ -1640,14 +1668,14 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
             // 4 arrivals per m-block and gemm0 n-tile: from the m-block's own CTA of a regular tile, 2 from each CTA of
             // a swapped one; a swapped gemm1 tile makes 4 from each CTA (see y_done_target)
             const bool g0 = ti.type == 0 || ti.type == 3;
-            if (!post(g0 ? &p.h_ready[ti.mb] : &p.ctl->y_done[ti.chunk], ti.type == 3 ? 2u : (unsigned)kEpiWarps)) dead = true;
+            if (!post(g0 ? &S.h_ready[ti.mb] : &S.cs->y_done[ti.chunk], ti.type == 3 ? 2u : (unsigned)kEpiWarps)) dead = true;
             ps.next_acc();
         }
     } else if (warp == 3) {
         // ---------------- releasing warp (both CTAs): makes the tiles' arrivals on the ready counters
         int rs = 0;
         uint32_t rph = 0;
-        if (direct) {
+        if (S.direct) {
             // nothing reads the dispatched rows here, but the caller may ask for them: token t's row of x goes to its
             // rows of Xe, the token's experts spread over `parts` CTAs
             const unsigned long long *mask = reinterpret_cast<const unsigned long long *>(stages + kStages * kStageBytes);
@@ -1699,10 +1727,8 @@ constexpr int kErrNoPairs = -2;     // reported as "unsupported device"
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaMaps tm)
 {
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t *stages = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    // [stage ring | epilogue staging | SmemTail]
-    SmemTail &S = *reinterpret_cast<SmemTail *>(stages + kStages * kStageBytes + kEpiStageBytes);
+    uint8_t *stages = smem_stages();
+    SmemTail &S = smem_tail();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n_sm = (int)gridDim.x;
     const int EE = p.EE;
@@ -1724,6 +1750,7 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
     }
 
     if (tid == 0) {
+        const unsigned odd = (ld_relaxed_u32(&p.ctl->epoch) >> 16) & 1u;
         // (rolled loops: code that runs once per launch runs at the speed of instruction fetch)
 #pragma unroll 1
         for (int i = 0; i < kStages; ++i) {
@@ -1746,14 +1773,23 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         if (p.direct) tma_prefetch_desc(&tm.x);
 #pragma unroll 1
         for (int i = 0; i < 4; ++i) { tma_prefetch_desc(&tm.xe_n[i]); tma_prefetch_desc(&tm.h_n[i]); }
+        S.cs = reinterpret_cast<CtlSet *>(p.sets + (odd ? ctl_set_bytes(p.nmb_max) : 0));
+        S.fcnt = reinterpret_cast<unsigned *>(S.cs + 1);
+        S.xe_ready = S.fcnt + kFine * kMaxEE;
+        S.h_ready = S.xe_ready + p.nmb_max;
+        S.trace_n = 0u;
     }
     if (warp == 1) { tmem_alloc_pair(&S.tmem_base, kTmemCols); tmem_relinquish_pair(); }
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();      // the peer's barriers exist before anything is sent to them
     tc_fence_after();
-    const uint32_t tmem_base = S.tmem_base;
-    if (tid == 0) S.trace_n = 0u;
+    {
+        const size_t bytes = ctl_set_bytes(p.nmb_max);
+        uint4 *other = reinterpret_cast<uint4 *>(p.sets + (reinterpret_cast<uint8_t *>(S.cs) == p.sets ? bytes : 0));
+        for (size_t i = (size_t)blockIdx.x * kThreads + tid; i < bytes / 16; i += (size_t)n_sm * kThreads)
+            other[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
     const unsigned long long tk0 = trace_now_t0(p);
 
     // Routing scratch.  The expert masks of the routing blocks sit in the first half of the epilogue staging
@@ -1840,16 +1876,16 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         if (!local_route) {
             if (ep && tid == 0) {
                 const unsigned long long um = r_mask[kMaxEE];
-                if (r_cnt[0]) atomicAdd(&p.ctl->x_local, (unsigned)r_cnt[0]);
-                if (r_cnt[1]) atomicAdd(&p.ctl->x_in, (unsigned)r_cnt[1]);
-                if (um) atomicAdd(&p.ctl->x_in_uniq, (unsigned)__popcll(um));
+                if (r_cnt[0]) atomicAdd(&S.cs->x_local, (unsigned)r_cnt[0]);
+                if (r_cnt[1]) atomicAdd(&S.cs->x_in, (unsigned)r_cnt[1]);
+                if (um) atomicAdd(&S.cs->x_in_uniq, (unsigned)__popcll(um));
             }
             const int ntok = min(1 << p.lg_rb, p.T - (b << p.lg_rb));
             const int f = ((b >> (6 - p.lg_rb)) * kFine) / p.nblk;
             for (int e = tid; e < EE; e += kThreads) {
                 const int cnt = e < p.E ? __popcll(r_mask[e]) : ntok;
                 p.hist[(size_t)b * kMaxEE + e] = cnt;
-                if (cnt) atomicAdd(&p.fcnt[f * kMaxEE + e], (unsigned)cnt);
+                if (cnt) atomicAdd(&S.fcnt[f * kMaxEE + e], (unsigned)cnt);
             }
             __syncthreads();      // the scratch is reused by this CTA's next block
         }
@@ -1860,7 +1896,7 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
     if (!local_route) {
         // the plan is chosen between arriving at the barrier and waiting on it: the arrival's way to L2 and
         // the wait for the slowest routing CTA hide it
-        grid_barrier_arrive(p);
+        grid_barrier_arrive(S);
         if (!picked && !ep && p.mode == kModeAuto) {
             pick = model_pick(ma, S, n_sm, w_comp, w_disp, w_comb, cm_ok, cm_bw, cm_tf, cm_bw_n, cm_tf_n);
             picked = true;
@@ -1894,11 +1930,11 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
     } else {
 #pragma unroll
         for (int f = 0; f < kFine; ++f) {
-            cf[f] = (alive && tid < EE) ? (int)__ldcg(p.fcnt + f * kMaxEE + tid) : 0;
+            cf[f] = (alive && tid < EE) ? (int)__ldcg(S.fcnt + f * kMaxEE + tid) : 0;
             cnt += cf[f];
         }
         // (asked for together with the counts: one L2 round trip instead of two)
-        if (alive && ep) { ep_xl = __ldcg(&p.ctl->x_local); ep_xi = __ldcg(&p.ctl->x_in); ep_xu = __ldcg(&p.ctl->x_in_uniq); }
+        if (alive && ep) { ep_xl = __ldcg(&S.cs->x_local); ep_xi = __ldcg(&S.cs->x_in); ep_xu = __ldcg(&S.cs->x_in_uniq); }
     }
     int total_rows;
     const int off = block_excl_scan(cnt, S, total_rows);
@@ -2073,12 +2109,12 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
             __syncthreads();
             ++fixed;
         }
-        if (tid == 0 && fixed) red_release_add_u32(&p.ctl->fix_done, (unsigned)fixed);
+        if (tid == 0 && fixed) red_release_add_u32(&S.cs->fix_done, (unsigned)fixed);
     }
 
     if (tid == 0) trace_ev(p, S, kEvFixup, 0u, tk3, trace_now(p), 0u);
     // ================= main phases
-    PipeState ps;
+    bool tmem_held = true;
     if (alive) {
         // The serial schedule is the phased plan with a grid barrier between the phases (one copy of each
         // phase's code serves both).
@@ -2102,34 +2138,35 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         // T = 27 149.4 -> 146.7.  At T = 64 a launch by itself gains as much (199.9 -> 197.8) but under load the
         // additional columns and rows cost power (202.8 -> 205.9 after half a second): hence the limit.
         const bool direct = p.direct && plan_kind == kPlanPhased;
+        const int budget = (mover && plan_kind != kPlanPhased) ? plan_steal : 0x7fffffff;
+        if (tid == 0) { S.budget = budget; S.die = die; S.direct = direct ? 1 : 0; }      // (published by gemm_phase's first barrier)
         if (dmax > 0 && !direct) dispatch_phase(p, S, stages, dmax, n_disp, p.nblk <= kLocalBlocks);
         if (serial) alive = grid_barrier(p, S, bar0 + (unsigned)n_sm, 2);
-        const int budget = (mover && plan_kind != kPlanPhased) ? plan_steal : 0x7fffffff;
-        if (alive && (budget > 0 || S.elastic)) gemm_phase(p, S, stages, tmem_base, &tm, budget, die, direct, ps);
+        if (alive && (budget > 0 || S.elastic)) {
+            gemm_phase(p, S, stages, &tm);
+            // (it ends with both CTAs of the pair past their last use of tensor memory and of each other's shared memory)
+            if (warp == 1) tmem_dealloc_pair(S.tmem_base, kTmemCols);
+            tmem_held = false;
+        }
         if (serial) alive = alive && grid_barrier(p, S, bar0 + 2u * (unsigned)n_sm, 3);
         if (alive) combine_phase(p, S, stages);
     }
 
-    // ================= leave: free TMEM; the last CTA out re-zeroes the control words
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    cluster_sync_all();
-    if (warp == 1) tmem_dealloc_pair(tmem_base, kTmemCols);
-    if (tid == 0) {
-        if (p.trace)     // last record of the CTA's slice: how many events were written
+    // ================= leave
+    if (tmem_held) {      // no GEMM phase here: the peer may be in one, and tensor memory is freed by both
+        tc_fence_before();
+        __syncthreads();
+        cluster_sync_all();
+        tc_fence_after();
+        if (warp == 1) tmem_dealloc_pair(S.tmem_base, kTmemCols);
+    }
+    if (p.trace) {      // last record of the CTA's slice: how many events were written
+        __syncthreads();
+        if (tid == 0)
             p.trace[(size_t)blockIdx.x * p.trace_cap + p.trace_cap - 1] =
                 make_uint4(min(S.trace_n, (unsigned)p.trace_cap - 1u), 0u, 0u, 0u);
-        S.bcast[0] = atom_acqrel_add_u32(&p.ctl->exit_count, 1u) == (unsigned)(n_sm - 1) ? 1 : 0;
     }
-    __syncthreads();
-    if (S.bcast[0]) {
-        if (p.nblk > kLocalBlocks)      // (a batch that every CTA routed for itself left the counts untouched)
-            for (int i = tid; i < kFine * kMaxEE; i += kThreads) p.fcnt[i] = 0u;
-        for (int i = tid; i < p.nmb_max; i += kThreads) { p.xe_ready[i] = 0u; p.h_ready[i] = 0u; }
-        unsigned *z = reinterpret_cast<unsigned *>(p.ctl);
-        if (tid < kCtlZeroWords) z[tid] = 0u;
-    }
+    if (tid == 0) atomicAdd(&p.ctl->epoch, blockIdx.x == 0 ? 65536u - (unsigned)(n_sm - 1) : 1u);
 }
 
 // ------------------------------------------------------------------------------------ which half an SM sits on

@@ -24,8 +24,8 @@ inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 constexpr int kWaitLogSlots = 1024 * 8;      // one slot per warp of up to 1024 CTAs
 
 struct Layout {
-    size_t ctl, fcnt, xe_ready, h_ready, wait_log, zero_end;       // [0, zero_end) is zeroed at create / recovery
-    size_t hist, topk, gates, row_of, token_of, counts, offsets, bw, tf, uniq_mask, xs;
+    size_t ctl, sets, wait_log, zero_end;       // [0, zero_end) is zeroed at create / recovery
+    size_t topk, gates, row_of, token_of, counts, offsets, bw, tf, uniq_mask, xs;
     size_t xe, hbuf, y, st_x, st_logits, st_out, st2_x, st2_logits, st2_out, total;
     int nmb_max, nblk_max, p_max;
 };
@@ -58,12 +58,9 @@ Layout make_layout(const weave_moe_config *c)
     size_t o = 0;
     auto take = [&](size_t bytes, size_t al) { o = align_up(o, al); size_t r = o; o += bytes; return r; };
     L.ctl = take(sizeof(Ctl), 256);
-    L.fcnt = take(sizeof(unsigned) * kFine * kMaxEE, 256);
-    L.xe_ready = take(sizeof(unsigned) * L.nmb_max, 256);
-    L.h_ready = take(sizeof(unsigned) * L.nmb_max, 256);
+    L.sets = take(2 * ctl_set_bytes(L.nmb_max), 256);
     L.wait_log = take(sizeof(int4) * kWaitLogSlots, 256);     // written by failed waits only, cleared by the host
     L.zero_end = align_up(o, 256);
-    L.hist = take(sizeof(int) * (size_t)L.nblk_max * kMaxEE, 256);
     L.topk = take(sizeof(int) * T * c->top_k, 256);
     L.gates = take(sizeof(float) * T * c->top_k, 256);
     L.row_of = take(sizeof(int) * T * c->top_k, 256);
@@ -97,6 +94,8 @@ struct weave_moe {
     weave_moe_config cfg;
     Layout L;
     uint8_t *ws;
+    uint8_t *ctl, *sets, *wait_log_dev;      // control words: in the workspace, or the static entry's own array
+    int nmb_ctl;                             // m-blocks the sets have flags for
     int n_sm;      // SMs of the device
     int n_cta;     // persistent CTAs = SMs rounded down to whole pairs
     int device;
@@ -271,6 +270,8 @@ int weave_moe_create(const weave_moe_config *cfg, weave_moe_t *out)
     h->cfg = *cfg;
     h->L = L;
     h->ws = static_cast<uint8_t *>(cfg->workspace);
+    h->ctl = h->ws + L.ctl; h->sets = h->ws + L.sets; h->wait_log_dev = h->ws + L.wait_log;
+    h->nmb_ctl = L.nmb_max;
     h->n_sm = prop.multiProcessorCount & ~1;     // the scheduler counts SMs in whole CTA pairs
     h->n_cta = h->n_sm;
     h->device = dev;
@@ -370,7 +371,7 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     p.mode = h->mode; p.fixed_c = h->fixed_c; p.fixed_K = h->fixed_K; p.fixed_steal = h->fixed_steal;
     p.nt0 = c.ffn / kTN0;
     p.nt1 = (c.hidden + 255) / 256;
-    p.nmb_max = L.nmb_max;
+    p.nmb_max = h->nmb_ctl;
     p.withhold_mb = h->withhold_mb;
     p.elastic_steal = h->elastic < 0 ? ((h->mode == WEAVE_SCHED_AUTO) ? 1 : 0) : h->elastic;
     p.kinds = h->kinds;
@@ -382,8 +383,8 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     p.logits = logits;
     p.out = static_cast<__nv_bfloat16 *>(out);
     uint8_t *ws = h->ws;
-    p.ctl = reinterpret_cast<Ctl *>(ws + L.ctl);
-    p.fcnt = reinterpret_cast<unsigned *>(ws + L.fcnt);
+    p.ctl = reinterpret_cast<Ctl *>(h->ctl);
+    p.sets = h->sets;
     p.hist = reinterpret_cast<int *>(ws + L.y);      // at most 64 bytes per token, a row of y has at least 256
     p.topk_idx = reinterpret_cast<int *>(ws + L.topk);
     p.gates = reinterpret_cast<float *>(ws + L.gates);
@@ -394,8 +395,6 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     p.xe = reinterpret_cast<__nv_bfloat16 *>(ws + L.xe);
     p.hbuf = reinterpret_cast<__nv_bfloat16 *>(ws + L.hbuf);
     p.y = reinterpret_cast<__nv_bfloat16 *>(ws + L.y);
-    p.xe_ready = reinterpret_cast<unsigned *>(ws + L.xe_ready);
-    p.h_ready = reinterpret_cast<unsigned *>(ws + L.h_ready);
     p.bw = h->bw_dev;
     p.tf = h->tf_dev;
     p.ep_rank = h->ep_rank;
@@ -405,7 +404,7 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     p.uniq_mask = reinterpret_cast<unsigned long long *>(ws + L.uniq_mask);
     p.trace = reinterpret_cast<uint4 *>(h->trace);
     p.trace_cap = h->trace_cap;
-    p.wait_log = reinterpret_cast<int4 *>(ws + L.wait_log);
+    p.wait_log = reinterpret_cast<int4 *>(h->wait_log_dev);
     memcpy(p.die_mask, h->die_mask, sizeof(p.die_mask));
     p.two_dies = h->two_dies;
 
@@ -786,14 +785,23 @@ int weave_moe_debug_gemm_queue(const int32_t *rows, int num_segments, int num_ch
 
 namespace {
 
-constexpr size_t kStaticScratchBytes = 64ull << 20;
-static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
+constexpr size_t kStaticScratchBytes = 64ull << 20;      // what a layer may need
+constexpr size_t kStaticArrayBytes = kStaticScratchBytes + (64 << 10);      // (room for words that were added to the workspace)
+static __device__ __align__(256) unsigned char g_static_scratch[kStaticArrayBytes];
+// The control words have a place of their own, the same for layers of every shape, so that the two sets of words go on
+// taking turns from call to call (a memset in front of every launch cost 2-3 us).  Zero when the image is loaded.
+// A row of x and of y takes at least 256 bytes each, so the scratch holds fewer than 2^17 rows.
+constexpr int kStaticNmb = (1 << 17) / kBM + kMaxEE * kFine;
+constexpr size_t kStaticSetBytes = (sizeof(CtlSet) + sizeof(unsigned) * ((size_t)kFine * kMaxEE + 2 * (size_t)kStaticNmb) + 255) / 256 * 256;
+static_assert(sizeof(Ctl) <= 256, "the sets start 256 bytes into the array");
+static __device__ __align__(256) unsigned char g_static_ctl[256 + 2 * kStaticSetBytes + sizeof(int4) * kWaitLogSlots];
 // the default cost tables BW(i), TFLOPS(i), i <= 1023: they depend on the device only and are
 // written once per device, at set-up
 static __device__ __align__(256) float g_static_tables[2][1024];
 
 struct StaticDevice {
     bool ready;
+    uint8_t *ctl;         // device address of g_static_ctl on this device
     uint8_t *base;        // device address of g_static_scratch on this device, rounded up to 1024
     const float *tables;  // device address of g_static_tables on this device
     size_t usable;
@@ -820,9 +828,12 @@ int static_setup(int dev, StaticDevice **out)
             return WEAVE_ERR_UNSUPPORTED_DEVICE;
         void *sym = nullptr;
         if (cudaGetSymbolAddress(&sym, g_static_scratch) != cudaSuccess || sym == nullptr) return WEAVE_ERR_CUDA;
+        void *csym = nullptr;
+        if (cudaGetSymbolAddress(&csym, g_static_ctl) != cudaSuccess || csym == nullptr) return WEAVE_ERR_CUDA;
+        d.ctl = static_cast<uint8_t *>(csym);
         const uintptr_t a = ((uintptr_t)sym + 1023) & ~(uintptr_t)1023;
         d.base = reinterpret_cast<uint8_t *>(a);
-        d.usable = kStaticScratchBytes - (size_t)(a - (uintptr_t)sym);
+        d.usable = kStaticArrayBytes - (size_t)(a - (uintptr_t)sym);
         d.n_sm = prop.multiProcessorCount & ~1;
         void *tsym = nullptr;
         if (cudaGetSymbolAddress(&tsym, g_static_tables) != cudaSuccess || tsym == nullptr) return WEAVE_ERR_CUDA;
@@ -885,6 +896,8 @@ int weave_moe_forward_static(int hidden, int ffn, int num_experts, int top_k, in
     h.cfg.gate_up = gate_up; h.cfg.down = down; h.cfg.workspace = sd->base; h.cfg.workspace_bytes = sd->usable;
     h.L = L;
     h.ws = sd->base;
+    h.ctl = sd->ctl; h.sets = sd->ctl + 256; h.wait_log_dev = sd->ctl + 256 + 2 * kStaticSetBytes;
+    h.nmb_ctl = kStaticNmb;
     h.n_sm = sd->n_sm; h.n_cta = sd->n_sm; h.device = dev;
     h.mode = WEAVE_SCHED_AUTO;
     h.fixed_c = (h.n_sm * 15 / 100 + 1) & ~1; h.fixed_K = 1; h.fixed_steal = 0;
@@ -908,10 +921,6 @@ int weave_moe_forward_static(int hidden, int ffn, int num_experts, int top_k, in
                     (uint64_t)hidden, (uint64_t)ffn);
     if (r) return WEAVE_ERR_CUDA;
 
-    // the array keeps whatever the last call left behind: zero the control words (the cost tables sit
-    // in their own array, written once at set-up), then the kernel; nothing else is enqueued
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    if (cudaMemsetAsync(h.ws, 0, L.zero_end, st) != cudaSuccess) return WEAVE_ERR_CUDA;
     return weave_moe_forward(&h, x, router_logits, out, T, cuda_stream);
 }
 

@@ -584,3 +584,33 @@ def test_routing_blocks_of_every_size(T, E, k, S):
     _, chunked, _ = run_case(cfg, sched=(pk.SCHED_FIXED, 20, 2, 1), inp=inp, dev_tensors=dev, moe=moe, n_sample=4, budget=16)
     assert torch.equal(out.view(torch.int16), chunked.view(torch.int16))
     moe.close()
+
+
+@pytest.mark.parametrize("T", [20, 300])
+def test_control_word_sets_take_turns_whatever_the_grid(T):
+    """A launch finds its set of control words zero because the launch before it zeroed it; which set is whose is
+    counted by the CTAs as they leave.  Odd numbers of launches on grids of 148, 4 and 100 CTAs, plain and with
+    chunks, and a launch right behind one that gave up (its host status not yet read)."""
+    cfg = _small(f"turns{T}", T, 256, 384, 16, 2, zipf=1.0)
+    inp = wl.make_inputs(cfg)
+    x, lg, gu, dn = to_dev(inp)
+    moe = pk.WeaveMoE(gu, dn, cfg.E, cfg.k, cfg.S, max_tokens=cfg.T)
+    n_sm = moe.geometry()["n_sm"]
+    ref = moe.forward(x, lg).view(torch.int16).clone()
+    for sm, n in [(4, 3), (n_sm, 1), (100, 1), (4, 1), (n_sm, 3)]:
+        moe.set_sm_count(sm)
+        for i in range(n):
+            moe.set_schedule(*((pk.SCHED_FIXED, 2, 2, 1) if i == 1 else (pk.SCHED_AUTO,)))
+            assert torch.equal(moe.forward(x, lg).view(torch.int16), ref), (sm, i)
+    moe.set_schedule(pk.SCHED_AUTO)
+    moe.check()
+    moe.set_timeout_ms(20)
+    moe.debug_withhold_flag(1)
+    moe.forward(x, lg)
+    moe.debug_withhold_flag(-1)
+    moe.set_timeout_ms(4000)
+    assert torch.equal(moe.forward(x, lg).view(torch.int16), ref)
+    assert moe.status() == pk.ERR_TIMEOUT
+    assert torch.equal(moe.forward(x, lg).view(torch.int16), ref)
+    moe.check()
+    moe.close()
