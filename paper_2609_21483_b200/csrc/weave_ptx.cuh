@@ -296,6 +296,15 @@ __device__ __forceinline__ void tma_kstep_pair(uint32_t dst_a, const void *map_a
         : "memory");
 }
 
+// one of those copies by itself, issued by the calling thread
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void *map, int x, int row, uint32_t leader_bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+        ::"r"(dst), "l"(map), "r"(x), "r"(row), "r"(leader_bar)
+        : "memory");
+}
+
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t *smem_slot, uint32_t ncols)   // one warp in each CTA
 {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_slot)),
