@@ -77,7 +77,7 @@ struct CtlSet {
     unsigned x_local, x_in, x_in_uniq;   // ... the workload descriptors of Section 3.1, counted while routing
     unsigned pad[12];
     // followed by fcnt [8][256]: rows per (fine chunk, expert);
-    //             xe_ready [nmb_max]: 1 when the m-block's rows are dispatched;
+    //             xe_ready [nmb_max]: the m-block's rows that are dispatched (or kBM at once);
     //             h_ready [nmb_max]: epilogue-warp arrivals of the m-block's gemm0 tiles
 };
 static_assert(sizeof(CtlSet) == 128, "the arrays behind it start on a line of their own");
@@ -111,7 +111,7 @@ enum { kPlanSplit = 0, kPlanDispatchAll = 1, kPlanPhased = 2, kPlanRejoin = 3 };
 struct KParams {
     int T, H, I, E, S, k, EE;
     int nblk;             // 64-token blocks = ceil(T / 64): the unit of the chunks, of small batches and of the expert-parallel share
-    int lg_rb, nrb;       // routing blocks of 1 << lg_rb tokens: 64, or 32 or 16 (8) where that gives no more blocks than CTAs
+    int lg_rb, nrb;       // routing blocks of 1 << lg_rb tokens, 4 to 64: as small as one block per CTA allows
     int mode, fixed_c, fixed_K, fixed_steal;
     int nt0, nt1;         // n-tiles per m-block: I / 128, ceil(H / 256)
     int nmb_max;          // allocated length of the per-m-block flag arrays
@@ -196,7 +196,7 @@ struct SmemTail {
     int scan_w[8];
     int scan_total;
     int c, K, steal, nmb, n_gemm, n_comb;
-    int budget, die, direct;     // see gemm_phase
+    int budget, die, direct, inline_disp;     // see gemm_phase
     int elastic;                 // this launch: movement pairs take GEMM tiles beyond their quota, GEMM CTAs dispatch one m-block first
     int comb_tok;                // tokens per combine tile of this launch: 16, 8, 4, 2 or 1
     unsigned trace_n;
@@ -221,6 +221,14 @@ struct MoveScratch {
     float cgate[kCombTile][kMaxTopK + 8];
 };
 static_assert(sizeof(MoveScratch) <= kEpiStageBytes / 2, "movement scratch must fit half of the staging area");
+// ... and of the dispatch in token order: destination row and m-block of every store out of a ring buffer
+constexpr int kTokEnt = 128;
+struct TokScratch {
+    int n[kStages];                    // stores out of the buffer (-1: no more work)
+    int row[kStages][kTokEnt], mb[kStages][kTokEnt];
+};
+static_assert(sizeof(TokScratch) <= kEpiStageBytes / 2, "as the movement scratch");
+static_assert(kMaxTopK + 8 <= 32 && 32 <= kTokEnt, "a token's rows fit a buffer's list, and a warp");
 static_assert(kLocalBlocks * (kMaxEE + 1) * 8 <= kEpiStageBytes / 2, "the routing masks must fit the other half");
 static_assert(kLocalBlocks * kMaxEE * 8 <= 2048, "the masks that the direct gate/up tiles read end below the first exchange buffer");
 static_assert(kFine == 8, "chunk of a fine chunk = f >> (3 - log2 K)");
@@ -485,7 +493,7 @@ struct RouteArgs {
     int *topk_idx;
     float *gates;
 };
-// kQuad: 64-token blocks, four threads per token.  Otherwise 32, 16 or 8 tokens with 8, 16 or 32 threads each: a thread
+// kQuad: 64-token blocks, four threads per token.  Otherwise 32 to 4 tokens with 8, 16 or 32 threads each: a thread
 // then goes through E / 8 to E / 32 experts instead of E / 4 (routing of a block, staging included: E = 256, k = 8, T = 1023 12.5 -> 7.4 us, E = 128, T = 1 7.8 -> 5.8).
 template <bool kQuad>
 __device__ __forceinline__ void route_block(int lg_rb, int T, int E, int k, int ep_size, int ep_rank, int ep_tshard, int *status,
@@ -493,10 +501,10 @@ __device__ __forceinline__ void route_block(int lg_rb, int T, int E, int k, int 
                                                uint32_t r_idx, uint32_t r_cnt, uint32_t r_p, bool write_out)
 {
     static_assert(kThreads == 4 * kRouteBlock, "four threads per token of a 64-token routing block");
-    const int lg = kQuad ? 2 : 8 - lg_rb, G = 1 << lg;      // G threads per token
+    const int lg = kQuad ? 2 : min(5, 8 - lg_rb), G = 1 << lg;      // G threads per token
     const int tl = threadIdx.x >> lg, q = threadIdx.x & (G - 1);
     const int t = (b << (kQuad ? 6 : lg_rb)) + tl;
-    const bool valid = t < T;
+    const bool valid = t < T && (kQuad || tl < (1 << lg_rb));
     const int e_lo = ep_size > 1 ? ep_rank * (E / ep_size) : 0;
     const int e_hi = ep_size > 1 ? e_lo + E / ep_size : E;
     const uint32_t row = lg_s + 4u * (uint32_t)(tl * route_row_stride(E));      // this token's logits, then keys
@@ -975,7 +983,7 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
                     if (pe_mb[s8] < 0) {
                         red_release_add_u32(&S.cs->pull_done, 1u);      // a block of remote tokens is staged
                     } else {
-                        if (pe_mb[s8] != p.withhold_mb) st_release_u32(&S.xe_ready[pe_mb[s8]], 1u);
+                        if (pe_mb[s8] != p.withhold_mb) st_release_u32(&S.xe_ready[pe_mb[s8]], (unsigned)kBM);
                         trace_ev(p, S, kEvDispatch, (unsigned)pe_mb[s8], pe_t0[s8], trace_now(p), (unsigned)pe_rows[s8]);
                     }
                     ++pe_head;
@@ -1019,6 +1027,180 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
             publish_upto(n);
         }
         __syncwarp();
+    }
+    __syncthreads();
+}
+
+// The dispatch in token order, for the plans in which every CTA dispatches and nothing is staged: a token's row of x is
+// read once and written to its k + S rows of Xe.  (In m-block order every row was read for each of its experts, from HBM
+// where x does not fit L2, an m-block's 128 rows were one SM's chain of copies, and nothing began before the
+// permutation of ALL tokens was final.)  The m-blocks' ready flags count their rows in.
+__device__ __forceinline__ void publish_row(const KParams &p, SmemTail &S, int mb, unsigned long long t0)
+{
+    if (mb == p.withhold_mb) return;
+    if (p.trace == nullptr) {
+        red_release_add_u32(&S.xe_ready[mb], 1u);
+    } else {      // the timeline has one record per m-block, made by whoever completes it
+        const unsigned before = atom_acqrel_add_u32(&S.xe_ready[mb], 1u);
+        int row0, nrows, seg;
+        decode_mblock(S, p.EE, mb, row0, nrows, seg);
+        if ((int)before + 1 == nrows) trace_ev(p, S, kEvDispatch, (unsigned)mb, t0, trace_now(p), (unsigned)nrows);
+    }
+}
+__device__ __forceinline__ int mblock_of(const SmemTail &S, int row, int e)      // K = 1: segment = expert
+{
+    return S.seg_mb0[e] + (row - S.seg_row0[e]) / kBM;
+}
+
+// Small batches (a few tokens per CTA): warps that have no work yet when the GEMM phase begins - the releasing warp and
+// the epilogue warps, wid = 0..kInlineWarps-1 - copy the rows with ordinary loads and stores, while the producers
+// already fetch the first tiles' weights.  Nothing stands in front of the GEMM phase then (8 experts, T = 256: 39.2 ->
+// 35.2 us; DSv2-Lite-shaped, T = 256: 214.3 -> 211.2; Qwen3.5-35B-shaped, T = 1023: 315.7 -> 310.2).
+//   one routing block (T <= 64, every CTA has all masks): unit = a token and a share of its experts, spread over all CTAs;
+//   otherwise: this CTA's own routing block, whose rows it placed itself.
+constexpr int kInlineWarps = 5;
+__device__ __forceinline__ void dispatch_inline(const KParams &p, SmemTail &S, uint8_t *stages, int wid)
+{
+    const int lane = threadIdx.x & 31, kk = p.k + p.S, n_sm = (int)gridDim.x;
+    const unsigned long long td0 = trace_now(p);
+    const bool local = p.nblk <= kLocalBlocks;
+    const unsigned long long *mask = reinterpret_cast<const unsigned long long *>(stages + kStages * kStageBytes);
+    const int parts = local ? max(1, min(kk, n_sm * kInlineWarps / p.T)) : 1;
+    const int unit0 = local ? (int)blockIdx.x * kInlineWarps + wid : wid;
+    const int units = local ? p.T * parts : 1 << p.lg_rb, step = local ? n_sm * kInlineWarps : kInlineWarps;
+    for (int w = unit0; w < units; w += step) {
+        const int t = local ? w % p.T : ((int)blockIdx.x << p.lg_rb) + w, part = local ? w / p.T : 0;
+        if (t >= p.T) break;
+        int n = 0, row = 0, mb = 0;      // lane i: the i-th destination of this unit and its m-block
+        if (local) {
+            int seen = 0;
+            for (int e0 = 0; e0 < p.EE; e0 += 32) {
+                const int e = e0 + lane;
+                unsigned all = __ballot_sync(0xffffffffu, e < p.EE && (e >= p.E || ((mask[e] >> t) & 1ull)));
+                for (; all; all &= all - 1u, ++seen) {
+                    if (seen % parts != part) continue;
+                    const int es = e0 + __ffs((int)all) - 1;
+                    if (lane == n) {
+                        row = S.offsets[es] + (es < p.E ? __popcll(mask[es] & ((1ull << t) - 1ull)) : t);
+                        mb = mblock_of(S, row, es);
+                    }
+                    ++n;
+                }
+            }
+        } else {
+            n = kk;
+            if (lane < p.k) {
+                const size_t at = (size_t)t * p.k + lane;
+                row = __ldcg(p.row_of + at);
+                mb = mblock_of(S, row, __ldcg(p.topk_idx + at));
+            } else if (lane < kk) {
+                row = S.offsets[p.E + lane - p.k] + t;
+                mb = mblock_of(S, row, p.E + lane - p.k);
+            }
+        }
+        const uint4 *src = reinterpret_cast<const uint4 *>(p.x + (size_t)t * p.H);
+        const int vecs = p.H >> 3;      // a multiple of 16
+        for (int v0 = 0; v0 < vecs; v0 += 128) {
+            uint4 q[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (v0 + 32 * i + lane < vecs) q[i] = __ldg(src + v0 + 32 * i + lane);
+            for (int j = 0; j < n; ++j) {
+                uint4 *dst = reinterpret_cast<uint4 *>(p.xe + (size_t)__shfl_sync(0xffffffffu, row, j) * p.H);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (v0 + 32 * i + lane < vecs) dst[v0 + 32 * i + lane] = q[i];
+            }
+        }
+        __syncwarp();      // the rows are written; the release below is cumulative
+        if (lane < n) {
+            fence_proxy_async_global();      // (TMA reads them)
+            publish_row(p, S, mb, td0);
+        }
+    }
+    __syncwarp();
+}
+
+// Large batches, 16-token tiles from the queue: bulk loads bring as many tokens as fit a 32 KB ring buffer (they are
+// neighbours in x: one copy); the lanes of the storing warp write each row out with one bulk store per destination and
+// publish it once those stores have completed, two buffers later.  Bound by HBM writes; T = 16384, H = 4096, k = 8:
+// 310 -> 230 us.
+__device__ __forceinline__ void dispatch_tokens(const KParams &p, SmemTail &S, uint8_t *stages)
+{
+    TokScratch &M = *reinterpret_cast<TokScratch *>(stages + kStages * kStageBytes + kEpiStageBytes / 2);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, n_sm = (int)gridDim.x;
+    fence_proxy_async_shared();      // the buffers held routing scratch written with ordinary stores
+    __syncthreads();
+    const uint32_t rowb = (uint32_t)p.H * 2u;
+    const int kk = p.k + p.S;
+    const int per_buf = min(kMvBuf / (int)rowb, kTokEnt / kk);      // tokens per buffer (at least 1: H <= 16384, kk <= 24)
+    if (warp == 0) {
+        // ---- loader
+        int b = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        if (lane == 0) ok = flag_wait_ge(&S.cs->fix_done, (unsigned)p.nrb, p, 10);
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        const int ntile = (p.T + 15) / 16;
+        for (int q = (int)blockIdx.x; ok && q < ntile;) {
+            const int t1 = min(p.T, q * 16 + 16);
+            for (int t = q * 16; t < t1; t += per_buf) {
+                const int nt = min(per_buf, t1 - t), n = nt * kk;
+                ok = __all_sync(0xffffffffu, mbar_wait(&S.dv_empty[b], ph ^ 1u, p, 11));
+                if (!ok) break;
+                for (int i = lane; i < n; i += 32) {
+                    const int tt = i / kk, j = i - tt * kk;
+                    const size_t at = (size_t)(t + tt) * p.k + j;
+                    const int row = j < p.k ? __ldcg(p.row_of + at) : S.offsets[p.E + j - p.k] + t + tt;
+                    M.row[b][i] = row;
+                    M.mb[b][i] = mblock_of(S, row, j < p.k ? __ldcg(p.topk_idx + at) : p.E + j - p.k);
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    M.n[b] = n;
+                    mbar_arrive_expect_tx(&S.dv_full[b], (uint32_t)nt * rowb);
+                    bulk_load(smem_u32(stages + b * kMvBuf), p.x + (size_t)t * p.H, (uint32_t)nt * rowb, &S.dv_full[b]);
+                }
+                if (++b == kStages) { b = 0; ph ^= 1u; }
+            }
+            if (lane == 0) q = n_sm + (int)atomicAdd(&S.cs->q_disp, 1u);
+            q = __shfl_sync(0xffffffffu, q, 0);
+        }
+        if (ok && __all_sync(0xffffffffu, mbar_wait(&S.dv_empty[b], ph ^ 1u, p, 12))) {
+            if (lane == 0) { M.n[b] = -1; mbar_arrive(&S.dv_full[b]); }
+        } else if (lane == 0) linger_after_abort();      // copies of this warp may still be landing in this CTA's buffers
+        __syncwarp();
+    } else if (warp == 1) {
+        // ---- storer
+        constexpr int kLag = 2;
+        int b = 0, n_buf = 0;
+        uint32_t ph = 0;
+        const unsigned long long td0 = trace_now(p);
+        auto publish = [&](int buf) {      // the stores out of `buf` have completed
+            fence_proxy_async_global();
+            const int n = M.n[buf];
+            for (int i = lane; i < n; i += 32) publish_row(p, S, M.mb[buf][i], td0);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&S.dv_empty[buf]);
+        };
+        bool ok = true;
+        for (;;) {
+            ok = __all_sync(0xffffffffu, mbar_wait(&S.dv_full[b], ph, p, 13));
+            if (!ok) break;
+            const int n = M.n[b];
+            if (n < 0) break;
+            const uint32_t src = smem_u32(stages + b * kMvBuf);
+            for (int i = lane; i < n; i += 32)
+                bulk_store(p.xe + (size_t)M.row[b][i] * p.H, src + (uint32_t)(i / kk) * rowb, rowb);
+            bulk_commit();
+            if (n_buf >= kLag) { bulk_wait<kLag>(); publish(b >= kLag ? b - kLag : b + kStages - kLag); }
+            ++n_buf;
+            if (++b == kStages) { b = 0; ph ^= 1u; }
+        }
+        bulk_wait<0>();
+        __syncwarp();
+        if (ok)
+            for (int i = min(n_buf, kLag); i > 0; --i) publish(b >= i ? b - i : b + kStages - i);
     }
     __syncthreads();
 }
@@ -1267,6 +1449,8 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
     fence_proxy_async_shared();     // the stage buffers were last touched by ordinary stores (routing scratch)
     __syncthreads();
 
+    if (S.inline_disp && warp >= 8 - kInlineWarps) dispatch_inline(p, S, stages, warp - (8 - kInlineWarps));
+
     if (warp == 2 && rank == 0) {
         // ---------------- scheduler (leader only): claims pair tiles in queue order, waits until their
         // inputs are ready, then publishes the tile to both CTAs' descriptor rings.  Runs up to
@@ -1301,9 +1485,9 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 const bool g0 = tl.type == 0 || tl.type == 3;
                 const unsigned *fl = tl.type == 2 ? nullptr : (g0 ? S.xe_ready : S.h_ready) + tl.mb;
                 const unsigned *fp = two ? (g0 ? S.xe_ready : S.h_ready) + tp.mb : fl;
-                const unsigned need = g0 ? 1u : (unsigned)(p.nt0 * kEpiWarps);
+                const unsigned need = g0 ? (unsigned)tl.nrows : (unsigned)(p.nt0 * kEpiWarps), need_p = g0 ? (unsigned)tp.nrows : need;
                 const bool waits = tl.type != 2 && !(S.direct && tl.type == 3);      // (x was there before the launch)
-                const bool late = waits && (ld_acquire_u32(fl) < need || (two && ld_acquire_u32(fp) < need));
+                const bool late = waits && (ld_acquire_u32(fl) < need || (two && ld_acquire_u32(fp) < need_p));
                 if (late) { tl.chunk |= kTileLate; tp.chunk |= kTileLate; }
                 if (!mbar_wait(&S.ti_empty[ps.slot], ps.slot_phase ^ 1u, p, 30)) break;
                 S.ti[ps.slot] = tl;
@@ -1321,7 +1505,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 mbar_arrive_cluster(mapa_u32(smem_u32(&S.ti_full[ps.slot]), 1u));
                 if (late) {
                     const int where = g0 ? 31 : 32;
-                    if (!flag_wait_ge(fl, need, p, where) || (two && !flag_wait_ge(fp, need, p, where))) break;
+                    if (!flag_wait_ge(fl, need, p, where) || (two && !flag_wait_ge(fp, need_p, p, where))) break;
                     fence_proxy_async_global();
                     mbar_arrive(&S.ti_late[ps.slot]);
                     mbar_arrive_cluster(mapa_u32(smem_u32(&S.ti_late[ps.slot]), 1u));
@@ -1719,29 +1903,6 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
         // ---------------- releasing warp (both CTAs): makes the tiles' arrivals on the ready counters
         int rs = 0;
         uint32_t rph = 0;
-        if (S.direct) {
-            // nothing reads the dispatched rows here, but the caller may ask for them: token t's row of x goes to its
-            // rows of Xe, the token's experts spread over `parts` CTAs
-            const unsigned long long *mask = reinterpret_cast<const unsigned long long *>(stages + kStages * kStageBytes);
-            const int parts = max(1, (int)gridDim.x / p.T), vecs = p.H >> 3;
-            for (int w = blockIdx.x; w < p.T * parts; w += gridDim.x) {
-                const int t = w % p.T;
-                int n = 0;
-                for (int e0 = 0; e0 < p.EE; e0 += 32) {
-                    const int e = e0 + lane;
-                    unsigned mine = __ballot_sync(0xffffffffu, e < p.EE && (e >= p.E || ((mask[e] >> t) & 1ull)));
-                    for (; mine; mine &= mine - 1u, ++n) {
-                        if (n % parts != w / p.T) continue;
-                        const int es = e0 + __ffs((int)mine) - 1;
-                        const int r = S.offsets[es] + (es < p.E ? __popcll(mask[es] & ((1ull << t) - 1ull)) : t);
-                        const uint4 *src = reinterpret_cast<const uint4 *>(p.x + (size_t)t * p.H);
-                        uint4 *dst = reinterpret_cast<uint4 *>(p.xe + (size_t)r * p.H);
-#pragma unroll 4
-                        for (int i = lane; i < vecs; i += 32) dst[i] = __ldg(src + i);
-                    }
-                }
-            }
-        }
         while (true) {
             if (!mbar_wait(&S.rel_full[rs], rph, p, 57)) break;
             unsigned *flag = S.rel_flag[rs];
@@ -2127,15 +2288,15 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
                     const int bstart = ((f * p.nblk + kFine - 1) / kFine) << (6 - p.lg_rb);
 #pragma unroll
                     for (int ff = 0; ff < kFine; ++ff) if (ff < f) base += cf[ff];
-#pragma unroll 4
+#pragma unroll 8
                     for (int bb = bstart; bb < b; ++bb) base += __ldcg(p.hist + (size_t)bb * kMaxEE + tid);
                 }
                 r_base[tid] = base;
             }
             __syncthreads();
             // the threads that routed a token place its rows (no divisions: this stands between routing and dispatch)
-            const int lg = 8 - p.lg_rb, tl = tid >> lg, t = (b << p.lg_rb) + tl;
-            if (t < p.T) {
+            const int lg = min(5, 8 - p.lg_rb), tl = tid >> lg, t = (b << p.lg_rb) + tl;
+            if (t < p.T && tl < (1 << p.lg_rb)) {
                 for (int j = tid & ((1 << lg) - 1); j < p.k; j += 1 << lg) {
                     const size_t at = (size_t)t * p.k + j;
                     const int e = from_smem ? idx_b[tl * kMaxTopK + j] : __ldcg(p.topk_idx + at);
@@ -2177,14 +2338,23 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         // A batch of at most 32 tokens under the phased plan: N = T columns cost a swapped tile's MMA no more than the
         // expert's few rows do (an instruction takes 48 cycles up to N = 64, and the weights set the pace), so the
         // gate/up tiles multiply ALL tokens, straight from x, and their epilogue keeps the expert's rows.  Nothing waits
-        // for a dispatch then (4-5 us); the GEMM phase's releasing warps write Xe, for whoever asks for it, before
-        // they have tiles to release.  T = 1 Qwen3-30B-shaped 46.8 -> 40.3 us, T = 7 DSv2-Lite-shaped 119.1 -> 112.7,
+        // for the dispatch then (4-5 us).  T = 1 Qwen3-30B-shaped 46.8 -> 40.3 us, T = 7 DSv2-Lite-shaped 119.1 -> 112.7,
         // T = 27 149.4 -> 146.7.  At T = 64 a launch by itself gains as much (199.9 -> 197.8) but under load the
         // additional columns and rows cost power (202.8 -> 205.9 after half a second): hence the limit.
         const bool direct = p.direct && plan_kind == kPlanPhased;
         const int budget = (mover && plan_kind != kPlanPhased) ? plan_steal : 0x7fffffff;
-        if (tid == 0) { S.budget = budget; S.die = die; S.direct = direct ? 1 : 0; }      // (published by gemm_phase's first barrier)
-        if (dmax > 0 && !direct) dispatch_phase(p, S, stages, dmax, n_disp, p.nblk <= kLocalBlocks);
+        const bool by_token = !two_roles && S.K == 1 && !ep;
+        const bool in_gemm = by_token && p.nrb <= n_sm && (p.lg_rb <= 4 || p.nblk <= kLocalBlocks);      // few tokens per CTA
+        if (tid == 0) {      // (published by gemm_phase's first barrier)
+            S.budget = budget; S.die = die; S.direct = direct ? 1 : 0;
+            S.inline_disp = in_gemm && !serial ? 1 : 0;
+        }
+        if (by_token) {
+            if (!in_gemm) dispatch_tokens(p, S, stages);
+            else if (serial && warp >= 8 - kInlineWarps) dispatch_inline(p, S, stages, warp - (8 - kInlineWarps));
+        } else if (dmax > 0) {
+            dispatch_phase(p, S, stages, dmax, n_disp, p.nblk <= kLocalBlocks);
+        }
         if (serial) alive = grid_barrier(p, S, bar0 + (unsigned)n_sm, 2);
         if (alive && (budget > 0 || S.elastic)) {
             gemm_phase(p, S, stages, &tm);

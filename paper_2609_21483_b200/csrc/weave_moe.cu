@@ -361,12 +361,13 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     p.T = T; p.H = c.hidden; p.I = c.ffn; p.E = c.num_experts; p.S = c.num_shared; p.k = c.top_k;
     p.EE = c.num_experts + c.num_shared;
     p.nblk = (T + kRouteBlock - 1) / kRouteBlock;
-    // Routing blocks of 16 or 32 tokens, with 16 or 8 threads per token, while each still has a CTA to itself (an
-    // expert-parallel share stages its remote tokens by 64).  A batch of at most 64 tokens is one block, routed by every
-    // CTA for itself, with as many threads per token as there are.
+    // Routing blocks of 4 to 32 tokens, with up to 32 threads per token, while each still has a CTA to itself (an
+    // expert-parallel share stages its remote tokens by 64).  Below 4 the fix-up's sum over the blocks of a fine chunk
+    // (at most 16 rows of the histogram from 4 on) would take longer than the routing saves.  A batch of at most 64
+    // tokens is one block, routed by every CTA for itself, with as many threads per token as there are.
     p.lg_rb = 6;
     if (p.nblk <= kLocalBlocks) p.lg_rb = T <= 8 ? 3 : T <= 16 ? 4 : T <= 32 ? 5 : 6;
-    else if (h->ep_size == 1) p.lg_rb = T <= 16 * h->n_cta ? 4 : T <= 32 * h->n_cta ? 5 : 6;
+    else if (h->ep_size == 1) for (p.lg_rb = 2; p.lg_rb < 6 && T > (h->n_cta << p.lg_rb);) ++p.lg_rb;
     p.nrb = (T + (1 << p.lg_rb) - 1) >> p.lg_rb;
     p.mode = h->mode; p.fixed_c = h->fixed_c; p.fixed_K = h->fixed_K; p.fixed_steal = h->fixed_steal;
     p.nt0 = c.ffn / kTN0;

@@ -614,3 +614,21 @@ def test_control_word_sets_take_turns_whatever_the_grid(T):
     assert torch.equal(moe.forward(x, lg).view(torch.int16), ref)
     moe.check()
     moe.close()
+
+
+@pytest.mark.parametrize("T", [33, 64, 65, 592, 593, 1184, 1185, 2368, 2369, 2400])
+@pytest.mark.parametrize("H,k,S", [(128, 1, 0), (1152, 3, 2), (16384, 2, 0), (256, 16, 8)])
+def test_dispatch_in_token_order(T, H, k, S):
+    """Token rows of 256 bytes to 32 KB, one to 24 destinations each, copied by idle warps of the GEMM phase (small
+    batches: shares of a token's experts, or the CTA's own routing block of 4 to 16 tokens) or by the bulk-copy
+    ring (from 2369 tokens on, 16-token tiles with a remainder).  Xe row by row, output on a sample; the same
+    bits as the m-block order that the chunked schedule uses."""
+    cfg = _small(f"tok_T{T}_H{H}_k{k}", T, H, 128, 24, k, S, zipf=0.8, cfg_id=980 + k)
+    inp = wl.make_inputs(cfg)
+    dev = to_dev(inp)
+    moe, out, _ = run_case(cfg, inp=inp, dev_tensors=dev, n_sample=8, budget=24)
+    xe, tok = moe.intermediates(T)["xe"].view(torch.int16), moe.routing(T)["token_of"].long()
+    assert torch.equal(xe, dev[0].view(torch.int16)[tok])
+    _, chunked, _ = run_case(cfg, sched=(pk.SCHED_FIXED, 20, 2, 1), inp=inp, dev_tensors=dev, moe=moe, n_sample=4, budget=8)
+    assert torch.equal(out.view(torch.int16), chunked.view(torch.int16))
+    moe.close()
