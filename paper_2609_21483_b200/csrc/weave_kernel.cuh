@@ -20,6 +20,8 @@
 #pragma once
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "weave_ptx.cuh"
 
 namespace weave {
@@ -32,7 +34,7 @@ constexpr int kStages = 6;
 constexpr int kStageA = kBM * kBK * 2;                  // 16 KB: this CTA's 128 rows of A
 constexpr int kStageB = 128 * kBK * 2;                  // 16 KB: this CTA's half (128 rows) of the 256-row B tile
 constexpr int kStageBytes = kStageA + kStageB;          // 32 KB
-constexpr int kEpiStageBytes = 4 * 4096;                // epilogue staging, per warp: 32 rows x 64 bytes, and two 1 KB exchange buffers
+constexpr int kEpiStageBytes = 4 * 4096;                // epilogue staging, per warp: 32 rows x 64 bytes (regular tiles); two 2 KB exchange buffers (swapped ones)
 constexpr int kRouteBlock = 64;  // tokens per routing block (one 64-bit mask per expert)
 constexpr int kLocalBlocks = 1;  // a batch of at most this many routing blocks is routed by every CTA for itself
                                  // (measured at two blocks: routing both in every CTA costs more than the grid barrier saves)
@@ -77,8 +79,8 @@ struct CtlSet {
     unsigned x_local, x_in, x_in_uniq;   // ... the workload descriptors of Section 3.1, counted while routing
     unsigned pad[12];
     // followed by fcnt [8][256]: rows per (fine chunk, expert);
-    //             xe_ready [nmb_max]: the m-block's rows that are dispatched (or kBM at once);
-    //             h_ready [nmb_max]: epilogue-warp arrivals of the m-block's gemm0 tiles
+    //             xe_ready [nmb_max]: the row tile's rows that are dispatched;
+    //             h_ready [nmb_max]: epilogue-warp arrivals of the row tile's gemm0 tiles
 };
 static_assert(sizeof(CtlSet) == 128, "the arrays behind it start on a line of their own");
 __host__ __device__ __forceinline__ size_t ctl_set_bytes(int nmb_max)
@@ -153,11 +155,12 @@ struct KParams {
 };
 
 struct TileInfo {
-    int type;   // 0 gemm0 (+SwiGLU), 1 gemm1, 2 no more tiles; 3 / 4 = gemm0 / gemm1 of a single m-block
-                // with the operands swapped (weights on the MMA's M axis, the m-block's rows on N)
-    int mb;     // this CTA's m-block (-1: the pair tile has no second half)
-    int row0;   // first row of this CTA's 128 rows of A
-    int nrows;  // valid rows (0 for a missing half)
+    int type;   // 0 gemm0 (+SwiGLU), 1 gemm1 of 256 rows, 2 no more tiles; 3 / 4 = gemm0 / gemm1 of a row tile of fewer
+                // rows, with the operands swapped (weights on the MMA's M axis, the tile's rows on N)
+    int mb;     // the m-block that this CTA's records name (row tile i of a segment stands for its m-blocks 2i, 2i + 1)
+    int rt;     // row tile: the index of its ready flags
+    int row0;   // first row of this CTA's 128 rows (regular) or of the tile (swapped)
+    int nrows;  // valid rows from there
     int e, n, chunk, nkb;      // chunk | kTileLate: handed over before the tile's rows are there
 };
 constexpr int kTileLate = 256;
@@ -202,7 +205,6 @@ struct SmemTail {
     unsigned trace_n;
     int chunk_mb0[kFine + 1];
     int chunk_pt0[kFine + 1];
-    int chunk_nswap[kFine];      // per chunk: segments with an odd number of m-blocks
     int chunk_tile0[kFine + 1];
     int split_pt, split_seg;     // K = 1: pair tiles [0, split_pt) = segments [0, split_seg) are list 0, the rest list 1
     int offsets[kMaxEE + 1];
@@ -221,11 +223,11 @@ struct MoveScratch {
     float cgate[kCombTile][kMaxTopK + 8];
 };
 static_assert(sizeof(MoveScratch) <= kEpiStageBytes / 2, "movement scratch must fit half of the staging area");
-// ... and of the dispatch in token order: destination row and m-block of every store out of a ring buffer
+// ... and of the dispatch in token order: destination row and row tile of every store out of a ring buffer
 constexpr int kTokEnt = 128;
 struct TokScratch {
     int n[kStages];                    // stores out of the buffer (-1: no more work)
-    int row[kStages][kTokEnt], mb[kStages][kTokEnt];
+    int row[kStages][kTokEnt], rt[kStages][kTokEnt];
 };
 static_assert(sizeof(TokScratch) <= kEpiStageBytes / 2, "as the movement scratch");
 static_assert(kMaxTopK + 8 <= 32 && 32 <= kTokEnt, "a token's rows fit a buffer's list, and a warp");
@@ -354,7 +356,7 @@ __device__ __forceinline__ void linger_after_abort()
 }
 
 // All CTAs are co-resident (cooperative launch); arrivals accumulate over the barriers of a launch.
-// Three exclusive scans in one pass: v = a | b << 24 | c << 48 with a, b < 2^24 and c < 2^16 in total.
+// Two exclusive scans in one pass: v = a | b << 32.
 __device__ __forceinline__ unsigned long long block_excl_scan_packed(unsigned long long v, SmemTail &S, unsigned long long &total)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -734,14 +736,33 @@ __device__ __forceinline__ void decode_mblock(const SmemTail &S, int EE, int mb,
     nrows = min(kBM, S.seg_rows[s] - m * kBM);
 }
 
+// A segment of R rows is worked on as ceil(R / 256) row tiles of almost equal size, in units of 16 rows (the MMA's N comes
+// in sixteens): the first ones have a unit more.  A tile of 256 rows runs as a regular tile, rows on the MMA's M axis;
+// any other runs swapped, weights on M and its 16 to 240 rows on N, so that it costs what its rows cost.  (With regular
+// tiles of 256 rows and a swapped one for the rest, eight rows over a multiple of 256 cost two thirds of a tile for
+// every panel of weights: Mixtral-shaped layer, T = 4096, 1014-1049 rows per expert 2117 us, 1024 each 1923.)
+__host__ __device__ __forceinline__ void rowtile_span(int rows, int pts, int i, int &first, int &n)
+{
+    const int units = (rows + 15) >> 4, q = units / pts, r = units - q * pts;
+    const int u0 = i * q + (i < r ? i : r), nu = q + (i < r ? 1 : 0);
+    first = u0 << 4;
+    n = nu << 4;
+    if (first + n > rows) n = rows - first;
+}
+// the row tile that row `rel` of a segment belongs to
+__host__ __device__ __forceinline__ int rowtile_of_rel(int rows, int pts, int rel)
+{
+    if (pts <= 1) return 0;
+    const int units = (rows + 15) >> 4, q = units / pts, r = units - q * pts, u = rel >> 4;
+    return u < r * (q + 1) ? u / (q + 1) : r + (u - r * (q + 1)) / q;
+}
+
 // GEMM queue order (the chunk-pipeline DAG order): chunk by chunk; inside a chunk all gemm0 tiles,
 // then all gemm1 tiles (every gemm0 tile a gemm1 tile waits for comes earlier in the queue and waits
 // only for dispatch, which keeps the in-order schedulers free of deadlock); inside those
 // expert-major, then groups of kPairGroup pair tiles, n-tile, pair tile fastest: consecutive tiles
-// share a weight panel, and a group's rows stay in L2 while all its n-tiles pass.  A pair tile = two
-// consecutive m-blocks of one segment; a segment's last, unpaired m-block is a member of its group
-// like any other pair tile (operands swapped), so it reads each weight panel right beside the
-// expert's regular tiles.  `lead` describes the leader CTA's half, `peer` the other CTA's.
+// share a weight panel, and a group's rows stay in L2 while all its n-tiles pass.  A pair tile = one row tile of a
+// segment, for one n-tile.  `lead` describes the leader CTA's half, `peer` the other CTA's.
 // Two other orders were measured and dropped: spreading the swapped tiles evenly over the queue
 // (no faster, and a large expert's panels were fetched a second time for its last m-block: +27 %
 // DRAM traffic on the Mixtral-shaped layer), and alternating gemm1 with gemm0 units (+1 % at
@@ -780,33 +801,34 @@ __host__ __device__ __forceinline__ void decode_pair_tile(const SmemTail &S, con
     const int wg = within - gi * kPairGroup * nt;
     const int gsize = (pts - gi * kPairGroup) < kPairGroup ? (pts - gi * kPairGroup) : kPairGroup;
     const int n = wg / gsize;
-    const int m0 = 2 * (gi * kPairGroup + (wg - n * gsize));
-    const int rows = S.seg_rows[s];
-    lead.type = peer.type = type;
-    lead.e = peer.e = s - j * p.EE;
-    lead.n = peer.n = n;
-    lead.chunk = peer.chunk = j;
-    lead.nkb = peer.nkb = (type == 0 ? p.H : p.I) / kBK;
-    lead.mb = S.seg_mb0[s] + m0;
-    lead.row0 = S.seg_row0[s] + m0 * kBM;
-    lead.nrows = (rows - m0 * kBM) < kBM ? (rows - m0 * kBM) : kBM;
-    if (rows - (m0 + 1) * kBM <= 0) {
-        // the segment's last, unpaired m-block: both CTAs work on it with the operands swapped,
-        // so the MMA costs ceil(nrows/16)*16 columns instead of a half-empty 256-row tile
-        lead.type = type + 3;
-        peer = lead;
-        return;
+    const int ti = gi * kPairGroup + (wg - n * gsize);
+    const int rows = S.seg_rows[s], mbs = S.seg_mb0[s + 1] - S.seg_mb0[s];
+    int first, nr;
+    rowtile_span(rows, pts, ti, first, nr);
+    lead.type = type;
+    lead.e = s - j * p.EE;
+    lead.n = n;
+    lead.chunk = j;
+    lead.nkb = (type == 0 ? p.H : p.I) / kBK;
+    lead.rt = S.seg_pt0[s] + ti;
+    lead.mb = S.seg_mb0[s] + 2 * ti;
+    lead.row0 = S.seg_row0[s] + first;
+    lead.nrows = nr;
+    const bool regular = nr > 240;      // 16 units, the last of them perhaps not full
+    if (!regular) lead.type = type + 3;
+    peer = lead;
+    if (2 * ti + 1 < mbs) peer.mb = lead.mb + 1;
+    if (regular) {
+        lead.nrows = kBM;
+        peer.row0 += kBM;
+        peer.nrows -= kBM;
     }
-    peer.nrows = (rows - (m0 + 1) * kBM) < kBM ? (rows - (m0 + 1) * kBM) : kBM;
-    peer.mb = lead.mb + 1;
-    peer.row0 = lead.row0 + kBM;
 }
 
-// epilogue-warp arrivals on y_done[j] when all gemm1 tiles of chunk j are finished: 4 per (m-block,
-// n-tile); an m-block processed as a swapped tile is finished by both CTAs of the pair (8)
+// epilogue-warp arrivals on y_done[j] when all gemm1 tiles of chunk j are finished: both CTAs' warps for every tile
 __device__ __forceinline__ unsigned y_done_target(const SmemTail &S, const KParams &p, int j)
 {
-    return (unsigned)(((S.chunk_mb0[j + 1] - S.chunk_mb0[j]) + S.chunk_nswap[j]) * p.nt1 * kEpiWarps);
+    return (unsigned)((S.chunk_pt0[j + 1] - S.chunk_pt0[j]) * p.nt1 * 2 * kEpiWarps);
 }
 
 // ------------------------------------------------------------------------------------ phase A: dispatch
@@ -983,7 +1005,17 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
                     if (pe_mb[s8] < 0) {
                         red_release_add_u32(&S.cs->pull_done, 1u);      // a block of remote tokens is staged
                     } else {
-                        if (pe_mb[s8] != p.withhold_mb) st_release_u32(&S.xe_ready[pe_mb[s8]], (unsigned)kBM);
+                        if (pe_mb[s8] != p.withhold_mb) {      // the m-block's rows count in on the row tiles they are part of
+                            int row0, nrows, seg;
+                            decode_mblock(S, p.EE, pe_mb[s8], row0, nrows, seg);
+                            const int rows = S.seg_rows[seg], pts = S.seg_pt0[seg + 1] - S.seg_pt0[seg], rel = row0 - S.seg_row0[seg];
+                            for (int i = rowtile_of_rel(rows, pts, rel); i < pts; ++i) {
+                                int first, n;
+                                rowtile_span(rows, pts, i, first, n);
+                                if (first >= rel + nrows) break;
+                                red_release_add_u32(&S.xe_ready[S.seg_pt0[seg] + i], (unsigned)(min(first + n, rel + nrows) - max(first, rel)));
+                            }
+                        }
                         trace_ev(p, S, kEvDispatch, (unsigned)pe_mb[s8], pe_t0[s8], trace_now(p), (unsigned)pe_rows[s8]);
                     }
                     ++pe_head;
@@ -1034,22 +1066,31 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
 // The dispatch in token order, for the plans in which every CTA dispatches and nothing is staged: a token's row of x is
 // read once and written to its k + S rows of Xe.  (In m-block order every row was read for each of its experts, from HBM
 // where x does not fit L2, an m-block's 128 rows were one SM's chain of copies, and nothing began before the
-// permutation of ALL tokens was final.)  The m-blocks' ready flags count their rows in.
-__device__ __forceinline__ void publish_row(const KParams &p, SmemTail &S, int mb, unsigned long long t0)
+// permutation of ALL tokens was final.)  The row tiles' ready flags count their rows in.
+__device__ __forceinline__ void publish_row(const KParams &p, SmemTail &S, int rt, unsigned long long t0)
 {
-    if (mb == p.withhold_mb) return;
+    if (rt == p.withhold_mb) return;
     if (p.trace == nullptr) {
-        red_release_add_u32(&S.xe_ready[mb], 1u);
-    } else {      // the timeline has one record per m-block, made by whoever completes it
-        const unsigned before = atom_acqrel_add_u32(&S.xe_ready[mb], 1u);
-        int row0, nrows, seg;
-        decode_mblock(S, p.EE, mb, row0, nrows, seg);
-        if ((int)before + 1 == nrows) trace_ev(p, S, kEvDispatch, (unsigned)mb, t0, trace_now(p), (unsigned)nrows);
+        red_release_add_u32(&S.xe_ready[rt], 1u);
+    } else {      // the timeline has one record per m-block, made by whoever completes its row tile
+        const unsigned before = atom_acqrel_add_u32(&S.xe_ready[rt], 1u);
+        int lo = 0, hi = p.EE;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (S.seg_pt0[mid] <= rt) lo = mid; else hi = mid;
+        }
+        const int i = rt - S.seg_pt0[lo], mb = S.seg_mb0[lo] + 2 * i;
+        int first, n;
+        rowtile_span(S.seg_rows[lo], S.seg_pt0[lo + 1] - S.seg_pt0[lo], i, first, n);
+        if ((int)before + 1 == n) {
+            trace_ev(p, S, kEvDispatch, (unsigned)mb, t0, trace_now(p), (unsigned)n);
+            if (mb + 1 < S.seg_mb0[lo + 1]) trace_ev(p, S, kEvDispatch, (unsigned)(mb + 1), t0, trace_now(p), 0u);
+        }
     }
 }
-__device__ __forceinline__ int mblock_of(const SmemTail &S, int row, int e)      // K = 1: segment = expert
+__device__ __forceinline__ int rowtile_of(const SmemTail &S, int row, int e)      // K = 1: segment = expert
 {
-    return S.seg_mb0[e] + (row - S.seg_row0[e]) / kBM;
+    return S.seg_pt0[e] + rowtile_of_rel(S.seg_rows[e], S.seg_pt0[e + 1] - S.seg_pt0[e], row - S.seg_row0[e]);
 }
 
 // Small batches (a few tokens per CTA): warps that have no work yet when the GEMM phase begins - the releasing warp and
@@ -1071,7 +1112,7 @@ __device__ __forceinline__ void dispatch_inline(const KParams &p, SmemTail &S, u
     for (int w = unit0; w < units; w += step) {
         const int t = local ? w % p.T : ((int)blockIdx.x << p.lg_rb) + w, part = local ? w / p.T : 0;
         if (t >= p.T) break;
-        int n = 0, row = 0, mb = 0;      // lane i: the i-th destination of this unit and its m-block
+        int n = 0, row = 0, rt = 0;      // lane i: the i-th destination of this unit and its row tile
         if (local) {
             int seen = 0;
             for (int e0 = 0; e0 < p.EE; e0 += 32) {
@@ -1082,7 +1123,7 @@ __device__ __forceinline__ void dispatch_inline(const KParams &p, SmemTail &S, u
                     const int es = e0 + __ffs((int)all) - 1;
                     if (lane == n) {
                         row = S.offsets[es] + (es < p.E ? __popcll(mask[es] & ((1ull << t) - 1ull)) : t);
-                        mb = mblock_of(S, row, es);
+                        rt = rowtile_of(S, row, es);
                     }
                     ++n;
                 }
@@ -1092,10 +1133,10 @@ __device__ __forceinline__ void dispatch_inline(const KParams &p, SmemTail &S, u
             if (lane < p.k) {
                 const size_t at = (size_t)t * p.k + lane;
                 row = __ldcg(p.row_of + at);
-                mb = mblock_of(S, row, __ldcg(p.topk_idx + at));
+                rt = rowtile_of(S, row, __ldcg(p.topk_idx + at));
             } else if (lane < kk) {
                 row = S.offsets[p.E + lane - p.k] + t;
-                mb = mblock_of(S, row, p.E + lane - p.k);
+                rt = rowtile_of(S, row, p.E + lane - p.k);
             }
         }
         const uint4 *src = reinterpret_cast<const uint4 *>(p.x + (size_t)t * p.H);
@@ -1115,7 +1156,7 @@ __device__ __forceinline__ void dispatch_inline(const KParams &p, SmemTail &S, u
         __syncwarp();      // the rows are written; the release below is cumulative
         if (lane < n) {
             fence_proxy_async_global();      // (TMA reads them)
-            publish_row(p, S, mb, td0);
+            publish_row(p, S, rt, td0);
         }
     }
     __syncwarp();
@@ -1153,7 +1194,7 @@ __device__ __forceinline__ void dispatch_tokens(const KParams &p, SmemTail &S, u
                     const size_t at = (size_t)(t + tt) * p.k + j;
                     const int row = j < p.k ? __ldcg(p.row_of + at) : S.offsets[p.E + j - p.k] + t + tt;
                     M.row[b][i] = row;
-                    M.mb[b][i] = mblock_of(S, row, j < p.k ? __ldcg(p.topk_idx + at) : p.E + j - p.k);
+                    M.rt[b][i] = rowtile_of(S, row, j < p.k ? __ldcg(p.topk_idx + at) : p.E + j - p.k);
                 }
                 __syncwarp();
                 if (lane == 0) {
@@ -1179,7 +1220,7 @@ __device__ __forceinline__ void dispatch_tokens(const KParams &p, SmemTail &S, u
         auto publish = [&](int buf) {      // the stores out of `buf` have completed
             fence_proxy_async_global();
             const int n = M.n[buf];
-            for (int i = lane; i < n; i += 32) publish_row(p, S, M.mb[buf][i], td0);
+            for (int i = lane; i < n; i += 32) publish_row(p, S, M.rt[buf][i], td0);
             __syncwarp();
             if (lane == 0) mbar_arrive(&S.dv_empty[buf]);
         };
@@ -1346,8 +1387,8 @@ __device__ __forceinline__ void combine_phase(const KParams &p, SmemTail &S, uin
 // ------------------------------------------------------------------------------------ phase B: GEMM
 
 // Tensor maps of the GEMM operands: bf16 matrices, boxes of 64 columns (one 128-byte swizzle row) by
-// 128 rows (64 rows for the gate and up halves of a swapped tile's weight operand; 8, 16, 32 or 64
-// rows for a swapped tile's row operand, whichever covers its half of the m-block's rows).
+// 128 rows (64 rows for the gate and up halves of a swapped tile's weight operand; 8, 16, 32 or 64 rows for its row
+// operand, whichever covers each CTA's half of the tile's rows, or what is left of it behind a first box of 64).
 // x: the input itself, boxes of half the batch's tokens rounded up to 8 or 16 (only where KParams::direct is set).
 struct TmaMaps { CUtensorMap xe, wgu, h, wd, wgu64, xe_n[4], h_n[4], x; };
 
@@ -1381,7 +1422,7 @@ __device__ __forceinline__ float silu_mul(float g, float u)
 // accumulator never handed back, a bounded wait running out.
 __device__ __forceinline__ void tile_info_landed(const TileInfo &ti, int *scratch)
 {
-    *reinterpret_cast<volatile int *>(scratch) = ti.type ^ ti.mb ^ ti.row0 ^ ti.nrows ^ ti.e ^ ti.n ^ ti.chunk ^ ti.nkb;
+    *reinterpret_cast<volatile int *>(scratch) = ti.type ^ ti.mb ^ ti.rt ^ ti.row0 ^ ti.nrows ^ ti.e ^ ti.n ^ ti.chunk ^ ti.nkb;
 }
 
 // bounded wait on a barrier whose guarded data may come from the peer CTA
@@ -1477,17 +1518,15 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 const int g = g_next;
                 const unsigned long long tp0 = trace_now(p);
                 TileInfo tl, tp;
-                if (g >= S.n_gemm) { tl.type = tp.type = 2; tl.mb = tp.mb = -1; tl.nrows = tp.nrows = 0; }
+                if (g >= S.n_gemm) { tl.type = tp.type = 2; tl.mb = tp.mb = -1; tl.nrows = tp.nrows = 0; tl.chunk = tp.chunk = 0; }
                 else decode_pair_tile(S, p, list, g, tl, tp);
                 // Are the tile's rows there?  If not, it is handed over all the same: the producers fetch the weights of its
                 // first k-steps meanwhile (8 experts, T = 256: 41.4 -> 39.2 us).
-                const bool two = tl.type != 2 && tp.mb != tl.mb;         // a regular pair tile has two m-blocks
                 const bool g0 = tl.type == 0 || tl.type == 3;
-                const unsigned *fl = tl.type == 2 ? nullptr : (g0 ? S.xe_ready : S.h_ready) + tl.mb;
-                const unsigned *fp = two ? (g0 ? S.xe_ready : S.h_ready) + tp.mb : fl;
-                const unsigned need = g0 ? (unsigned)tl.nrows : (unsigned)(p.nt0 * kEpiWarps), need_p = g0 ? (unsigned)tp.nrows : need;
+                const unsigned *fl = tl.type == 2 ? nullptr : (g0 ? S.xe_ready : S.h_ready) + tl.rt;
+                const unsigned need = g0 ? (unsigned)(tl.type == 0 ? kBM + tp.nrows : tl.nrows) : (unsigned)(p.nt0 * 2 * kEpiWarps);
                 const bool waits = tl.type != 2 && !(S.direct && tl.type == 3);      // (x was there before the launch)
-                const bool late = waits && (ld_acquire_u32(fl) < need || (two && ld_acquire_u32(fp) < need_p));
+                const bool late = waits && ld_acquire_u32(fl) < need;
                 if (late) { tl.chunk |= kTileLate; tp.chunk |= kTileLate; }
                 if (!mbar_wait(&S.ti_empty[ps.slot], ps.slot_phase ^ 1u, p, 30)) break;
                 S.ti[ps.slot] = tl;
@@ -1504,8 +1543,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 mbar_arrive(&S.ti_full[ps.slot]);
                 mbar_arrive_cluster(mapa_u32(smem_u32(&S.ti_full[ps.slot]), 1u));
                 if (late) {
-                    const int where = g0 ? 31 : 32;
-                    if (!flag_wait_ge(fl, need, p, where) || (two && !flag_wait_ge(fp, need_p, p, where))) break;
+                    if (!flag_wait_ge(fl, need, p, g0 ? 31 : 32)) break;
                     fence_proxy_async_global();
                     mbar_arrive(&S.ti_late[ps.slot]);
                     mbar_arrive_cluster(mapa_u32(smem_u32(&S.ti_late[ps.slot]), 1u));
@@ -1551,13 +1589,14 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
             if (ti.type == 2) break;
             {
                 const CUtensorMap *tma_a, *tma_b;
-                int arow, brow, arow2 = -1;
+                int arow, brow, arow2 = -1, brow2 = -1;
                 // swapped tiles: rows per CTA on the N axis (the MMA's N, a multiple of 16, split in two)
                 const bool from_x = S.direct && ti.type == 3;
                 const int nhalf = ((((from_x ? p.T : ti.nrows) + 15) >> 4) << 4) >> 1;
-                // ... fetched with the smallest box that covers them (the copy engine takes in a fixed
-                // number of rows per cycle, so rows nobody reads cost as much as the others)
-                const int bi = nhalf <= 8 ? 0 : nhalf <= 16 ? 1 : nhalf <= 32 ? 2 : 3;
+                // ... fetched with the smallest box that covers them (the copy engine takes in a fixed number of rows per
+                // cycle, so rows nobody reads cost as much as the others), from 65 on with a box of 64 and another one
+                const int rest = nhalf > 64 ? nhalf - 64 : nhalf;
+                const int bi = rest <= 8 ? 0 : rest <= 16 ? 1 : rest <= 32 ? 2 : 3;
                 uint32_t tx = 2u * kStageBytes;                  // bytes landing in both CTAs per k-step
                 if (ti.type == 0) {      // leader holds the gate rows of the n-tile, peer the up rows
                     tma_a = &tm->xe; tma_b = &tm->wgu;
@@ -1569,16 +1608,21 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                     brow = ti.e * p.H + ti.n * 256 + (int)rank * 128;
                 } else if (ti.type == 3) {   // M axis: 64 gate rows then 64 up rows of this CTA's 64 h-columns
                     tma_a = &tm->wgu64; tma_b = &tm->xe_n[bi];
-                    tx = 2u * (kStageA + (1024u << bi));
+                    tx = 2u * (kStageA + (1024u << bi) + (nhalf > 64 ? 8192u : 0u));
                     arow = ti.e * 2 * p.I + ti.n * kTN0 + (int)rank * 64;
                     arow2 = arow + p.I;
                     brow = ti.row0 + (int)rank * nhalf;
                     if (from_x) { tma_b = &tm->x; brow = (int)rank * nhalf; }
                 } else {                     // M axis: this CTA's 128 of the n-tile's 256 out-columns
                     tma_a = &tm->wd; tma_b = &tm->h_n[bi];
-                    tx = 2u * (kStageA + (1024u << bi));
+                    tx = 2u * (kStageA + (1024u << bi) + (nhalf > 64 ? 8192u : 0u));
                     arow = ti.e * p.H + ti.n * 256 + (int)rank * 128;
                     brow = ti.row0 + (int)rank * nhalf;
+                }
+                const CUtensorMap *tma_b2 = tma_b;      // (swapped tiles of more than 128 rows: rows 64 and up of this half)
+                if (ti.type >= 3 && nhalf > 64) {
+                    brow2 = brow + 64;
+                    tma_b = ti.type == 3 ? &tm->xe_n[3] : &tm->h_n[3];
                 }
                 // The whole warp walks the loop, one elected thread issues.  The next stage's barrier is looked at
                 // before this k-step's copies are issued, so that the answer is there when it is needed (the
@@ -1615,23 +1659,33 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                         const uint32_t sa = ring + (uint32_t)(st * kStageBytes), lb = full0_lead + (uint32_t)(st * 8);
                         if (elect_one()) {
                             if (ti.type < 3) tma_load_2d_pair(sa, tma_a, i * kBK, arow, lb);
-                            else tma_load_2d_pair(sa + kStageA, tma_b, i * kBK, brow, lb);
+                            else {
+                                tma_load_2d_pair(sa + kStageA, tma_b, i * kBK, brow, lb);
+                                if (brow2 >= 0) tma_load_2d_pair(sa + kStageA + 8192u, tma_b2, i * kBK, brow2, lb);
+                            }
                         }
                         __syncwarp();
                     }
                 }
                 bool freed = __all_sync(0xffffffffu, mbar_test_wait(&S.empty[ps.stage], ps.stage_phase ^ 1u));
-                for (; kb < ti.nkb; ++kb) {
-                    if (!freed && !__all_sync(0xffffffffu, mbar_wait(&S.empty[ps.stage], ps.stage_phase ^ 1u, p, 33))) {
-                        dead = true;
-                        break;
+                auto ksteps = [&](auto two_boxes) {
+                    for (; kb < ti.nkb; ++kb) {
+                        if (!freed && !__all_sync(0xffffffffu, mbar_wait(&S.empty[ps.stage], ps.stage_phase ^ 1u, p, 33))) {
+                            dead = true;
+                            break;
+                        }
+                        const uint32_t sa = ring + (uint32_t)(ps.stage * kStageBytes), fo = (uint32_t)(ps.stage * 8);
+                        ps.next_stage();
+                        freed = __all_sync(0xffffffffu, mbar_test_wait(&S.empty[ps.stage], ps.stage_phase ^ 1u));
+                        if (decltype(two_boxes)::value)
+                            tma_kstep_pair_b2(sa, tma_a, sa + kStageA, tma_b, kb * kBK, arow, arow2, brow, full0_lead + fo, full0 + fo, tx,
+                                              rank == 0 ? 1u : 0u, arow2 >= 0 ? 1u : 0u, tma_b2, brow2);
+                        else
+                            tma_kstep_pair(sa, tma_a, sa + kStageA, tma_b, kb * kBK, arow, arow2, brow, full0_lead + fo, full0 + fo, tx,
+                                           rank == 0 ? 1u : 0u, arow2 >= 0 ? 1u : 0u);
                     }
-                    const uint32_t sa = ring + (uint32_t)(ps.stage * kStageBytes), fo = (uint32_t)(ps.stage * 8);
-                    ps.next_stage();
-                    freed = __all_sync(0xffffffffu, mbar_test_wait(&S.empty[ps.stage], ps.stage_phase ^ 1u));
-                    tma_kstep_pair(sa, tma_a, sa + kStageA, tma_b, kb * kBK, arow, arow2, brow, full0_lead + fo, full0 + fo, tx,
-                                   rank == 0 ? 1u : 0u, arow2 >= 0 ? 1u : 0u);
-                }
+                };
+                if (brow2 >= 0) ksteps(std::true_type()); else ksteps(std::false_type());
             }
         }
         if (dead && lane == 0) linger_after_abort();
@@ -1736,89 +1790,112 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
             const uint32_t taddr = S.tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)ps.acc * 256u;
             if (ti.type == 3) {
                 // swapped gemm0: lanes 0..63 hold the gate projection of this CTA's 64 h-columns, lanes 64..127 the up
-                // projection; TMEM columns are the m-block's rows.  Gate warp q and up warp q + 2 trade halves of every
-                // 16 rows through shared memory, 1 KB each way: the gate warp finishes rows 0..7, the up warp rows
-                // 8..15.  Each warp writes only its own two buffers (the upper half of its staging area), in turn; it
-                // fills one again two batches later, after a barrier at which the partner arrived with the older
-                // batch's values already used in stores.
-                // (With the gate warps alone doing the arithmetic and the stores 64 rows took 5.5 us.)
+                // projection; TMEM columns are the tile's rows.  Gate warp q and up warp q + 2 trade halves of every 32
+                // rows through shared memory, 2 KB each way: the gate warp finishes rows 0..15, the up warp rows
+                // 16..31.  (With the gate warps alone doing the arithmetic and the stores 64 rows took 5.5 us; trading 16
+                // rows at a time and fetching from tensor memory only when needed, 200 rows took 7.2 us.)  The next 32
+                // rows come out of tensor memory meanwhile.  Each warp writes only its own two buffers (its staging
+                // area, upper half first), in turn, behind a barrier at which the partner arrived with the buffer's
+                // last values in its registers; one more barrier ends the tile.
                 //
-                // direct: TMEM columns are the batch's tokens, and the expert's rows are those with a bit in its mask.
+                // direct: TMEM columns are the batch's tokens (at most 32, so the lower buffers, where the masks are, stay
+                // untouched), and the expert's rows are those with a bit in its mask.
                 const int up = q >> 1;
                 const bool direct = S.direct != 0;
-                const uint32_t xbase = smem_u32(stages + kStages * kStageBytes) + 2048u + (uint32_t)lane * 16u;
-                const uint32_t xmine = xbase + (uint32_t)q * 4096u, xtheirs = xbase + (uint32_t)(q ^ 2) * 4096u;
+                const uint32_t xmine = smem_u32(stages + kStages * kStageBytes) + (uint32_t)(q * 4096 + lane * 16);
+                const uint32_t xtheirs = smem_u32(stages + kStages * kStageBytes) + (uint32_t)((q ^ 2) * 4096 + lane * 16);
                 uint64_t *const xbar = &S.xg[q & 1];
-                const int col = ti.n * kTN0 + (int)rank * 64 + (q & 1) * 32 + lane;      // this thread's h-column
                 const int ncol = direct ? p.T : ti.nrows;
-                unsigned long long sel = ~0ull;                  // direct: the tokens of this expert
+                unsigned sel = ~0u;                  // direct: the tokens of this expert
                 if (direct) {
-                    sel = (2ull << (p.T - 1)) - 1ull;
-                    if (ti.e < p.E) sel = *reinterpret_cast<const unsigned long long *>(stages + kStages * kStageBytes + 8 * ti.e);
+                    sel = (2u << (p.T - 1)) - 1u;
+                    if (ti.e < p.E) sel = *reinterpret_cast<const unsigned *>(stages + kStages * kStageBytes + 8 * ti.e);
                 }
-                for (int c0 = 0; c0 < ncol && !dead; c0 += 32) {
-                    uint32_t v[32];
-                    tmem_ld_32x32(taddr + c0, v);
-                    tmem_ld_wait32(v);
-                    if (c0 + 32 >= ncol) release_acc();
+                auto meet = [&]() {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(xbar);
+                    if (!mbar_wait(xbar, xg_phase, p, 53)) dead = true;
+                    dead = __any_sync(0xffffffffu, dead);
+                    xg_phase ^= 1u;
+                };
+                __nv_bfloat16 *dst = p.hbuf + (size_t)ti.row0 * p.I + ti.n * kTN0 + (int)rank * 64 + (q & 1) * 32 + lane;
+                uint32_t v[2][32];
+                tmem_ld_32x32(taddr, v[0]);
+                for (int c0 = 0; c0 < ncol && !dead; c0 += 64) {
 #pragma unroll
-                    for (int b = 0; b < 2; ++b) {
-                        const int c = c0 + 16 * b;
-                        if (c >= ncol || (direct && ((sel >> c) & 0xFFFFull) == 0ull)) continue;      // (the same for both warps)
-                        const uint32_t xo = xg_phase ? 1024u : 0u;
-                        if (up) {
-                            st_shared_v4(xmine + xo, make_uint4(v[16 * b], v[16 * b + 1], v[16 * b + 2], v[16 * b + 3]));
-                            st_shared_v4(xmine + xo + 512u, make_uint4(v[16 * b + 4], v[16 * b + 5], v[16 * b + 6], v[16 * b + 7]));
-                        } else {
-                            st_shared_v4(xmine + xo, make_uint4(v[16 * b + 8], v[16 * b + 9], v[16 * b + 10], v[16 * b + 11]));
-                            st_shared_v4(xmine + xo + 512u, make_uint4(v[16 * b + 12], v[16 * b + 13], v[16 * b + 14], v[16 * b + 15]));
+                    for (int hh = 0; hh < 2; ++hh) {
+                        const int c = c0 + 32 * hh;
+                        if (c >= ncol || dead) break;
+                        tmem_ld_wait32(v[hh]);
+                        if (c + 32 < ncol) tmem_ld_32x32(taddr + c + 32, v[hh ^ 1]);
+                        else release_acc();
+                        const uint32_t xo = hh ? 0u : 2048u;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            if (up) st_shared_v4(xmine + xo + 512u * i, make_uint4(v[hh][4 * i], v[hh][4 * i + 1], v[hh][4 * i + 2], v[hh][4 * i + 3]));
+                            else st_shared_v4(xmine + xo + 512u * i, make_uint4(v[hh][16 + 4 * i], v[hh][17 + 4 * i], v[hh][18 + 4 * i], v[hh][19 + 4 * i]));
                         }
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(xbar);
-                        if (!mbar_wait(xbar, xg_phase, p, 53)) dead = true;
-                        dead = __any_sync(0xffffffffu, dead);
+                        meet();
                         if (dead) break;
-                        xg_phase ^= 1u;
-                        const uint4 t0 = ld_shared_v4(xtheirs + xo), t1 = ld_shared_v4(xtheirs + xo + 512u);
-                        const uint32_t o[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
-                        // this warp's eight rows of the batch, as bits (warp-uniform: a row that is not there costs a branch)
-                        const int r0 = c + 8 * up;
-                        unsigned rows8 = (unsigned)(sel >> r0) & 0xFFu;
-                        if (!direct) rows8 = ncol - r0 >= 8 ? 0xFFu : (1u << max(0, ncol - r0)) - 1u;
-                        const int first = direct ? __popcll(sel & ((1ull << r0) - 1ull)) : r0;
-                        __nv_bfloat16 *dst = p.hbuf + (size_t)(ti.row0 + first) * p.I + col;
-                        __nv_bfloat16 hv[8];
+                        // this warp's sixteen rows, as bits (warp-uniform)
+                        const int r0 = c + 16 * up;
+                        unsigned rows16 = ncol - r0 >= 16 ? 0xFFFFu : (1u << max(0, ncol - r0)) - 1u;
+                        int first = r0;
+                        if (direct) {
+                            rows16 &= sel >> (16 * up);
+                            first = up ? __popc(sel & 0xFFFFu) : 0;
+                        }
 #pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            hv[i] = __float2bfloat16_rn(silu_mul(__uint_as_float(up ? o[i] : v[16 * b + i]), __uint_as_float(up ? v[16 * b + 8 + i] : o[i])));
+                        for (int h8 = 0; h8 < 2; ++h8) {
+                            const uint4 t0 = ld_shared_v4(xtheirs + xo + 1024u * h8), t1 = ld_shared_v4(xtheirs + xo + 1024u * h8 + 512u);
+                            const uint32_t o[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+                            const unsigned r8 = (rows16 >> (8 * h8)) & 0xFFu;
+                            if (r8) {
+                                __nv_bfloat16 hv[8];
 #pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            if ((rows8 >> i) & 1u) {
-                                *dst = hv[i];
-                                dst += p.I;
+                                for (int i = 0; i < 8; ++i) {
+                                    const uint32_t own = up ? v[hh][16 + 8 * h8 + i] : v[hh][8 * h8 + i];
+                                    hv[i] = __float2bfloat16_rn(silu_mul(__uint_as_float(up ? o[i] : own), __uint_as_float(up ? own : o[i])));
+                                }
+                                __nv_bfloat16 *dr = dst + (size_t)(first + __popc(rows16 & (h8 ? 0xFFu : 0u))) * p.I;
+#pragma unroll
+                                for (int i = 0; i < 8; ++i)
+                                    if ((r8 >> i) & 1u) {
+                                        *dr = hv[i];
+                                        dr += p.I;
+                                    }
                             }
-                        // (values that no row used have to land all the same before the partner fills the buffer again)
-                        *reinterpret_cast<volatile int *>(&S.scan_w[warp]) = (int)(o[0] ^ o[4]);
+                            // (values that no row used have to land all the same before the partner fills the buffer again)
+                            *reinterpret_cast<volatile int *>(&S.scan_w[warp]) = (int)(o[0] ^ o[4]);
+                        }
                     }
                 }
+                if (!dead) meet();
                 if (dead) break;
             } else if (ti.type == 4) {
-                // swapped gemm1: lane = one of this CTA's 128 out-columns, TMEM columns = the m-block's rows
+                // swapped gemm1: lane = one of this CTA's 128 out-columns, TMEM columns = the tile's rows, 32 at a time with the
+                // next 32 on their way while these are converted and stored
                 if (ti.n * 256 + (int)rank * 128 < p.H) {
                     __nv_bfloat16 *dst = p.y + (size_t)ti.row0 * p.H + ti.n * 256 + (int)rank * 128 + q * 32 + lane;
-                    for (int c0 = 0; c0 < ti.nrows; c0 += 32) {
-                        uint32_t v[32];
-                        tmem_ld_32x32(taddr + c0, v);
-                        tmem_ld_wait32(v);
-                        if (c0 + 32 >= ti.nrows) release_acc();
+                    uint32_t v[2][32];
+                    tmem_ld_32x32(taddr, v[0]);
+                    for (int c0 = 0; c0 < ti.nrows; c0 += 64) {
 #pragma unroll
-                        for (int g = 0; g < 4; ++g) {
-                            if (c0 + 8 * g >= ti.nrows) break;
-                            __nv_bfloat16 *dg = dst + (size_t)(c0 + 8 * g) * p.H;
+                        for (int hh = 0; hh < 2; ++hh) {
+                            const int c = c0 + 32 * hh;
+                            if (c >= ti.nrows) break;
+                            tmem_ld_wait32(v[hh]);
+                            if (c + 32 < ti.nrows) tmem_ld_32x32(taddr + c + 32, v[hh ^ 1]);
+                            else release_acc();
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                if (c0 + 8 * g + j < ti.nrows) *dg = __float2bfloat16_rn(__uint_as_float(v[8 * g + j]));
-                                dg += p.H;
+                            for (int g = 0; g < 4; ++g) {
+                                if (c + 8 * g >= ti.nrows) break;
+                                __nv_bfloat16 *dg = dst + (size_t)(c + 8 * g) * p.H;
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) {
+                                    if (c + 8 * g + j < ti.nrows) *dg = __float2bfloat16_rn(__uint_as_float(v[hh][8 * g + j]));
+                                    dg += p.H;
+                                }
                             }
                         }
                     }
@@ -1893,10 +1970,9 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                 if (q == 0) trace_ev(p, S, kEvGemmEpi, (unsigned)(ti.mb & 0xFFFFFF), te0, trace_now(p),
                                      (unsigned)(ti.type << 16 | (int)min(65535ull, te1 - te0)));
             }
-            // 4 arrivals per m-block and gemm0 n-tile: from the m-block's own CTA of a regular tile, 2 from each CTA of
-            // a swapped one; a swapped gemm1 tile makes 4 from each CTA (see y_done_target)
+            // every tile makes 4 arrivals from each CTA
             const bool g0 = ti.type == 0 || ti.type == 3;
-            if (!post(g0 ? &S.h_ready[ti.mb] : &S.cs->y_done[ti.chunk & (kTileLate - 1)], ti.type == 3 ? 2u : (unsigned)kEpiWarps)) dead = true;
+            if (!post(g0 ? &S.h_ready[ti.rt] : &S.cs->y_done[ti.chunk & (kTileLate - 1)], (unsigned)kEpiWarps)) dead = true;
             ps.next_acc();
         }
     } else if (warp == 3) {
@@ -2209,12 +2285,10 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
 #pragma unroll
             for (int f = 0; f < kFine; ++f) if ((f >> sh) == j) rows += cf[f];
             const int mbs = (rows + kBM - 1) / kBM;
-            // m-blocks, pair tiles and unpaired m-blocks of the experts before this one: one packed scan
-            unsigned long long tot3;
-            const unsigned long long ex3 = block_excl_scan_packed((unsigned long long)mbs | ((unsigned long long)((mbs + 1) >> 1) << 24) |
-                                                                      ((unsigned long long)(mbs & 1) << 48), S, tot3);
-            const int ex = (int)(ex3 & 0xFFFFFFull), pex = (int)((ex3 >> 24) & 0xFFFFFFull);
-            const int tot = (int)(tot3 & 0xFFFFFFull), ptot = (int)((tot3 >> 24) & 0xFFFFFFull), nodd = (int)(tot3 >> 48);
+            // m-blocks and row tiles of the experts before this one: one packed scan
+            unsigned long long tot2;
+            const unsigned long long ex2 = block_excl_scan_packed((unsigned long long)mbs | ((unsigned long long)((mbs + 1) >> 1) << 32), S, tot2);
+            const int ex = (int)(unsigned)ex2, pex = (int)(ex2 >> 32), tot = (int)(unsigned)tot2, ptot = (int)(tot2 >> 32);
             if (tid < EE) {
                 S.seg_mb0[j * EE + tid] = mb_base + ex;
                 S.seg_pt0[j * EE + tid] = pt_base + pex;
@@ -2238,7 +2312,6 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
                 S.chunk_mb0[j] = mb_base;
                 S.chunk_pt0[j] = pt_base;
                 S.chunk_tile0[j] = pt_base * (p.nt0 + p.nt1);
-                S.chunk_nswap[j] = nodd;
             }
             run_row += rows;
             mb_base += tot;

@@ -748,16 +748,14 @@ int weave_moe_debug_gemm_queue(const int32_t *rows, int num_segments, int num_ch
     int mb = 0, pt = 0, row = 0;
     for (int j = 0; j < num_chunks; ++j) {
         S.chunk_mb0[j] = mb; S.chunk_pt0[j] = pt; S.chunk_tile0[j] = pt * (nt0 + nt1);
-        int nodd = 0;
         for (int e = 0; e < num_segments; ++e) {
             const int r = rows[j * num_segments + e];
             if (r < 0) return WEAVE_ERR_INVALID_ARG;
             const int mbs = (r + kBM - 1) / kBM;
             S.seg_mb0[j * num_segments + e] = mb; S.seg_pt0[j * num_segments + e] = pt;
             S.seg_row0[j * num_segments + e] = row; S.seg_rows[j * num_segments + e] = r;
-            mb += mbs; pt += (mbs + 1) / 2; row += r; nodd += mbs & 1;
+            mb += mbs; pt += (mbs + 1) / 2; row += r;
         }
-        S.chunk_nswap[j] = nodd;
     }
     S.seg_mb0[num_chunks * num_segments] = mb; S.seg_pt0[num_chunks * num_segments] = pt;
     S.chunk_mb0[num_chunks] = mb; S.chunk_pt0[num_chunks] = pt; S.chunk_tile0[num_chunks] = pt * (nt0 + nt1);
@@ -767,8 +765,12 @@ int weave_moe_debug_gemm_queue(const int32_t *rows, int num_segments, int num_ch
     for (int g = 0; g < n && g < max_tiles && out; ++g) {
         TileInfo tl, tp;
         decode_pair_tile(S, p, 0, g, tl, tp);
+        // in terms of m-blocks: row tile i of a segment stands for its m-blocks 2i and 2i + 1
+        const int seg = tl.chunk * num_segments + tl.e, rel = tl.mb - S.seg_mb0[seg];
+        const bool pair = tp.mb != tl.mb;
         int32_t *o = out + (size_t)g * 6;
-        o[0] = tl.type; o[1] = tl.mb; o[2] = tl.type >= 3 ? -1 : tp.mb; o[3] = tl.n; o[4] = tl.chunk; o[5] = tl.nrows;
+        o[0] = tl.type % 3 + (pair ? 0 : 3); o[1] = tl.mb; o[2] = pair ? tp.mb : -1; o[3] = tl.n; o[4] = tl.chunk;
+        o[5] = std::min(kBM, S.seg_rows[seg] - rel * kBM);
     }
     return n;
 }

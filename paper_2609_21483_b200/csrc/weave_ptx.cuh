@@ -295,6 +295,27 @@ __device__ __forceinline__ void tma_kstep_pair(uint32_t dst_a, const void *map_a
           "r"(tx), "r"(expect), "r"(a2), "r"(row_a2)
         : "memory");
 }
+// the same with the second operand in two boxes, 8 KB apart (a form of its own: each instruction of the other counts)
+__device__ __forceinline__ void tma_kstep_pair_b2(uint32_t dst_a, const void *map_a, uint32_t dst_b, const void *map_b, int x,
+                                               int row_a, int row_a2, int row_b, uint32_t leader_bar, uint32_t local_bar,
+                                               uint32_t tx, uint32_t expect, uint32_t a2, const void *map_b2, int row_b2)
+{
+    asm volatile(
+        "{\n\t.reg .pred pe, px, p2;\n\t.reg .b32 d2, d3;\n\t"
+        "elect.sync _|pe, 0xffffffff;\n\t"
+        "setp.ne.and.u32 px, %10, 0, pe;\n\t"
+        "setp.ne.and.u32 p2, %11, 0, pe;\n\t"
+        "add.u32 d2, %0, 8192;\n\t"
+        "add.u32 d3, %2, 8192;\n\t"
+        "@px mbarrier.arrive.expect_tx.shared::cta.b64 _, [%8], %9;\n\t"
+        "@pe cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%4, %5}], [%7];\n\t"
+        "@p2 cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [d2], [%1, {%4, %12}], [%7];\n\t"
+        "@pe cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%2], [%3, {%4, %6}], [%7];\n\t"
+        "@pe cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [d3], [%13, {%4, %14}], [%7];\n\t}"
+        ::"r"(dst_a), "l"(map_a), "r"(dst_b), "l"(map_b), "r"(x), "r"(row_a), "r"(row_b), "r"(leader_bar), "r"(local_bar),
+          "r"(tx), "r"(expect), "r"(a2), "r"(row_a2), "l"(map_b2), "r"(row_b2)
+        : "memory");
+}
 
 // one of those copies by itself, issued by the calling thread
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void *map, int x, int row, uint32_t leader_bar)

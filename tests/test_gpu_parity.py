@@ -632,3 +632,23 @@ def test_dispatch_in_token_order(T, H, k, S):
     _, chunked, _ = run_case(cfg, sched=(pk.SCHED_FIXED, 20, 2, 1), inp=inp, dev_tensors=dev, moe=moe, n_sample=4, budget=8)
     assert torch.equal(out.view(torch.int16), chunked.view(torch.int16))
     moe.close()
+
+
+@pytest.mark.parametrize("H,ffn", [(256, 256), (384, 128), (640, 896)])
+@pytest.mark.parametrize("rows", [[1, 15, 16, 17], [127, 128, 129, 143], [240, 241, 255, 256], [257, 271, 272, 273],
+                                  [496, 497, 511, 512], [513, 768, 769, 1027], [2049, 0, 3, 130]])
+def test_row_tiles_of_every_size(rows, H, ffn):
+    """An expert's rows are split into tiles of almost equal size in units of 16 rows: tiles of 16 to 240 rows with
+    the operands swapped, 256-row tiles regular (the last one perhaps not full), mixtures of both; H and I with
+    half n-tiles.  k = 1 and crafted logits; whole output against the oracle, the same bits with two chunks."""
+    T = sum(rows)
+    cfg = _small(f"tiles_{rows[0]}_{H}", T, H, ffn, len(rows), 1, cfg_id=990)
+    want = np.repeat(np.arange(len(rows)), rows)[np.random.default_rng(7).permutation(T)]
+    inp = wl.make_inputs(cfg)
+    inp.logits[np.arange(T), want] = 50.0
+    dev = to_dev(inp)
+    moe, out, _ = run_case(cfg, inp=inp, dev_tensors=dev)
+    assert moe.routing(T)["counts"].cpu().tolist() == rows
+    _, chunked, _ = run_case(cfg, sched=(pk.SCHED_FIXED, 20, 2, 1), inp=inp, dev_tensors=dev, moe=moe)
+    assert torch.equal(out.view(torch.int16), chunked.view(torch.int16))
+    moe.close()
