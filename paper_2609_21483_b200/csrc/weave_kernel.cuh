@@ -150,7 +150,7 @@ struct KParams {
     uint4 *trace;         // optional [n_sm][trace_cap] event records (nullptr = off)
     int trace_cap;
     unsigned die_mask[32]; // bit smid: which half of the chip (die) the SM sits on
-    int two_dies;          // 0: not known, one list of GEMM tiles
+    int lists_pt;          // one chunk: two lists of GEMM tiles from this many row tiles on (see tile_lists_from)
     int4 *wait_log;       // [n_sm][8 warps]: written only by a wait that gives up or is cut short by the abort word
 };
 
@@ -2100,7 +2100,7 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
     if (p.mode == kModeAuto) { cm_bw_n = p.bw[n_sm]; cm_tf_n = p.tf[n_sm]; }
     unsigned smid;
     asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
-    const int die = p.two_dies && smid < 1024u ? (int)((p.die_mask[smid >> 5] >> (smid & 31u)) & 1u) : 0;
+    const int die = smid < 1024u ? (int)((p.die_mask[smid >> 5] >> (smid & 31u)) & 1u) : 0;
     const int P = p.T * (p.k + p.S);
     // Eq. 1-3 (single-GPU reading: every pair moves through HBM)
     const float B = (float)(2 * p.H);
@@ -2300,7 +2300,8 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
             // half, a weight panel and the expert's rows cross to the other half once instead of being fetched by
             // both (under the power cap every byte moved costs time: Mixtral-shaped T = 4096 2421 -> 2362 us,
             // Qwen3-30B-shaped T = 8192 skewed 778 -> 760; no difference where nothing is shared, T = 64).
-            if (K == 1 && tid < EE && p.two_dies) {
+            const bool two_lists = K == 1 && ptot >= p.lists_pt;
+            if (two_lists && tid < EE) {
                 const int mypt = (mbs + 1) >> 1, before = ptot - 2 * pex, after = 2 * (pex + mypt) - ptot;
                 if (before >= 0 && after > 0) {
                     S.split_pt = before <= after ? pex : pex + mypt;
@@ -2308,7 +2309,7 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
                 }
             }
             if (tid == 0) {
-                if (K > 1 || !p.two_dies || ptot == 0) { S.split_pt = ptot; S.split_seg = EE; }
+                if (!two_lists) { S.split_pt = ptot; S.split_seg = EE; }
                 S.chunk_mb0[j] = mb_base;
                 S.chunk_pt0[j] = pt_base;
                 S.chunk_tile0[j] = pt_base * (p.nt0 + p.nt1);

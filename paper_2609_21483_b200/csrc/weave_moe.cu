@@ -225,6 +225,19 @@ int find_dies(int n_sm, uint8_t *scratch, unsigned (&mask)[32])
     return 1;
 }
 
+// The number of row tiles from which the GEMM tiles of one chunk are kept in two lists, one for each half of the chip: any,
+// unless a gemm1 tile takes long (64 k-steps and more) and a pair gets few of them.  The half that is later, or that has
+// fewer SMs (chips with 74/74, 72/76 and 70/78 were measured), then starts its last ones late, and that costs more than a
+// panel that both halves fetch.  Mixtral-shaped, T = 64 to 700 (1.7 per pair): two lists 482-628 us, one 450-576; T = 1024
+// (2.2) 796 / 744 (72/76), 803 / 845 (70/78); T = 1500 (3.5, two row tiles per expert) 1006 / 1029.  Phi-3.5-shaped, T = 512 (3.5, one row tile per
+// expert) 446 / 442; T = 2048 (5.0) 748 / 787.  Short tiles: 8 experts, T = 256 35.3 / 37.0.
+int tile_lists_from(int two_dies, int pairs, int EE, int ffn, int nt1)
+{
+    if (!two_dies) return 0x7fffffff;
+    if (ffn < 64 * kBK) return 1;
+    return std::max(1, std::min((9 * pairs + 2 * nt1 - 1) / (2 * nt1), std::max((3 * pairs + nt1 - 1) / nt1, (3 * EE + 1) / 2)));
+}
+
 int upload_tables(weave_moe *h, const float *bw, const float *tf)
 {
     cudaError_t e = cudaMemcpy(h->ws + h->L.bw, bw, sizeof(float) * (h->n_sm + 1), cudaMemcpyHostToDevice);
@@ -407,7 +420,7 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     p.trace_cap = h->trace_cap;
     p.wait_log = reinterpret_cast<int4 *>(h->wait_log_dev);
     memcpy(p.die_mask, h->die_mask, sizeof(p.die_mask));
-    p.two_dies = h->two_dies;
+    p.lists_pt = tile_lists_from(h->two_dies, h->n_cta / 2, p.EE, c.ffn, p.nt1);
 
     // A small batch under AUTO: its gate/up tiles may read x itself (kernel body).  Not in an expert-parallel share, whose
     // remote tokens are to be read from their staged copies, and not under the withheld-flag hook, which is about a wait

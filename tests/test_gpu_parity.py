@@ -652,3 +652,22 @@ def test_row_tiles_of_every_size(rows, H, ffn):
     _, chunked, _ = run_case(cfg, sched=(pk.SCHED_FIXED, 20, 2, 1), inp=inp, dev_tensors=dev, moe=moe)
     assert torch.equal(out.view(torch.int16), chunked.view(torch.int16))
     moe.close()
+
+
+@pytest.mark.parametrize("rows", [[16] * 8, [16] * 9, [300, 300, 20, 20], [300, 20, 20, 20], [300, 300, 600, 0, 0],
+                                  [2000] + [7] * 9, [7] * 9 + [2000]])
+@pytest.mark.parametrize("ffn", [128, 4096])
+def test_one_list_of_tiles_or_two(rows, ffn):
+    """Row-tile counts on both sides of the lines between one list of GEMM tiles and two: for long down tiles and two
+    CTA pairs, 9 of them, or 6 of experts with more than one and a half on average.  k = 1 and crafted logits; whole
+    output against the oracle, the same bits on all SMs."""
+    T = sum(rows)
+    cfg = _small(f"lists_{len(rows)}_{rows[0]}_{ffn}", T, 128, ffn, len(rows), 1, cfg_id=995)
+    inp = wl.make_inputs(cfg)
+    inp.logits[np.arange(T), np.repeat(np.arange(len(rows)), rows)] = 50.0
+    dev = to_dev(inp)
+    moe, out, _ = run_case(cfg, inp=inp, dev_tensors=dev)
+    moe.set_sm_count(4)
+    _, few, _ = run_case(cfg, inp=inp, dev_tensors=dev, moe=moe)
+    assert torch.equal(out.view(torch.int16), few.view(torch.int16))
+    moe.close()
