@@ -192,11 +192,11 @@ int weave_moe_set_model_options(weave_moe_t h, int kinds_mask, int elastic);
 
 /* Geometry the scheduler works with: number of SMs used (= persistent CTAs; an even number,
  * because the GEMM phase runs on pairs of neighbouring SMs), rows per m-block (the unit of the
- * dispatch queue and of the ready flags), h-columns per gemm0 tile, out-columns per gemm1 tile,
+ * dispatch queue), h-columns per gemm0 tile, out-columns per gemm1 tile,
  * tokens per routing block, tokens per combine tile (the largest size: a batch that would give
  * fewer tiles than SMs is cut into tiles of half that size, repeatedly, down to one token), rows
- * per GEMM tile (two m-blocks of one expert segment; a segment with an odd number of m-blocks ends
- * in a half-empty tile).
+ * per GEMM tile at most (the rows of an expert's segment are split into as few tiles as that allows, of almost
+ * equal size; the ready flags count rows per such tile).
  * Any pointer may be NULL. */
 int weave_moe_get_geometry(weave_moe_t h, int *n_sm, int *block_m, int *tile_n0, int *tile_n1,
                            int *route_block, int *combine_tile, int *gemm_tile_m);
@@ -241,8 +241,9 @@ int weave_moe_debug_wait_log(weave_moe_t h, int32_t *out, int max_records);
  * mbarrier); after it the kernel records WEAVE_ERR_TIMEOUT and every CTA returns.  Default 4000. */
 int weave_moe_set_timeout_ms(weave_moe_t h, int ms);
 
-/* Test hook for the give-up path: the m-block with this index never publishes its
- * "dispatched" flag (-1 = off), so its consumer's bounded wait expires.  Host-side injection
+/* Test hook for the give-up path: the rows of the m-block with this index (of the row tile, where the
+ * dispatch goes through the tokens in order) are never counted as dispatched (-1 = off), so
+ * their consumer's bounded wait expires.  Host-side injection
  * only; nothing faults or traps. */
 int weave_moe_debug_withhold_flag(weave_moe_t h, int m_block);
 
@@ -287,7 +288,7 @@ int weave_moe_debug_gemm_queue(const int32_t *rows, int num_segments, int num_ch
  *     calls fail with WEAVE_ERR_WORKSPACE and must use a handle.  Every GPU on which the library
  *     is loaded holds those 64 MiB until the process exits.
  *   - The first call on each device performs a one-time set-up with that device current (it looks
- *     up the device addresses of the built-in arrays, fills the built-in cost tables with a
+ *     up the device addresses of the built-in arrays, finds out which half of the chip each SM sits on, fills the built-in cost tables with a
  *     synchronous copy, raises the kernel's shared-memory limit and resolves the TMA descriptor
  *     encoder).  Make that first call outside any stream capture.
  *   - All calls on a device share the one array, and it keeps the previous call's contents; every

@@ -1,13 +1,13 @@
 // The persistent MoE-layer megakernel: one CTA per SM, one launch per layer.
 //
-//   phase R  (all CTAs)   top-k routing of 64-token blocks (four threads per token, lists merged by
-//                         shuffles), per-block expert bitmasks -> in-block ranks and a
-//                         [block][expert] histogram; grid barrier (bounded)
+//   phase R  (all CTAs)   top-k routing of blocks of 4 to 64 tokens (32 to 4 threads per token),
+//                         per-block expert bitmasks -> in-block ranks and a [block][expert]
+//                         histogram; grid barrier (bounded; none up to 64 tokens)
 //   set-up   (every CTA, redundantly) counts, offsets, candidate tile counts, cost model -> plan
 //                         (c, K, n_steal), segment tables of the chosen K; permutation fix-up
-//   phase A  (movement CTAs: blockIdx < c)  dispatch tiles: gather x rows into expert-major Xe
+//   phase A  (movement CTAs: blockIdx < c; every CTA in the phased plan)  x rows into expert-major Xe
 //   phase B  (GEMM CTA pairs until the queue is empty; movement pairs for n_steal tiles)
-//                         two neighbouring CTAs (a cluster of 2) share a 256-row tile: a scheduler
+//                         two neighbouring CTAs (a cluster of 2) share a tile of up to 256 rows: a scheduler
 //                         warp claims tiles and waits for their inputs, TMA producers feed a
 //                         6-stage smem ring, one thread issues tcgen05.mma.cta_group::2 into TMEM,
 //                         four epilogue warps per CTA drain it through a staged, coalesced store,
@@ -52,7 +52,7 @@ constexpr int kTmemCols = 512;
 constexpr int kEpiWarps = 4;     // warps 4..7
 constexpr int kRel = 3;          // mailbox ring between the epilogue warps and the releasing warp (warp 3)
 constexpr unsigned kRelEnd = 0xFFFFFFFFu;
-constexpr int kPairGroup = 8;    // 256-row pair tiles (= 16 m-blocks) kept L2-resident while all n-tiles pass
+constexpr int kPairGroup = 8;    // row tiles of an expert kept L2-resident while all n-tiles pass
 
 constexpr int kErrNonFinite = -5;
 constexpr int kErrTimeout = -6;
@@ -115,8 +115,8 @@ struct KParams {
     int nblk;             // 64-token blocks = ceil(T / 64): the unit of the chunks, of small batches and of the expert-parallel share
     int lg_rb, nrb;       // routing blocks of 1 << lg_rb tokens, 4 to 64: as small as one block per CTA allows
     int mode, fixed_c, fixed_K, fixed_steal;
-    int nt0, nt1;         // n-tiles per m-block: I / 128, ceil(H / 256)
-    int nmb_max;          // allocated length of the per-m-block flag arrays
+    int nt0, nt1;         // n-tiles per row tile: I / 128, ceil(H / 256)
+    int nmb_max;          // allocated length of the flag arrays (row tiles are never more than m-blocks)
     int ep_rank, ep_size; // expert-parallel share (ep_size <= 1: off): this rank hosts experts
                           // [ep_rank*E/ep_size, (ep_rank+1)*E/ep_size) and owns token shard ep_rank
     int ep_tshard;        // tokens per shard = ceil(T / ep_size)
@@ -125,7 +125,7 @@ struct KParams {
     int elastic_steal;    // movement pairs keep stealing past their quota while no combine chunk is ready
     int kinds;            // bit mask of the plan kinds the cost model may choose (bit kPlanSplit, ...)
     int direct;           // the gate/up tiles may read x itself (T <= kDirectTokens, see the kernel body); tm.x is set
-    int withhold_mb;      // test hook: this m-block's "dispatched" flag is never published (-1 = off)
+    int withhold_mb;      // test hook: the rows of this m-block (dispatch in token order: row tile) are never counted in (-1 = off)
     int c_min, c_max, c_step;
     float alpha;
     float eff[4];
@@ -209,7 +209,7 @@ struct SmemTail {
     int split_pt, split_seg;     // K = 1: pair tiles [0, split_pt) = segments [0, split_seg) are list 0, the rest list 1
     int offsets[kMaxEE + 1];
     int seg_mb0[kMaxSeg + 1];
-    int seg_pt0[kMaxSeg + 1];    // prefix of pair tiles: ceil(m-blocks / 2) per segment
+    int seg_pt0[kMaxSeg + 1];    // prefix of row tiles: ceil(m-blocks / 2) per segment
     int seg_row0[kMaxSeg];
     int seg_rows[kMaxSeg];
 };
