@@ -1,6 +1,8 @@
 """GPU parity: the CUDA layer, called through its C ABI, against the CPU oracle on the same seeded
 inputs.  Routing, counts, offsets and permutation bit-exact; values within
 |gpu - ref| <= 2e-2 + 2e-2*|ref| and relative L2 <= 5e-3 (see tests/parity.py)."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -670,4 +672,27 @@ def test_one_list_of_tiles_or_two(rows, ffn):
     moe.set_sm_count(4)
     _, few, _ = run_case(cfg, inp=inp, dev_tensors=dev, moe=moe)
     assert torch.equal(out.view(torch.int16), few.view(torch.int16))
+    moe.close()
+
+
+@pytest.mark.parametrize("T", [16, 48])
+@pytest.mark.parametrize("entry", ["forward", "static"])
+def test_calls_from_a_thread_without_a_context(T, entry):
+    """A fresh thread whose first CUDA call is the layer: the tensor maps that a call encodes (a small batch's x, all of
+    the static entry's) need the device's context there.  The same bits as from this thread."""
+    cfg = _small(f"thread_{entry}_{T}", T, 256, 256, 8, 2, cfg_id=996)
+    x, logits, gu, dn = to_dev(wl.make_inputs(cfg))
+    moe = pk.WeaveMoE(gu, dn, cfg.E, cfg.k, 0, max_tokens=T)
+    run = (lambda out: moe.forward(x, logits, out=out, stream=0)) if entry == "forward" else \
+        (lambda out: pk.load().weave_moe_forward_static(cfg.H, cfg.I, cfg.E, cfg.k, 0, gu.data_ptr(), dn.data_ptr(), x.data_ptr(),
+                                                        logits.data_ptr(), out.data_ptr(), T, 0))
+    want, out, got = torch.empty_like(x), torch.zeros_like(x), []
+    run(want)
+    torch.cuda.synchronize()
+    th = threading.Thread(target=lambda: got.append(run(out)))
+    th.start()
+    th.join()
+    torch.cuda.synchronize()
+    assert got and (entry == "forward" or got[0] == 0)
+    assert torch.equal(out.view(torch.int16), want.view(torch.int16))
     moe.close()
