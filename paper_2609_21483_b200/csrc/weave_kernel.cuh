@@ -2418,7 +2418,9 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         const bool direct = p.direct && plan_kind == kPlanPhased;
         const int budget = (mover && plan_kind != kPlanPhased) ? plan_steal : 0x7fffffff;
         const bool by_token = !two_roles && S.K == 1 && !ep;
-        const bool in_gemm = by_token && p.nrb <= n_sm && (p.lg_rb <= 4 || p.nblk <= kLocalBlocks);      // few tokens per CTA
+        // few tokens per CTA, and every CTA enters the GEMM phase (with elastic stealing off, dispatch-all's movers do not)
+        const bool all_gemm = plan_kind == kPlanPhased || S.elastic;
+        const bool in_gemm = by_token && all_gemm && p.nrb <= n_sm && (p.lg_rb <= 4 || p.nblk <= kLocalBlocks);
         if (tid == 0) {      // (published by gemm_phase's first barrier)
             S.budget = budget; S.die = die; S.direct = direct ? 1 : 0;
             S.inline_disp = in_gemm && !serial ? 1 : 0;

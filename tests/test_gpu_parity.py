@@ -696,3 +696,25 @@ def test_calls_from_a_thread_without_a_context(T, entry):
     assert got and (entry == "forward" or got[0] == 0)
     assert torch.equal(out.view(torch.int16), want.view(torch.int16))
     moe.close()
+
+
+@pytest.mark.parametrize("T", [7, 64, 65, 256, 2368])
+@pytest.mark.parametrize("kinds", [2, 3, 10])
+def test_dispatch_all_with_and_without_elastic_stealing(T, kinds):
+    """AUTO restricted to dispatch-all (alone, beside the split, beside the rejoin kind).  With elastic stealing off its
+    movement CTAs take no GEMM tiles, so nothing of the dispatch may be left to the GEMM phase.  Whole output against
+    the oracle, the same bits as SERIAL."""
+    cfg = _small(f"dispatch_all_T{T}", T, 256, 256, 8, 2, 1, cfg_id=997)
+    inp = wl.make_inputs(cfg)
+    dev = to_dev(inp)
+    moe, ref, _ = run_case(cfg, sched=(pk.SCHED_SERIAL, 0, 1, 0), inp=inp, dev_tensors=dev, n_sample=None if T < 300 else 16)
+    moe.set_schedule(pk.SCHED_AUTO)
+    moe.set_timeout_ms(500)
+    for elastic in (0, 1):
+        moe.set_model_options(kinds, elastic)
+        out = moe.forward(dev[0], dev[1])
+        moe.check()
+        plan = moe.plan()
+        assert kinds != 2 or (plan["kind"], plan["K"]) == (pk.PLAN_DISPATCH_ALL, 1)      # (the dispatch in token order)
+        assert torch.equal(out.view(torch.int16), ref.view(torch.int16)), elastic
+    moe.close()
