@@ -135,7 +135,8 @@ struct KParams {
     __nv_bfloat16 *out;
     Ctl *ctl;
     uint8_t *sets;        // two CtlSets with their arrays, ctl_set_bytes(nmb_max) each
-    int *hist;            // [nrb][256]; shares its place with y, whose rows are written long after the last look at it
+    int *hist;            // [nrb][256]; shares its place with xs, which only an expert-parallel share uses: every CTA waits
+                          // for fix_done == nrb, and with it for the last look at hist, before it stages a row there
     int *topk_idx;        // [T][k]
     float *gates;         // [T][k]
     int *row_of;          // [T][k]

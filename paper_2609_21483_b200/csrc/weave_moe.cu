@@ -70,7 +70,9 @@ Layout make_layout(const weave_moe_config *c)
     L.bw = take(sizeof(float) * 1024, 256);
     L.tf = take(sizeof(float) * 1024, 256);
     L.uniq_mask = take(sizeof(unsigned long long) * (size_t)L.nblk_max, 256);
-    L.xs = take(T * c->hidden * 2, 1024);       // expert-parallel share: staged copies of remote tokens
+    // expert-parallel share: staged copies of remote tokens; before them the routing histogram of every batch, 1 KB per
+    // routing block of at least 4 tokens (see KParams::hist)
+    L.xs = take(std::max(T * c->hidden * 2, (T + 3) / 4 * kMaxEE * sizeof(int)), 1024);
     L.xe = take((size_t)L.p_max * c->hidden * 2, 1024);
     L.hbuf = take((size_t)L.p_max * c->ffn * 2, 1024);
     L.y = take((size_t)L.p_max * c->hidden * 2, 1024);
@@ -407,7 +409,7 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     uint8_t *ws = h->ws;
     p.ctl = reinterpret_cast<Ctl *>(h->ctl);
     p.sets = h->sets;
-    p.hist = reinterpret_cast<int *>(ws + L.y);      // at most 64 bytes per token, a row of y has at least 256
+    p.hist = reinterpret_cast<int *>(ws + L.xs);
     p.topk_idx = reinterpret_cast<int *>(ws + L.topk);
     p.gates = reinterpret_cast<float *>(ws + L.gates);
     p.row_of = reinterpret_cast<int *>(ws + L.row_of);

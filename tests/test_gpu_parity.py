@@ -718,3 +718,44 @@ def test_dispatch_all_with_and_without_elastic_stealing(T, kinds):
         assert kinds != 2 or (plan["kind"], plan["K"]) == (pk.PLAN_DISPATCH_ALL, 1)      # (the dispatch in token order)
         assert torch.equal(out.view(torch.int16), ref.view(torch.int16)), elastic
     moe.close()
+
+
+def _fill_y(moe, T, n_behind, value=0x5A):
+    """Fills y of a batch of T tokens and the n_behind bytes behind it with a value; returns the view of both."""
+    y = moe.intermediates(T)["y"].view(torch.uint8)
+    off = y.data_ptr() - moe.workspace.data_ptr()
+    view = moe.workspace[off:off + y.numel() + n_behind]
+    view.fill_(value)
+    return view
+
+
+@pytest.mark.parametrize("T", [65, 66, 67])
+def test_routing_histogram_keeps_out_of_y_and_what_is_behind_it(T):
+    """Routing blocks of 4 tokens, 256 experts, the narrowest rows and max_tokens = T: the histogram takes more bytes than
+    y has, and the CTAs that still read it are not waited for by those that already store rows of y.  Nothing but y's
+    own rows changes there: the bytes up to the next 1024-byte boundary stay as they were."""
+    cfg = _small(f"hist_T{T}", T, 128, 128, 256, 1, cfg_id=998)
+    inp = wl.make_inputs(cfg)
+    dev = to_dev(inp)
+    moe = pk.WeaveMoE(dev[2], dev[3], cfg.E, cfg.k, cfg.S, max_tokens=T)
+    pad = -(T * cfg.H * 2) % 1024
+    view = _fill_y(moe, T, pad)
+    run_case(cfg, inp=inp, dev_tensors=dev, moe=moe)
+    assert pad > 0 and (view[-pad:] == 0x5A).all()
+    moe.close()
+
+
+@pytest.mark.parametrize("T", [64, 65, 2000])
+def test_a_rank_without_rows_leaves_y_alone(T):
+    """An expert-parallel share none of whose experts is selected has no row of y; the routing leaves none there either."""
+    cfg = _small(f"no_rows_T{T}", T, 256, 128, 16, 2, cfg_id=999)
+    inp = wl.make_inputs(cfg)
+    inp.logits[:, 8:] += 100.0
+    x, lg, gu, dn = to_dev(inp)
+    moe = pk.WeaveMoE(gu, dn, cfg.E, cfg.k, cfg.S, max_tokens=T)
+    moe.set_expert_parallel(0, 2)
+    view = _fill_y(moe, T, 0)
+    out = moe.forward(x, lg)
+    moe.check()
+    assert (view == 0x5A).all() and not out.any()
+    moe.close()
