@@ -233,7 +233,8 @@ struct TokScratch {
 static_assert(sizeof(TokScratch) <= kEpiStageBytes / 2, "as the movement scratch");
 static_assert(kMaxTopK + 8 <= 32 && 32 <= kTokEnt, "a token's rows fit a buffer's list, and a warp");
 static_assert(kLocalBlocks * (kMaxEE + 1) * 8 <= kEpiStageBytes / 2, "the routing masks must fit the other half");
-static_assert(kLocalBlocks * kMaxEE * 8 <= 2048, "the masks that the direct gate/up tiles read end below the first exchange buffer");
+static_assert(kLocalBlocks * kMaxEE * 8 <= 2048, "the masks end below the first upper exchange buffer, the only kind that tiles of at most 32 rows use");
+static_assert(kDirectTokens <= 32, "gate/up tiles that read the masks stay out of the lower exchange buffers");
 static_assert(kFine == 8, "chunk of a fine chunk = f >> (3 - log2 K)");
 __device__ __forceinline__ MoveScratch &move_scratch(uint8_t *stages)
 {
@@ -1491,7 +1492,13 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
     fence_proxy_async_shared();     // the stage buffers were last touched by ordinary stores (routing scratch)
     __syncthreads();
 
-    if (S.inline_disp && warp >= 8 - kInlineWarps) dispatch_inline(p, S, stages, warp - (8 - kInlineWarps));
+    if (S.inline_disp && warp >= 8 - kInlineWarps) {
+        dispatch_inline(p, S, stages, warp - (8 - kInlineWarps));
+        // Its warps look rows up in the routing masks, and a swapped gate/up tile of more than 32 rows trades values where
+        // the masks are (lower exchange buffers): no warp goes on to its epilogue before the others are done with them.
+        // Tiles of a batch of at most 32 tokens use the upper buffers only.
+        if (p.nblk <= kLocalBlocks && p.T > kDirectTokens) named_barrier_sync<1, kInlineWarps * 32>();
+    }
 
     if (warp == 2 && rank == 0) {
         // ---------------- scheduler (leader only): claims pair tiles in queue order, waits until their

@@ -102,6 +102,15 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity)
     return ok != 0;
 }
 
+// ---------------------------------------------------------------- a barrier of some of the CTA's warps
+
+// the block barrier number ID (0 is __syncthreads) for THREADS threads in whole warps
+template <int ID, int THREADS>
+__device__ __forceinline__ void named_barrier_sync()
+{
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
+}
+
 // ---------------------------------------------------------------- TMA
 // (the tiled loads themselves are in the CTA-pair section below; none of them uses multicast)
 

@@ -759,3 +759,26 @@ def test_a_rank_without_rows_leaves_y_alone(T):
     moe.check()
     assert (view == 0x5A).all() and not out.any()
     moe.close()
+
+
+@pytest.mark.parametrize("T", [33, 63, 64])
+@pytest.mark.parametrize("n_sm", [4, 6, 148])
+def test_masks_outlive_the_first_wide_gate_up_tiles(T, n_sm):
+    """Batches of 33 to 64 tokens: idle warps dispatch by the routing masks, in shared memory that a gate/up tile of more
+    than 32 rows uses for its epilogue.  One expert has all tokens, long rows, few CTAs (each warp takes several
+    tokens while that tile may already be finished): Xe row by row and the whole output against the oracle, 20 launches."""
+    cfg = _small(f"masks_T{T}", T, 4096, 128, 12, 3, 1, cfg_id=1000)
+    inp = wl.make_inputs(cfg)
+    inp.logits[:, 0] = 50.0
+    dev = to_dev(inp)
+    moe = pk.WeaveMoE(dev[2], dev[3], cfg.E, cfg.k, cfg.S, max_tokens=T)
+    moe.set_sm_count(min(n_sm, moe.geometry()["n_sm"]))
+    _, ref, _ = run_case(cfg, inp=inp, dev_tensors=dev, moe=moe)
+    tok = moe.routing(T)["token_of"].long().clone()
+    for _ in range(20):
+        moe.intermediates(T)["xe"].zero_()
+        out = moe.forward(dev[0], dev[1])
+        assert torch.equal(moe.intermediates(T)["xe"].view(torch.int16), dev[0].view(torch.int16)[tok])
+        assert torch.equal(out.view(torch.int16), ref.view(torch.int16))
+    moe.check()
+    moe.close()
