@@ -241,10 +241,9 @@ int weave_moe_debug_wait_log(weave_moe_t h, int32_t *out, int max_records);
  * mbarrier); after it the kernel records WEAVE_ERR_TIMEOUT and every CTA returns.  Default 4000. */
 int weave_moe_set_timeout_ms(weave_moe_t h, int ms);
 
-/* Test hook for the give-up path: the rows of the m-block with this index (of the row tile, where the
- * dispatch goes through the tokens in order) are never counted as dispatched (-1 = off), so
- * their consumer's bounded wait expires.  Host-side injection
- * only; nothing faults or traps. */
+/* Test hook for the give-up path: the rows of the m-block with this index are never counted as
+ * dispatched (-1 = off; an index that the batch does not reach withholds nothing), so the bounded wait of
+ * the GEMM tiles that share rows with it expires.  Host-side injection only; nothing faults or traps. */
 int weave_moe_debug_withhold_flag(weave_moe_t h, int m_block);
 
 /* Optional in-kernel timeline (our analogue of the utilisation profile of the paper's Section 5.4).

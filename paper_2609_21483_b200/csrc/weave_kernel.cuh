@@ -125,7 +125,7 @@ struct KParams {
     int elastic_steal;    // movement pairs keep stealing past their quota while no combine chunk is ready
     int kinds;            // bit mask of the plan kinds the cost model may choose (bit kPlanSplit, ...)
     int direct;           // the gate/up tiles may read x itself (T <= kDirectTokens, see the kernel body); tm.x is set
-    int withhold_mb;      // test hook: the rows of this m-block (dispatch in token order: row tile) are never counted in (-1 = off)
+    int withhold_mb;      // test hook: the rows of this m-block are never counted in (-1 = off)
     int c_min, c_max, c_step;
     float alpha;
     float eff[4];
@@ -1069,9 +1069,19 @@ __device__ __forceinline__ void dispatch_phase(const KParams &p, SmemTail &S, ui
 // read once and written to its k + S rows of Xe.  (In m-block order every row was read for each of its experts, from HBM
 // where x does not fit L2, an m-block's 128 rows were one SM's chain of copies, and nothing began before the
 // permutation of ALL tokens was final.)  The row tiles' ready flags count their rows in.
+// (test hook) does row tile rt have rows of the withheld m-block?
+__device__ __noinline__ bool withheld(int mb, int EE, int rt)
+{
+    const SmemTail &S = smem_tail();
+    if (mb >= S.nmb) return false;
+    int row0, nrows, seg;
+    decode_mblock(S, EE, mb, row0, nrows, seg);
+    const int rows = S.seg_rows[seg], pts = S.seg_pt0[seg + 1] - S.seg_pt0[seg], rel = row0 - S.seg_row0[seg], i = rt - S.seg_pt0[seg];
+    return i >= rowtile_of_rel(rows, pts, rel) && i <= rowtile_of_rel(rows, pts, rel + nrows - 1);
+}
 __device__ __forceinline__ void publish_row(const KParams &p, SmemTail &S, int rt, unsigned long long t0)
 {
-    if (rt == p.withhold_mb) return;
+    if (p.withhold_mb >= 0 && withheld(p.withhold_mb, p.EE, rt)) return;
     if (p.trace == nullptr) {
         red_release_add_u32(&S.xe_ready[rt], 1u);
     } else {      // the timeline has one record per m-block, made by whoever completes its row tile

@@ -782,3 +782,26 @@ def test_masks_outlive_the_first_wide_gate_up_tiles(T, n_sm):
         assert torch.equal(out.view(torch.int16), ref.view(torch.int16))
     moe.check()
     moe.close()
+
+
+@pytest.mark.parametrize("T", [40, 640, 2400])
+@pytest.mark.parametrize("sched", [(pk.SCHED_AUTO, 0, 1, 0), (pk.SCHED_SERIAL, 0, 1, 0), (pk.SCHED_FIXED, 20, 1, 0)])
+def test_a_withheld_m_block_is_an_m_block_whatever_the_dispatch_order(T, sched):
+    """One expert: T rows are more m-blocks of 128 rows than row tiles of up to 256.  The last m-block's index names
+    rows in every dispatch order (idle warps, token tiles, m-block order), the one behind it names none."""
+    cfg = _small(f"withheld_T{T}", T, 128, 128, 1, 1, cfg_id=1001)
+    inp = wl.make_inputs(cfg)
+    x, lg, gu, dn = to_dev(inp)
+    moe = pk.WeaveMoE(gu, dn, cfg.E, cfg.k, cfg.S, max_tokens=T)
+    moe.set_schedule(*sched)
+    ref = moe.forward(x, lg).view(torch.int16).clone()
+    moe.check()
+    moe.set_timeout_ms(20)
+    last = (T + 127) // 128 - 1
+    moe.debug_withhold_flag(last)
+    moe.forward(x, lg)
+    assert moe.status() == pk.ERR_TIMEOUT
+    moe.debug_withhold_flag(last + 1)
+    assert torch.equal(moe.forward(x, lg).view(torch.int16), ref)
+    moe.check()
+    moe.close()
