@@ -1566,7 +1566,7 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                     mbar_arrive(&S.ti_late[ps.slot]);
                     mbar_arrive_cluster(mapa_u32(smem_u32(&S.ti_late[ps.slot]), 1u));
                 }
-                if (tl.type != 2) trace_ev(p, S, kEvGemmLoad, (unsigned)g, tp0, trace_now(p), 0u);
+                if (tl.type != 2) trace_ev(p, S, kEvGemmLoad, (unsigned)(list ? n_list0 + g : g), tp0, trace_now(p), 0u);
                 ps.next_slot();
                 if (tl.type == 2) break;
                 // the next claim's round trip comes after the hand-over

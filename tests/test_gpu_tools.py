@@ -121,3 +121,25 @@ def test_utilisation_report_from_the_kernel_timeline():
     assert serial["overlap_ratio"] < 0.01
     txt = timeline.ascii_timeline(trace, width=60).splitlines()
     assert len(txt) == auto["n_cta"] + 1 and any("G" in l for l in txt[1:])
+
+
+@pytest.mark.parametrize("T", [20, 1000])
+def test_timeline_names_every_scheduled_tile_once(T):
+    """The record that a GEMM tile's scheduler writes is named by the tile's place in the queue, whether the queue is
+    one list or two: 0 .. n-1, each once."""
+    cfg = wl.MoEConfig("trace_ids", 92, T=T, H=512, I=768, E=16, k=4)
+    x, lg, gu, dn = to_dev(wl.make_inputs(cfg))
+    moe = pk.WeaveMoE(gu, dn, cfg.E, cfg.k, cfg.S, max_tokens=cfg.T)
+    geo = moe.geometry()
+    moe.enable_trace(4096)
+    for sched in [(pk.SCHED_AUTO, 0, 1, 0), (pk.SCHED_FIXED, 10, 1, 3)]:
+        moe.set_schedule(*sched)
+        moe.forward(x, lg)
+        moe.check()
+        assert moe.plan()["K"] == 1
+        ev = np.concatenate([a for a in moe.read_trace() if len(a)])
+        counts = moe.routing(cfg.T)["counts"].cpu().numpy()
+        tiles = int(((counts + geo["gemm_tile_m"] - 1) // geo["gemm_tile_m"]).sum())
+        nt = cfg.I // geo["tile_n0"] + (cfg.H + geo["tile_n1"] - 1) // geo["tile_n1"]
+        np.testing.assert_array_equal(np.sort(ev[(ev[:, 2] >> 24) == 5, 2] & 0xFFFFFF), np.arange(tiles * nt))
+    moe.close()
