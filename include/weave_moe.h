@@ -261,15 +261,27 @@ int weave_moe_set_trace(weave_moe_t h, void *buf, int events_per_cta);
 /* HOST-ONLY (no GPU needed, no handle): the order in which the kernel's GEMM schedulers claim pair
  * tiles (Section 4: the queues follow the dependency order of the chunk pipeline), for `num_chunks` chunks of
  * `num_segments` expert segments whose row counts are rows[chunk * num_segments + expert], n-tile
- * counts nt0 (gemm0) and nt1 (gemm1).  Writes up to max_tiles records of
- * 6 ints {type (0 gemm0, 1 gemm1, +3 when the operands are swapped), leader m-block, peer m-block
- * (-1 for a swapped tile), n-tile, chunk, rows of the leader m-block} to `out` (host memory, may be
+ * counts nt0 (gemm0) and nt1 (gemm1), in terms of m-blocks: row tile i of a segment stands for its
+ * m-blocks 2i and 2i + 1 (how the rows are really cut, and which tiles run with the operands swapped, is
+ * weave_moe_debug_gemm_tiles()'s to say).  Writes up to max_tiles records of
+ * 6 ints {type (0 gemm0, 1 gemm1, +3 where the segment's last m-block has no partner), leader m-block,
+ * peer m-block (-1 without one), n-tile, chunk, rows of the leader m-block} to `out` (host memory, may be
  * NULL) and returns the total number of tiles, or a negative error for bad arguments (chunks not
- * in {1,2,4,8}, more than 1024 segments in total, non-positive tile counts).  This is the same
+ * in {1,2,4,8}, more than 1024 segments in total, non-positive tile counts).  The order comes from the
  * decoding routine the device runs; tests use it to check that every tile a gemm1 tile waits for
  * comes earlier in the queue. */
 int weave_moe_debug_gemm_queue(const int32_t *rows, int num_segments, int num_chunks, int nt0, int nt1,
                                int32_t *out, int max_tiles);
+
+/* HOST-ONLY: the same tiles as the device's decoding routine gives them out.  split: with one chunk, the
+ * segments before it are the first list of tiles, the others the second (the kernel cuts near half of the
+ * tiles, or not at all: split = num_segments, the only value with more chunks).  Writes up to
+ * max_tiles records of 10 ints, the first list's in front, {type (0 / 1 = gemm0 / gemm1 of 256 rows, 3 / 4 = of
+ * fewer, with the operands swapped), list, chunk, expert, n-tile, row tile (the index of its ready counter),
+ * first row, rows, first row of the peer CTA's half (regular) or of the tile (swapped), how many of its rows
+ * the dispatch counts in on that row tile} and returns the number of tiles or a negative error. */
+int weave_moe_debug_gemm_tiles(const int32_t *rows, int num_segments, int num_chunks, int split, int nt0,
+                               int nt1, int32_t *out, int max_tiles);
 
 /* ---- for callers that cannot allocate ---------------------------------------------------------
  *

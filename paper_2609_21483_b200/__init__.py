@@ -65,7 +65,7 @@ EXPORTS = [
     "weave_moe_set_expert_parallel", "weave_moe_get_ep_descriptors",
     "weave_moe_forward_host_pipelined", "weave_moe_host_wait", "weave_moe_debug_gemm_queue",
     "weave_moe_get_plan_kind", "weave_moe_set_model_options", "weave_moe_last_timeout_where",
-    "weave_moe_debug_wait_log",
+    "weave_moe_debug_wait_log", "weave_moe_debug_gemm_tiles",
 ]
 
 
@@ -136,6 +136,8 @@ def load():
     lib.weave_moe_last_cuda_error.argtypes = [vp]
     lib.weave_moe_debug_gemm_queue.restype = ci
     lib.weave_moe_debug_gemm_queue.argtypes = [vp, ci, ci, ci, ci, vp, ci]
+    lib.weave_moe_debug_gemm_tiles.restype = ci
+    lib.weave_moe_debug_gemm_tiles.argtypes = [vp, ci, ci, ci, ci, ci, vp, ci]
     lib.weave_moe_strerror.restype = ctypes.c_char_p
     lib.weave_moe_strerror.argtypes = [ci]
     _lib = lib
@@ -161,6 +163,24 @@ def gemm_queue(rows, nt0: int, nt1: int):
     if n:
         _check(0 if load().weave_moe_debug_gemm_queue(rows.ctypes.data, EE, K, nt0, nt1, out.ctypes.data, n) == n
                else WEAVE_ERR_INVALID_ARG, "weave_moe_debug_gemm_queue")
+    return out
+
+
+def gemm_tiles(rows, nt0: int, nt1: int, split: Optional[int] = None):
+    """Host-only: the GEMM tiles as the device decodes them -> int32 array [n_tiles, 10] of (type, list, chunk, expert,
+    n-tile, row tile, first row, rows, peer's first row, rows counted in); split = first segment of the second list."""
+    import numpy as np
+    rows = np.ascontiguousarray(rows, dtype=np.int32)
+    if rows.ndim == 1:
+        rows = rows[None, :]
+    K, EE = rows.shape
+    args = (rows.ctypes.data, EE, K, EE if split is None else split, nt0, nt1)
+    n = load().weave_moe_debug_gemm_tiles(*args, None, 0)
+    if n < 0:
+        raise WeaveError(n, "weave_moe_debug_gemm_tiles")
+    out = np.zeros((n, 10), np.int32)
+    if n:
+        load().weave_moe_debug_gemm_tiles(*args, out.ctypes.data, n)
     return out
 
 

@@ -756,16 +756,14 @@ int weave_moe_debug_wait_log(weave_moe_t h, int32_t *out, int max_records)
     return n;
 }
 
-int weave_moe_debug_gemm_queue(const int32_t *rows, int num_segments, int num_chunks, int nt0, int nt1, int32_t *out,
-                               int max_tiles)
+// the tables that the kernel's set-up builds in shared memory, built here the same way, with one list of tiles; returns
+// their number or an error
+static int queue_tables(const int32_t *rows, int num_segments, int num_chunks, int nt0, int nt1, SmemTail &S, KParams &p)
 {
     if (!rows || num_segments < 1 || nt0 < 1 || nt1 < 1) return WEAVE_ERR_INVALID_ARG;
     if (num_chunks != 1 && num_chunks != 2 && num_chunks != 4 && num_chunks != 8) return WEAVE_ERR_INVALID_ARG;
     if (num_segments * num_chunks > kMaxSeg) return WEAVE_ERR_INVALID_ARG;
-    // the tables the kernel's set-up builds in shared memory, built here the same way
-    std::vector<unsigned char> raw(sizeof(SmemTail), 0);
-    SmemTail &S = *reinterpret_cast<SmemTail *>(raw.data());
-    KParams p;
+    memset(static_cast<void *>(&S), 0, sizeof(S));
     memset(&p, 0, sizeof(p));
     p.EE = num_segments; p.nt0 = nt0; p.nt1 = nt1; p.H = kBK; p.I = kBK;
     int mb = 0, pt = 0, row = 0;
@@ -783,8 +781,16 @@ int weave_moe_debug_gemm_queue(const int32_t *rows, int num_segments, int num_ch
     S.seg_mb0[num_chunks * num_segments] = mb; S.seg_pt0[num_chunks * num_segments] = pt;
     S.chunk_mb0[num_chunks] = mb; S.chunk_pt0[num_chunks] = pt; S.chunk_tile0[num_chunks] = pt * (nt0 + nt1);
     S.K = num_chunks;
-    S.split_pt = pt; S.split_seg = num_segments;      // (one list: the order inside either of two is this one's)
-    const int n = pt * (nt0 + nt1);
+    S.split_pt = pt; S.split_seg = num_segments;
+    return pt * (nt0 + nt1);
+}
+
+int weave_moe_debug_gemm_queue(const int32_t *rows, int num_segments, int num_chunks, int nt0, int nt1, int32_t *out,
+                               int max_tiles)
+{
+    SmemTail S;
+    KParams p;
+    const int n = queue_tables(rows, num_segments, num_chunks, nt0, nt1, S, p);
     for (int g = 0; g < n && g < max_tiles && out; ++g) {
         TileInfo tl, tp;
         decode_pair_tile(S, p, 0, g, tl, tp);
@@ -794,6 +800,30 @@ int weave_moe_debug_gemm_queue(const int32_t *rows, int num_segments, int num_ch
         int32_t *o = out + (size_t)g * 6;
         o[0] = tl.type % 3 + (pair ? 0 : 3); o[1] = tl.mb; o[2] = pair ? tp.mb : -1; o[3] = tl.n; o[4] = tl.chunk;
         o[5] = std::min(kBM, S.seg_rows[seg] - rel * kBM);
+    }
+    return n;
+}
+
+int weave_moe_debug_gemm_tiles(const int32_t *rows, int num_segments, int num_chunks, int split, int nt0, int nt1, int32_t *out,
+                               int max_tiles)
+{
+    SmemTail S;
+    KParams p;
+    const int n = queue_tables(rows, num_segments, num_chunks, nt0, nt1, S, p);
+    if (n < 0) return n;
+    if (split < 0 || split > num_segments || (num_chunks > 1 && split != num_segments)) return WEAVE_ERR_INVALID_ARG;
+    if (num_chunks == 1) { S.split_seg = split; S.split_pt = S.seg_pt0[split]; }
+    const int n_list0 = num_chunks == 1 ? S.split_pt * (nt0 + nt1) : n;
+    for (int g = 0; g < n && g < max_tiles && out; ++g) {
+        TileInfo tl, tp;
+        const int list = g >= n_list0;
+        decode_pair_tile(S, p, list, list ? g - n_list0 : g, tl, tp);
+        const int seg = tl.chunk * num_segments + tl.e, pts = S.seg_pt0[seg + 1] - S.seg_pt0[seg];
+        const int n_rows = tl.type < 3 ? tl.nrows + tp.nrows : tl.nrows, rel = tl.row0 - S.seg_row0[seg];
+        int mapped = 0;
+        for (int i = 0; i < n_rows; ++i) mapped += S.seg_pt0[seg] + rowtile_of_rel(S.seg_rows[seg], pts, rel + i) == tl.rt;
+        const int32_t rec[10] = {tl.type, list, tl.chunk, tl.e, tl.n, tl.rt, tl.row0, n_rows, tp.row0, mapped};
+        memcpy(out + (size_t)g * 10, rec, sizeof(rec));
     }
     return n;
 }
