@@ -202,23 +202,23 @@ int find_dies(int n_sm, uint8_t *scratch, unsigned (&mask)[32])
     memset(mask, 0, sizeof(mask));
     const int smem = 120 * 1024;      // one block per SM
     if (cudaFuncSetAttribute(weave_die_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 0;
-    unsigned *out = reinterpret_cast<unsigned *>(scratch);
-    weave_die_probe_kernel<<<n_sm, 32, smem>>>(reinterpret_cast<unsigned *>(scratch + kMaxSm * kDieLines * 4), 1024, out);
-    std::vector<unsigned> lat((size_t)kMaxSm * kDieLines);
-    if (cudaGetLastError() != cudaSuccess ||
-        cudaMemcpy(lat.data(), out, lat.size() * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
+    unsigned *lines_dev = reinterpret_cast<unsigned *>(scratch + kMaxSm * kDieLines * 4), *out = reinterpret_cast<unsigned *>(scratch);
+    int stride = 1024;
+    void *args[] = {&lines_dev, &stride, &out};
+    unsigned lat[kMaxSm * kDieLines];      // (no host heap here: an allocation could throw through the C entry points)
+    if (cudaLaunchKernel((const void *)weave_die_probe_kernel, dim3(n_sm), dim3(32), args, smem, nullptr) != cudaSuccess ||
+        cudaMemcpy(lat, out, sizeof(lat), cudaMemcpyDeviceToHost) != cudaSuccess)
         return 0;
-    std::vector<int> sms;
+    int sms[kMaxSm], n = 0;
     for (int i = 0; i < kMaxSm; ++i)
-        if (lat[(size_t)i * kDieLines]) sms.push_back(i);
-    const int n = (int)sms.size();
+        if (lat[(size_t)i * kDieLines]) sms[n++] = i;
     if (n < 8) return 0;
-    std::vector<int> votes(n, 0);
+    int votes[kMaxSm] = {0};
     int lines = 0;
     for (int a = 0; a < kDieLines; ++a) {
-        std::vector<unsigned> v;
-        for (int i : sms) v.push_back(lat[(size_t)i * kDieLines + a]);
-        std::sort(v.begin(), v.end());
+        unsigned v[kMaxSm];
+        for (int i = 0; i < n; ++i) v[i] = lat[(size_t)sms[i] * kDieLines + a];
+        std::sort(v, v + n);
         int cut = n / 4;      // the widest gap with at least a quarter of the SMs on either side
         for (int i = n / 4; i < n - n / 4; ++i)
             if (v[i] - v[i - 1] > v[cut] - v[cut - 1]) cut = i;
