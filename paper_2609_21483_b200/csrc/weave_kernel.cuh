@@ -200,7 +200,8 @@ struct SmemTail {
     int scan_w[8];
     int scan_total;
     int c, K, steal, nmb, n_gemm, n_comb;
-    int budget, die, direct, inline_disp;     // see gemm_phase
+    int budget, die, direct;     // see gemm_phase
+    int inline_disp;             // 1 = idle warps of the GEMM phase dispatch, 2 = and meet before their epilogues
     int elastic;                 // this launch: movement pairs take GEMM tiles beyond their quota, GEMM CTAs dispatch one m-block first
     int comb_tok;                // tokens per combine tile of this launch: 16, 8, 4, 2 or 1
     unsigned trace_n;
@@ -1506,8 +1507,9 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
         dispatch_inline(p, S, stages, warp - (8 - kInlineWarps));
         // Its warps look rows up in the routing masks, and a swapped gate/up tile of more than 32 rows trades values where
         // the masks are (lower exchange buffers): no warp goes on to its epilogue before the others are done with them.
-        // Tiles of a batch of at most 32 tokens use the upper buffers only.
-        if (p.nblk <= kLocalBlocks && p.T > kDirectTokens) named_barrier_sync<1, kInlineWarps * 32>();
+        // No barrier (inline_disp = 1) where the batch has at most 32 tokens, whose tiles use the upper buffers only, or more
+        // than one routing block, whose rows are not looked up in masks.
+        if (S.inline_disp > 1) named_barrier_sync<1, kInlineWarps * 32>();
     }
 
     if (warp == 2 && rank == 0) {
@@ -1566,7 +1568,8 @@ __device__ __forceinline__ void gemm_phase(const KParams &p, SmemTail &S, uint8_
                     mbar_arrive(&S.ti_late[ps.slot]);
                     mbar_arrive_cluster(mapa_u32(smem_u32(&S.ti_late[ps.slot]), 1u));
                 }
-                if (tl.type != 2) trace_ev(p, S, kEvGemmLoad, (unsigned)(list ? n_list0 + g : g), tp0, trace_now(p), 0u);
+                if (p.trace && tl.type != 2)      // (the id is the tile's place in the whole queue, the second list behind the first)
+                    trace_ev(p, S, kEvGemmLoad, (unsigned)(list ? S.split_pt * per_pt + g : g), tp0, trace_now(p), 0u);
                 ps.next_slot();
                 if (tl.type == 2) break;
                 // the next claim's round trip comes after the hand-over
@@ -2441,7 +2444,7 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         const bool in_gemm = by_token && all_gemm && p.nrb <= n_sm && (p.lg_rb <= 4 || p.nblk <= kLocalBlocks);
         if (tid == 0) {      // (published by gemm_phase's first barrier)
             S.budget = budget; S.die = die; S.direct = direct ? 1 : 0;
-            S.inline_disp = in_gemm && !serial ? 1 : 0;
+            S.inline_disp = in_gemm && !serial ? (p.nblk <= kLocalBlocks && p.T > kDirectTokens ? 2 : 1) : 0;
         }
         if (by_token) {
             if (!in_gemm) dispatch_tokens(p, S, stages);
