@@ -304,7 +304,9 @@ int weave_moe_debug_gemm_tiles(const int32_t *rows, int num_segments, int num_ch
  *     encoder).  Make that first call outside any stream capture.
  *   - All calls on a device share the one array, and it keeps the previous call's contents; every
  *     call enqueues the kernel and nothing else.  Calls that overlap on the GPU (different streams,
- *     no ordering between them) race on the array: order them.
+ *     no ordering between them) race on the array: order them.  Such an overlap can also spoil the
+ *     call behind it, because calls take turns with two sets of control words and each cleans the
+ *     set that it does not use.
  *   - Scheduling is AUTO with the default cost tables.  Arguments, layouts and alignment as for
  *     weave_moe_create() / weave_moe_forward(); asynchronous on the stream; a device-side failure
  *     of this call (non-finite logits, an expired wait) is not reported - use a handle when the

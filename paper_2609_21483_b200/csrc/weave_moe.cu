@@ -238,9 +238,11 @@ int find_dies(int n_sm, uint8_t *scratch, unsigned (&mask)[32])
 // The number of row tiles from which the GEMM tiles of one chunk are kept in two lists, one for each half of the chip: any,
 // unless a gemm1 tile takes long (64 k-steps and more) and a pair gets few of them.  The half that is later, or that has
 // fewer SMs (chips with 74/74, 72/76 and 70/78 were measured), then starts its last ones late, and that costs more than a
-// panel that both halves fetch.  Mixtral-shaped, T = 64 to 700 (1.7 per pair): two lists 482-628 us, one 450-576; T = 1024
-// (2.2) 796 / 744 (72/76), 803 / 845 (70/78); T = 1500 (3.5, two row tiles per expert) 1006 / 1029.  Phi-3.5-shaped, T = 512 (3.5, one row tile per
-// expert) 446 / 442; T = 2048 (5.0) 748 / 787.  Short tiles: 8 experts, T = 256 35.3 / 37.0.
+// panel that both halves fetch.  Two lists / one, us.  Mixtral-shaped, T = 64 to 700 (1.7 gemm1 tiles per pair) 482-628 /
+// 450-576; T = 1024 (2.2) 796 / 744 on a 72/76 chip, but 803 / 845 on a 70/78 chip, where this rule takes the slower side;
+// T = 1500 (3.5, two row tiles per expert) 1006 / 1029.  Phi-3.5-shaped, T = 512 (3.5, one row tile per expert) 446 / 442;
+// T = 2048 (5.0) 748 / 787.  Short tiles: 8 experts, T = 256 35.3 / 37.0.  The lines at 64 k-steps, 4.5 and 3 tiles per pair
+// and 1.5 row tiles per expert stand on these two shapes and three chips.
 int tile_lists_from(int two_dies, int pairs, int EE, int ffn, int nt1)
 {
     if (!two_dies) return 0x7fffffff;
@@ -386,7 +388,7 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     p.nblk = (T + kRouteBlock - 1) / kRouteBlock;
     // Routing blocks of 4 to 32 tokens, with up to 32 threads per token, while each still has a CTA to itself (an
     // expert-parallel share stages its remote tokens by 64).  Below 4 the fix-up's sum over the blocks of a fine chunk
-    // (at most 16 rows of the histogram from 4 on) would take longer than the routing saves.  A batch of at most 64
+    // (up to 31 rows of the histogram with blocks of 4) would take longer than the routing saves.  A batch of at most 64
     // tokens is one block, routed by every CTA for itself, with as many threads per token as there are.
     p.lg_rb = 6;
     if (p.nblk <= kLocalBlocks) p.lg_rb = T <= 8 ? 3 : T <= 16 ? 4 : T <= 32 ? 5 : 6;
