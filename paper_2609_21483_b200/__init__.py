@@ -14,7 +14,7 @@ from typing import Optional
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _SRC_DIR = os.path.join(_HERE, "csrc")
 LIB_PATH = os.path.join(_HERE, "libweave_moe.so")
-_SOURCES = ["weave_moe.cu", "weave_kernel.cuh", "weave_ptx.cuh"]
+_SOURCES = ["weave_moe.cu", "weave_kernel.cuh", "weave_stream.cuh", "weave_ptx.cuh"]
 
 WEAVE_OK = 0
 WEAVE_ERR_INVALID_ARG = -1

@@ -153,6 +153,8 @@ struct KParams {
     unsigned die_mask[32]; // bit smid: which half of the chip (die) the SM sits on
     int lists_pt;          // one chunk: two lists of GEMM tiles from this many row tiles on (see tile_lists_from)
     int4 *wait_log;       // [n_sm][8 warps]: written only by a wait that gives up or is cut short by the abort word
+    int st_slots;         // weave_stream_kernel: slots of its ring, and the modelled time of its plan
+    float st_plan_t;
 };
 
 struct TileInfo {
@@ -272,9 +274,9 @@ __device__ __noinline__ void give_up(Ctl *ctl, int where)
 __device__ __noinline__ void note_failed_wait(int4 *log, int where, unsigned what, unsigned want, int how)
 {
     // the first failed wait of a warp is the one that tells where it stood; what it runs into afterwards,
-    // on its way out with the abort word set, is not recorded
-    if (log && log[blockIdx.x * 8 + (threadIdx.x >> 5)].w == 0)
-        log[blockIdx.x * 8 + (threadIdx.x >> 5)] = make_int4(where, (int)what, (int)want, how);
+    // on its way out with the abort word set, is not recorded  (warps 8 and up of the streaming kernel share the slots)
+    int4 *slot = log + blockIdx.x * 8 + ((threadIdx.x >> 5) & 7);
+    if (log && slot->w == 0) *slot = make_int4(where, (int)what, (int)want, how);
 }
 
 // Optional timeline: one 16-byte record {start ns, end ns, kind<<24 | id, extra} per event, per CTA.

@@ -14,6 +14,7 @@
 
 #include "../../include/weave_moe.h"
 #include "weave_kernel.cuh"
+#include "weave_stream.cuh"
 
 using namespace weave;
 
@@ -114,6 +115,8 @@ struct weave_moe {
     int kinds;         // plan kinds AUTO may choose (bit mask)
     int elastic;       // -1 = on under AUTO only, 0 = off, 1 = on
     const float *bw_dev, *tf_dev;     // cost tables on the device (in the workspace unless set otherwise)
+    const float *bw_host, *tf_host;   // the same on the host: tables[], or the static entry's
+    float tables[2][1024];
     void *trace;
     int trace_cap;
     int ep_rank, ep_size;
@@ -125,10 +128,14 @@ struct weave_moe {
     cudaStream_t pipe_h2d, pipe_d2h;
     cudaEvent_t pipe_in_ready[2], pipe_k_done[2], pipe_out_done[2];
     TmaMaps tm;
+    StreamMaps sm;
+    int maps;                   // which of them are encoded (kMapsTiles | kMapsStream): the static entry encodes what a call needs
     EncodeTiledFn encode;
 };
 
 namespace {
+
+enum { kMapsTiles = 1, kMapsStream = 2 };
 
 int cuda_fail(weave_moe *h, cudaError_t e)
 {
@@ -136,19 +143,14 @@ int cuda_fail(weave_moe *h, cudaError_t e)
     return WEAVE_ERR_CUDA;
 }
 
-// bf16 matrix [rows][cols] row-major, box = 64 columns (128 bytes) x 128 rows, 128-byte swizzle
-int encode_map(EncodeTiledFn fn, CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, bool weights,
-               uint32_t box_rows = kBM)
+// bf16 tensor of `rank` dimensions, innermost first, 128-byte swizzle
+int encode_tiled(EncodeTiledFn fn, CUtensorMap *m, const void *base, int rank, const cuuint64_t *dims, const cuuint64_t *strides,
+                 const cuuint32_t *box, CUtensorMapL2promotion promotion)
 {
-    cuuint64_t dims[2] = {cols, rows};
-    cuuint64_t strides[1] = {cols * 2};
-    cuuint32_t box[2] = {kBK, box_rows};
-    cuuint32_t estr[2] = {1, 1};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
     auto encode = [&]() {
-        return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                  weights ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void *>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, promotion, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     };
     CUresult r = encode();
     if (r == CUDA_ERROR_INVALID_CONTEXT || r == CUDA_ERROR_NOT_INITIALIZED) {
@@ -157,6 +159,15 @@ int encode_map(EncodeTiledFn fn, CUtensorMap *m, const void *base, uint64_t rows
         if (cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess) r = encode();
     }
     return r == CUDA_SUCCESS ? 0 : (int)r;
+}
+
+// bf16 matrix [rows][cols] row-major, box = 64 columns (128 bytes) x 128 rows
+int encode_map(EncodeTiledFn fn, CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, bool weights,
+               uint32_t box_rows = kBM)
+{
+    const cuuint64_t dims[2] = {cols, rows}, strides[1] = {cols * 2};
+    const cuuint32_t box[2] = {kBK, box_rows};
+    return encode_tiled(fn, m, base, 2, dims, strides, box, weights ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
 }
 
 int encode_maps(EncodeTiledFn fn, TmaMaps *m, const void *xe, const void *hbuf, const void *gate_up, const void *down,
@@ -173,6 +184,79 @@ int encode_maps(EncodeTiledFn fn, TmaMaps *m, const void *xe, const void *hbuf, 
         r |= encode_map(fn, &m->h_n[i], hbuf, p_max, ffn, false, 8u << i);
     }
     return r;
+}
+
+// the weights as weave_stream_kernel reads them: one box is 1 to 8 units of columns (for gate_up the gate and the up rows) x
+// 128 or 64 of K, with the 64-column blocks of K as a dimension of their own
+int encode_stream_maps(EncodeTiledFn fn, StreamMaps *m, const void *gate_up, const void *down, uint64_t EE, uint64_t hidden, uint64_t ffn)
+{
+    int r = 0;
+    for (cuuint32_t w = 1; w <= kStWarps; ++w) {
+        const cuuint32_t kb = (cuuint32_t)stream_kblocks((int)w);
+        const cuuint64_t gd[4] = {64, EE * 2 * ffn - ffn, 2, hidden / 64}, gs[3] = {hidden * 2, ffn * hidden * 2, 128};
+        const cuuint32_t gb[4] = {64, kStUnitG * w, 2, kb};
+        r |= encode_tiled(fn, &m->g[w - 1], gate_up, 4, gd, gs, gb, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+        const cuuint64_t dd[3] = {64, EE * hidden, ffn / 64}, ds[2] = {ffn * 2, 128};
+        const cuuint32_t db[3] = {64, kStUnitD * w, kb};
+        r |= encode_tiled(fn, &m->d[w - 1], down, 3, dd, ds, db, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+    }
+    return r;
+}
+
+// the tensor maps of one kernel or the other, unless they are there already
+int need_maps(weave_moe *h, int which)
+{
+    if (h->maps & which) return 0;
+    const weave_moe_config &c = h->cfg;
+    const uint64_t EE = (uint64_t)(c.num_experts + c.num_shared), hidden = (uint64_t)c.hidden, ffn = (uint64_t)c.ffn;
+    const int r = which == kMapsTiles ? encode_maps(h->encode, &h->tm, h->ws + h->L.xe, h->ws + h->L.hbuf, c.gate_up, c.down,
+                                                    (uint64_t)h->L.p_max, EE, hidden, ffn)
+                                      : encode_stream_maps(h->encode, &h->sm, c.gate_up, c.down, EE, hidden, ffn);
+    if (r) { h->last_cuda_error = r; return WEAVE_ERR_CUDA; }
+    h->maps |= which;
+    return 0;
+}
+
+// Is the phased plan AUTO's pick for a batch of T tokens (no expert-parallel share)?  The kernel's arg-min in the same
+// fp32 operations: the phased plan loses ties to the split and to dispatch-all and wins them against rejoin.
+bool phased_is_picked(const weave_moe *h, int T, float *t_phased)
+{
+    const weave_moe_config &c = h->cfg;
+    if (!(h->kinds & (1 << kPlanPhased))) return false;
+    const float *bw = h->bw_host, *tf = h->tf_host;
+    const int n_sm = h->n_cta, EE = c.num_experts + c.num_shared, P = T * (c.top_k + c.num_shared);
+    const float B = (float)(2 * c.hidden);
+    const float w_comp = (((float)P * 6.0f) * (float)c.hidden) * (float)c.ffn, w_disp = (float)(T + P) * B, w_comb = (float)(P + T) * B;
+    const float one_a = 1.0f - h->alpha, bw_n = bw[n_sm], tf_n = tf[n_sm], t_disp = w_disp / bw_n;
+    const float t = (t_disp + w_comp / tf_n) + one_a * (w_comb / bw_n);
+    for (int i = 0; i < 64; ++i) {
+        const int cc = h->c_min + i * h->c_step;
+        if (cc < 2 || cc > h->c_max || cc > n_sm - 2) continue;
+        const float b = bw[cc], f = tf[n_sm - cc];
+        for (int ki = 0; ki < 4; ++ki) {
+            if ((EE << ki) > kMaxSeg) break;
+            const float t_comp = w_comp / (f * h->eff[ki]), t_tail = one_a * (w_comb / (b * (float)(1 << ki)));
+            if ((h->kinds & (1 << kPlanSplit)) && std::max(t_comp + t_tail, (w_disp + w_comb) / b) <= t) return false;
+            if ((h->kinds & (1 << kPlanDispatchAll)) && t_disp + std::max(t_comp + t_tail, w_comb / b) <= t) return false;
+        }
+        if (h->kinds & (1 << kPlanRejoin)) {
+            const float td = w_disp / b, rest = std::max(0.0f, w_comp - std::min(td * f, w_comp * 0.6666667f));
+            if ((td + rest / tf_n) + one_a * (w_comb / bw_n) < t) return false;
+        }
+    }
+    *t_phased = t;
+    return true;
+}
+
+// Batches that weave_stream_kernel takes: the number of its ring's slots, 0 where the general kernel runs.  (A timeline and the
+// withheld-flag hook are about the general kernel's tiles and flags.)
+int stream_slots(const weave_moe *h, int T)
+{
+    const weave_moe_config &c = h->cfg;
+    if (T > kStMaxT || h->mode != WEAVE_SCHED_AUTO || h->ep_size != 1 || h->withhold_mb >= 0 || h->trace) return 0;
+    const size_t rows = (size_t)T * ((size_t)std::max(c.hidden, c.ffn) * 2 + kStPad);
+    if (rows > (size_t)(kStArea - kStMinSlots * kStSlot)) return 0;
+    return std::min(kStMaxSlots, (int)((kStArea - rows) / kStSlot));
 }
 
 void default_tables(int n_sm, std::vector<float> &bw, std::vector<float> &tf)
@@ -256,6 +340,9 @@ int upload_tables(weave_moe *h, const float *bw, const float *tf)
     if (e != cudaSuccess) return cuda_fail(h, e);
     e = cudaMemcpy(h->ws + h->L.tf, tf, sizeof(float) * (h->n_sm + 1), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(h, e);
+    memcpy(h->tables[0], bw, sizeof(float) * (h->n_sm + 1));
+    memcpy(h->tables[1], tf, sizeof(float) * (h->n_sm + 1));
+    h->bw_host = h->tables[0]; h->tf_host = h->tables[1];
     return WEAVE_OK;
 }
 
@@ -329,6 +416,8 @@ int weave_moe_create(const weave_moe_config *cfg, weave_moe_t *out)
 
     e = cudaFuncSetAttribute(weave_moe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) { int rc = cuda_fail(h, e); delete h; return rc; }
+    e = cudaFuncSetAttribute(weave_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e != cudaSuccess) { int rc = cuda_fail(h, e); delete h; return rc; }
     e = cudaFuncSetAttribute(weave_moe_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 0);
     int occ = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, weave_moe_kernel, kThreads, kSmemBytes);
@@ -347,13 +436,9 @@ int weave_moe_create(const weave_moe_config *cfg, weave_moe_t *out)
     cudaDriverEntryPointQueryResult qres;
     e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fnp, cudaEnableDefault, &qres);
     if (e != cudaSuccess || !fnp || qres != cudaDriverEntryPointSuccess) { delete h; return WEAVE_ERR_UNSUPPORTED_DEVICE; }
-    EncodeTiledFn enc = reinterpret_cast<EncodeTiledFn>(fnp);
-    const int EE = cfg->num_experts + cfg->num_shared;
-    int r = 0;
-    r = encode_maps(enc, &h->tm, h->ws + L.xe, h->ws + L.hbuf, cfg->gate_up, cfg->down, (uint64_t)L.p_max, (uint64_t)EE,
-                    (uint64_t)cfg->hidden, (uint64_t)cfg->ffn);
-    if (r) { h->last_cuda_error = r; delete h; return WEAVE_ERR_CUDA; }
-    h->encode = enc;
+    h->encode = reinterpret_cast<EncodeTiledFn>(fnp);
+    h->maps = 0;
+    if (need_maps(h, kMapsTiles) || need_maps(h, kMapsStream)) { delete h; return WEAVE_ERR_CUDA; }
 
     e = cudaMemset(h->ws, 0, L.zero_end);
     if (e != cudaSuccess) { int rc = cuda_fail(h, e); delete h; return rc; }
@@ -434,6 +519,19 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     memcpy(p.die_mask, h->die_mask, sizeof(p.die_mask));
     p.lists_pt = tile_lists_from(h->two_dies, h->n_cta / 2, p.EE, c.ffn, p.nt1);
 
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    p.st_slots = stream_slots(h, T);
+    if (p.st_slots && phased_is_picked(h, T, &p.st_plan_t)) {
+        if (const int rc = need_maps(h, kMapsStream)) return rc;
+        void *sargs[] = {&p, &h->sm};
+        cudaError_t e = cudaLaunchCooperativeKernel((const void *)weave_stream_kernel, dim3(h->n_cta), dim3(kStThreads), sargs,
+                                                    (size_t)kSmemBytes, st);
+        if (e != cudaSuccess) return cuda_fail(h, e);
+        h->last_T = T;
+        h->last_stream = st;
+        return WEAVE_OK;
+    }
+
     // A small batch under AUTO: its gate/up tiles may read x itself (kernel body).  Not in an expert-parallel share, whose
     // remote tokens are to be read from their staged copies, and not under the withheld-flag hook, which is about a wait
     // that does not exist then.
@@ -444,8 +542,8 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
         if (r) { h->last_cuda_error = r; return WEAVE_ERR_CUDA; }
     }
 
+    if (const int rc = need_maps(h, kMapsTiles)) return rc;
     void *args[] = {&p, &h->tm};
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     // one CTA per SM; the kernel is compiled with a cluster shape of two neighbouring CTAs (the GEMM
     // phase's CTA pairs); cooperative, so that all CTAs are co-resident for the in-kernel grid
     // barrier and flag waits
@@ -862,6 +960,7 @@ struct StaticDevice {
     uint8_t *ctl;         // device address of g_static_ctl on this device
     uint8_t *base;        // device address of g_static_scratch on this device, rounded up to 1024
     const float *tables;  // device address of g_static_tables on this device
+    float host_tables[2][1024];
     size_t usable;
     int n_sm;
     unsigned die_mask[32];
@@ -899,13 +998,16 @@ int static_setup(int dev, StaticDevice **out)
         {
             std::vector<float> bw, tf;      // host heap only; filled and copied once per device
             default_tables(d.n_sm, bw, tf);
+            std::copy(bw.begin(), bw.end(), d.host_tables[0]);
+            std::copy(tf.begin(), tf.end(), d.host_tables[1]);
             if (cudaMemcpy(tsym, bw.data(), sizeof(float) * (d.n_sm + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
                 cudaMemcpy(static_cast<float *>(tsym) + 1024, tf.data(), sizeof(float) * (d.n_sm + 1),
                            cudaMemcpyHostToDevice) != cudaSuccess)
                 return WEAVE_ERR_CUDA;
         }
         if (cudaFuncSetAttribute(weave_moe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) !=
-            cudaSuccess)
+            cudaSuccess ||
+            cudaFuncSetAttribute(weave_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
             return WEAVE_ERR_CUDA;
         if (cudaMemset(d.base, 0, 64 * 1024) != cudaSuccess) return WEAVE_ERR_CUDA;
         d.two_dies = find_dies(prop.multiProcessorCount, d.base, d.die_mask);
@@ -970,15 +1072,11 @@ int weave_moe_forward_static(int hidden, int ffn, int num_experts, int top_k, in
     h.elastic = -1;
     h.bw_dev = sd->tables;
     h.tf_dev = sd->tables + 1024;
+    h.bw_host = sd->host_tables[0];
+    h.tf_host = sd->host_tables[1];
     memcpy(h.die_mask, sd->die_mask, sizeof(h.die_mask));
     h.two_dies = sd->two_dies;
     h.encode = sd->encode;
-    const int EE = num_experts + num_shared;
-    int r = 0;
-    r = encode_maps(sd->encode, &h.tm, h.ws + L.xe, h.ws + L.hbuf, gate_up, down, (uint64_t)L.p_max, (uint64_t)EE,
-                    (uint64_t)hidden, (uint64_t)ffn);
-    if (r) return WEAVE_ERR_CUDA;
-
     return weave_moe_forward(&h, x, router_logits, out, T, cuda_stream);
 }
 

@@ -1,0 +1,74 @@
+"""The streaming kernel of the smallest batches against the oracle and, bit for bit, against the general kernel
+(the SERIAL schedule): outputs, routing, dispatched rows, h and y, and the plan that is reported."""
+import numpy as np
+import pytest
+import torch
+
+import workloads as wl
+import paper_2609_21483_b200 as pk
+from oracle import cost_model as cm
+from parity import run_case, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def _state(moe, T):
+    r = {k: v.clone() for k, v in moe.routing(T).items()}
+    r.update({k: v.view(torch.int16).clone() for k, v in moe.intermediates(T).items()})
+    return r
+
+
+@pytest.mark.parametrize("T", [1, 2, 7, 8, 9, 13, 16, 17, 27, 32])
+@pytest.mark.parametrize("H,I,E,k,S", [(128, 128, 4, 1, 0),        # fewer units than CTAs
+                                       (1152, 384, 256, 16, 0),    # k and E at their limits, tiles of every width
+                                       (2048, 1408, 12, 3, 2),     # ring used many times over; shared experts: 8 rows and more
+                                       (256, 7168, 3, 2, 0),       # long rows of h
+                                       (16384, 128, 5, 2, 1),      # one row of x takes 32 KB
+                                       (512, 1024, 1, 1, 0)])      # one expert has every token
+def test_smallest_batches_match_oracle_and_general_kernel(T, H, I, E, k, S):
+    cfg = wl.MoEConfig(f"stream_{T}_{H}", 1000 + E, T=T, H=H, I=I, E=E, k=k, S=S, zipf_s=0.8 if E > 4 else None)
+    inp = wl.make_inputs(cfg)
+    dev = to_dev(inp)
+    moe, out, _ = run_case(cfg, inp=inp, dev_tensors=dev)
+    assert moe.plan()["kind"] == pk.PLAN_PHASED
+    got = _state(moe, T)
+    for sm in (4, 100, moe.geometry()["n_sm"]):      # shares of a few tiles and of many
+        moe.set_sm_count(sm)
+        for _ in range(3):
+            assert torch.equal(moe.forward(dev[0], dev[1]).view(torch.int16), out.view(torch.int16)), sm
+    _, general, _ = run_case(cfg, sched=(pk.SCHED_SERIAL, 0, 1, 0), inp=inp, dev_tensors=dev, moe=moe)
+    assert torch.equal(out.view(torch.int16), general.view(torch.int16))
+    want = _state(moe, T)
+    for name in want:
+        assert torch.equal(got[name], want[name]), name
+    moe.close()
+
+
+def test_smallest_batches_report_the_plan_of_the_cost_model():
+    """Whichever kernel runs, the plan is the arg-min over the candidates for the tables that are set."""
+    H, I, E, k = 256, 256, 130, 4
+    cfg = wl.MoEConfig("stream_plan", 1200, T=8, H=H, I=I, E=E, k=k)
+    x, lg, gu, dn = to_dev(wl.make_inputs(cfg))
+    moe = pk.WeaveMoE(gu, dn, E, k, 0, max_tokens=8)
+    N = moe.geometry()["n_sm"]
+    rng = np.random.default_rng(3)
+    seen = set()
+    for trial in range(24):
+        T, kinds = int(rng.integers(1, 9)), int(rng.choice([4, 5, 6, 7, 15]))
+        idx = np.arange(N + 1, dtype=np.float64)
+        bw = (10 ** rng.uniform(3.0, 5.5) * np.minimum(idx, rng.uniform(20, 148))).astype(np.float32)
+        tf = (10 ** rng.uniform(6, 8.0) * idx ** rng.uniform(0.2, 1.0)).astype(np.float32)
+        bw[0], tf[0] = bw[1], tf[1]
+        eff, alpha = np.array([1.0, .9, .8, .7], np.float32), float(rng.uniform(0, 0.95))
+        tab = cm.CostTables(N, bw, tf, eff, alpha, c_min=2, c_max=N // 2, c_step=2, steal_workers=N // 2, max_segments=1024, kinds=kinds)
+        moe.set_cost_tables(bw, tf, eff, alpha, 2, N // 2, 2)
+        moe.set_model_options(kinds, -1)
+        moe.forward(x[:T].contiguous(), lg[:T].contiguous())
+        moe.check()
+        tiles = int((moe.routing(T)["counts"] > 0).sum()) * (I // 128 + (H + 255) // 256)
+        want, got = cm.plan(tab, T, T * k, H, I, [tiles] * 4, n_experts=E), moe.plan()
+        assert (got["kind"], got["c"], got["K"]) == (want.kind, want.c, want.K), (trial, got, want)
+        assert got["t_total_us"] == pytest.approx(float(want.t_total), rel=1e-6)
+        seen.add(got["kind"])
+    assert pk.PLAN_PHASED in seen and len(seen) > 1
+    moe.close()
