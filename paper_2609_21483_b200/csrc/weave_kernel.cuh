@@ -153,8 +153,7 @@ struct KParams {
     unsigned die_mask[32]; // bit smid: which half of the chip (die) the SM sits on
     int lists_pt;          // one chunk: two lists of GEMM tiles from this many row tiles on (see tile_lists_from)
     int4 *wait_log;       // [n_sm][8 warps]: written only by a wait that gives up or is cut short by the abort word
-    int st_slots;         // weave_stream_kernel: slots of its ring, and the modelled time of its plan
-    float st_plan_t;
+    float st_plan_t;      // weave_stream_kernel: the modelled time of its plan
 };
 
 struct TileInfo {

@@ -191,15 +191,15 @@ int encode_maps(EncodeTiledFn fn, TmaMaps *m, const void *xe, const void *hbuf, 
 int encode_stream_maps(EncodeTiledFn fn, StreamMaps *m, const void *gate_up, const void *down, uint64_t EE, uint64_t hidden, uint64_t ffn)
 {
     int r = 0;
-    for (cuuint32_t w = 1; w <= kStWarps; ++w) {
-        const cuuint32_t kb = (cuuint32_t)stream_kblocks((int)w);
-        const cuuint64_t gd[4] = {64, EE * 2 * ffn - ffn, 2, hidden / 64}, gs[3] = {hidden * 2, ffn * hidden * 2, 128};
-        const cuuint32_t gb[4] = {64, kStUnitG * w, 2, kb};
-        r |= encode_tiled(fn, &m->g[w - 1], gate_up, 4, gd, gs, gb, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
-        const cuuint64_t dd[3] = {64, EE * hidden, ffn / 64}, ds[2] = {ffn * 2, 128};
-        const cuuint32_t db[3] = {64, kStUnitD * w, kb};
-        r |= encode_tiled(fn, &m->d[w - 1], down, 3, dd, ds, db, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
-    }
+    const cuuint64_t gd[4] = {64, EE * 2 * ffn - ffn, 2, hidden / 64}, gs[3] = {hidden * 2, ffn * hidden * 2, 128};
+    const cuuint64_t dd[3] = {64, EE * hidden, ffn / 64}, ds[2] = {ffn * 2, 128};
+    for (cuuint32_t kb = 1; kb <= 2; ++kb)
+        for (cuuint32_t w = 1; w <= kStWarps / kb; ++w) {
+            const cuuint32_t gb[4] = {64, kStUnitG * w, 2, kb}, db[3] = {64, kStUnitD * w, kb};
+            const int i = stream_map((int)w, (int)kb);
+            r |= encode_tiled(fn, &m->g[i], gate_up, 4, gd, gs, gb, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+            r |= encode_tiled(fn, &m->d[i], down, 3, dd, ds, db, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+        }
     return r;
 }
 
@@ -248,15 +248,14 @@ bool phased_is_picked(const weave_moe *h, int T, float *t_phased)
     return true;
 }
 
-// Batches that weave_stream_kernel takes: the number of its ring's slots, 0 where the general kernel runs.  (A timeline and the
-// withheld-flag hook are about the general kernel's tiles and flags.)
-int stream_slots(const weave_moe *h, int T)
+// Batches that weave_stream_kernel takes: up to eight tokens (the N of one product), whose rows of x, or of h if they all went to
+// one expert, leave room for a ring of 80 KB.  (A timeline and the withheld-flag hook are about the general kernel's tiles and
+// flags.)
+bool streams(const weave_moe *h, int T)
 {
     const weave_moe_config &c = h->cfg;
-    if (T > kStMaxT || h->mode != WEAVE_SCHED_AUTO || h->ep_size != 1 || h->withhold_mb >= 0 || h->trace) return 0;
-    const size_t rows = (size_t)T * ((size_t)std::max(c.hidden, c.ffn) * 2 + kStPad);
-    if (rows > (size_t)(kStArea - kStMinSlots * kStSlot)) return 0;
-    return std::min(kStMaxSlots, (int)((kStArea - rows) / kStSlot));
+    if (T > kStTokens || h->mode != WEAVE_SCHED_AUTO || h->ep_size != 1 || h->withhold_mb >= 0 || h->trace) return false;
+    return (size_t)T * ((size_t)std::max(c.hidden, c.ffn) * 2 + kStPad) <= (size_t)(kStArea - kStMinRing);
 }
 
 void default_tables(int n_sm, std::vector<float> &bw, std::vector<float> &tf)
@@ -520,8 +519,7 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     p.lists_pt = tile_lists_from(h->two_dies, h->n_cta / 2, p.EE, c.ffn, p.nt1);
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    p.st_slots = stream_slots(h, T);
-    if (p.st_slots && phased_is_picked(h, T, &p.st_plan_t)) {
+    if (streams(h, T) && phased_is_picked(h, T, &p.st_plan_t)) {
         if (const int rc = need_maps(h, kMapsStream)) return rc;
         void *sargs[] = {&p, &h->sm};
         cudaError_t e = cudaLaunchCooperativeKernel((const void *)weave_stream_kernel, dim3(h->n_cta), dim3(kStThreads), sargs,

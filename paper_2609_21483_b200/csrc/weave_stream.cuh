@@ -8,6 +8,13 @@
 // rows the M axis; the products are summed 16 of K at a time in ascending order, as the general kernel's
 // tcgen05.mma sums them, and the results carry the same bits.
 //
+// One launch behind another, us, the general kernel / this one, and the time of the bytes: Qwen3-30B-shaped T = 1 37.7 / 26.3 (11.5), T = 8
+// 97.9 / 88.5 (77.8); Qwen3-235B-shaped T = 1 81 / 60.2 (46.1); Mixtral-shaped T = 1 159 / 119 (107.5), T = 4 314 / 295 (269);
+// DSv2-Lite-shaped T = 7 112.5 / 102.8 (87.1); 8 experts T = 1 25.3 / 14.6.  Bound by HBM but for a chain of 10 us in front of the first
+// weights (launch, routing) and around the exchange of h and y.  Measured and left: with 9 to 16 tokens +-2 %, slower above (the
+// general kernel is at HBM speed there); a quarter of the units claimed in tiles of one or two (their chain of products is one
+// warp's: 282 us where 189 were); a unit per warp with a ring and a claim of its own (every warp holds a unit to the end: 120 / 103).
+//
 //   warp 0        producer: one tensor copy per ring slot (a tile's rows x 64 or 128 of K)
 //   warp 1        makes the finished tiles' arrivals on the ready counters
 //   warps 2..7    write down the routing and the dispatched rows
@@ -21,18 +28,38 @@
 namespace weave {
 
 constexpr int kStThreads = 512;
-constexpr int kStTokens = 32;                     // one 32-bit mask per expert
-constexpr int kStMaxT = 8;                        // largest batch (see stream_slots)
-constexpr int kStSlot = 16384;                    // bytes of a ring slot
-constexpr int kStMaxSlots = 12, kStMinSlots = 5;
+constexpr int kStTokens = 8;                      // largest batch: one N tile (see stream_slots)
+constexpr int kStMaxSlot = 16384;                 // bytes of a ring slot, at most
+constexpr int kStMaxSlots = 16;
+constexpr int kStMinRing = 5 * kStMaxSlot, kStFullRing = 10 * kStMaxSlot;      // bytes
 constexpr int kStArea = kStages * kStageBytes + kEpiStageBytes;      // shared memory in front of the SmemTail: ring, then rows
 constexpr int kStUnitG = 8, kStUnitD = 16;        // columns of h / of y that one warp works on: 8 gate + 8 up rows, or 16 rows
 constexpr int kStWarps = 8;                       // ... so a tile has up to 8 units
 constexpr int kStPad = 16;                        // bytes between two rows of x or h in shared memory (no bank conflicts)
 
-// boxes of 1 to 8 units: gate_up as [K/64][gate, up][row][64], down as [K/64][row][64]; 128 of K up to 4 units, 64 from 5 on
-struct StreamMaps { CUtensorMap g[kStWarps], d[kStWarps]; };
-__host__ __device__ __forceinline__ constexpr int stream_kblocks(int w) { return w <= kStWarps / 2 ? 2 : 1; }
+// Boxes of 1 to 8 units: gate_up as [K/64][gate, up][row][64], down as [K/64][row][64], with one or two blocks of K.
+constexpr int kStMaps = kStWarps + kStWarps / 2;
+struct StreamMaps { CUtensorMap g[kStMaps], d[kStMaps]; };
+__host__ __device__ __forceinline__ constexpr int stream_map(int units, int kblocks) { return units - 1 + (kblocks - 1) * kStWarps; }
+
+// This CTA's share of a phase: n units from unit c of active expert a on (the units of all active experts' columns, one
+// expert behind the other, are dealt out evenly), in tiles of `cap` units, at most 8.  A tile may go over from one expert to
+// the next (w1 units of the first): a tile is a chain of K / 16 dependent products however narrow it is, and two short
+// ones where an expert ends cost the CTA 2 to 3 us more than one (T = 1 Qwen3-30B-shaped).
+struct StreamShare {
+    int a, c, n, cap, upe;      // upe: units per expert
+    __device__ __forceinline__ StreamShare() {}
+    __device__ __forceinline__ StreamShare(int n_act, int upe_, int cta, int ctas) : upe(upe_)
+    {
+        const unsigned total = (unsigned)(n_act * upe_);      // (at most 2^18 units, 2^10 CTAs)
+        const unsigned u = total * (unsigned)cta / (unsigned)ctas;
+        n = (int)(total * (unsigned)(cta + 1) / (unsigned)ctas - u);
+        a = (int)(u / (unsigned)upe);
+        c = (int)u - a * upe;
+        const int tiles = max(1, (n + kStWarps - 1) / kStWarps);
+        cap = max(1, (n + tiles - 1) / tiles);
+    }
+};
 
 struct StreamShared {      // lies over the SmemTail's segment tables, which this kernel does not use
     uint64_t full[kStMaxSlots], empty[kStMaxSlots];
@@ -42,8 +69,11 @@ struct StreamShared {      // lies over the SmemTail's segment tables, which thi
     int act[kMaxEE];                              // experts with rows
     int n_act, failed;
     unsigned wsum[8];
+    int wmax[8];
+    StreamShare share[2];                         // gate/up, down
     int idx[kStTokens][kMaxTopK], row[kStTokens][kMaxTopK];
     float gate[kStTokens][kMaxTopK];
+    __device__ __forceinline__ int rows(int a) const { return off[act[a] + 1] - off[act[a]]; }
 };
 constexpr size_t kStSharedAt = (offsetof(SmemTail, seg_mb0) + 15) / 16 * 16;      // (the tail starts on a 1024-byte boundary)
 static_assert(kStSharedAt + sizeof(StreamShared) <= sizeof(SmemTail), "must fit the segment tables");
@@ -71,25 +101,21 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const void *map, int c
                  ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar)) : "memory");
 }
 
-// This CTA's share of a phase: units [u, end) of all active experts' columns, in tiles of 1 to 8 units (equal ones where
-// an expert's part is cut) that never span two experts.
-struct StreamWalk {
-    int u, end, upe;      // upe: units per expert
-    int a, c, w;          // the current tile: active expert, first unit in it, units
-    __device__ __forceinline__ StreamWalk(int n_act, int upe_, int cta, int ctas) : upe(upe_)
+struct StreamWalk : StreamShare {
+    int w, w1, at_a, at_c;      // the current tile: units, units of its first expert, that expert and the first unit of it
+    __device__ __forceinline__ StreamWalk(const StreamShare &s) : StreamShare(s) {}
+    // rows: rows of h that fit shared memory (0: no limit)
+    __device__ __forceinline__ bool next(const StreamShared &X, int rows)
     {
-        const int total = n_act * upe_;
-        u = (int)((long long)total * cta / ctas);
-        end = (int)((long long)total * (cta + 1) / ctas);
-    }
-    __device__ __forceinline__ bool next()
-    {
-        if (u >= end) return false;
-        a = u / upe;
-        c = u - a * upe;
-        const int n = min(upe - c, end - u), tiles = (n + kStWarps - 1) / kStWarps;
-        w = (n + tiles - 1) / tiles;
-        u += w;
+        if (n == 0) return false;
+        at_a = a;
+        at_c = c;
+        w = min(cap, n);
+        w1 = min(w, upe - c);
+        if (rows && w1 < w && X.rows(a) + X.rows(a + 1) > rows) w = w1;
+        n -= w;
+        c += w;
+        if (c >= upe) { c -= upe; ++a; }
         return true;
     }
 };
@@ -114,18 +140,13 @@ __device__ __forceinline__ void stream_route(const KParams &p, StreamShared &X, 
         if (key[i] > bk) { bk = key[i]; be = e; }
     }
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicCAS(&p.ctl->status, 0, kErrNonFinite);
-    float vmax = 0.f, sum = 0.f, mine = 0.f;
+    float mine = 0.f;      // lane j: logit and expert of slot j
     int my_e = 0;
 #pragma unroll 1
     for (int j = 0; j < p.k; ++j) {
         const unsigned top = __reduce_max_sync(0xffffffffu, bk);
         const int hi = (int)__reduce_min_sync(0xffffffffu, bk == top ? (unsigned)be : 0x7fffffffu);
-        const float v = float_from_order_key(top);
-        if (j == 0) vmax = v;
-        const float pj = expf(v - vmax);
-        sum += pj;
-        if (lane == j) { mine = pj; my_e = hi; }
-        if (lane == 0) atomicOr(&X.mask[hi], 1u << t);
+        if (lane == j) { mine = float_from_order_key(top); my_e = hi; }
         if ((hi & 31) == lane) {
             bk = 0u; be = 0x7fffffff;
 #pragma unroll
@@ -135,54 +156,69 @@ __device__ __forceinline__ void stream_route(const KParams &p, StreamShared &X, 
             }
         }
     }
+    mine = expf(mine - __shfl_sync(0xffffffffu, mine, 0));
+    float sum = 0.f;
+#pragma unroll 1
+    for (int j = 0; j < p.k; ++j) sum += __shfl_sync(0xffffffffu, mine, j);      // slot order
     if (lane < p.k) {
+        atomicOr(&X.mask[my_e], 1u << t);
         X.idx[t][lane] = my_e;
         X.gate[t][lane] = __fdiv_rn(mine, sum);
     }
 }
 
-// One tile for a warp: 16 weight rows x 8 * NT tokens, KB blocks of 64 of K per ring slot.  a_off: this lane's ldmatrix row in a
-// slot, blk: bytes of a block of K in the slot, b_row: this lane's rows of x or h.  The rows' values are fetched before the wait for the slot.
-template <int NT, int KB>
-__device__ __forceinline__ bool stream_tile(const KParams &p, StreamShared &X, uint32_t ring, int slots, int &slot, uint32_t &ph,
-                                            int nk, bool works, uint32_t a_off, uint32_t blk, const uint32_t (&b_row)[4], float (&acc)[NT][4])
+// One tile for a warp: 16 weight rows x 8 tokens, KB blocks of 64 of K per ring slot.  a_off: this lane's ldmatrix row in a slot,
+// blk: bytes of a block of K in the slot, b_row: this lane's row of x or h.  A block's operands are fetched between the
+// products of the block before: the chain of dependent products (and nothing else) sets the pace.
+struct StreamRing { uint32_t base, bytes; int slots, slot; uint32_t ph; };
+template <int KB>
+__device__ __forceinline__ bool stream_tile(const KParams &p, StreamShared &X, StreamRing &r, int K, bool works, uint32_t a_off, uint32_t blk,
+                                            uint32_t b_row, float (&acc)[4])
 {
     const int lane = threadIdx.x & 31;
     const uint32_t sw = (uint32_t)(lane & 7), kh = (uint32_t)(lane >> 4);
     bool ok = true;
+    uint32_t a[2][4][4], b[2][2][4], a0 = 0;
 #pragma unroll
-    for (int n = 0; n < NT; ++n)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[n][i] = 0.f;
-    for (int kk = 0; kk < nk; ++kk) {
-        uint32_t b[NT][2][4];
-#pragma unroll
-        for (int n = 0; n < NT; ++n)
-#pragma unroll
-            for (int i = 0; i < 2; ++i) ldmatrix_x4(b_row[n] + (uint32_t)(kk * (KB * 128) + i * 64), b[n][i]);
-        ok = mbar_wait(&X.full[slot], ph, p, 61) && ok;
-        if (works) {
-            const uint32_t a0 = ring + (uint32_t)(slot * kStSlot) + a_off;
-#pragma unroll
-            for (int kb = 0; kb < KB; ++kb) {
-                uint32_t a[4][4];
-#pragma unroll
-                for (int s = 0; s < 4; ++s) ldmatrix_x4(a0 + (uint32_t)kb * blk + (((2u * (uint32_t)s + kh) ^ sw) << 4), a[s]);
-                if (kb > 0) {
-#pragma unroll
-                    for (int n = 0; n < NT; ++n)
-#pragma unroll
-                        for (int i = 0; i < 2; ++i) ldmatrix_x4(b_row[n] + (uint32_t)(kk * (KB * 128) + kb * 128 + i * 64), b[n][i]);
-                }
-#pragma unroll
-                for (int s = 0; s < 4; ++s)
-#pragma unroll
-                    for (int n = 0; n < NT; ++n) mma_16816(acc[n], a[s], b[n][s >> 1][2 * (s & 1)], b[n][s >> 1][2 * (s & 1) + 1]);
-            }
-        }
+    for (int i = 0; i < 4; ++i) acc[i] = 0.f;
+    auto arrived = [&](int j) {      // block j (of parity j & 1): its slot is there
+        if (KB == 1 || (j & 1) == 0) {
+            ok = mbar_wait(&X.full[r.slot], r.ph, p, 61) && ok;
+            a0 = r.base + (uint32_t)r.slot * r.bytes + a_off;
+            if (++r.slot == r.slots) { r.slot = 0; r.ph ^= 1u; }
+        } else a0 += blk;
+    };
+    auto fetch = [&](int buf, int j, int s) {      // 16 of K
+        ldmatrix_x4(a0 + (((2u * (uint32_t)s + kh) ^ sw) << 4), a[buf][s]);
+        if ((s & 1) == 0) ldmatrix_x4(b_row + (uint32_t)(j * 128 + s * 32), b[buf][s >> 1]);
+    };
+    auto free_slot = [&](int slot) {      // the slot's values are in registers
         __syncwarp();
         if (lane == 0) mbar_arrive(&X.empty[slot]);
-        if (++slot == slots) { slot = 0; ph ^= 1u; }
+    };
+    const int nb = K / 64;      // even
+    int held = r.slot;
+    arrived(0);
+#pragma unroll
+    for (int s = 0; s < 4; ++s) fetch(0, 0, s);
+    for (int j = 0; j < nb; j += 2) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const bool more = h == 0 || j + 2 < nb;
+            const int last = held;
+            if (more) {
+                if (KB == 1 || h == 1) held = r.slot;
+                arrived(j + h + 1);
+            }
+            if (works) {
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    mma_16816(acc, a[h][s], b[h][s >> 1][2 * (s & 1)], b[h][s >> 1][2 * (s & 1) + 1]);
+                    if (more) fetch(h ^ 1, j + h + 1, s);
+                }
+            }
+            if (KB == 1 || h == 1) free_slot(last);
+        }
     }
     return ok;
 }
@@ -195,38 +231,32 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
     StreamShared &X = *reinterpret_cast<StreamShared *>(reinterpret_cast<uint8_t *>(&S) + kStSharedAt);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cta = (int)blockIdx.x, ctas = (int)gridDim.x;
-    const int slots = p.st_slots;
-    const uint32_t ring = smem_u32(stages), rows_s = ring + (uint32_t)(slots * kStSlot);
+    const uint32_t ring = smem_u32(stages), area_end = ring + (uint32_t)kStArea;
 
-    // the logits of this warp's tokens and the batch's rows of x start on their way before anything else
-    float lg[2][8];
+    // the logits of this warp's token and the batch's rows of x start on their way before anything else
+    float lg[8];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const int t = warp + 16 * r;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int e = lane + 32 * i;
-            lg[r][i] = t < p.T && e < p.E ? __ldcg(p.logits + (size_t)t * p.E + e) : 0.f;
-        }
+    for (int i = 0; i < 8; ++i) {
+        const int e = lane + 32 * i;
+        lg[i] = warp < p.T && e < p.E ? __ldcg(p.logits + (size_t)warp * p.E + e) : 0.f;
     }
-    const uint32_t pitch_x = (uint32_t)p.H * 2u + kStPad;
+    const uint32_t pitch_x = (uint32_t)p.H * 2u + kStPad, pitch_h = (uint32_t)p.I * 2u + kStPad, x_s = area_end - (uint32_t)p.T * pitch_x;
     if (warp > 0) {
         const int per_row = p.H >> 3;
         for (int t = 0; t < p.T; ++t)
             for (int c = tid - 32; c < per_row; c += kStThreads - 32)
-                cp_async_16(rows_s + (uint32_t)t * pitch_x + (uint32_t)(c * 16), p.x + (size_t)t * p.H + c * 8);
+                cp_async_16(x_s + (uint32_t)t * pitch_x + (uint32_t)(c * 16), p.x + (size_t)t * p.H + c * 8);
     }
     if (tid == 0) {
         const unsigned odd = (ld_relaxed_u32(&p.ctl->epoch) >> 16) & 1u;
-#pragma unroll 1
-        for (int i = 0; i < slots; ++i) { mbar_init(&X.full[i], 1); mbar_init(&X.empty[i], kStWarps); }
-#pragma unroll 1
-        for (int i = 0; i < 2; ++i) { mbar_init(&X.done[i], kStWarps); mbar_init(&X.freed[i], 1); }
-        fence_mbar_init();
         S.cs = reinterpret_cast<CtlSet *>(p.sets + (odd ? ctl_set_bytes(p.nmb_max) : 0));
         S.h_ready = reinterpret_cast<unsigned *>(S.cs + 1) + kFine * kMaxEE + p.nmb_max;
         X.failed = 0;
     }
+    if (warp == 14 && lane < kStMaxSlots) { mbar_init(&X.full[lane], 1); mbar_init(&X.empty[lane], kStWarps); }
+    if (warp == 14 && lane >= 30) { mbar_init(&X.done[lane - 30], kStWarps); mbar_init(&X.freed[lane - 30], 1); }
+    if (warp == 14) fence_mbar_init();
+    if (warp == 15 && lane < 2 * kStMaps) tma_prefetch_desc(lane < kStMaps ? &tm.g[lane] : &tm.d[lane - kStMaps]);
     if (tid < kMaxEE) X.mask[tid] = tid >= p.E && tid < p.EE ? (2u << (p.T - 1)) - 1u : 0u;
     __syncthreads();
     {
@@ -236,8 +266,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
             other[i] = make_uint4(0u, 0u, 0u, 0u);
     }
     // ================= routing, counts, offsets, active experts
-    if (warp < p.T) stream_route(p, X, warp, lg[0]);
-    if (warp + 16 < p.T) stream_route(p, X, warp + 16, lg[1]);
+    if (warp < p.T) stream_route(p, X, warp, lg);
     __syncthreads();
     unsigned v = 0, inc = 0;      // rows | (has rows) << 16
     if (warp < kMaxEE / 32) {
@@ -250,6 +279,8 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
             if (lane >= o) inc += q;
         }
         if (lane == 31) X.wsum[warp] = inc;
+        const int most = (int)__reduce_max_sync(0xffffffffu, n);
+        if (lane == 0) X.wmax[warp] = most;
     }
     __syncthreads();
     if (warp < kMaxEE / 32) {
@@ -266,6 +297,22 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
     }
     __syncthreads();
     const int A = X.n_act;
+    if (lane == 0 && (warp == 0 || warp == 8)) X.share[warp >> 3] = StreamShare(A, warp ? p.H / kStUnitD : p.I / kStUnitG, cta, ctas);
+    __syncthreads();
+    // Shared memory: the ring, then the rows of x and, later, in the same place, of h: of one expert, of two where the ring stays
+    // deep all the same (fewer than about 160 KB on their way make the stream slower).
+    int most = 0;      // rows of an expert
+#pragma unroll
+    for (int w = 0; w < kMaxEE / 32; ++w) most = max(most, X.wmax[w]);
+    int rows_h = 2 * most;
+    if (kStArea - rows_h * (int)pitch_h < kStFullRing) rows_h = most;
+    const int ring_bytes = (kStArea - max(p.T * (int)pitch_x, rows_h * (int)pitch_h)) & ~2047;
+    const uint32_t h_s = ring + (uint32_t)ring_bytes;
+    // The ring's slots, as large as this CTA's widest tiles want them: a block of K of five units and more, two of fewer.  (With
+    // slots for eight units throughout, a share of ten in two tiles of five had 120 KB of the ring's 192 in flight.)
+    const int cap0 = X.share[0].cap, cap1 = X.share[1].cap;
+    const int slot_units = max(cap0 <= kStWarps / 2 ? 2 * cap0 : cap0, cap1 <= kStWarps / 2 ? 2 * cap1 : cap1);
+    const int slots = min(kStMaxSlots, ring_bytes / (slot_units * 2048));
 
     if (warp == 0) {
         // ---------------- producer
@@ -274,17 +321,24 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
             uint32_t ph = 0;
             bool ok = true;
             for (int phase = 0; phase < 2 && ok; ++phase) {
-                StreamWalk wk(A, phase ? p.H / kStUnitD : p.I / kStUnitG, cta, ctas);
-                while (ok && wk.next()) {
-                    const int e = X.act[wk.a], kb = stream_kblocks(wk.w), nk = (phase ? p.I : p.H) / (64 * kb);
-                    const int row = phase ? e * p.H + wk.c * kStUnitD : e * 2 * p.I + wk.c * kStUnitG;
-                    const CUtensorMap *map = phase ? &tm.d[wk.w - 1] : &tm.g[wk.w - 1];
+                StreamWalk wk(X.share[phase]);
+                while (ok && wk.next(X, phase ? rows_h : 0)) {
+                    const int kb = 2 * wk.w <= slot_units ? 2 : 1, nk = (phase ? p.I : p.H) / (64 * kb), w2 = wk.w - wk.w1;
+                    const int e1 = X.act[wk.at_a], e2 = w2 ? X.act[wk.at_a + 1] : 0;
+                    const int row1 = phase ? e1 * p.H + wk.at_c * kStUnitD : e1 * 2 * p.I + wk.at_c * kStUnitG, row2 = phase ? e2 * p.H : e2 * 2 * p.I;
+                    const CUtensorMap *maps = phase ? tm.d : tm.g;
+                    const CUtensorMap *map1 = maps + stream_map(wk.w1, kb), *map2 = w2 ? maps + stream_map(w2, kb) : nullptr;
                     for (int kk = 0; kk < nk; ++kk) {
                         if (!mbar_wait(&X.empty[slot], ph ^ 1u, p, 60)) { ok = false; break; }
                         mbar_arrive_expect_tx(&X.full[slot], (uint32_t)(wk.w * kb * 2048));
-                        const uint32_t dst = ring + (uint32_t)(slot * kStSlot);
-                        if (phase) tma_load_3d(dst, map, 0, row, kb * kk, &X.full[slot]);
-                        else tma_load_4d(dst, map, 0, row, 0, kb * kk, &X.full[slot]);
+                        const uint32_t dst = ring + (uint32_t)(slot * slot_units * 2048), dst2 = dst + (uint32_t)(wk.w1 * kb * 2048);
+                        if (phase) {
+                            tma_load_3d(dst, map1, 0, row1, kb * kk, &X.full[slot]);
+                            if (w2) tma_load_3d(dst2, map2, 0, row2, kb * kk, &X.full[slot]);
+                        } else {
+                            tma_load_4d(dst, map1, 0, row1, 0, kb * kk, &X.full[slot]);
+                            if (w2) tma_load_4d(dst2, map2, 0, row2, 0, kb * kk, &X.full[slot]);
+                        }
                         if (++slot == slots) { slot = 0; ph ^= 1u; }
                     }
                 }
@@ -301,10 +355,11 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                 int tile = 0;
                 bool ok = true;
                 for (int phase = 0; phase < 2 && ok; ++phase) {
-                    StreamWalk wk(A, phase ? p.H / kStUnitD : p.I / kStUnitG, cta, ctas);
-                    for (; ok && wk.next(); ++tile) {
+                    StreamWalk wk(X.share[phase]);
+                    for (; ok && wk.next(X, phase ? rows_h : 0); ++tile) {
                         ok = mbar_wait(&X.done[tile & 1], (uint32_t)((tile >> 1) & 1), p, 64);
-                        if (ok) red_release_add_u32(phase ? &S.cs->y_done[0] : &S.h_ready[wk.a], (unsigned)wk.w);
+                        if (ok) red_release_add_u32(phase ? &S.cs->y_done[0] : &S.h_ready[wk.at_a], (unsigned)(phase ? wk.w : wk.w1));
+                        if (ok && !phase && wk.w1 < wk.w) red_release_add_u32(&S.h_ready[wk.at_a + 1], (unsigned)(wk.w - wk.w1));
                         mbar_arrive(&X.freed[tile & 1]);
                     }
                 }
@@ -347,68 +402,60 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
         } else {
             // ---------------- the products
             const int wi = warp - 8;
-            int slot = 0, tile = 0;
-            uint32_t ph = 0;
+            int tile = 0;
+            StreamRing r = {ring, (uint32_t)(slot_units * 2048), slots, 0, 0u};
             bool ok = true;
             for (int phase = 0; phase < 2; ++phase) {
-                StreamWalk wk(A, phase ? p.H / kStUnitD : p.I / kStUnitG, cta, ctas);
-                const uint32_t pitch = phase ? (uint32_t)p.I * 2u + kStPad : pitch_x;
-                int cur = -1;
-                for (; wk.next(); ++tile) {
-                    const int e = X.act[wk.a], n_e = X.off[e + 1] - X.off[e], row0 = X.off[e];
-                    const int nk = (phase ? p.I : p.H) / (64 * stream_kblocks(wk.w));
-                    if (phase && wk.a != cur) {
-                        // the next expert's rows of h, once all of them are there and nobody reads what they replace
-                        cur = wk.a;
+                StreamWalk wk(X.share[phase]);
+                const uint32_t pitch = phase ? pitch_h : pitch_x, rows_s = phase ? h_s : x_s;
+                int first = -1, second = -1;      // active experts whose rows of h are in shared memory, one behind the other
+                for (; wk.next(X, phase ? rows_h : 0); ++tile) {
+                    const bool two = wk.w1 < wk.w;
+                    const int kb = 2 * wk.w <= slot_units ? 2 : 1;
+                    if (phase && ((wk.at_a != first && wk.at_a != second) || (two && wk.at_a + 1 != second))) {
+                        // the next rows of h, once all of them are there and nobody reads what they replace
+                        first = wk.at_a; second = two ? wk.at_a + 1 : -1;
                         named_barrier_sync<2, kStWarps * 32>();
-                        if (lane == 0) ok = flag_wait_ge(&S.h_ready[wk.a], (unsigned)(p.I / kStUnitG), p, 62) && ok;
+                        if (lane == 0) ok = flag_wait_ge(&S.h_ready[first], (unsigned)(p.I / kStUnitG), p, 62) && ok;
+                        if (lane == 0 && two) ok = flag_wait_ge(&S.h_ready[second], (unsigned)(p.I / kStUnitG), p, 62) && ok;
                         __syncwarp();
-                        const int per_row = p.I >> 3, ctid = tid - 256;
-                        const __nv_bfloat16 *src = p.hbuf + (size_t)row0 * p.I;
-                        for (int t = 0; t < n_e; ++t)
+                        const int per_row = p.I >> 3, ctid = tid - 256, n = X.rows(first) + (two ? X.rows(second) : 0);
+                        const __nv_bfloat16 *src = p.hbuf + (size_t)X.off[X.act[first]] * p.I;      // (the two experts' rows are neighbours)
+                        for (int t = 0; t < n; ++t)
                             for (int c = ctid; c < per_row; c += kStWarps * 32)
                                 cp_async_16(rows_s + (uint32_t)t * pitch + (uint32_t)(c * 16), src + (size_t)t * p.I + c * 8);
                         cp_async_wait_all();
                         named_barrier_sync<2, kStWarps * 32>();
                     }
-                    uint32_t b_row[4];
-#pragma unroll
-                    for (int n = 0; n < 4; ++n) {
-                        const int i = 8 * n + (lane & 7);
-                        const int r = phase ? (i < n_e ? i : 0) : (int)__fns(X.mask[e], 0u, i < n_e ? i + 1 : 1);
-                        b_row[n] = rows_s + (uint32_t)r * pitch + (uint32_t)((lane >> 3) * 16);
-                    }
+                    // this warp's unit: unit li of the ones that the tile has of active expert a
+                    const bool works = wi < wk.w, later = works && wi >= wk.w1;
+                    const int a = later ? wk.at_a + 1 : wk.at_a, li = later ? wi - wk.w1 : wi, wp = later ? wk.w - wk.w1 : wk.w1;
+                    const int unit = later ? li : wk.at_c + li, e = X.act[a], n_e = X.rows(a), row0 = X.off[e];
+                    const int i8 = lane & 7;
+                    const int src_row = phase ? (a == second ? X.rows(first) : 0) + (i8 < n_e ? i8 : 0) : (int)__fns(X.mask[e], 0u, i8 < n_e ? i8 + 1 : 1);
+                    const uint32_t b_row = rows_s + (uint32_t)src_row * pitch + (uint32_t)((lane >> 3) * 16);
                     const uint32_t half = (uint32_t)((lane >> 3) & 1);      // rows 8..15 of the warp's sixteen
-                    const uint32_t a_off = phase ? (uint32_t)(wi * 16 + (lane & 7) + 8 * (int)half) * 128u
-                                                 : (uint32_t)(wi * 8 + (lane & 7)) * 128u + half * (uint32_t)(wk.w * 1024);
-                    const uint32_t blk = (uint32_t)(wk.w * 2048);
-                    const bool works = wi < wk.w;
-                    const int col = phase ? wk.c * kStUnitD + wi * 16 + (lane >> 2) : wk.c * kStUnitG + wi * 8 + (lane >> 2);
-                    __nv_bfloat16 *dst = phase ? p.y + (size_t)row0 * p.H + col : p.hbuf + (size_t)row0 * p.I + col;
-                    const size_t dpitch = phase ? (size_t)p.H : (size_t)p.I;
-                    auto run = [&](auto nt, auto kb) {
-                        constexpr int NT = decltype(nt)::value;
-                        float acc[NT][4];
-                        ok = stream_tile<NT, decltype(kb)::value>(p, X, ring, slots, slot, ph, nk, works, a_off, blk, b_row, acc) && ok;
-                        if (works) {
+                    const uint32_t part = later ? (uint32_t)(wk.w1 * kb * 2048) : 0u;
+                    const uint32_t a_off = part + (phase ? (uint32_t)(li * 16 + i8 + 8 * (int)half) * 128u : (uint32_t)(li * 8 + i8) * 128u + half * (uint32_t)(wp * 1024));
+                    const uint32_t blk = (uint32_t)(wp * 2048);
+                    const int K = phase ? p.I : p.H;
+                    float acc[4];
+                    ok = (kb == 2 ? stream_tile<2>(p, X, r, K, works, a_off, blk, b_row, acc)
+                                               : stream_tile<1>(p, X, r, K, works, a_off, blk, b_row, acc)) && ok;
+                    if (works) {
+                        const int col = (phase ? unit * kStUnitD : unit * kStUnitG) + (lane >> 2);
 #pragma unroll
-                            for (int n = 0; n < NT; ++n)
-#pragma unroll
-                                for (int i = 0; i < 2; ++i) {      // this lane has tokens 2q and 2q + 1 of every eight
-                                    const int r = 8 * n + 2 * (lane & 3) + i;
-                                    if (r < n_e) {
-                                        __nv_bfloat16 *d = dst + (size_t)r * dpitch;
-                                        if (phase) { d[0] = __float2bfloat16_rn(acc[n][i]); d[8] = __float2bfloat16_rn(acc[n][2 + i]); }
-                                        else d[0] = __float2bfloat16_rn(silu_mul(acc[n][i], acc[n][2 + i]));
-                                    }
-                                }
+                        for (int i = 0; i < 2; ++i) {      // this lane has rows 2q and 2q + 1 of the expert
+                            const int t = 2 * (lane & 3) + i;
+                            if (t < n_e) {
+                                if (phase) {
+                                    __nv_bfloat16 *d = p.y + (size_t)(row0 + t) * p.H + col;
+                                    d[0] = __float2bfloat16_rn(acc[i]);
+                                    d[8] = __float2bfloat16_rn(acc[2 + i]);
+                                } else p.hbuf[(size_t)(row0 + t) * p.I + col] = __float2bfloat16_rn(silu_mul(acc[i], acc[2 + i]));
+                            }
                         }
-                    };
-                    using C1 = std::integral_constant<int, 1>;
-                    using C2 = std::integral_constant<int, 2>;
-                    using C4 = std::integral_constant<int, 4>;
-                    if (wk.w <= kStWarps / 2) { if (n_e <= 8) run(C1(), C2()); else if (n_e <= 16) run(C2(), C2()); else run(C4(), C2()); }
-                    else { if (n_e <= 8) run(C1(), C1()); else if (n_e <= 16) run(C2(), C1()); else run(C4(), C1()); }
+                    }
                     __syncwarp();
                     if (lane == 0) {
                         if (tile >= 2) ok = mbar_wait(&X.freed[tile & 1], (uint32_t)(((tile >> 1) - 1) & 1), p, 65) && ok;
