@@ -2354,6 +2354,7 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
             // per tile, not a bandwidth problem  (ceil(T / ct) < N  <=>  T <= (N - 1) * ct)
             int ct = kCombTile;
             while (ct > 1 && p.T <= (n_sm - 1) * ct) ct >>= 1;
+            if (ct == 1 && p.T > n_sm) ct = 2;      // one round of two tokens each, not two rounds of claims (8 experts, T = 200: 35.1 -> 33.3 us)
             S.comb_tok = ct;
             S.n_comb = (p.T + ct - 1) / ct;
             if (blockIdx.x == 0) {
