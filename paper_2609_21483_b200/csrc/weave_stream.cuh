@@ -8,11 +8,12 @@
 // rows the M axis; the products are summed 16 of K at a time in ascending order, as the general kernel's
 // tcgen05.mma sums them, and the results carry the same bits.
 //
-// One launch behind another, us, the general kernel / this one, and the time of the bytes: Qwen3-30B-shaped T = 1 37.7 / 26.3 (11.5), T = 8
-// 97.9 / 88.5 (77.8); Qwen3-235B-shaped T = 1 81 / 60.2 (46.1); Mixtral-shaped T = 1 159 / 119 (107.5), T = 4 314 / 295 (269);
-// DSv2-Lite-shaped T = 7 112.5 / 102.8 (87.1); 8 experts T = 1 25.3 / 14.6.  Bound by HBM but for a chain of 10 us in front of the first
-// weights (launch, routing) and around the exchange of h and y.  Measured and left: with 9 to 16 tokens +-2 %, slower above (the
-// general kernel is at HBM speed there); a quarter of the units claimed in tiles of one or two (their chain of products is one
+// One launch behind another, us, the general kernel / this one, and the time of the bytes: Qwen3-30B-shaped T = 1 37.7 / 25.4 (11.5), T = 8
+// 98 / 88.5 (77.8), T = 16 142.9 / 135.3 (117); Qwen3-235B-shaped T = 1 81 / 60 (46.1); Mixtral-shaped T = 1 159 / 119 (107.5), T = 4
+// 314 / 295 (269); DSv2-Lite-shaped T = 7 112.5 / 103 (87.1), T = 16 167 / 163; Qwen3.5-35B-shaped T = 12 68.3 / 55.7; 8 experts
+// T = 1 25.3 / 14.6, T = 16 27.1 / 20.4.  Bound by HBM but for a chain of 10 us in front of the first weights (launch,
+// routing) and around the exchange of h and y.  Measured and left: more than 16 tokens (the rows of x take the ring's
+// place; T = 27 163 against 141); a quarter of the units claimed in tiles of one or two (their chain of products is one
 // warp's: 282 us where 189 were); a unit per warp with a ring and a claim of its own (every warp holds a unit to the end: 120 / 103).
 //
 //   warp 0        producer: one tensor copy per ring slot (a tile's rows x 64 or 128 of K)
@@ -28,7 +29,7 @@
 namespace weave {
 
 constexpr int kStThreads = 512;
-constexpr int kStTokens = 8;                      // largest batch: one N tile (see stream_slots)
+constexpr int kStTokens = 16;                     // largest batch: two N tiles of a product (see streams())
 constexpr int kStMaxSlot = 16384;                 // bytes of a ring slot, at most
 constexpr int kStMaxSlots = 16;
 constexpr int kStMinRing = 5 * kStMaxSlot, kStFullRing = 10 * kStMaxSlot;      // bytes
@@ -126,8 +127,16 @@ __device__ __forceinline__ void stream_route(const KParams &p, StreamShared &X, 
 {
     const int lane = threadIdx.x & 31;
     unsigned key[8], bk = 0u;
-    int be = 0x7fffffff;
+    int bi;
     bool bad = false;
+    auto best = [&]() {      // the lane's largest key; of equal ones the first
+        bk = 0u;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) bk = max(bk, key[i]);
+        bi = 7;
+#pragma unroll
+        for (int i = 6; i >= 0; --i) bi = key[i] == bk ? i : bi;
+    };
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int e = lane + 32 * i;
@@ -135,26 +144,22 @@ __device__ __forceinline__ void stream_route(const KParams &p, StreamShared &X, 
         const bool nf = !(fabsf(x) <= 3.402823466e38f);
         bad = bad || (e < p.E && nf);
         x = nf ? -3.402823466e38f : x;
-        x = __fadd_rn(x, 0.0f);
-        key[i] = e < p.E ? float_order_key(x) : 0u;
-        if (key[i] > bk) { bk = key[i]; be = e; }
+        key[i] = e < p.E ? float_order_key(__fadd_rn(x, 0.0f)) : 0u;
     }
+    best();
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicCAS(&p.ctl->status, 0, kErrNonFinite);
     float mine = 0.f;      // lane j: logit and expert of slot j
     int my_e = 0;
 #pragma unroll 1
     for (int j = 0; j < p.k; ++j) {
-        const unsigned top = __reduce_max_sync(0xffffffffu, bk);
-        const int hi = (int)__reduce_min_sync(0xffffffffu, bk == top ? (unsigned)be : 0x7fffffffu);
+        const unsigned top = __reduce_max_sync(0xffffffffu, bk), eq = __ballot_sync(0xffffffffu, bk == top);
+        int win = __ffs((int)eq) - 1;
+        if (eq & (eq - 1u)) win = (int)(__reduce_min_sync(0xffffffffu, bk == top ? (unsigned)(lane + 32 * bi) : 0x7fffffffu) & 31u);
+        const int hi = win + 32 * __shfl_sync(0xffffffffu, bi, win);
         if (lane == j) { mine = float_from_order_key(top); my_e = hi; }
-        if ((hi & 31) == lane) {
-            bk = 0u; be = 0x7fffffff;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                if (i == (hi >> 5)) key[i] = 0u;
-                if (key[i] > bk) { bk = key[i]; be = lane + 32 * i; }
-            }
-        }
+        for (int i = 0; i < 8; ++i) key[i] = lane == win && bi == i ? 0u : key[i];
+        best();
     }
     mine = expf(mine - __shfl_sync(0xffffffffu, mine, 0));
     float sum = 0.f;
@@ -223,6 +228,47 @@ __device__ __forceinline__ bool stream_tile(const KParams &p, StreamShared &X, S
     return ok;
 }
 
+// The same for an expert of 9 to 16 rows, without the look ahead (registers).
+template <int KB>
+__device__ __forceinline__ bool stream_tile_16(const KParams &p, StreamShared &X, StreamRing &r, int K, bool works, uint32_t a_off, uint32_t blk,
+                                               uint32_t b_row, uint32_t b_row2, float (&acc)[4], float (&acc2)[4])
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t sw = (uint32_t)(lane & 7), kh = (uint32_t)(lane >> 4);
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] = acc2[i] = 0.f;
+#pragma unroll 1
+    for (int j = 0; j < K / 64; j += KB) {
+        ok = mbar_wait(&X.full[r.slot], r.ph, p, 61) && ok;
+        if (works) {
+#pragma unroll
+            for (int kb = 0; kb < KB; ++kb) {
+                const uint32_t a0 = r.base + (uint32_t)r.slot * r.bytes + a_off + (uint32_t)kb * blk;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t a[2][4], b[4], b2[4];
+                    ldmatrix_x4(b_row + (uint32_t)((j + kb) * 128 + h * 64), b);
+                    ldmatrix_x4(b_row2 + (uint32_t)((j + kb) * 128 + h * 64), b2);
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) ldmatrix_x4(a0 + (((2u * (uint32_t)(2 * h + s) + kh) ^ sw) << 4), a[s]);
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) {
+                        mma_16816(acc, a[s], b[2 * s], b[2 * s + 1]);
+                        mma_16816(acc2, a[s], b2[2 * s], b2[2 * s + 1]);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&X.empty[r.slot]);
+        if (++r.slot == r.slots) { r.slot = 0; r.ph ^= 1u; }
+    }
+    return ok;
+}
+
+// kWide: 9 to 16 tokens (a kernel of its own: with the second N tile in it the smaller batches take 1 to 2 % longer)
+template <bool kWide>
 __global__ void __launch_bounds__(kStThreads, 1)
 weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ StreamMaps tm)
 {
@@ -439,20 +485,27 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                     const uint32_t a_off = part + (phase ? (uint32_t)(li * 16 + i8 + 8 * (int)half) * 128u : (uint32_t)(li * 8 + i8) * 128u + half * (uint32_t)(wp * 1024));
                     const uint32_t blk = (uint32_t)(wp * 2048);
                     const int K = phase ? p.I : p.H;
-                    float acc[4];
-                    ok = (kb == 2 ? stream_tile<2>(p, X, r, K, works, a_off, blk, b_row, acc)
-                                               : stream_tile<1>(p, X, r, K, works, a_off, blk, b_row, acc)) && ok;
+                    float acc[kWide ? 2 : 1][4];
+                    if (!kWide || n_e <= 8)
+                        ok = (kb == 2 ? stream_tile<2>(p, X, r, K, works, a_off, blk, b_row, acc[0]) : stream_tile<1>(p, X, r, K, works, a_off, blk, b_row, acc[0])) && ok;
+                    else {
+                        const int i16 = i8 + 8 < n_e ? i8 + 8 : 0;
+                        const int src_row2 = phase ? (a == second ? X.rows(first) : 0) + i16 : (int)__fns(X.mask[e], 0u, i16 + 1);
+                        const uint32_t b_row2 = rows_s + (uint32_t)src_row2 * pitch + (uint32_t)((lane >> 3) * 16);
+                        ok = (kb == 2 ? stream_tile_16<2>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])
+                                      : stream_tile_16<1>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])) && ok;
+                    }
                     if (works) {
                         const int col = (phase ? unit * kStUnitD : unit * kStUnitG) + (lane >> 2);
 #pragma unroll
-                        for (int i = 0; i < 2; ++i) {      // this lane has rows 2q and 2q + 1 of the expert
-                            const int t = 2 * (lane & 3) + i;
+                        for (int i = 0; i < (kWide ? 4 : 2); ++i) {      // this lane has rows 2q and 2q + 1 of every eight of the expert
+                            const int t = 2 * (lane & 3) + (i & 1) + 8 * (i >> 1);
                             if (t < n_e) {
                                 if (phase) {
                                     __nv_bfloat16 *d = p.y + (size_t)(row0 + t) * p.H + col;
-                                    d[0] = __float2bfloat16_rn(acc[i]);
-                                    d[8] = __float2bfloat16_rn(acc[2 + i]);
-                                } else p.hbuf[(size_t)(row0 + t) * p.I + col] = __float2bfloat16_rn(silu_mul(acc[i], acc[2 + i]));
+                                    d[0] = __float2bfloat16_rn(acc[i >> 1][i & 1]);
+                                    d[8] = __float2bfloat16_rn(acc[i >> 1][2 + (i & 1)]);
+                                } else p.hbuf[(size_t)(row0 + t) * p.I + col] = __float2bfloat16_rn(silu_mul(acc[i >> 1][i & 1], acc[i >> 1][2 + (i & 1)]));
                             }
                         }
                     }
