@@ -194,7 +194,8 @@ int weave_moe_set_model_options(weave_moe_t h, int kinds_mask, int elastic);
  * because the GEMM phase runs on pairs of neighbouring SMs), rows per m-block (the unit of the
  * dispatch queue), h-columns per gemm0 tile, out-columns per gemm1 tile,
  * tokens per routing block, tokens per combine tile (the largest size: a batch that would give
- * fewer tiles than SMs is cut into tiles of half that size, repeatedly, down to one token), rows
+ * fewer tiles than SMs is cut into tiles of half that size, repeatedly, down to one token, or to two where
+ * that many tiles are one round on all SMs), rows
  * per GEMM tile at most (the rows of an expert's segment are split into as few tiles as that allows, of almost
  * equal size; the ready flags count rows per such tile).
  * Any pointer may be NULL. */
@@ -221,7 +222,8 @@ int weave_moe_get_intermediates(weave_moe_t h, const void **xe, const void **hbu
 int weave_moe_status(weave_moe_t h);
 
 /* After weave_moe_status() returned WEAVE_ERR_TIMEOUT: a small integer naming the wait that gave
- * up first (1-3 grid barriers, 10-16 dispatch, 20-24 combine, 30-57 GEMM phase); 0 otherwise.
+ * up first (1-3 grid barriers, 10-16 dispatch, 20-24 combine, 30-57 GEMM phase, 60-65 the streaming kernel of the
+ * smallest batches); 0 otherwise.
  * Diagnostic only. */
 int weave_moe_last_timeout_where(weave_moe_t h);
 
@@ -255,7 +257,8 @@ int weave_moe_debug_withhold_flag(weave_moe_t h, int m_block);
  * extra = type << 16 | ns spent before the release), 7 combine tile, 8 wait for a chunk's gemm1,
  * 9 grid barrier (the one behind the routing; a batch of at most 64 tokens is routed by every CTA for itself
  * and has none), 11 GEMM tile main loop on the MMA issuer (id = type << 16 | rows, extra = ns spent
- * waiting for a free accumulator). */
+ * waiting for a free accumulator).  The records are the general kernel's: while a timeline is set, or a flag withheld, a
+ * batch of up to 16 tokens runs on it too (same results) and not on the streaming kernel. */
 int weave_moe_set_trace(weave_moe_t h, void *buf, int events_per_cta);
 
 /* HOST-ONLY (no GPU needed, no handle): the order in which the kernel's GEMM schedulers claim pair
