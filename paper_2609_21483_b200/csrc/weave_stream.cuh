@@ -445,6 +445,9 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                 uint4 *dst = reinterpret_cast<uint4 *>(p.xe + (size_t)r * p.H);
                 for (int c = lane; c < (p.H >> 3); c += 32) dst[c] = __ldg(src + c);
             }
+            // (counted in with y: nothing is written to `out`, which may be x itself, before its last reader is done)
+            __syncwarp();
+            if (lane == 0) red_release_add_u32(&S.cs->y_done[0], 1u);
         } else {
             // ---------------- the products
             const int wi = warp - 8;
@@ -522,7 +525,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
 
     // ================= combine: out[t] = sum over the slots, in slot order, then the shared experts
     __syncthreads();
-    if (tid == 0 && !flag_wait_ge(&S.cs->y_done[0], (unsigned)(A * (p.H / kStUnitD)), p, 63)) X.failed = 1;
+    if (tid == 0 && !flag_wait_ge(&S.cs->y_done[0], (unsigned)(A * (p.H / kStUnitD) + 6 * ctas), p, 63)) X.failed = 1;
     __syncthreads();
     if (!X.failed) {
         const int vecs = p.H >> 3, total = p.T * vecs;      // 16-byte pieces, four neighbours to a CTA

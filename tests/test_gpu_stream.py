@@ -72,3 +72,39 @@ def test_smallest_batches_report_the_plan_of_the_cost_model():
         seen.add(got["kind"])
     assert pk.PLAN_PHASED in seen and len(seen) > 1
     moe.close()
+
+
+@pytest.mark.parametrize("T", [1, 8, 16])
+def test_smallest_batches_in_place_and_captured_between_larger_ones(T):
+    """out = x; a CUDA graph of two layers; calls of 1 to 40 tokens in turn on one handle, so that both kernels hand the
+    control words to each other: the same bits every time."""
+    cfg = wl.MoEConfig(f"stream_mix_{T}", 1300, T=40, H=1024, I=512, E=64, k=4, S=1, zipf_s=0.5)
+    x, lg, gu, dn = to_dev(wl.make_inputs(cfg))
+    moe = pk.WeaveMoE(gu, dn, cfg.E, cfg.k, cfg.S, max_tokens=40)
+    xs, ls = x[:T].contiguous(), lg[:T].contiguous()
+    ref = moe.forward(xs, ls).view(torch.int16).clone()
+    xe = moe.intermediates(T)["xe"].view(torch.int16).clone()
+    for _ in range(200):
+        buf = xs.clone()
+        moe.forward(buf, ls, buf)
+    assert torch.equal(buf.view(torch.int16), ref)
+    assert torch.equal(moe.intermediates(T)["xe"].view(torch.int16), xe)
+    second = moe.forward(buf, ls).view(torch.int16).clone()
+    s, g, o1, o2 = torch.cuda.Stream(), torch.cuda.CUDAGraph(), torch.empty_like(xs), torch.empty_like(xs)
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        with torch.cuda.graph(g, stream=s):
+            moe.forward(xs, ls, o1)
+            moe.forward(o1, ls, o2)
+    for _ in range(3):
+        o2.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(o1.view(torch.int16), ref) and torch.equal(o2.view(torch.int16), second)
+    refs = {}
+    for i in range(400):
+        n = (7 * i) % 40 + 1
+        out = moe.forward(x[:n].contiguous(), lg[:n].contiguous()).view(torch.int16)
+        assert torch.equal(out, refs.setdefault(n, out.clone())), n
+    moe.check()
+    moe.close()
