@@ -396,7 +396,8 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
         cp_async_wait_all();
         named_barrier_sync<1, kStThreads - 32>();      // x is in shared memory
         if (warp == 1) {
-            // ---------------- a release at GPU scope waits until the tile's stores are performed: not the products' business
+            // ---------------- a release at GPU scope waits until the tile's stores are performed: not the products' business (made by
+            // their own warps: T = 8 Qwen3-30B-shaped 87.5 -> 95.3 us)
             if (lane == 0) {
                 int tile = 0;
                 bool ok = true;
