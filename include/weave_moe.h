@@ -245,7 +245,9 @@ int weave_moe_set_timeout_ms(weave_moe_t h, int ms);
 
 /* Test hook for the give-up path: the rows of the m-block with this index are never counted as
  * dispatched (-1 = off; an index that the batch does not reach withholds nothing), so the bounded wait of
- * the GEMM tiles that share rows with it expires.  Host-side injection only; nothing faults or traps. */
+ * the GEMM tiles that share rows with it expires.  In the streaming kernel of the smallest batches, where
+ * every expert with rows is one m-block, its finished columns of h are never counted in, and the wait of
+ * its down tiles expires.  Host-side injection only; nothing faults or traps. */
 int weave_moe_debug_withhold_flag(weave_moe_t h, int m_block);
 
 /* Optional in-kernel timeline (our analogue of the utilisation profile of the paper's Section 5.4).
@@ -257,7 +259,7 @@ int weave_moe_debug_withhold_flag(weave_moe_t h, int m_block);
  * extra = type << 16 | ns spent before the release), 7 combine tile, 8 wait for a chunk's gemm1,
  * 9 grid barrier (the one behind the routing; a batch of at most 64 tokens is routed by every CTA for itself
  * and has none), 11 GEMM tile main loop on the MMA issuer (id = type << 16 | rows, extra = ns spent
- * waiting for a free accumulator).  The records are the general kernel's: while a timeline is set, or a flag withheld, a
+ * waiting for a free accumulator).  The records are the general kernel's: while a timeline is set, a
  * batch of up to 16 tokens runs on it too (same results) and not on the streaming kernel. */
 int weave_moe_set_trace(weave_moe_t h, void *buf, int events_per_cta);
 

@@ -251,12 +251,11 @@ bool phased_is_picked(const weave_moe *h, int T, float *t_phased)
 const void *stream_kernel(int T) { return T > 8 ? (const void *)weave_stream_kernel<true> : (const void *)weave_stream_kernel<false>; }
 
 // Batches that weave_stream_kernel takes: up to 16 tokens (the N of two products) whose rows of x, or of h if they all went to
-// one expert, leave room for a ring of 80 KB, or of 128 KB from nine tokens on.  (A timeline and the withheld-flag hook are about the general kernel's tiles and
-// flags.)
+// one expert, leave room for a ring of 80 KB, or of 128 KB from nine tokens on.  (A timeline is about the general kernel's tiles.)
 bool streams(const weave_moe *h, int T)
 {
     const weave_moe_config &c = h->cfg;
-    if (T > kStTokens || h->mode != WEAVE_SCHED_AUTO || h->ep_size != 1 || h->withhold_mb >= 0 || h->trace) return false;
+    if (T > kStTokens || h->mode != WEAVE_SCHED_AUTO || h->ep_size != 1 || h->trace) return false;
     return (size_t)T * ((size_t)std::max(c.hidden, c.ffn) * 2 + kStPad) <= (size_t)(kStArea - (T > 8 ? 8 * kStMaxSlot : kStMinRing));
 }
 

@@ -175,6 +175,8 @@ __device__ __forceinline__ void stream_route(const KParams &p, StreamShared &X, 
 // One tile for a warp: 16 weight rows x 8 tokens, KB blocks of 64 of K per ring slot.  a_off: this lane's ldmatrix row in a slot,
 // blk: bytes of a block of K in the slot, b_row: this lane's row of x or h.  A block's operands are fetched between the
 // products of the block before: the chain of dependent products (and nothing else) sets the pace.
+// A lane whose wait ended without success waits for nothing more and hands no slot back: the tile's arrival is then missing,
+// and nobody reads what it gave.
 struct StreamRing { uint32_t base, bytes; int slots, slot; uint32_t ph; };
 template <int KB>
 __device__ __forceinline__ bool stream_tile(const KParams &p, StreamShared &X, StreamRing &r, int K, bool works, uint32_t a_off, uint32_t blk,
@@ -188,7 +190,7 @@ __device__ __forceinline__ bool stream_tile(const KParams &p, StreamShared &X, S
     for (int i = 0; i < 4; ++i) acc[i] = 0.f;
     auto arrived = [&](int j) {      // block j (of parity j & 1): its slot is there
         if (KB == 1 || (j & 1) == 0) {
-            ok = mbar_wait(&X.full[r.slot], r.ph, p, 61) && ok;
+            if (ok) ok = mbar_wait(&X.full[r.slot], r.ph, p, 61);
             a0 = r.base + (uint32_t)r.slot * r.bytes + a_off;
             if (++r.slot == r.slots) { r.slot = 0; r.ph ^= 1u; }
         } else a0 += blk;
@@ -199,7 +201,7 @@ __device__ __forceinline__ bool stream_tile(const KParams &p, StreamShared &X, S
     };
     auto free_slot = [&](int slot) {      // the slot's values are in registers
         __syncwarp();
-        if (lane == 0) mbar_arrive(&X.empty[slot]);
+        if (lane == 0 && ok) mbar_arrive(&X.empty[slot]);
     };
     const int nb = K / 64;      // even
     int held = r.slot;
@@ -240,7 +242,7 @@ __device__ __forceinline__ bool stream_tile_16(const KParams &p, StreamShared &X
     for (int i = 0; i < 4; ++i) acc[i] = acc2[i] = 0.f;
 #pragma unroll 1
     for (int j = 0; j < K / 64; j += KB) {
-        ok = mbar_wait(&X.full[r.slot], r.ph, p, 61) && ok;
+        if (ok) ok = mbar_wait(&X.full[r.slot], r.ph, p, 61);
         if (works) {
 #pragma unroll
             for (int kb = 0; kb < KB; ++kb) {
@@ -261,7 +263,7 @@ __device__ __forceinline__ bool stream_tile_16(const KParams &p, StreamShared &X
             }
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(&X.empty[r.slot]);
+        if (lane == 0 && ok) mbar_arrive(&X.empty[r.slot]);
         if (++r.slot == r.slots) { r.slot = 0; r.ph ^= 1u; }
     }
     return ok;
@@ -405,8 +407,10 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                     StreamWalk wk(X.share[phase]);
                     for (; ok && wk.next(X, phase ? rows_h : 0); ++tile) {
                         ok = mbar_wait(&X.done[tile & 1], (uint32_t)((tile >> 1) & 1), p, 64);
-                        if (ok) red_release_add_u32(phase ? &S.cs->y_done[0] : &S.h_ready[wk.at_a], (unsigned)(phase ? wk.w : wk.w1));
-                        if (ok && !phase && wk.w1 < wk.w) red_release_add_u32(&S.h_ready[wk.at_a + 1], (unsigned)(wk.w - wk.w1));
+                        if (!ok) break;
+                        // (the test hook's m-block is an active expert here)
+                        if (phase || wk.at_a != p.withhold_mb) red_release_add_u32(phase ? &S.cs->y_done[0] : &S.h_ready[wk.at_a], (unsigned)(phase ? wk.w : wk.w1));
+                        if (!phase && wk.w1 < wk.w && wk.at_a + 1 != p.withhold_mb) red_release_add_u32(&S.h_ready[wk.at_a + 1], (unsigned)(wk.w - wk.w1));
                         mbar_arrive(&X.freed[tile & 1]);
                     }
                 }
@@ -450,7 +454,8 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
             __syncwarp();
             if (lane == 0) red_release_add_u32(&S.cs->y_done[0], 1u);
         } else {
-            // ---------------- the products
+            // ---------------- the products.  `ok` is the warp's: once a wait of it has failed it only goes on to meet the others
+            // at the barriers around a reload of h.
             const int wi = warp - 8;
             int tile = 0;
             StreamRing r = {ring, (uint32_t)(slot_units * 2048), slots, 0, 0u};
@@ -466,17 +471,20 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                         // the next rows of h, once all of them are there and nobody reads what they replace
                         first = wk.at_a; second = two ? wk.at_a + 1 : -1;
                         named_barrier_sync<2, kStWarps * 32>();
-                        if (lane == 0) ok = flag_wait_ge(&S.h_ready[first], (unsigned)(p.I / kStUnitG), p, 62) && ok;
-                        if (lane == 0 && two) ok = flag_wait_ge(&S.h_ready[second], (unsigned)(p.I / kStUnitG), p, 62) && ok;
-                        __syncwarp();
+                        if (lane == 0 && ok) {
+                            ok = flag_wait_ge(&S.h_ready[first], (unsigned)(p.I / kStUnitG), p, 62);
+                            if (ok && two) ok = flag_wait_ge(&S.h_ready[second], (unsigned)(p.I / kStUnitG), p, 62);
+                        }
+                        ok = __all_sync(0xffffffffu, ok);
                         const int per_row = p.I >> 3, ctid = tid - 256, n = X.rows(first) + (two ? X.rows(second) : 0);
                         const __nv_bfloat16 *src = p.hbuf + (size_t)X.off[X.act[first]] * p.I;      // (the two experts' rows are neighbours)
-                        for (int t = 0; t < n; ++t)
+                        for (int t = 0; t < n && ok; ++t)
                             for (int c = ctid; c < per_row; c += kStWarps * 32)
                                 cp_async_16(rows_s + (uint32_t)t * pitch + (uint32_t)(c * 16), src + (size_t)t * p.I + c * 8);
                         cp_async_wait_all();
                         named_barrier_sync<2, kStWarps * 32>();
                     }
+                    if (!ok) continue;
                     // this warp's unit: unit li of the ones that the tile has of active expert a
                     const bool works = wi < wk.w, later = works && wi >= wk.w1;
                     const int a = later ? wk.at_a + 1 : wk.at_a, li = later ? wi - wk.w1 : wi, wp = later ? wk.w - wk.w1 : wk.w1;
@@ -491,15 +499,16 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                     const int K = phase ? p.I : p.H;
                     float acc[kWide ? 2 : 1][4];
                     if (!kWide || n_e <= 8)
-                        ok = (kb == 2 ? stream_tile<2>(p, X, r, K, works, a_off, blk, b_row, acc[0]) : stream_tile<1>(p, X, r, K, works, a_off, blk, b_row, acc[0])) && ok;
+                        ok = kb == 2 ? stream_tile<2>(p, X, r, K, works, a_off, blk, b_row, acc[0]) : stream_tile<1>(p, X, r, K, works, a_off, blk, b_row, acc[0]);
                     else {
                         const int i16 = i8 + 8 < n_e ? i8 + 8 : 0;
                         const int src_row2 = phase ? (a == second ? X.rows(first) : 0) + i16 : (int)__fns(X.mask[e], 0u, i16 + 1);
                         const uint32_t b_row2 = rows_s + (uint32_t)src_row2 * pitch + (uint32_t)((lane >> 3) * 16);
-                        ok = (kb == 2 ? stream_tile_16<2>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])
-                                      : stream_tile_16<1>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])) && ok;
+                        ok = kb == 2 ? stream_tile_16<2>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])
+                                     : stream_tile_16<1>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide]);
                     }
-                    if (works) {
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (works && ok) {
                         const int col = (phase ? unit * kStUnitD : unit * kStUnitG) + (lane >> 2);
 #pragma unroll
                         for (int i = 0; i < (kWide ? 4 : 2); ++i) {      // this lane has rows 2q and 2q + 1 of every eight of the expert
@@ -514,10 +523,11 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                         }
                     }
                     __syncwarp();
-                    if (lane == 0) {
-                        if (tile >= 2) ok = mbar_wait(&X.freed[tile & 1], (uint32_t)(((tile >> 1) - 1) & 1), p, 65) && ok;
-                        mbar_arrive(&X.done[tile & 1]);
+                    if (lane == 0 && ok) {
+                        if (tile >= 2) ok = mbar_wait(&X.freed[tile & 1], (uint32_t)(((tile >> 1) - 1) & 1), p, 65);
+                        if (ok) mbar_arrive(&X.done[tile & 1]);
                     }
+                    ok = __all_sync(0xffffffffu, ok);
                 }
             }
             if (!ok) X.failed = 1;
@@ -526,7 +536,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
 
     // ================= combine: out[t] = sum over the slots, in slot order, then the shared experts
     __syncthreads();
-    if (tid == 0 && !flag_wait_ge(&S.cs->y_done[0], (unsigned)(A * (p.H / kStUnitD) + 6 * ctas), p, 63)) X.failed = 1;
+    if (tid == 0 && !X.failed && !flag_wait_ge(&S.cs->y_done[0], (unsigned)(A * (p.H / kStUnitD) + 6 * ctas), p, 63)) X.failed = 1;
     __syncthreads();
     if (!X.failed) {
         const int vecs = p.H >> 3, total = p.T * vecs;      // 16-byte pieces, four neighbours to a CTA

@@ -108,3 +108,51 @@ def test_smallest_batches_in_place_and_captured_between_larger_ones(T):
         assert torch.equal(out, refs.setdefault(n, out.clone())), n
     moe.check()
     moe.close()
+
+
+@pytest.mark.parametrize("T", [1, 8, 16])
+@pytest.mark.parametrize("which", [0, 1, -1])
+def test_a_wait_that_gives_up_ends_the_streaming_launch(T, which):
+    """The finished h tiles of one active expert are never counted in: the waits for them run out, nobody works on with what
+    is not there (the expert's rows of y and the output stay as they were), the launch ends without a second limit, and
+    the next ones, the one that was queued behind it included, are right again on either kernel."""
+    cfg = wl.MoEConfig(f"stream_fail_{T}", 1400, T=64, H=2048, I=1408, E=24, k=3, S=1)
+    x, lg, gu, dn = to_dev(wl.make_inputs(cfg))
+    moe = pk.WeaveMoE(gu, dn, cfg.E, cfg.k, cfg.S, max_tokens=64)
+    xs, ls = x[:T].contiguous(), lg[:T].contiguous()
+    ref64 = moe.forward(x, lg).view(torch.int16).clone()
+    ref = moe.forward(xs, ls).view(torch.int16).clone()
+    moe.check()
+    counts, offsets = (moe.routing(T)[n].cpu().numpy() for n in ("counts", "offsets"))
+    active = np.flatnonzero(counts)
+    e = active[which]
+    y, out = moe.intermediates(T)["y"].view(torch.int16), torch.full_like(xs, -3.0)
+    y.fill_(0x7fc1)
+    limit_ms, t0, t1 = 100, torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    moe.set_timeout_ms(limit_ms)
+    moe.debug_withhold_flag(which % len(active))
+    t0.record()
+    moe.forward(xs, ls, out)
+    t1.record()
+    moe.debug_withhold_flag(-1)
+    moe.set_timeout_ms(4000)
+    assert moe.status() == pk.ERR_TIMEOUT
+    assert 60 <= moe.last_timeout_where() <= 65
+    assert limit_ms <= t0.elapsed_time(t1) < 2 * limit_ms
+    assert (y[offsets[e]:offsets[e + 1]] == 0x7fc1).all() and (out == -3.0).all()
+    for _ in range(3):
+        assert torch.equal(moe.forward(xs, ls).view(torch.int16), ref)
+        assert torch.equal(moe.forward(x, lg).view(torch.int16), ref64)
+    moe.check()
+    moe.set_timeout_ms(20)      # ... and right behind a failed launch, its host status not yet read
+    moe.debug_withhold_flag(which % len(active))
+    moe.forward(xs, ls)
+    moe.debug_withhold_flag(-1)
+    moe.set_timeout_ms(4000)
+    assert torch.equal(moe.forward(xs, ls).view(torch.int16), ref)
+    assert torch.equal(moe.forward(x, lg).view(torch.int16), ref64)
+    assert moe.status() == pk.ERR_TIMEOUT
+    moe.debug_withhold_flag(len(active))      # an index that the batch does not reach
+    assert torch.equal(moe.forward(xs, ls).view(torch.int16), ref)
+    moe.check()
+    moe.close()
