@@ -229,9 +229,10 @@ int weave_moe_last_timeout_where(weave_moe_t h);
 
 /* Post-mortem of the launch whose failure the last weave_moe_status() reported.  Every bounded wait
  * that ended without success - its own limit ran out, or it saw the abort word another wait had raised -
- * left a record in its warp's slot.  Copies up to max_records records of six ints to `out` (host):
+ * left a record in its warp's slot (16 warps in the streaming kernel, 8 in the general one).  Copies up to max_records records of six ints to `out` (host):
  * {CTA, warp, wait id (as weave_moe_last_timeout_where), the object waited on (for a shared-memory
- * barrier its address, whose low 10 bits are the barrier's byte offset among the CTA's barriers; for
+ * barrier its address, whose low 10 bits are the barrier's byte offset from the start of the kernel's
+ * structure of them; for
  * a ready flag the low 32 bits of its device address), the parity or count waited for, 1 = this
  * wait's limit ran out / 2 = cut short by the abort word}.  Returns the number of records there
  * are (may exceed max_records), 0 when the last status was clean.  Diagnostic only: which warps

@@ -152,7 +152,7 @@ struct KParams {
     int trace_cap;
     unsigned die_mask[32]; // bit smid: which half of the chip (die) the SM sits on
     int lists_pt;          // one chunk: two lists of GEMM tiles from this many row tiles on (see tile_lists_from)
-    int4 *wait_log;       // [n_sm][8 warps]: written only by a wait that gives up or is cut short by the abort word
+    int4 *wait_log;       // [kWaitLogCtas][kWaitLogWarps]: written only by a wait that gives up or is cut short by the abort word
     float st_plan_t;      // weave_stream_kernel: the modelled time of its plan
 };
 
@@ -270,12 +270,14 @@ __device__ __noinline__ void give_up(Ctl *ctl, int where)
 // barrier or low bits of the flag's address), the parity or target it waited for, 1 = timed out / 2 = cut
 // short} in its warp's slot (the warp's first such wait only).  Together the slots show who was waiting
 // for whom when the launch stopped.
+constexpr int kWaitLogCtas = 512, kWaitLogWarps = 16;      // (the streaming kernel has 16 warps; no sm_100 device has as many SMs)
 __device__ __noinline__ void note_failed_wait(int4 *log, int where, unsigned what, unsigned want, int how)
 {
     // the first failed wait of a warp is the one that tells where it stood; what it runs into afterwards,
-    // on its way out with the abort word set, is not recorded  (warps 8 and up of the streaming kernel share the slots)
-    int4 *slot = log + blockIdx.x * 8 + ((threadIdx.x >> 5) & 7);
-    if (log && slot->w == 0) *slot = make_int4(where, (int)what, (int)want, how);
+    // on its way out with the abort word set, is not recorded
+    if (!log || blockIdx.x >= kWaitLogCtas) return;
+    int4 *slot = log + blockIdx.x * kWaitLogWarps + (threadIdx.x >> 5);
+    if (slot->w == 0) *slot = make_int4(where, (int)what, (int)want, how);
 }
 
 // Optional timeline: one 16-byte record {start ns, end ns, kind<<24 | id, extra} per event, per CTA.

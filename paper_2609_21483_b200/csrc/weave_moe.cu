@@ -22,7 +22,7 @@ namespace {
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-constexpr int kWaitLogSlots = 1024 * 8;      // one slot per warp of up to 1024 CTAs
+constexpr int kWaitLogSlots = kWaitLogCtas * kWaitLogWarps;
 
 struct Layout {
     size_t ctl, sets, wait_log, zero_end;       // [0, zero_end) is zeroed at create / recovery
@@ -774,7 +774,7 @@ int weave_moe_status(weave_moe_t h)
             if (cudaMemcpy(raw.data(), h->ws + h->L.wait_log, sizeof(int4) * kWaitLogSlots, cudaMemcpyDeviceToHost) == cudaSuccess)
                 for (int i = 0; i < kWaitLogSlots; ++i)
                     if (raw[i].w != 0) {
-                        const int32_t rec[6] = {i / 8, i % 8, raw[i].x, raw[i].y, raw[i].z, raw[i].w};
+                        const int32_t rec[6] = {i / kWaitLogWarps, i % kWaitLogWarps, raw[i].x, raw[i].y, raw[i].z, raw[i].w};
                         h->wait_log->insert(h->wait_log->end(), rec, rec + 6);
                     }
         }

@@ -76,7 +76,8 @@ struct StreamShared {      // lies over the SmemTail's segment tables, which thi
     float gate[kStTokens][kMaxTopK];
     __device__ __forceinline__ int rows(int a) const { return off[act[a] + 1] - off[act[a]]; }
 };
-constexpr size_t kStSharedAt = (offsetof(SmemTail, seg_mb0) + 15) / 16 * 16;      // (the tail starts on a 1024-byte boundary)
+constexpr size_t kStSharedAt = (offsetof(SmemTail, seg_mb0) + 1023) / 1024 * 1024;      // (the tail starts on a 1024-byte boundary; on another one,
+                                                                                        // the low bits of a barrier's address name it in the wait log)
 static_assert(kStSharedAt + sizeof(StreamShared) <= sizeof(SmemTail), "must fit the segment tables");
 static_assert(alignof(StreamShared) <= 16, "aligned where it lies");
 

@@ -156,3 +156,25 @@ def test_a_wait_that_gives_up_ends_the_streaming_launch(T, which):
     assert torch.equal(moe.forward(xs, ls).view(torch.int16), ref)
     moe.check()
     moe.close()
+
+
+def test_wait_log_of_the_streaming_kernel_tells_its_sixteen_warps_apart():
+    """Every failed wait is in its own warp's slot: the producer's (60), the products' (61, 62, 65), the releasing warp's (64)
+    and the combine's (63, thread 0); a barrier is named by its offset among the kernel's barriers."""
+    cfg = wl.MoEConfig("stream_log", 1450, T=8, H=2048, I=1408, E=24, k=3)
+    x, lg, gu, dn = to_dev(wl.make_inputs(cfg))
+    moe = pk.WeaveMoE(gu, dn, cfg.E, cfg.k, cfg.S, max_tokens=8)
+    moe.set_timeout_ms(20)
+    moe.debug_withhold_flag(0)
+    moe.forward(x, lg)
+    assert moe.status() == pk.ERR_TIMEOUT
+    log = moe.wait_log()
+    assert len({r[:2] for r in log}) == len(log) and all(0 <= r[0] < moe.geometry()["n_sm"] for r in log)
+    warps = {60: {0}, 61: set(range(8, 16)), 62: set(range(8, 16)), 63: {0}, 64: {1}, 65: set(range(8, 16))}
+    assert all(r[1] in warps[r[2]] for r in log), log
+    failed = [r for r in log if r[2] == 62]
+    assert {r[0] for r in failed if r[1] == 8} and {r[1] for r in failed} == set(range(8, 16))
+    places = {60: (128, 256), 61: (0, 128), 64: (256, 272), 65: (272, 288)}      # empty, full, done, freed
+    assert all(places[r[2]][0] <= (r[3] & 1023) < places[r[2]][1] for r in log if r[2] in places), log
+    assert any(r[5] == 1 for r in log) and moe.last_timeout_where() in {r[2] for r in log if r[5] == 1}
+    moe.close()
