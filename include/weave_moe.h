@@ -260,8 +260,9 @@ int weave_moe_debug_withhold_flag(weave_moe_t h, int m_block);
  * extra = type << 16 | ns spent before the release), 7 combine tile, 8 wait for a chunk's gemm1,
  * 9 grid barrier (the one behind the routing; a batch of at most 64 tokens is routed by every CTA for itself
  * and has none), 11 GEMM tile main loop on the MMA issuer (id = type << 16 | rows, extra = ns spent
- * waiting for a free accumulator).  The records are the general kernel's: while a timeline is set, a
- * batch of up to 16 tokens runs on it too (same results) and not on the streaming kernel. */
+ * waiting for a free accumulator).  The streaming kernel of the smallest batches writes 1, 2, 4 (one per
+ * dispatched row, id = row), 12 tile of up to 8 units of columns on the CTA's product warps (id = (0 gate/up, 1 down) << 16 | units,
+ * extra = ns spent waiting for h before it), 8 (wait for the last y) and 7 (the CTA's share of the combine, id = CTA). */
 int weave_moe_set_trace(weave_moe_t h, void *buf, int events_per_cta);
 
 /* HOST-ONLY (no GPU needed, no handle): the order in which the kernel's GEMM schedulers claim pair

@@ -282,7 +282,7 @@ __device__ __noinline__ void note_failed_wait(int4 *log, int where, unsigned wha
 
 // Optional timeline: one 16-byte record {start ns, end ns, kind<<24 | id, extra} per event, per CTA.
 enum { kEvRoute = 1, kEvSetup = 2, kEvFixup = 3, kEvDispatch = 4, kEvGemmLoad = 5, kEvGemmEpi = 6,
-       kEvCombine = 7, kEvWaitChunk = 8, kEvBarrier = 9, kEvMma = 11 };
+       kEvCombine = 7, kEvWaitChunk = 8, kEvBarrier = 9, kEvMma = 11, kEvStream = 12 };
 __device__ __forceinline__ void trace_ev(const KParams &p, SmemTail &S, int kind, unsigned id,
                                          unsigned long long t0, unsigned long long t1, unsigned extra)
 {

@@ -248,14 +248,24 @@ bool phased_is_picked(const weave_moe *h, int T, float *t_phased)
     return true;
 }
 
-const void *stream_kernel(int T) { return T > 8 ? (const void *)weave_stream_kernel<true> : (const void *)weave_stream_kernel<false>; }
+const void *stream_kernel(int T, bool trace)
+{
+    if (trace) return T > 8 ? (const void *)weave_stream_kernel<true, true> : (const void *)weave_stream_kernel<false, true>;
+    return T > 8 ? (const void *)weave_stream_kernel<true, false> : (const void *)weave_stream_kernel<false, false>;
+}
+
+cudaError_t size_stream_kernels(bool trace)
+{
+    const cudaError_t e = cudaFuncSetAttribute(stream_kernel(1, trace), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(stream_kernel(kStTokens, trace), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+}
 
 // Batches that weave_stream_kernel takes: up to 16 tokens (the N of two products) whose rows of x, or of h if they all went to
-// one expert, leave room for a ring of 80 KB, or of 128 KB from nine tokens on.  (A timeline is about the general kernel's tiles.)
+// one expert, leave room for a ring of 80 KB, or of 128 KB from nine tokens on.
 bool streams(const weave_moe *h, int T)
 {
     const weave_moe_config &c = h->cfg;
-    if (T > kStTokens || h->mode != WEAVE_SCHED_AUTO || h->ep_size != 1 || h->trace) return false;
+    if (T > kStTokens || h->mode != WEAVE_SCHED_AUTO || h->ep_size != 1) return false;
     return (size_t)T * ((size_t)std::max(c.hidden, c.ffn) * 2 + kStPad) <= (size_t)(kStArea - (T > 8 ? 8 * kStMaxSlot : kStMinRing));
 }
 
@@ -416,10 +426,7 @@ int weave_moe_create(const weave_moe_config *cfg, weave_moe_t *out)
 
     e = cudaFuncSetAttribute(weave_moe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) { int rc = cuda_fail(h, e); delete h; return rc; }
-    for (int T : {1, kStTokens}) {
-        e = cudaFuncSetAttribute(stream_kernel(T), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) break;
-    }
+    for (int trace = 0; trace < 2 && e == cudaSuccess; ++trace) e = size_stream_kernels(trace != 0);
     if (e != cudaSuccess) { int rc = cuda_fail(h, e); delete h; return rc; }
     e = cudaFuncSetAttribute(weave_moe_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 0);
     int occ = 0;
@@ -526,7 +533,7 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     if (streams(h, T) && phased_is_picked(h, T, &p.st_plan_t)) {
         if (const int rc = need_maps(h, kMapsStream)) return rc;
         void *sargs[] = {&p, &h->sm};
-        cudaError_t e = cudaLaunchCooperativeKernel(stream_kernel(T), dim3(h->n_cta), dim3(kStThreads), sargs,
+        cudaError_t e = cudaLaunchCooperativeKernel(stream_kernel(T, p.trace != nullptr), dim3(h->n_cta), dim3(kStThreads), sargs,
                                                     (size_t)kSmemBytes, st);
         if (e != cudaSuccess) return cuda_fail(h, e);
         h->last_T = T;
@@ -1009,8 +1016,7 @@ int static_setup(int dev, StaticDevice **out)
         }
         if (cudaFuncSetAttribute(weave_moe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) !=
             cudaSuccess ||
-            cudaFuncSetAttribute(stream_kernel(1), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess ||
-            cudaFuncSetAttribute(stream_kernel(kStTokens), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
+            size_stream_kernels(false) != cudaSuccess)
             return WEAVE_ERR_CUDA;
         if (cudaMemset(d.base, 0, 64 * 1024) != cudaSuccess) return WEAVE_ERR_CUDA;
         d.two_dies = find_dies(prop.multiProcessorCount, d.base, d.die_mask);

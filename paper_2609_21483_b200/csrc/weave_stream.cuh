@@ -270,8 +270,9 @@ __device__ __forceinline__ bool stream_tile_16(const KParams &p, StreamShared &X
     return ok;
 }
 
-// kWide: 9 to 16 tokens (a kernel of its own: with the second N tile in it the smaller batches take 1 to 2 % longer)
-template <bool kWide>
+// kWide: 9 to 16 tokens (a kernel of its own: with the second N tile in it the smaller batches take 1 to 2 % longer);
+// kTrace: with the timeline's records (apart, so that the kernels that are timed carry none of it)
+template <bool kWide, bool kTrace>
 __global__ void __launch_bounds__(kStThreads, 1)
 weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ StreamMaps tm)
 {
@@ -282,6 +283,8 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
     const int cta = (int)blockIdx.x, ctas = (int)gridDim.x;
     const uint32_t ring = smem_u32(stages), area_end = ring + (uint32_t)kStArea;
 
+    auto now = [] { return kTrace ? globaltimer_ns() : 0ull; };
+    const unsigned long long tk0 = now();
     // the logits of this warp's token and the batch's rows of x start on their way before anything else
     float lg[8];
 #pragma unroll
@@ -301,6 +304,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
         S.cs = reinterpret_cast<CtlSet *>(p.sets + (odd ? ctl_set_bytes(p.nmb_max) : 0));
         S.h_ready = reinterpret_cast<unsigned *>(S.cs + 1) + kFine * kMaxEE + p.nmb_max;
         X.failed = 0;
+        S.trace_n = 0;
     }
     if (warp == 14 && lane < kStMaxSlots) { mbar_init(&X.full[lane], 1); mbar_init(&X.empty[lane], kStWarps); }
     if (warp == 14 && lane >= 30) { mbar_init(&X.done[lane - 30], kStWarps); mbar_init(&X.freed[lane - 30], 1); }
@@ -317,6 +321,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
     // ================= routing, counts, offsets, active experts
     if (warp < p.T) stream_route(p, X, warp, lg);
     __syncthreads();
+    const unsigned long long tk1 = now();
     unsigned v = 0, inc = 0;      // rows | (has rows) << 16
     if (warp < kMaxEE / 32) {
         const unsigned n = (unsigned)__popc(X.mask[tid]);
@@ -362,6 +367,10 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
     const int cap0 = X.share[0].cap, cap1 = X.share[1].cap;
     const int slot_units = max(cap0 <= kStWarps / 2 ? 2 * cap0 : cap0, cap1 <= kStWarps / 2 ? 2 * cap1 : cap1);
     const int slots = min(kStMaxSlots, ring_bytes / (slot_units * 2048));
+    if (kTrace && tid == 0) {
+        trace_ev(p, S, kEvRoute, 0u, tk0, tk1, 0u);
+        trace_ev(p, S, kEvSetup, 0u, tk1, now(), 0u);
+    }
 
     if (warp == 0) {
         // ---------------- producer
@@ -441,6 +450,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
             // the dispatched rows, row r by CTA r mod N
             const int P = p.T * (p.k + p.S);
             for (int r = cta + ctas * (warp - 2); r < P; r += ctas * 6) {
+                const unsigned long long td = now();
                 int lo = 0, hi = p.EE;      // largest expert that starts at or before r (empty ones share a start with the next)
                 while (hi - lo > 1) {
                     const int mid = (lo + hi) >> 1;
@@ -450,6 +460,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                 const uint4 *src = reinterpret_cast<const uint4 *>(p.x + (size_t)t * p.H);
                 uint4 *dst = reinterpret_cast<uint4 *>(p.xe + (size_t)r * p.H);
                 for (int c = lane; c < (p.H >> 3); c += 32) dst[c] = __ldg(src + c);
+                if (kTrace && lane == 0) trace_ev(p, S, kEvDispatch, (unsigned)r, td, now(), 0u);
             }
             // (counted in with y: nothing is written to `out`, which may be x itself, before its last reader is done)
             __syncwarp();
@@ -467,6 +478,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                 int first = -1, second = -1;      // active experts whose rows of h are in shared memory, one behind the other
                 for (; wk.next(X, phase ? rows_h : 0); ++tile) {
                     const bool two = wk.w1 < wk.w;
+                    const unsigned long long th = now();
                     const int kb = 2 * wk.w <= slot_units ? 2 : 1;
                     if (phase && ((wk.at_a != first && wk.at_a != second) || (two && wk.at_a + 1 != second))) {
                         // the next rows of h, once all of them are there and nobody reads what they replace
@@ -486,6 +498,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                         named_barrier_sync<2, kStWarps * 32>();
                     }
                     if (!ok) continue;
+                    const unsigned long long tt = now();
                     // this warp's unit: unit li of the ones that the tile has of active expert a
                     const bool works = wi < wk.w, later = works && wi >= wk.w1;
                     const int a = later ? wk.at_a + 1 : wk.at_a, li = later ? wi - wk.w1 : wi, wp = later ? wk.w - wk.w1 : wk.w1;
@@ -527,6 +540,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                     if (lane == 0 && ok) {
                         if (tile >= 2) ok = mbar_wait(&X.freed[tile & 1], (uint32_t)(((tile >> 1) - 1) & 1), p, 65);
                         if (ok) mbar_arrive(&X.done[tile & 1]);
+                        if (kTrace && wi == 0) trace_ev(p, S, kEvStream, (unsigned)(phase << 16 | wk.w), tt, now(), (unsigned)(tt - th));
                     }
                     ok = __all_sync(0xffffffffu, ok);
                 }
@@ -537,8 +551,10 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
 
     // ================= combine: out[t] = sum over the slots, in slot order, then the shared experts
     __syncthreads();
+    const unsigned long long tw = now();
     if (tid == 0 && !X.failed && !flag_wait_ge(&S.cs->y_done[0], (unsigned)(A * (p.H / kStUnitD) + 6 * ctas), p, 63)) X.failed = 1;
     __syncthreads();
+    const unsigned long long tc = now();
     if (!X.failed) {
         const int vecs = p.H >> 3, total = p.T * vecs;      // 16-byte pieces, four neighbours to a CTA
         for (int i = ((tid >> 2) * ctas + cta) * 4 + (tid & 3); i < total; i += kStThreads * ctas) {
@@ -560,6 +576,14 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                                                                  pack_bf16x2(a0[4], a0[5]), pack_bf16x2(a0[6], a0[7])));
         }
     } else if (tid == 0) linger_after_abort();      // copies may still be landing in this CTA's shared memory
+    if (kTrace) {      // the slice's last record: how many there are
+        __syncthreads();
+        if (tid == 0) {
+            trace_ev(p, S, kEvWaitChunk, 0u, tw, tc, 0u);
+            trace_ev(p, S, kEvCombine, (unsigned)cta, tc, now(), 0u);
+            p.trace[(size_t)cta * p.trace_cap + p.trace_cap - 1] = make_uint4(min(S.trace_n, (unsigned)p.trace_cap - 1u), 0u, 0u, 0u);
+        }
+    }
     if (tid == 0) atomicAdd(&p.ctl->epoch, cta == 0 ? 65536u - (unsigned)(ctas - 1) : 1u);
 }
 

@@ -36,7 +36,8 @@ if ROOT not in sys.path:
 # event kinds written by the kernel
 EV_ROUTE, EV_SETUP, EV_FIXUP, EV_DISPATCH, EV_CLAIM, EV_EPILOGUE, EV_COMBINE, EV_WAIT_CHUNK, EV_BARRIER = range(1, 10)
 EV_MMA = 11
-_BUSY_KINDS = (EV_SETUP, EV_FIXUP, EV_DISPATCH, EV_EPILOGUE, EV_COMBINE, EV_MMA)
+EV_STREAM = 12      # a tile of the streaming kernel of the smallest batches, on one CTA
+_BUSY_KINDS = (EV_SETUP, EV_FIXUP, EV_DISPATCH, EV_EPILOGUE, EV_COMBINE, EV_MMA, EV_STREAM)
 
 
 def flatten(trace):
@@ -115,11 +116,14 @@ def analyse(trace, shape=None):
     mv = ev[(ev[:, 3] == EV_DISPATCH) | (ev[:, 3] == EV_COMBINE)]
     mm = ev[ev[:, 3] == EV_MMA]
     mm_s = np.minimum(mm[:, 1] + mm[:, 5], mm[:, 2])
-    breaks = np.unique(np.concatenate([[w0, w1], np.clip(mv[:, 1], w0, w1), np.clip(mv[:, 2], w0, w1),
+    st = ev[ev[:, 3] == EV_STREAM]
+    breaks = np.unique(np.concatenate([[w0, w1], np.clip(st[:, 1], w0, w1), np.clip(st[:, 2], w0, w1), np.clip(mv[:, 1], w0, w1), np.clip(mv[:, 2], w0, w1),
                                        np.clip(mm_s, w0, w1), np.clip(mm[:, 2], w0, w1)]))
     seg = np.diff(breaks)
     n_mv = _coverage(np.clip(mv[:, 1], w0, w1), np.clip(mv[:, 2], w0, w1), breaks)
-    n_mm = _coverage(np.clip(mm_s, w0, w1), np.clip(mm[:, 2], w0, w1), breaks)
+    # CTAs in a main loop: both of a pair, or the one that works on a tile of the streaming kernel
+    n_mm = (2 * _coverage(np.clip(mm_s, w0, w1), np.clip(mm[:, 2], w0, w1), breaks)
+            + _coverage(np.clip(st[:, 1], w0, w1), np.clip(st[:, 2], w0, w1), breaks))
     rep = {
         "n_cta": n_cta,
         "window_us": window / 1e3,
@@ -130,7 +134,7 @@ def analyse(trace, shape=None):
         "tensor_active": float((seg * (n_mm > 0)).sum() / window),
         "overlap_ratio": float((seg * ((n_mv > 0) & (n_mm > 0))).sum() / window),
         "mean_ctas_moving": float((seg * n_mv).sum() / window),
-        "mean_ctas_gemm": float((seg * n_mm).sum() * 2 / window),
+        "mean_ctas_gemm": float((seg * n_mm).sum() / window),
         "events": int(len(ev)),
     }
     if shape is not None:
@@ -161,7 +165,7 @@ def ascii_timeline(trace, width=120):
     ev = flatten(trace)
     end = int(ev[:, 2].max())
     edges = np.linspace(0, end, width + 1)
-    classes = [("R", (EV_ROUTE,)), ("s", (EV_SETUP, EV_FIXUP)), ("D", (EV_DISPATCH,)), ("G", (EV_MMA, EV_EPILOGUE)),
+    classes = [("R", (EV_ROUTE,)), ("s", (EV_SETUP, EV_FIXUP)), ("D", (EV_DISPATCH,)), ("G", (EV_MMA, EV_EPILOGUE, EV_STREAM)),
                ("C", (EV_COMBINE,))]
     occ = np.zeros((len(classes), n_cta, width))
     for ci, (_, kinds) in enumerate(classes):

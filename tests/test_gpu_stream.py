@@ -178,3 +178,31 @@ def test_wait_log_of_the_streaming_kernel_tells_its_sixteen_warps_apart():
     assert all(places[r[2]][0] <= (r[3] & 1023) < places[r[2]][1] for r in log if r[2] in places), log
     assert any(r[5] == 1 for r in log) and moe.last_timeout_where() in {r[2] for r in log if r[5] == 1}
     moe.close()
+
+
+@pytest.mark.parametrize("T", [1, 8, 9, 16])
+@pytest.mark.parametrize("H,I,E,k,S", [(2048, 1408, 12, 3, 2), (128, 128, 4, 1, 0), (1152, 384, 256, 16, 0)])
+def test_timeline_of_the_smallest_batches_is_the_streaming_kernels(T, H, I, E, k, S):
+    """With a timeline set the same kernel runs, with the same bits, and its records account for every unit of columns of
+    both phases, every dispatched row, and every CTA's routing, set-up, wait and combine."""
+    cfg = wl.MoEConfig(f"stream_trace_{T}", 1460, T=T, H=H, I=I, E=E, k=k, S=S)
+    x, lg, gu, dn = to_dev(wl.make_inputs(cfg))
+    moe = pk.WeaveMoE(gu, dn, E, k, S, max_tokens=T)
+    ref = moe.forward(x, lg).view(torch.int16).clone()
+    moe.enable_trace(512)
+    assert torch.equal(moe.forward(x, lg).view(torch.int16), ref)
+    moe.check()
+    trace = moe.read_trace()
+    ev = np.concatenate(trace).astype(np.int64)
+    kind, ident = ev[:, 2] >> 24, ev[:, 2] & 0xFFFFFF
+    active, n_sm = int((moe.routing(T)["counts"] > 0).sum()), moe.geometry()["n_sm"]
+    tiles = ident[kind == 12]
+    assert ((tiles & 0xFFFF) >= 1).all() and ((tiles & 0xFFFF) <= 8).all()
+    for phase, units in ((0, I // 8), (1, H // 16)):
+        assert (tiles[tiles >> 16 == phase] & 0xFFFF).sum() == active * units
+    np.testing.assert_array_equal(np.sort(ident[kind == 4]), np.arange(T * (k + S)))
+    assert all((kind == q).sum() == n_sm for q in (1, 2, 7, 8)) and set(kind) <= {1, 2, 4, 7, 8, 12}
+    from paper_2609_21483_b200 import timeline
+    rep = timeline.analyse(trace, {"T": T, "H": H, "I": I, "k": k, "S": S})
+    assert 0 < rep["tensor_active"] <= 1 and rep["mean_ctas_gemm"] <= n_sm and rep["gemm_TFLOPs"] > 0
+    moe.close()

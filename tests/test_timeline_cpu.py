@@ -61,3 +61,15 @@ def test_ascii_timeline_marks_the_roles():
     assert txt[1].split()[1].startswith("RsGGGGGGGGGG")      # CTA 0: routing, set-up, GEMM
     assert "D" in txt[3] and "C" not in txt[3]
     assert txt[4].rstrip().endswith("CCCCC")
+
+
+def test_streaming_tiles_keep_one_cta_busy_each():
+    """A tile of the streaming kernel is its own CTA's tensor work, not a pair's."""
+    ctas = [np.array([_rec(0, 100, tl.EV_ROUTE), _rec(100, 200, tl.EV_SETUP), _rec(200, 200 + 500 * (c + 1), tl.EV_STREAM, 8)],
+                     dtype=np.uint32) for c in range(3)]
+    rep = tl.analyse(ctas)
+    assert rep["window_us"] == 1.6 and rep["tensor_active"] == 1500 / 1600
+    assert abs(rep["mean_ctas_gemm"] - 3000 / 1600) < 1e-12 and rep["overlap_ratio"] == 0.0
+    assert abs(rep["sm_busy"] - (600 + 1100 + 1600) / 4800) < 1e-12
+    txt = tl.ascii_timeline(ctas, width=17).splitlines()
+    assert [l.split()[1].count("G") for l in txt[1:]] == [5, 10, 15]
