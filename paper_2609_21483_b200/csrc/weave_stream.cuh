@@ -176,8 +176,8 @@ __device__ __forceinline__ void stream_route(const KParams &p, StreamShared &X, 
 // One tile for a warp: 16 weight rows x 8 tokens, KB blocks of 64 of K per ring slot.  a_off: this lane's ldmatrix row in a slot,
 // blk: bytes of a block of K in the slot, b_row: this lane's row of x or h.  A block's operands are fetched between the
 // products of the block before: the chain of dependent products (and nothing else) sets the pace.
-// A lane whose wait ended without success waits for nothing more and hands no slot back: the tile's arrival is then missing,
-// and nobody reads what it gave.
+// False: a wait has failed, and the results are not to be used.  (The rest of the tile is run through; slots are handed back all the
+// same, to a producer that is on its way out.)
 struct StreamRing { uint32_t base, bytes; int slots, slot; uint32_t ph; };
 template <int KB>
 __device__ __forceinline__ bool stream_tile(const KParams &p, StreamShared &X, StreamRing &r, int K, bool works, uint32_t a_off, uint32_t blk,
@@ -191,7 +191,7 @@ __device__ __forceinline__ bool stream_tile(const KParams &p, StreamShared &X, S
     for (int i = 0; i < 4; ++i) acc[i] = 0.f;
     auto arrived = [&](int j) {      // block j (of parity j & 1): its slot is there
         if (KB == 1 || (j & 1) == 0) {
-            if (ok) ok = mbar_wait(&X.full[r.slot], r.ph, p, 61);
+            ok = mbar_wait(&X.full[r.slot], r.ph, p, 61) && ok;
             a0 = r.base + (uint32_t)r.slot * r.bytes + a_off;
             if (++r.slot == r.slots) { r.slot = 0; r.ph ^= 1u; }
         } else a0 += blk;
@@ -202,7 +202,7 @@ __device__ __forceinline__ bool stream_tile(const KParams &p, StreamShared &X, S
     };
     auto free_slot = [&](int slot) {      // the slot's values are in registers
         __syncwarp();
-        if (lane == 0 && ok) mbar_arrive(&X.empty[slot]);
+        if (lane == 0) mbar_arrive(&X.empty[slot]);
     };
     const int nb = K / 64;      // even
     int held = r.slot;
@@ -243,7 +243,7 @@ __device__ __forceinline__ bool stream_tile_16(const KParams &p, StreamShared &X
     for (int i = 0; i < 4; ++i) acc[i] = acc2[i] = 0.f;
 #pragma unroll 1
     for (int j = 0; j < K / 64; j += KB) {
-        if (ok) ok = mbar_wait(&X.full[r.slot], r.ph, p, 61);
+        ok = mbar_wait(&X.full[r.slot], r.ph, p, 61) && ok;
         if (works) {
 #pragma unroll
             for (int kb = 0; kb < KB; ++kb) {
@@ -264,7 +264,7 @@ __device__ __forceinline__ bool stream_tile_16(const KParams &p, StreamShared &X
             }
         }
         __syncwarp();
-        if (lane == 0 && ok) mbar_arrive(&X.empty[r.slot]);
+        if (lane == 0) mbar_arrive(&X.empty[r.slot]);
         if (++r.slot == r.slots) { r.slot = 0; r.ph ^= 1u; }
     }
     return ok;
@@ -466,8 +466,9 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
             __syncwarp();
             if (lane == 0) red_release_add_u32(&S.cs->y_done[0], 1u);
         } else {
-            // ---------------- the products.  `ok` is the warp's: once a wait of it has failed it only goes on to meet the others
-            // at the barriers around a reload of h.
+            // ---------------- the products.  `ok` is the warp's at the start of a tile: once a wait of it has failed it only goes on
+            // to meet the others at the barriers around a reload of h (the wide kernel through tiles of no length, as a jump over
+            // them costs it 1 to 1.5 %: T = 16 Qwen3-30B-shaped 129.5 -> 131.0 us; the narrow one loses 0.8 % by them).
             const int wi = warp - 8;
             int tile = 0;
             StreamRing r = {ring, (uint32_t)(slot_units * 2048), slots, 0, 0u};
@@ -486,7 +487,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                         named_barrier_sync<2, kStWarps * 32>();
                         if (lane == 0 && ok) {
                             ok = flag_wait_ge(&S.h_ready[first], (unsigned)(p.I / kStUnitG), p, 62);
-                            if (ok && two) ok = flag_wait_ge(&S.h_ready[second], (unsigned)(p.I / kStUnitG), p, 62);
+                            if (two && ok) ok = flag_wait_ge(&S.h_ready[second], (unsigned)(p.I / kStUnitG), p, 62);
                         }
                         ok = __all_sync(0xffffffffu, ok);
                         const int per_row = p.I >> 3, ctid = tid - 256, n = X.rows(first) + (two ? X.rows(second) : 0);
@@ -497,7 +498,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                         cp_async_wait_all();
                         named_barrier_sync<2, kStWarps * 32>();
                     }
-                    if (!ok) continue;
+                    if (!kWide && !ok) continue;
                     const unsigned long long tt = now();
                     // this warp's unit: unit li of the ones that the tile has of active expert a
                     const bool works = wi < wk.w, later = works && wi >= wk.w1;
@@ -510,17 +511,20 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                     const uint32_t part = later ? (uint32_t)(wk.w1 * kb * 2048) : 0u;
                     const uint32_t a_off = part + (phase ? (uint32_t)(li * 16 + i8 + 8 * (int)half) * 128u : (uint32_t)(li * 8 + i8) * 128u + half * (uint32_t)(wp * 1024));
                     const uint32_t blk = (uint32_t)(wp * 2048);
-                    const int K = phase ? p.I : p.H;
+                    const int K = !kWide || ok ? (phase ? p.I : p.H) : 0;
                     float acc[kWide ? 2 : 1][4];
-                    if (!kWide || n_e <= 8)
+                    if (!kWide || n_e <= 8) {
+                        const bool before = ok;
                         ok = kb == 2 ? stream_tile<2>(p, X, r, K, works, a_off, blk, b_row, acc[0]) : stream_tile<1>(p, X, r, K, works, a_off, blk, b_row, acc[0]);
-                    else {
+                        if (kWide) ok = ok && before;      // (there was no wait in a tile of no length to fail)
+                    } else {
                         const int i16 = i8 + 8 < n_e ? i8 + 8 : 0;
                         const int src_row2 = phase ? (a == second ? X.rows(first) : 0) + i16 : (int)__fns(X.mask[e], 0u, i16 + 1);
                         const uint32_t b_row2 = rows_s + (uint32_t)src_row2 * pitch + (uint32_t)((lane >> 3) * 16);
-                        ok = kb == 2 ? stream_tile_16<2>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])
-                                     : stream_tile_16<1>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide]);
+                        ok = (kb == 2 ? stream_tile_16<2>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])
+                                      : stream_tile_16<1>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])) && ok;
                     }
+                    if (lane == 0 && tile >= 2) ok = mbar_wait(&X.freed[tile & 1], (uint32_t)(((tile >> 1) - 1) & 1), p, 65) && ok;
                     ok = __all_sync(0xffffffffu, ok);
                     if (works && ok) {
                         const int col = (phase ? unit * kStUnitD : unit * kStUnitG) + (lane >> 2);
@@ -537,12 +541,8 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                         }
                     }
                     __syncwarp();
-                    if (lane == 0 && ok) {
-                        if (tile >= 2) ok = mbar_wait(&X.freed[tile & 1], (uint32_t)(((tile >> 1) - 1) & 1), p, 65);
-                        if (ok) mbar_arrive(&X.done[tile & 1]);
-                        if (kTrace && wi == 0) trace_ev(p, S, kEvStream, (unsigned)(phase << 16 | wk.w), tt, now(), (unsigned)(tt - th));
-                    }
-                    ok = __all_sync(0xffffffffu, ok);
+                    if (lane == 0 && ok) mbar_arrive(&X.done[tile & 1]);
+                    if (kTrace && lane == 0 && ok && wi == 0) trace_ev(p, S, kEvStream, (unsigned)(phase << 16 | wk.w), tt, now(), (unsigned)(tt - th));
                 }
             }
             if (!ok) X.failed = 1;
@@ -552,7 +552,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
     // ================= combine: out[t] = sum over the slots, in slot order, then the shared experts
     __syncthreads();
     const unsigned long long tw = now();
-    if (tid == 0 && !X.failed && !flag_wait_ge(&S.cs->y_done[0], (unsigned)(A * (p.H / kStUnitD) + 6 * ctas), p, 63)) X.failed = 1;
+    if (tid == 0 && !flag_wait_ge(&S.cs->y_done[0], (unsigned)(A * (p.H / kStUnitD) + 6 * ctas), p, 63)) X.failed = 1;
     __syncthreads();
     const unsigned long long tc = now();
     if (!X.failed) {
