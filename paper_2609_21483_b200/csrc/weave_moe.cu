@@ -261,12 +261,21 @@ cudaError_t size_stream_kernels(bool trace)
 }
 
 // Batches that weave_stream_kernel takes: up to 16 tokens (the N of two products) whose rows of x, or of h if they all went to
-// one expert, leave room for a ring of 80 KB, or of 128 KB from nine tokens on.
+// one expert, leave a ring of 128 KB from nine tokens on (all that were measured are faster than the general kernel then, by 3 %
+// and more) and of six 16 KB slots up to eight.  Five slots cost 6 % of the rate of a long stream, which is more than the
+// shorter prologue saves once there is much to read.  General kernel / this one with five slots, us: rows of x (7680 columns,
+// T = 8), all experts that the batch can reach 0.8 GB 117 / 107, 1.5 GB 171 / 177, 3 GB 327 / 339; rows of h (T = 2 and 4, all
+// tokens on the same experts), these experts 0.8 GB 182 / 171, 1.5 GB 311 / 293, 1.9 GB 380 / 396.  Hence the two lines.
 bool streams(const weave_moe *h, int T)
 {
     const weave_moe_config &c = h->cfg;
     if (T > kStTokens || h->mode != WEAVE_SCHED_AUTO || h->ep_size != 1) return false;
-    return (size_t)T * ((size_t)std::max(c.hidden, c.ffn) * 2 + kStPad) <= (size_t)(kStArea - (T > 8 ? 8 * kStMaxSlot : kStMinRing));
+    if ((size_t)T * st_pitch(std::max(c.hidden, c.ffn), true) > (size_t)(kStArea - (T > 8 ? kStWideRing : kStMinRing))) return false;
+    const size_t six = (size_t)(kStArea - kStGoodRing), expert = 6 * (size_t)c.hidden * (size_t)c.ffn;      // bytes
+    const size_t any = (size_t)(std::min(c.num_experts, T * c.top_k) + c.num_shared), same = (size_t)(c.top_k + c.num_shared);
+    if (T * st_pitch(c.hidden, false) > six && any * expert > 1000000000u) return false;
+    if (T * st_pitch(c.ffn, false) > six && same * expert > 1600000000u) return false;
+    return true;
 }
 
 void default_tables(int n_sm, std::vector<float> &bw, std::vector<float> &tf)

@@ -206,3 +206,33 @@ def test_timeline_of_the_smallest_batches_is_the_streaming_kernels(T, H, I, E, k
     rep = timeline.analyse(trace, {"T": T, "H": H, "I": I, "k": k, "S": S})
     assert 0 < rep["tensor_active"] <= 1 and rep["mean_ctas_gemm"] <= n_sm and rep["gemm_TFLOPs"] > 0
     moe.close()
+
+
+@pytest.mark.parametrize("T,H,I,E,k,S,streams", [
+    (16, 128, 128, 4, 1, 0, True), (17, 128, 128, 4, 1, 0, False),          # the largest batch
+    (8, 7168, 512, 64, 8, 0, True),                                           # x leaves six ring slots, to the byte
+    (8, 7296, 512, 64, 8, 0, False), (8, 7296, 512, 40, 4, 0, True),          # five: 1.43 GB of experts within reach, 0.72 GB
+    (3, 4096, 14464, 6, 4, 1, True), (4, 4096, 14336, 6, 4, 1, True),         # h of one expert leaves six
+    (4, 4096, 14464, 6, 4, 1, False), (4, 4096, 14464, 6, 3, 1, True),        # five: 1.78 GB of experts at least, 1.42 GB
+    (8, 128, 8064, 2, 1, 0, True), (8, 128, 8192, 2, 1, 0, False),            # no room for five
+    (9, 4480, 128, 8, 2, 0, True), (9, 4608, 128, 8, 2, 0, False),            # nine tokens and more: eight slots
+    (10, 3968, 128, 8, 2, 0, True), (10, 4096, 128, 8, 2, 0, False)])
+def test_which_batches_stream(T, H, I, E, k, S, streams):
+    """The kernel that runs on both sides of every line of the rule, told by the timeline's records, and its bits against the
+    SERIAL schedule's."""
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    gu, dn = (torch.empty(s, dtype=torch.bfloat16, device="cuda").normal_(0, 0.02, generator=gen) for s in ((E + S, 2 * I, H), (E + S, H, I)))
+    x = torch.empty((T, H), dtype=torch.bfloat16, device="cuda").normal_(0, 1, generator=gen)
+    lg = torch.empty((T, E), device="cuda").normal_(0, 1, generator=gen)
+    moe = pk.WeaveMoE(gu, dn, E, k, S, max_tokens=T)
+    moe.enable_trace(4096)
+    for same in (False, True):      # all tokens on the same experts
+        out = moe.forward(x, lg[:1].expand(T, E).contiguous() if same else lg).view(torch.int16).clone()
+        moe.check()
+        kinds = set((np.concatenate([a for a in moe.read_trace() if len(a)])[:, 2] >> 24).tolist())
+        assert (12 in kinds, 6 in kinds) == (streams, not streams)
+        moe.set_schedule(pk.SCHED_SERIAL)
+        assert torch.equal(moe.forward(x, lg[:1].expand(T, E).contiguous() if same else lg).view(torch.int16), out)
+        moe.set_schedule(pk.SCHED_AUTO)
+    moe.check()
+    moe.close()
