@@ -7,7 +7,7 @@ import torch
 import workloads as wl
 import paper_2609_21483_b200 as pk
 from oracle import cost_model as cm
-from parity import run_case, to_dev
+from parity import check_routing, run_case, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -235,4 +235,50 @@ def test_which_batches_stream(T, H, I, E, k, S, streams):
         assert torch.equal(moe.forward(x, lg[:1].expand(T, E).contiguous() if same else lg).view(torch.int16), out)
         moe.set_schedule(pk.SCHED_AUTO)
     moe.check()
+    moe.close()
+
+
+def _edge_logits(kind, T, E, rng):
+    if kind == "equal":                       # ties decide everything
+        return np.full((T, E), rng.standard_normal(), np.float32)
+    if kind == "quantised":                   # a few values: ties in one lane (e, e + 32) and across lanes
+        return rng.integers(-1, 2, (T, E)).astype(np.float32)
+    if kind == "signed_zeros":                # -0 == +0
+        lg = np.where(rng.random((T, E)) < 0.5, np.float32(0.0), np.float32(-0.0))
+        lg[:, rng.integers(0, E)] = -1.0
+        return lg.astype(np.float32)
+    if kind == "extreme":                     # the largest finite values of either sign, denormals, zeros
+        return rng.choice(np.array([3.4028235e38, -3.4028235e38, 1e-45, -1e-45, 0.0, 1.0], np.float32), (T, E))
+    lg = rng.standard_normal((T, E)).astype(np.float32)
+    lg[T // 2, rng.integers(0, E)] = {"nan": np.nan, "+inf": np.inf, "-inf": -np.inf}[kind]
+    return lg
+
+
+@pytest.mark.parametrize("T", [1, 8, 9, 16])
+@pytest.mark.parametrize("E,k", [(4, 2), (4, 4), (40, 5), (130, 16), (256, 8)])
+def test_routing_of_the_smallest_batches_at_the_edges(T, E, k):
+    """Ties within a lane and across lanes, signed zeros, the largest finite logits, non-finite ones: indices, permutation
+    and counts of the oracle where the logits are finite, and the general kernel's status and bits always."""
+    cfg = wl.MoEConfig(f"stream_edge_{T}_{E}", 1470 + E, T=T, H=128, I=128, E=E, k=k)
+    inp = wl.make_inputs(cfg)
+    x, lg, gu, dn = to_dev(inp)
+    moe = pk.WeaveMoE(gu, dn, E, k, 0, max_tokens=T)
+    moe.enable_trace(256)      # (its records tell which kernel ran)
+    rng = np.random.default_rng(T * 1000 + E)
+    for kind in ("equal", "quantised", "quantised", "signed_zeros", "extreme", "nan", "+inf", "-inf"):
+        inp.logits[:] = _edge_logits(kind, T, E, rng)
+        lg.copy_(torch.from_numpy(inp.logits))
+        got = []
+        for sched in (pk.SCHED_AUTO, pk.SCHED_SERIAL):
+            moe.set_schedule(sched)
+            out = moe.forward(x, lg).view(torch.int16).clone()
+            assert moe.status() == (0 if np.isfinite(inp.logits).all() else pk.ERR_NONFINITE_LOGITS)
+            kinds = set((np.concatenate([a for a in moe.read_trace() if len(a)])[:, 2] >> 24).tolist())
+            assert (12 in kinds) == (sched == pk.SCHED_AUTO)
+            got.append((out, _state(moe, T)))
+            if np.isfinite(inp.logits).all():
+                check_routing(moe, inp)
+        assert torch.equal(got[0][0], got[1][0]), kind
+        for name in got[0][1]:
+            assert torch.equal(got[0][1][name], got[1][1][name]), (kind, name)
     moe.close()
