@@ -465,7 +465,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                 const int t = (int)__fns(X.mask[lo], 0u, r - X.off[lo] + 1);
                 const uint4 *src = reinterpret_cast<const uint4 *>(p.x + (size_t)t * p.H);
                 uint4 *dst = reinterpret_cast<uint4 *>(p.xe + (size_t)r * p.H);
-                for (int c = lane; c < (p.H >> 3); c += 32) dst[c] = __ldg(src + c);
+                for (int c = lane; c < (p.H >> 3); c += 32) dst[c] = __ldcg(src + c);      // (x may be the output: not read-only)
                 if (kTrace && lane == 0) trace_ev(p, S, kEvDispatch, (unsigned)r, td, now(), 0u);
             }
             // (counted in with y: nothing is written to `out`, which may be x itself, before its last reader is done)

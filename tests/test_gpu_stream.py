@@ -84,11 +84,12 @@ def test_smallest_batches_in_place_and_captured_between_larger_ones(T):
     xs, ls = x[:T].contiguous(), lg[:T].contiguous()
     ref = moe.forward(xs, ls).view(torch.int16).clone()
     xe = moe.intermediates(T)["xe"].view(torch.int16).clone()
-    for _ in range(200):
+    wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(200):      # every launch is looked at: a read of x behind the first write of out is a matter of timing
         buf = xs.clone()
         moe.forward(buf, ls, buf)
-    assert torch.equal(buf.view(torch.int16), ref)
-    assert torch.equal(moe.intermediates(T)["xe"].view(torch.int16), xe)
+        wrong += (buf.view(torch.int16) != ref).sum() + (moe.intermediates(T)["xe"].view(torch.int16) != xe).sum()
+    assert wrong.item() == 0
     second = moe.forward(buf, ls).view(torch.int16).clone()
     s, g, o1, o2 = torch.cuda.Stream(), torch.cuda.CUDAGraph(), torch.empty_like(xs), torch.empty_like(xs)
     s.wait_stream(torch.cuda.current_stream())
