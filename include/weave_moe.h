@@ -85,7 +85,9 @@ int weave_moe_create(const weave_moe_config *cfg, weave_moe_t *out_handle);
  * (WEAVE_ERR_NONFINITE_LOGITS, WEAVE_ERR_TIMEOUT) are reported by weave_moe_status().
  * The call makes no other CUDA call (no allocation, copy, memset or synchronisation: the kernel
  * re-zeroes its own control words), so a sequence of layers may be captured into a CUDA graph on
- * `cuda_stream`; the replay reads the arguments and the schedule settings given at capture time. */
+ * `cuda_stream`; the replay reads the arguments and the schedule settings given at capture time, but
+ * for BW and TFLOPS, which a replay of the general kernel reads as they are then (see
+ * weave_moe_set_cost_tables()). */
 int weave_moe_forward(weave_moe_t h, const void *x, const float *router_logits, void *out, int T,
                       void *cuda_stream);
 
@@ -148,7 +150,10 @@ int weave_moe_set_sm_count(weave_moe_t h, int n_sm);
  * ignored); eff_chunk[4] = Eq. 9's correction factor for K = 1,2,4,8; alpha = Section 3.1's
  * overlap ratio in [0,1); candidate grid c = c_min, c_min+c_step, ... <= c_max (at most 64
  * values; c_min and c_step even, c_min >= 2).  A candidate (c, K) is skipped when K*(E+S) > 1024
- * (the kernel's table of (chunk, expert) segments).  Synchronous copy to the device. */
+ * (the kernel's table of (chunk, expert) segments).  Synchronous copy to the device.
+ * The streaming kernel of the smallest batches (AUTO, up to 16 tokens) is launched for plans that the
+ * host has found to be PHASED with its own copy of the tables: in a CUDA graph such a layer keeps the
+ * plan, and the modelled time, of the tables that were set at its capture. */
 int weave_moe_set_cost_tables(weave_moe_t h, const float *bw, const float *tflops,
                               const float *eff_chunk, float alpha, int c_min, int c_max, int c_step);
 

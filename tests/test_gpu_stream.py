@@ -283,3 +283,39 @@ def test_routing_of_the_smallest_batches_at_the_edges(T, E, k):
         for name in got[0][1]:
             assert torch.equal(got[0][1][name], got[1][1][name]), (kind, name)
     moe.close()
+
+
+def test_a_captured_batch_keeps_its_plan_as_the_header_says():
+    """Tables set behind a capture: a replay of the streaming kernel reports the plan that was made with the old ones, a replay
+    of the general kernel the new arg-min; a direct call the new one, whatever the size."""
+    cfg = wl.MoEConfig("stream_graph_plan", 1480, T=40, H=512, I=256, E=16, k=2)
+    x, lg, gu, dn = to_dev(wl.make_inputs(cfg))
+    moe = pk.WeaveMoE(gu, dn, cfg.E, cfg.k, max_tokens=40)
+    N = moe.geometry()["n_sm"]
+    moe.set_model_options(1 << pk.PLAN_PHASED, -1)
+    want, graphs, refs = {}, {}, {}
+    s = torch.cuda.Stream()
+    for T in (8, 40):
+        xs, ls = x[:T].contiguous(), lg[:T].contiguous()
+        refs[T] = (xs, ls, moe.forward(xs, ls).view(torch.int16).clone())
+        want[T] = moe.plan()["t_total_us"]
+        out = torch.empty_like(xs)
+        s.wait_stream(torch.cuda.current_stream())
+        graphs[T] = (torch.cuda.CUDAGraph(), out)
+        with torch.cuda.stream(s):
+            with torch.cuda.graph(graphs[T][0], stream=s):
+                moe.forward(xs, ls, out)
+    idx = np.arange(N + 1, dtype=np.float32)
+    moe.set_cost_tables(1e3 * np.maximum(idx, 1), 1e6 * np.maximum(idx, 1), np.array([1.0, .9, .8, .7], np.float32), 0.5, 2, N // 2, 2)
+    for T, (g, out) in graphs.items():
+        g.replay()
+        torch.cuda.synchronize()
+        replayed = moe.plan()["t_total_us"]
+        assert torch.equal(out.view(torch.int16), refs[T][2])
+        moe.forward(refs[T][0], refs[T][1])
+        direct = moe.plan()["t_total_us"]
+        assert direct > 10 * want[T] and moe.plan()["kind"] == pk.PLAN_PHASED
+        # (the general kernel reads BW and TFLOPS on the device; alpha is an argument of the launch)
+        assert replayed == want[T] if T <= 16 else replayed > 10 * want[T]
+    moe.check()
+    moe.close()
