@@ -559,7 +559,8 @@ def test_load_distributions_around_the_cut_between_the_two_tile_lists(rows, ffn)
 @pytest.mark.parametrize("E,k,S", [(4, 1, 0), (5, 5, 1), (130, 8, 2), (256, 16, 0)])
 def test_batches_whose_gate_up_tiles_read_x_itself(T, E, k, S):
     """Up to 32 tokens under the phased plan: the gate/up tiles multiply all tokens and keep the expert's rows.
-    T around that limit and around the row boxes of 8 and 16; experts below and above a warp's width, odd
+    T around that limit and around the row boxes of 8 and 16 (up to 16 tokens these shapes run on the streaming kernel; the
+    next test has the boxes of 8); experts below and above a warp's width, odd
     counts, a shared expert; whole output against the oracle, and the dispatched rows are still written."""
     cfg = _small(f"direct_T{T}_E{E}", T, 256, 256, E, k, S, cfg_id=960 + E)
     inp = wl.make_inputs(cfg)
@@ -568,6 +569,27 @@ def test_batches_whose_gate_up_tiles_read_x_itself(T, E, k, S):
     assert moe.plan()["kind"] == pk.PLAN_PHASED
     xe, tok = moe.intermediates(T)["xe"].view(torch.int16), moe.routing(T)["token_of"].long()
     assert torch.equal(xe, dev[0].view(torch.int16)[tok])
+    _, serial, _ = run_case(cfg, sched=(pk.SCHED_SERIAL, 0, 1, 0), inp=inp, dev_tensors=dev, moe=moe)
+    assert torch.equal(out.view(torch.int16), serial.view(torch.int16))
+    moe.close()
+
+
+@pytest.mark.parametrize("T,H", [(4, 16384), (7, 16384), (8, 16384), (9, 5120), (15, 5120), (16, 5120)])
+@pytest.mark.parametrize("E,k,S", [(4, 1, 0), (5, 5, 1), (130, 8, 2)])
+def test_wide_layers_whose_gate_up_tiles_read_x_in_boxes_of_8_rows(T, H, E, k, S):
+    """The same up to 16 tokens, where only layers too wide for the streaming kernel come this way."""
+    cfg = _small(f"direct_wide_T{T}_E{E}", T, H, 128, E, k, S, cfg_id=980 + E)
+    inp = wl.make_inputs(cfg)
+    dev = to_dev(inp)
+    moe, out, _ = run_case(cfg, inp=inp, dev_tensors=dev)
+    assert moe.plan()["kind"] == pk.PLAN_PHASED
+    xe, tok = moe.intermediates(T)["xe"].view(torch.int16), moe.routing(T)["token_of"].long()
+    assert torch.equal(xe, dev[0].view(torch.int16)[tok])
+    moe.enable_trace(4096)
+    assert torch.equal(moe.forward(dev[0], dev[1]).view(torch.int16), out.view(torch.int16))
+    kinds = set((np.concatenate([a for a in moe.read_trace() if len(a)])[:, 2] >> 24).tolist())
+    assert 6 in kinds and 12 not in kinds
+    moe.enable_trace(0)
     _, serial, _ = run_case(cfg, sched=(pk.SCHED_SERIAL, 0, 1, 0), inp=inp, dev_tensors=dev, moe=moe)
     assert torch.equal(out.view(torch.int16), serial.view(torch.int16))
     moe.close()

@@ -12,6 +12,10 @@ from parity import check_routing, run_case, to_dev
 pytestmark = pytest.mark.gpu
 
 
+def _kinds(moe):
+    return set((np.concatenate([a for a in moe.read_trace() if len(a)])[:, 2] >> 24).tolist())
+
+
 def _state(moe, T):
     r = {k: v.clone() for k, v in moe.routing(T).items()}
     r.update({k: v.view(torch.int16).clone() for k, v in moe.intermediates(T).items()})
@@ -36,6 +40,10 @@ def test_smallest_batches_match_oracle_and_general_kernel(T, H, I, E, k, S):
         moe.set_sm_count(sm)
         for _ in range(3):
             assert torch.equal(moe.forward(dev[0], dev[1]).view(torch.int16), out.view(torch.int16)), sm
+    moe.enable_trace(4096)      # its records tell which kernel the rule picks: beyond it this compares the general one with itself
+    assert torch.equal(moe.forward(dev[0], dev[1]).view(torch.int16), out.view(torch.int16))
+    assert (12 in _kinds(moe)) == (T <= 16 and T * (2 * max(H, I) + 16) <= 212992 - 16384 * (8 if T > 8 else 5))
+    moe.enable_trace(0)
     _, general, _ = run_case(cfg, sched=(pk.SCHED_SERIAL, 0, 1, 0), inp=inp, dev_tensors=dev, moe=moe)
     assert torch.equal(out.view(torch.int16), general.view(torch.int16))
     want = _state(moe, T)
@@ -230,8 +238,7 @@ def test_which_batches_stream(T, H, I, E, k, S, streams):
     for same in (False, True):      # all tokens on the same experts
         out = moe.forward(x, lg[:1].expand(T, E).contiguous() if same else lg).view(torch.int16).clone()
         moe.check()
-        kinds = set((np.concatenate([a for a in moe.read_trace() if len(a)])[:, 2] >> 24).tolist())
-        assert (12 in kinds, 6 in kinds) == (streams, not streams)
+        assert (12 in _kinds(moe), 6 in _kinds(moe)) == (streams, not streams)
         moe.set_schedule(pk.SCHED_SERIAL)
         assert torch.equal(moe.forward(x, lg[:1].expand(T, E).contiguous() if same else lg).view(torch.int16), out)
         moe.set_schedule(pk.SCHED_AUTO)
@@ -274,8 +281,7 @@ def test_routing_of_the_smallest_batches_at_the_edges(T, E, k):
             moe.set_schedule(sched)
             out = moe.forward(x, lg).view(torch.int16).clone()
             assert moe.status() == (0 if np.isfinite(inp.logits).all() else pk.ERR_NONFINITE_LOGITS)
-            kinds = set((np.concatenate([a for a in moe.read_trace() if len(a)])[:, 2] >> 24).tolist())
-            assert (12 in kinds) == (sched == pk.SCHED_AUTO)
+            assert (12 in _kinds(moe)) == (sched == pk.SCHED_AUTO)
             got.append((out, _state(moe, T)))
             if np.isfinite(inp.logits).all():
                 check_routing(moe, inp)
