@@ -2437,9 +2437,10 @@ weave_moe_kernel(const __grid_constant__ KParams p, const __grid_constant__ TmaM
         // A batch of at most 32 tokens under the phased plan: N = T columns cost a swapped tile's MMA no more than the
         // expert's few rows do (an instruction takes 48 cycles up to N = 64, and the weights set the pace), so the
         // gate/up tiles multiply ALL tokens, straight from x, and their epilogue keeps the expert's rows.  Nothing waits
-        // for the dispatch then (4-5 us).  T = 1 Qwen3-30B-shaped 46.8 -> 40.3 us, T = 7 DSv2-Lite-shaped 119.1 -> 112.7,
-        // T = 27 149.4 -> 146.7 (batches of up to 16 tokens mostly run on the streaming kernel now).  At T = 64 a launch by itself gains as much (199.9 -> 197.8) but under load the
-        // additional columns and rows cost power (202.8 -> 205.9 after half a second): hence the limit.
+        // for the dispatch then (4-5 us).  T = 27 Qwen3-30B-shaped 149.4 -> 146.7 us; of the batches of up to 16 tokens, which
+        // gained 6 us, only those of layers too wide for the streaming kernel still come here under AUTO.  At T = 64 a launch by
+        // itself gains as much (199.9 -> 197.8) but under load the additional columns and rows cost power (202.8 -> 205.9 after
+        // half a second): hence the limit.
         const bool direct = p.direct && plan_kind == kPlanPhased;
         const int budget = (mover && plan_kind != kPlanPhased) ? plan_steal : 0x7fffffff;
         const bool by_token = !two_roles && S.K == 1 && !ep;

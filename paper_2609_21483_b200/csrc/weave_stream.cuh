@@ -450,7 +450,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
             if (cta == ctas - 1 && tid == 64) {
                 p.ctl->plan_c = ctas; p.ctl->plan_K = 1; p.ctl->plan_steal = 0; p.ctl->plan_t = p.st_plan_t; p.ctl->plan_kind = kPlanPhased;
                 p.ctl->ep_x_local = 0u; p.ctl->ep_x_in = 0u; p.ctl->ep_x_in_uniq = 0u;
-                p.ctl->plan_nmb = A;      // (at most 32 rows per expert: one m-block and one row tile each)
+                p.ctl->plan_nmb = A;      // (at most 16 rows per expert: one m-block and one row tile each)
                 p.ctl->plan_ngemm = A * (p.nt0 + p.nt1);
             }
             // the dispatched rows, row r by CTA r mod N
