@@ -325,3 +325,38 @@ def test_a_captured_batch_keeps_its_plan_as_the_header_says():
         assert replayed == want[T] if T <= 16 else replayed > 10 * want[T]
     moe.check()
     moe.close()
+
+
+def test_smallest_batches_through_the_other_entry_points():
+    """forward_static, forward_host and forward_host_pipelined with batches on both sides of the largest streamed one, in turn,
+    plain and captured: the handle's bits."""
+    cfg = wl.MoEConfig("stream_entries", 1500, T=40, H=1024, I=512, E=24, k=3, S=1)
+    x, lg, gu, dn = to_dev(wl.make_inputs(cfg))
+    moe = pk.WeaveMoE(gu, dn, cfg.E, cfg.k, cfg.S, max_tokens=40)
+    cut = {T: (x[:T].contiguous(), lg[:T].contiguous()) for T in (1, 8, 9, 16, 17, 40)}
+    refs = {T: moe.forward(*c).view(torch.int16).clone() for T, c in cut.items()}
+    for T in (1, 40, 8, 8, 16, 17, 9, 1, 16, 40):
+        out = torch.zeros_like(cut[T][0])
+        pk.forward_static(*cut[T], gu, dn, cfg.E, cfg.k, cfg.S, out=out)
+        assert torch.equal(out.view(torch.int16), refs[T]), T
+    s, g, outs = torch.cuda.Stream(), torch.cuda.CUDAGraph(), {T: torch.zeros_like(c[0]) for T, c in cut.items()}
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        with torch.cuda.graph(g, stream=s):
+            for T, c in cut.items():
+                pk.forward_static(*c, gu, dn, cfg.E, cfg.k, cfg.S, out=outs[T])
+    for _ in range(2):
+        g.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(outs[T].view(torch.int16), refs[T]) for T in cut)
+    host = [(T, *[t.cpu().pin_memory() for t in cut[T]], torch.zeros_like(cut[T][0], device="cpu").pin_memory()) for T in (8, 40, 1, 16, 9, 17)]
+    for call in (moe.forward_host, moe.forward_host_pipelined):
+        for T, xh, lh, oh in host:
+            call(xh, lh, oh)
+        moe.host_wait()
+        torch.cuda.synchronize()
+        for T, xh, lh, oh in host:
+            assert torch.equal(oh.view(torch.int16), refs[T].cpu()), (call, T)
+            oh.zero_()
+    moe.check()
+    moe.close()
