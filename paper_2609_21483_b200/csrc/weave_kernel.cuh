@@ -182,10 +182,10 @@ constexpr int kMvBuf = kStageBytes;     // 32 KB
 constexpr int kCombWarps = 6;           // warps 2..7 reduce
 
 struct SmemTail {
+    uint64_t full[kStages], empty[kStages];      // (the streaming kernel's rows of x and h reach over these 128 bytes)
+    uint64_t tmem_full[2], tmem_empty[2];
     CtlSet *cs;                  // this launch's set of control words, and its arrays
     unsigned *fcnt, *xe_ready, *h_ready;
-    uint64_t full[kStages], empty[kStages];
-    uint64_t tmem_full[2], tmem_empty[2];
     uint64_t ti_full[kTinfo], ti_empty[kTinfo], ti_late[kTinfo];     // ti_late: the rows of a kTileLate tile are there
     uint64_t dv_full[kStages], dv_empty[kStages];   // dispatch: loader -> storer ring over the stage buffers
     uint64_t cb_full[kStages], cb_empty[kStages];   // combine: loader -> reducing warps

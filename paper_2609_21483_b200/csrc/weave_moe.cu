@@ -270,11 +270,12 @@ bool streams(const weave_moe *h, int T)
 {
     const weave_moe_config &c = h->cfg;
     if (T > kStTokens || h->mode != WEAVE_SCHED_AUTO || h->ep_size != 1) return false;
-    if ((size_t)T * st_pitch(std::max(c.hidden, c.ffn), true) > (size_t)(kStArea - (T > 8 ? kStWideRing : kStMinRing))) return false;
-    const size_t six = (size_t)(kStArea - kStGoodRing), expert = 6 * (size_t)c.hidden * (size_t)c.ffn;      // bytes
+    const size_t x_rows = (size_t)T * (size_t)(c.hidden * 2 + kStPad), h_rows = (size_t)T * ((size_t)c.ffn * 2 + kStPad);
+    if (std::max(x_rows, h_rows) > (size_t)(kStArea - (T > 8 ? kStWideRing : kStMinRing))) return false;
+    const size_t six = (size_t)(kStRowsEnd - kStGoodRing), expert = 6 * (size_t)c.hidden * (size_t)c.ffn;      // bytes
     const size_t any = (size_t)(std::min(c.num_experts, T * c.top_k) + c.num_shared), same = (size_t)(c.top_k + c.num_shared);
-    if (T * st_pitch(c.hidden, false) > six && any * expert > 1000000000u) return false;
-    if (T * st_pitch(c.ffn, false) > six && same * expert > 1600000000u) return false;
+    if (x_rows > six && any * expert > 1000000000u) return false;
+    if (h_rows > six && same * expert > 1600000000u) return false;
     return true;
 }
 

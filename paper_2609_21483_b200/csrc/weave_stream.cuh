@@ -36,13 +36,11 @@ constexpr int kStMinRing = 5 * kStMaxSlot, kStGoodRing = 6 * kStMaxSlot, kStWide
 constexpr int kStArea = kStages * kStageBytes + kEpiStageBytes;      // shared memory in front of the SmemTail: ring, then rows
 constexpr int kStUnitG = 8, kStUnitD = 16;        // columns of h / of y that one warp works on: 8 gate + 8 up rows, or 16 rows
 constexpr int kStWarps = 8;                       // ... so a tile has up to 8 units
-// Rows of x and h in shared memory must not start on the same bank.  Up to 8 tokens the 16-byte pieces of row r are swapped by
-// r & 7 in every 128 bytes: eight rows of 7168 columns and six ring slots then fill the area to the byte (DSv3-shaped T = 8: 795 us
-// with 16 bytes between the rows and five slots, 753 with six; the general kernel 750).  With more tokens, where that is never
-// the limit, there are 16 bytes between the rows (the swap costs the wide kernel 0.3 to 1 %).
-__host__ __device__ __forceinline__ constexpr uint32_t st_pitch(int cols, bool wide) { return (uint32_t)cols * 2u + (wide ? 16u : 0u); }
-template <bool kWide>
-__device__ __forceinline__ uint32_t st_piece(int row, int piece) { return (uint32_t)(kWide ? piece : piece ^ (row & 7)) * 16u; }
+constexpr int kStPad = 16;                        // bytes between two rows of x or h in shared memory (no bank conflicts)
+// The rows end over the general kernel's ring barriers: with these 128 bytes eight rows of 7168 columns leave six ring slots
+// (DSv3-shaped T = 8: 795 us with five, 753 with six; the general kernel 750).
+constexpr int kStRowsEnd = kStArea + 128;
+static_assert(offsetof(SmemTail, cs) >= kStRowsEnd - kStArea, "the general kernel's barriers only");
 
 // Boxes of 1 to 8 units: gate_up as [K/64][gate, up][row][64], down as [K/64][row][64], with one or two blocks of K.
 constexpr int kStMaps = kStWarps + kStWarps / 2;
@@ -185,7 +183,7 @@ __device__ __forceinline__ void stream_route(const KParams &p, StreamShared &X, 
 // False: a wait has failed, and the results are not to be used.  (The rest of the tile is run through; slots are handed back all the
 // same, to a producer that is on its way out.)
 struct StreamRing { uint32_t base, bytes; int slots, slot; uint32_t ph; };
-template <bool kWide, int KB>
+template <int KB>
 __device__ __forceinline__ bool stream_tile(const KParams &p, StreamShared &X, StreamRing &r, int K, bool works, uint32_t a_off, uint32_t blk,
                                             uint32_t b_row, float (&acc)[4])
 {
@@ -204,7 +202,7 @@ __device__ __forceinline__ bool stream_tile(const KParams &p, StreamShared &X, S
     };
     auto fetch = [&](int buf, int j, int s) {      // 16 of K
         ldmatrix_x4(a0 + (((2u * (uint32_t)s + kh) ^ sw) << 4), a[buf][s]);
-        if ((s & 1) == 0) ldmatrix_x4((kWide ? b_row + (uint32_t)(s * 32) : b_row ^ (uint32_t)(s * 32)) + (uint32_t)(j * 128), b[buf][s >> 1]);
+        if ((s & 1) == 0) ldmatrix_x4(b_row + (uint32_t)(j * 128 + s * 32), b[buf][s >> 1]);
     };
     auto free_slot = [&](int slot) {      // the slot's values are in registers
         __syncwarp();
@@ -287,7 +285,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
     StreamShared &X = *reinterpret_cast<StreamShared *>(reinterpret_cast<uint8_t *>(&S) + kStSharedAt);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cta = (int)blockIdx.x, ctas = (int)gridDim.x;
-    const uint32_t ring = smem_u32(stages), area_end = ring + (uint32_t)kStArea;
+    const uint32_t ring = smem_u32(stages), area_end = ring + (uint32_t)kStRowsEnd;
 
     auto now = [] { return kTrace ? globaltimer_ns() : 0ull; };
     const unsigned long long tk0 = now();
@@ -298,12 +296,12 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
         const int e = lane + 32 * i;
         lg[i] = warp < p.T && e < p.E ? __ldcg(p.logits + (size_t)warp * p.E + e) : 0.f;
     }
-    const uint32_t pitch_x = st_pitch(p.H, kWide), pitch_h = st_pitch(p.I, kWide), x_s = area_end - (uint32_t)p.T * pitch_x;
+    const uint32_t pitch_x = (uint32_t)p.H * 2u + kStPad, pitch_h = (uint32_t)p.I * 2u + kStPad, x_s = area_end - (uint32_t)p.T * pitch_x;
     if (warp > 0) {
         const int per_row = p.H >> 3;
         for (int t = 0; t < p.T; ++t)
             for (int c = tid - 32; c < per_row; c += kStThreads - 32)
-                cp_async_16(x_s + (uint32_t)t * pitch_x + st_piece<kWide>(t, c), p.x + (size_t)t * p.H + c * 8);
+                cp_async_16(x_s + (uint32_t)t * pitch_x + (uint32_t)(c * 16), p.x + (size_t)t * p.H + c * 8);
     }
     if (tid == 0) {
         const unsigned odd = (ld_relaxed_u32(&p.ctl->epoch) >> 16) & 1u;
@@ -365,8 +363,8 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
 #pragma unroll
     for (int w = 0; w < kMaxEE / 32; ++w) most = max(most, X.wmax[w]);
     int rows_h = 2 * most;
-    if (kStArea - rows_h * (int)pitch_h < kStFullRing) rows_h = most;
-    const int ring_bytes = (kStArea - max(p.T * (int)pitch_x, rows_h * (int)pitch_h)) & ~2047;
+    if (kStRowsEnd - rows_h * (int)pitch_h < kStFullRing) rows_h = most;
+    const int ring_bytes = (kStRowsEnd - max(p.T * (int)pitch_x, rows_h * (int)pitch_h)) & ~2047;
     const uint32_t h_s = ring + (uint32_t)ring_bytes;
     // The ring's slots, as large as this CTA's widest tiles want them: a block of K of five units and more, two of fewer.  (With
     // slots for eight units throughout, a share of ten in two tiles of five had 120 KB of the ring's 192 in flight.)
@@ -500,7 +498,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                         const __nv_bfloat16 *src = p.hbuf + (size_t)X.off[X.act[first]] * p.I;      // (the two experts' rows are neighbours)
                         for (int t = 0; t < n && ok; ++t)
                             for (int c = ctid; c < per_row; c += kStWarps * 32)
-                                cp_async_16(rows_s + (uint32_t)t * pitch + st_piece<kWide>(t, c), src + (size_t)t * p.I + c * 8);
+                                cp_async_16(rows_s + (uint32_t)t * pitch + (uint32_t)(c * 16), src + (size_t)t * p.I + c * 8);
                         cp_async_wait_all();
                         named_barrier_sync<2, kStWarps * 32>();
                     }
@@ -512,7 +510,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                     const int unit = later ? li : wk.at_c + li, e = X.act[a], n_e = X.rows(a), row0 = X.off[e];
                     const int i8 = lane & 7;
                     const int src_row = phase ? (a == second ? X.rows(first) : 0) + (i8 < n_e ? i8 : 0) : (int)__fns(X.mask[e], 0u, i8 < n_e ? i8 + 1 : 1);
-                    const uint32_t b_row = rows_s + (uint32_t)src_row * pitch + st_piece<kWide>(src_row, lane >> 3);
+                    const uint32_t b_row = rows_s + (uint32_t)src_row * pitch + (uint32_t)((lane >> 3) * 16);
                     const uint32_t half = (uint32_t)((lane >> 3) & 1);      // rows 8..15 of the warp's sixteen
                     const uint32_t part = later ? (uint32_t)(wk.w1 * kb * 2048) : 0u;
                     const uint32_t a_off = part + (phase ? (uint32_t)(li * 16 + i8 + 8 * (int)half) * 128u : (uint32_t)(li * 8 + i8) * 128u + half * (uint32_t)(wp * 1024));
@@ -521,12 +519,12 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                     float acc[kWide ? 2 : 1][4];
                     if (!kWide || n_e <= 8) {
                         const bool before = ok;
-                        ok = kb == 2 ? stream_tile<kWide, 2>(p, X, r, K, works, a_off, blk, b_row, acc[0]) : stream_tile<kWide, 1>(p, X, r, K, works, a_off, blk, b_row, acc[0]);
+                        ok = kb == 2 ? stream_tile<2>(p, X, r, K, works, a_off, blk, b_row, acc[0]) : stream_tile<1>(p, X, r, K, works, a_off, blk, b_row, acc[0]);
                         if (kWide) ok = ok && before;      // (there was no wait in a tile of no length to fail)
                     } else {
                         const int i16 = i8 + 8 < n_e ? i8 + 8 : 0;
                         const int src_row2 = phase ? (a == second ? X.rows(first) : 0) + i16 : (int)__fns(X.mask[e], 0u, i16 + 1);
-                        const uint32_t b_row2 = rows_s + (uint32_t)src_row2 * pitch + st_piece<kWide>(src_row2, lane >> 3);
+                        const uint32_t b_row2 = rows_s + (uint32_t)src_row2 * pitch + (uint32_t)((lane >> 3) * 16);
                         ok = (kb == 2 ? stream_tile_16<2>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])
                                       : stream_tile_16<1>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])) && ok;
                     }
