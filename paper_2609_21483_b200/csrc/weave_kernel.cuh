@@ -274,10 +274,9 @@ constexpr int kWaitLogCtas = 512, kWaitLogWarps = 16;      // (the streaming ker
 __device__ __noinline__ void note_failed_wait(int4 *log, int where, unsigned what, unsigned want, int how)
 {
     // the first failed wait of a warp is the one that tells where it stood; what it runs into afterwards,
-    // on its way out with the abort word set, is not recorded
-    if (!log || blockIdx.x >= kWaitLogCtas) return;
-    int4 *slot = log + blockIdx.x * kWaitLogWarps + (threadIdx.x >> 5);
-    if (slot->w == 0) *slot = make_int4(where, (int)what, (int)want, how);
+    // on its way out with the abort word set, is not recorded  (no log for grids of more than kWaitLogCtas)
+    int4 *slot = log + blockIdx.x * kWaitLogWarps + ((threadIdx.x >> 5) & (kWaitLogWarps - 1));
+    if (log && slot->w == 0) *slot = make_int4(where, (int)what, (int)want, how);
 }
 
 // Optional timeline: one 16-byte record {start ns, end ns, kind<<24 | id, extra} per event, per CTA.

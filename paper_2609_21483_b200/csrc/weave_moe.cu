@@ -535,7 +535,7 @@ int weave_moe_forward(weave_moe_t h, const void *x, const float *logits, void *o
     p.uniq_mask = reinterpret_cast<unsigned long long *>(ws + L.uniq_mask);
     p.trace = reinterpret_cast<uint4 *>(h->trace);
     p.trace_cap = h->trace_cap;
-    p.wait_log = reinterpret_cast<int4 *>(h->wait_log_dev);
+    p.wait_log = h->n_cta <= kWaitLogCtas ? reinterpret_cast<int4 *>(h->wait_log_dev) : nullptr;
     memcpy(p.die_mask, h->die_mask, sizeof(p.die_mask));
     p.lists_pt = tile_lists_from(h->two_dies, h->n_cta / 2, p.EE, c.ffn, p.nt1);
 

@@ -308,7 +308,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
         S.cs = reinterpret_cast<CtlSet *>(p.sets + (odd ? ctl_set_bytes(p.nmb_max) : 0));
         S.h_ready = reinterpret_cast<unsigned *>(S.cs + 1) + kFine * kMaxEE + p.nmb_max;
         X.failed = 0;
-        S.trace_n = 0;
+        if (kTrace) S.trace_n = 0;
     }
     if (warp == 14 && lane < kStMaxSlots) { mbar_init(&X.full[lane], 1); mbar_init(&X.empty[lane], kStWarps); }
     if (warp == 14 && lane >= 30) { mbar_init(&X.done[lane - 30], kStWarps); mbar_init(&X.freed[lane - 30], 1); }
@@ -470,9 +470,9 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
             __syncwarp();
             if (lane == 0) red_release_add_u32(&S.cs->y_done[0], 1u);
         } else {
-            // ---------------- the products.  `ok` is the warp's at the start of a tile: once a wait of it has failed it only goes on
-            // to meet the others at the barriers around a reload of h (the wide kernel through tiles of no length, as a jump over
-            // them costs it 1 to 1.5 %: T = 16 Qwen3-30B-shaped 129.5 -> 131.0 us; the narrow one loses 0.8 % by them).
+            // ---------------- the products.  Once a wait of a warp has failed (`ok`: the warp's at the start of a tile) it stores and
+            // hands over nothing; it goes through the tiles that are left as ones of no length, to meet the others at the barriers
+            // around a reload of h.  (A jump over them costs 8 experts, T = 2 15.2 -> 15.9 us; the wide kernel 1 to 1.5 %.)
             const int wi = warp - 8;
             int tile = 0;
             StreamRing r = {ring, (uint32_t)(slot_units * 2048), slots, 0, 0u};
@@ -489,10 +489,8 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                         // the next rows of h, once all of them are there and nobody reads what they replace
                         first = wk.at_a; second = two ? wk.at_a + 1 : -1;
                         named_barrier_sync<2, kStWarps * 32>();
-                        if (lane == 0 && ok) {
-                            ok = flag_wait_ge(&S.h_ready[first], (unsigned)(p.I / kStUnitG), p, 62);
-                            if (two && ok) ok = flag_wait_ge(&S.h_ready[second], (unsigned)(p.I / kStUnitG), p, 62);
-                        }
+                        if (lane == 0 && ok) ok = flag_wait_ge(&S.h_ready[first], (unsigned)(p.I / kStUnitG), p, 62);
+                        if (lane == 0 && ok && two) ok = flag_wait_ge(&S.h_ready[second], (unsigned)(p.I / kStUnitG), p, 62);
                         ok = __all_sync(0xffffffffu, ok);
                         const int per_row = p.I >> 3, ctid = tid - 256, n = X.rows(first) + (two ? X.rows(second) : 0);
                         const __nv_bfloat16 *src = p.hbuf + (size_t)X.off[X.act[first]] * p.I;      // (the two experts' rows are neighbours)
@@ -502,7 +500,6 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                         cp_async_wait_all();
                         named_barrier_sync<2, kStWarps * 32>();
                     }
-                    if (!kWide && !ok) continue;
                     const unsigned long long tt = now();
                     // this warp's unit: unit li of the ones that the tile has of active expert a
                     const bool works = wi < wk.w, later = works && wi >= wk.w1;
@@ -515,20 +512,17 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                     const uint32_t part = later ? (uint32_t)(wk.w1 * kb * 2048) : 0u;
                     const uint32_t a_off = part + (phase ? (uint32_t)(li * 16 + i8 + 8 * (int)half) * 128u : (uint32_t)(li * 8 + i8) * 128u + half * (uint32_t)(wp * 1024));
                     const uint32_t blk = (uint32_t)(wp * 2048);
-                    const int K = !kWide || ok ? (phase ? p.I : p.H) : 0;
+                    const int K = ok ? (phase ? p.I : p.H) : 0;
                     float acc[kWide ? 2 : 1][4];
-                    if (!kWide || n_e <= 8) {
-                        const bool before = ok;
-                        ok = kb == 2 ? stream_tile<2>(p, X, r, K, works, a_off, blk, b_row, acc[0]) : stream_tile<1>(p, X, r, K, works, a_off, blk, b_row, acc[0]);
-                        if (kWide) ok = ok && before;      // (there was no wait in a tile of no length to fail)
-                    } else {
+                    if (!kWide || n_e <= 8)
+                        ok = (kb == 2 ? stream_tile<2>(p, X, r, K, works, a_off, blk, b_row, acc[0]) : stream_tile<1>(p, X, r, K, works, a_off, blk, b_row, acc[0])) && ok;
+                    else {
                         const int i16 = i8 + 8 < n_e ? i8 + 8 : 0;
                         const int src_row2 = phase ? (a == second ? X.rows(first) : 0) + i16 : (int)__fns(X.mask[e], 0u, i16 + 1);
                         const uint32_t b_row2 = rows_s + (uint32_t)src_row2 * pitch + (uint32_t)((lane >> 3) * 16);
                         ok = (kb == 2 ? stream_tile_16<2>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])
                                       : stream_tile_16<1>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])) && ok;
                     }
-                    if (lane == 0 && tile >= 2) ok = mbar_wait(&X.freed[tile & 1], (uint32_t)(((tile >> 1) - 1) & 1), p, 65) && ok;
                     ok = __all_sync(0xffffffffu, ok);
                     if (works && ok) {
                         const int col = (phase ? unit * kStUnitD : unit * kStUnitG) + (lane >> 2);
@@ -545,7 +539,10 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                         }
                     }
                     __syncwarp();
-                    if (lane == 0 && ok) mbar_arrive(&X.done[tile & 1]);
+                    if (lane == 0 && ok) {
+                        if (tile >= 2) ok = mbar_wait(&X.freed[tile & 1], (uint32_t)(((tile >> 1) - 1) & 1), p, 65);
+                        if (ok) mbar_arrive(&X.done[tile & 1]);
+                    }
                     if (kTrace && lane == 0 && ok && wi == 0) trace_ev(p, S, kEvStream, (unsigned)(phase << 16 | wk.w), tt, now(), (unsigned)(tt - th));
                 }
             }
