@@ -38,7 +38,7 @@ constexpr int kStUnitG = 8, kStUnitD = 16;        // columns of h / of y that on
 constexpr int kStWarps = 8;                       // ... so a tile has up to 8 units
 constexpr int kStPad = 16;                        // bytes between two rows of x or h in shared memory (no bank conflicts)
 // The rows end over the general kernel's ring barriers: with these 128 bytes eight rows of 7168 columns leave six ring slots
-// (DSv3-shaped T = 8: 795 us with five, 753 with six; the general kernel 750).
+// (DSv3-shaped T = 8: 826 us with five, 783 with six; the general kernel 776).
 constexpr int kStRowsEnd = kStArea + 128;
 static_assert(offsetof(SmemTail, cs) >= kStRowsEnd - kStArea, "the general kernel's barriers only");
 
