@@ -523,6 +523,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                         ok = (kb == 2 ? stream_tile_16<2>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])
                                       : stream_tile_16<1>(p, X, r, K, works, a_off, blk, b_row, b_row2, acc[0], acc[kWide])) && ok;
                     }
+                    if (lane == 0 && ok && tile >= 2) ok = mbar_wait(&X.freed[tile & 1], (uint32_t)(((tile >> 1) - 1) & 1), p, 65);
                     ok = __all_sync(0xffffffffu, ok);
                     if (works && ok) {
                         const int col = (phase ? unit * kStUnitD : unit * kStUnitG) + (lane >> 2);
@@ -539,10 +540,7 @@ weave_stream_kernel(const __grid_constant__ KParams p, const __grid_constant__ S
                         }
                     }
                     __syncwarp();
-                    if (lane == 0 && ok) {
-                        if (tile >= 2) ok = mbar_wait(&X.freed[tile & 1], (uint32_t)(((tile >> 1) - 1) & 1), p, 65);
-                        if (ok) mbar_arrive(&X.done[tile & 1]);
-                    }
+                    if (lane == 0 && ok) mbar_arrive(&X.done[tile & 1]);
                     if (kTrace && lane == 0 && ok && wi == 0) trace_ev(p, S, kEvStream, (unsigned)(phase << 16 | wk.w), tt, now(), (unsigned)(tt - th));
                 }
             }

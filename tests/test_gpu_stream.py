@@ -360,3 +360,33 @@ def test_smallest_batches_through_the_other_entry_points():
             oh.zero_()
     moe.check()
     moe.close()
+
+
+@pytest.mark.parametrize("T", [8, 16])
+def test_an_abort_in_the_middle_of_a_long_stream(T):
+    """Four CTAs take milliseconds for the layer.  The one that waits for the withheld h gives up after 1 ms while the others are
+    among their down tiles: their releasing and product warps are cut short at whatever they wait for, and all of them
+    leave together."""
+    cfg = wl.MoEConfig(f"stream_abort_{T}", 1510, T=T, H=2048, I=1408, E=64, k=8)
+    inp = wl.make_inputs(cfg)
+    x, lg, gu, dn = to_dev(inp)
+    moe = pk.WeaveMoE(gu, dn, cfg.E, cfg.k, max_tokens=T)
+    ref = moe.forward(x, lg).view(torch.int16).clone()
+    moe.check()
+    active = int((moe.routing(T)["counts"] > 0).sum())
+    moe.set_sm_count(4)
+    for which in (0, active // 4, active // 2, active - 1):
+        out = torch.full_like(x, -3.0)
+        moe.set_timeout_ms(1)
+        moe.debug_withhold_flag(which)
+        moe.forward(x, lg, out)
+        moe.debug_withhold_flag(-1)
+        moe.set_timeout_ms(4000)
+        assert moe.status() == pk.ERR_TIMEOUT
+        assert (out == -3.0).all() and 60 <= moe.last_timeout_where() <= 65
+        assert torch.equal(moe.forward(x, lg).view(torch.int16), ref)
+        moe.check()
+    moe.set_sm_count(moe.geometry()["n_sm"])
+    assert torch.equal(moe.forward(x, lg).view(torch.int16), ref)
+    moe.check()
+    moe.close()
